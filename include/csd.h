@@ -158,7 +158,7 @@ csd_status csd_tree_accept_greedy(const float* target_logits_dev, const int32_t*
 /* Prompt prefill: the model takes the input tokens in one run (Section 2).  Appends n tokens
  * (any n >= 1 with kv_len + n <= max_seq) at positions kv_len .. kv_len+n-1 to the cache of every
  * layer and produces no logits.  Models whose layer matrices are large enough for the tensor-core
- * kernels go through the weights once per 128 tokens (wide blocks, two bf16 terms per fp32
+ * kernels go through the weights once per 1024 tokens (wide blocks, two bf16 terms per fp32
  * activation); the rest, and a remainder of at most max_rows tokens, go through the review
  * kernels.  arch 1: decoder tokens, after csd_encoder_forward. */
 csd_status csd_prefill(csd_model* m, const int32_t* tokens_dev, int n, int kv_len, void* stream);

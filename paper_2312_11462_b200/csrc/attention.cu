@@ -11,6 +11,7 @@
 // Rows see keys [0, n_keys + r) when causal, all n_keys otherwise (cross-attention, encoder).
 #include <cooperative_groups.h>
 #include "attention.cuh"
+#include "gemm_tc.cuh"
 #include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
@@ -845,7 +846,7 @@ csd_status launch_attention(const AttnArgs& a, cudaStream_t st) {
 }
 
 static csd_status launch_attention_rows(const AttnArgs& a, cudaStream_t st) {
-    if (a.k_new || a.tree_mask || a.out_xs || a.m > 128) return CSD_ERR_INVALID_ARG;   // 128: the widest block the model driver forms
+    if (a.k_new || a.tree_mask || a.out_xs || a.m > CSD_WIDE_ROWS) return CSD_ERR_INVALID_ARG;
     if ((a.Dh == 64 || a.Dh == 128) && !g_attn_cuda_cores) return launch_attention_block(a, 32, st);
     for (int r0 = 0; r0 < a.m; r0 += MAXM) {
         AttnArgs s = a;

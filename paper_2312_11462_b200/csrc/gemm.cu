@@ -326,7 +326,7 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual) {
     return align_up(worst, 256);
 }
 
-int linear_ticket_count(int N) { return N + 1; }   // one ticket per row group, at least one row each
+int linear_ticket_count(int N) { return N + 1; }   // one ticket per row group, at least one row each (the wide kernel needs fewer)
 
 bool linear_uses_tensor_cores(int m, int N, int K, bool dual) {
     const int path = gemm_path();
@@ -400,12 +400,12 @@ struct LinearWs { size_t tickets, partial, xs, ssq, total; };
 static LinearWs linear_ws(int m, int N, int K) {
     LinearWs w;
     size_t off = 0;
-    const int rows = m > CSD_MAX_ROWS ? CSD_WIDE_ROWS : CSD_MAX_ROWS;
+    const int rows = m > CSD_MAX_ROWS ? CSD_LINEAR_ROWS : CSD_MAX_ROWS;
     w.tickets = off; off += align_up((size_t)linear_ticket_count(N) * sizeof(unsigned), 256);
     w.partial = off;
     {
         size_t pb = linear_scratch_bytes(m > CSD_MAX_ROWS ? CSD_MAX_ROWS : m, N, K, false);
-        if (m > CSD_MAX_ROWS && wide_partial_bytes(m, N, K, false) > pb) pb = wide_partial_bytes(m, N, K, false);
+        if (m > CSD_MAX_ROWS && wide_partial_bytes(m) > pb) pb = wide_partial_bytes(m);
         off += pb;
     }
     w.xs = off;      off += align_up((size_t)3 * rows * K * 2, 256);
@@ -415,7 +415,7 @@ static LinearWs linear_ws(int m, int N, int K) {
 }
 
 extern "C" size_t csd_linear_workspace_bytes(int m, int N, int K) {
-    if (m < 1 || m > CSD_WIDE_ROWS || N < 1 || K < 8) return 0;
+    if (m < 1 || m > CSD_LINEAR_ROWS || N < 1 || K < 8) return 0;
     return linear_ws(m, N, K).total;
 }
 
@@ -423,7 +423,7 @@ extern "C" size_t csd_linear_workspace_bytes(int m, int N, int K) {
 // leaves the tickets zero again, so one cudaMemset after allocation is enough.
 extern "C" csd_status csd_linear(const void* W_bf16_dev, int N, int K, const float* X_dev, int m, float* Y_dev,
                                  void* workspace_dev, size_t workspace_bytes, void* stream) {
-    if (m < 1 || m > CSD_WIDE_ROWS || N < 1 || K < 8 || (K & 7)) return CSD_ERR_INVALID_ARG;
+    if (m < 1 || m > CSD_LINEAR_ROWS || N < 1 || K < 8 || (K & 7)) return CSD_ERR_INVALID_ARG;
     if (!W_bf16_dev || !X_dev || !Y_dev || !workspace_dev) return CSD_ERR_INVALID_ARG;
     const LinearWs w = linear_ws(m, N, K);
     if (workspace_bytes < w.total) return CSD_ERR_CAPACITY;
@@ -436,6 +436,7 @@ extern "C" csd_status csd_linear(const void* W_bf16_dev, int N, int K, const flo
         WideArgs wa;
         wa.W = (const __nv_bfloat16*)W_bf16_dev; wa.N = N; wa.K = K; wa.m = m; wa.xs = (const __nv_bfloat16*)(ws + w.xs);
         wa.Y = Y_dev; wa.ldy = N; wa.epilogue = EPI_STORE; wa.partial = (float*)(ws + w.partial);
+        wa.tickets = (unsigned*)(ws + w.tickets);
         return launch_linear_wide(wa, (cudaStream_t)stream);
     }
     LinearArgs a;

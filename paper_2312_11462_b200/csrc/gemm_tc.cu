@@ -169,27 +169,7 @@ __device__ __forceinline__ float tc_gelu(float x) {
 }
 __device__ __forceinline__ float tc_silu(float x) { return x / (1.f + expf(-x)); }
 
-// Units of work are (tile of 128 output columns, 64-wide K block) pairs in tile-major order; CTA c
-// owns the contiguous range [unit_begin(c), unit_begin(c+1)), so every SM streams the same
-// number of weight bytes whatever N and K are.
-// (units * ctas fits 32 bits: the planner refuses shapes where it would not)
-__device__ __forceinline__ unsigned unit_begin(unsigned c, unsigned units, unsigned ctas) { return c * units / ctas; }
-__device__ __forceinline__ int cta_of_unit(unsigned u, unsigned units, unsigned ctas) {
-    unsigned c = ((u + 1) * ctas - 1) / units;
-    while (c + 1 < ctas && unit_begin(c + 1, units, ctas) <= u) ++c;
-    while (c > 0 && unit_begin(c, units, ctas) > u) --c;
-    return (int)c;
-}
-
 // ---- distributed shared memory (cluster split) ---------------------------------------------------
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
 __device__ __forceinline__ void remote_store(uint32_t cluster_addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
@@ -202,12 +182,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
         if (ok) return true;
     }
     return false;
-}
-
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
 }
 
 template <int M, bool DUAL>

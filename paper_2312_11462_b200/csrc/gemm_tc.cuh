@@ -18,7 +18,8 @@ int rs_box_rows(int m, int N, int K, bool dual);       // weight rows per CTA an
 csd_status launch_linear_rs(const LinearArgs& a, cudaStream_t st);
 
 // wide-block variant (gemm_wide.cu): up to CSD_WIDE_ROWS rows per pass, two bf16 terms per value
-constexpr int CSD_WIDE_ROWS = 128;
+constexpr int CSD_WIDE_ROWS = 1024;
+constexpr int CSD_LINEAR_ROWS = 128;     // most rows csd_linear takes
 struct WideArgs {
     const __nv_bfloat16* W = nullptr;    // [N, K] row-major
     const __nv_bfloat16* W2 = nullptr;   // gated feed-forward only
@@ -27,18 +28,20 @@ struct WideArgs {
     const float* ssq = nullptr;          // with an RMS norm: pieces [ssq_cnt][m] of the rows' sums of squares
     int ssq_cnt = 0;
     float eps = 0.f;
-    float* Y = nullptr;                  // [m, ldy]
+    float* Y = nullptr;                  // [m, ldy]; may be null for the gated pair with out_xs
     int ldy = 0, epilogue = EPI_STORE;
     __nv_bfloat16* out_xs = nullptr;     // optional: (Y * out_gain) in two-term form [2][mpad][out_ld] for the next wide GEMM
     int out_ld = 0;
     const __nv_bfloat16* out_gain = nullptr;
     float* out_ssq = nullptr;            // optional: [wide_ssq_pieces(...)][m] pieces of the sums of squares of the rows of Y
-    float* partial = nullptr;            // scratch of wide_partial_bytes(...) for K-partitioned launches (optional)
+    float* partial = nullptr;            // scratch of wide_partial_bytes(m) for partial sums
+    unsigned* tickets = nullptr;         // zero-initialised, wide_ticket_count(m, N) entries
 };
 bool wide_supported(int m, int N, int K, bool dual);
 int wide_ssq_pieces(int m, int N, int K, bool dual);
 int wide_ssq_capacity(int N);
-size_t wide_partial_bytes(int m, int N, int K, bool dual);
+size_t wide_partial_bytes(int m);
+int wide_ticket_count(int m, int N);
 int wide_split_pieces(int K);
 csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_bfloat16* gain, __nv_bfloat16* xs,
                              float* ssq, cudaStream_t st);

@@ -1,125 +1,137 @@
-// Wide-block variant of the tensor-core GEMM  Y[m, N] = X[m, K] . W[N, K]^T  for up to 128 rows:
-// the prompt prefill and the encoder pass, where the model takes many tokens in one run
-// (Section 2) and the weights should stream once per 128 tokens instead of once per 17.
+// Wide-block variant of the tensor-core GEMM  Y[m, N] = X[m, K] . W[N, K]^T  for up to
+// CSD_WIDE_ROWS rows: the prompt prefill and the encoder pass, where the model takes many tokens in
+// one run (Section 2) and the weights should stream once per pass.
 //
-// Same plan as the row-range kernel (gemm_rs.cu): every CTA owns contiguous ranges of at most 128
-// weight rows over the whole K extent, nothing is shared between CTAs.  The rows of X are the
-// narrow operand of tcgen05.mma with up to 256 columns: each fp32 value enters as TWO bf16 terms
-// x = hi + lo (16 mantissa bits, relative error 2^-17, the size of the tensor cores' own fp32
-// accumulation error), laid out as [2][mpad][K] with mpad = m rounded up to 16, so one TMA box of
-// 2*mpad rows brings both terms of a 64-wide K block.  With 128 rows a stage moves 32 KB of X for
-// 11 to 16 KB of weights, all CTAs re-read X from L2, and the kernel is bound by what an SM can
-// take in (about 63 GB/s), not by HBM; it still is one pass over the weights instead of eight.
-// One CTA per SM (the ring takes most of the shared memory).
+// Each fp32 value of X enters as TWO bf16 terms x = hi + lo (16 mantissa bits, relative error
+// 2^-17), laid out as [2][mpad][K].  A tile is 256 weight rows x nt tokens (the gated pair: 256 rows
+// of both matrices x nt tokens; nt <= 256, <= 128 for the pair) and belongs to a PAIR of CTAs on
+// neighbouring SMs: tcgen05.mma with cta_group::2, 128 weight rows and half of the tokens staged by
+// each CTA, both terms accumulated into the same fp32 columns.
 //
-// Epilogue per output column (one thread per weight row): hi + lo sums, rms factor, residual add or
-// gated activation, optional two-term split and sum-of-squares pieces for the next wide GEMM.
-// Every mbarrier wait is bounded; on a time-out the CTA records CSD_ERR_TIMEOUT, stops, frees its
-// tensor memory, returns.
+// What bounds it: the bytes an SM takes in (about 70 GB/s) and the tensor pipe, nearly level.  A full tile takes
+// 48 KB per 1024 tensor clocks and SM; at 1024 rows, N 12288, K 4096 the copies alone need 114 us, the MMAs alone
+// 89 us, the kernel 157 us (1.29 PFLOP/s of two-term products, 77 % of the measured one-term cuBLAS rate; the
+// earlier kernel, one CTA per 84 weight rows and 128 tokens, took in 32 KB of token terms for every 11 KB of
+// weights: 8 x 46 us).  At 128 rows both kernels need 40 us; below, the weight stream bounds.
+//
+// fp32 accumulation.  The tensor core loses a little with every add of a long chain, so after WG_DRAIN
+// K blocks (64 adds) the accumulator set is added into fp32 registers of the epilogue warps while
+// the MMAs continue on the other set: shorter chains than in the earlier kernel (256 to 700
+// adds), and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to 11008:
+// 2.7e-6 (earlier 5.0e-6), which is what the two-term form itself leaves.
+//
+// Roles inside a CTA (384 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 of the pair's first CTA
+// issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
+// tokens) and finish tiles; they hold 128 accumulators each, hence the register split.  Every
+// mbarrier wait is bounded; on a time-out the CTA records CSD_ERR_TIMEOUT, stops, frees its tensor
+// memory, returns.
 #include "gemm_tc.cuh"
 #include "tc_common.cuh"
 
 namespace csd {
 
-constexpr size_t WG_SMEM_MAX = 200 * 1024;
-constexpr int WG_MAX_STAGES = 8;
-constexpr int WG_THREADS = 320;              // TMA warp, MMA warp, eight epilogue warps (two per tensor-memory quadrant)
-
-struct WgPlan {
-    int mpad, npad, grid, T, V, box, rows8, ks, nkb, nks, stages, qp, chunks, tmem_cols, pk;
-    size_t stage, smem;
-};
+constexpr size_t WG_SMEM_MAX = 227 * 1024;
+constexpr int WG_MAX_STAGES = 10;
+constexpr int WG_THREADS = 384;              // one control warpgroup, two epilogue warpgroups
+// Registers a thread: 168 at launch (65536 / 384); 128 x 56 + 256 x 224 = 384 x 168.  Without the split the
+// accumulators spill.
+constexpr int WG_REGS_CTL = 56, WG_REGS_EPI = 224;
+constexpr int WG_ROWS = 256;                 // weight rows of a pair's tile
+constexpr int WG_DRAIN = 8;                  // K blocks per accumulator set before it is added into registers
+constexpr int WG_SET = 256;                  // tensor-memory columns of a set
 
 struct __align__(8) WgCtrl {
     uint64_t full[WG_MAX_STAGES], empty[WG_MAX_STAGES], acc_full[2], acc_empty[2];
+    uint64_t part_full;                      // parked partial sums have landed in the ring
     uint32_t tmem_base;
     int abort_flag;
-    float scale[CSD_WIDE_ROWS];
+    float scale[256];                        // rms-norm factors of the tile's tokens
+};
+// Epilogue staging: per token half two buffers of 16 tokens x 128 weight rows.  An accumulator thread owns one
+// weight row, memory wants the rows of a token side by side: through these buffers a warp gets 4 whole
+// 128-row stretches per chunk and moves 16 bytes per lane.
+constexpr size_t WG_STAGING = 2 * 2 * 16 * TILE_N * sizeof(float);
+
+// How a launch is divided.  tiles = row tiles x token tiles, tokens fastest, so that pairs running at the
+// same time share weight rows in L2.  Three ways:
+//   planes   few tiles (pairs / tiles >= 3): every tile goes to pk pairs that share its K range, each writes
+//            an fp32 plane and wide_reduce_kernel adds the planes and runs the epilogue;
+//   whole    pair c takes whole tiles (no partial sums) where that leaves little of the last round empty;
+//   shares   otherwise the (tile, K block) units are dealt out in equal contiguous shares; a tile cut by a
+//            share boundary is finished by its first contributor from the partial sums the later
+//            ones parked before they went on (the same scheme, and the same order of waiting, as in
+//            gemm_tc.cu).
+// whole or shares: by the K blocks of the busiest pair, a fix-up (park, fetch, add: about 5 us) counted as 8 blocks
+// of a full tile (0.55 us each).
+struct WgPlan {
+    int mpad, nt, ntok, tiles, nkb, pairs, pk, gran, stages;
+    size_t stage, smem;
 };
 
-// K partitions: a matrix with few rows per CTA (the projections back to d_model) makes every CTA
-// re-read all of X for a sliver of weights.  Cutting K in `pk` parts and the rows in grid / pk
-// ranges of up to 128 divides the X traffic per CTA by pk; the pk partial results go to planes of
-// a scratch buffer and a small kernel adds them (and runs the epilogue).  Only without an input
-// norm, for single matrices with N a multiple of 8.
 int wide_split_pieces(int K) { return (K + 1023) / 1024; }
 
-int wide_pk(int m, int N, int K, bool dual) {
-    (void)m;
-    if (dual || (N & 7)) return 1;
-    const int sms = tc_sm_count();
-    if ((N + sms - 1) / sms >= 64 || K < 2048) return 1;
-    int pk = sms / ((N + TILE_N - 1) / TILE_N);
-    if (pk > 4) pk = 4;
-    return pk < 2 ? 1 : pk;
-}
-
-static WgPlan wg_plan(int m, int N, int K, bool dual, int pk = 1) {
+static WgPlan wg_plan(int m, int N, int K, bool dual) {
     WgPlan p{};
+    const int P = tc_sm_count() / 2, most = dual ? 128 : 256;
     p.mpad = (m + 15) & ~15;
-    p.npad = 2 * p.mpad;
-    p.pk = pk;
-    p.grid = tc_sm_count();
-    const int per = (N + p.grid - 1) / p.grid;
-    p.T = (per + TILE_N - 1) / TILE_N;
-    p.V = p.grid * p.T;
-    if (pk > 1) { p.T = 1; p.V = p.grid / pk; p.grid = p.V * pk; }
-    p.box = (N + p.V - 1) / p.V;
-    p.rows8 = (p.box + 7) & ~7;
-    p.qp = (p.box + 31) / 32;
+    p.ntok = (m + most - 1) / most;
+    p.nt = ((m + p.ntok - 1) / p.ntok + 31) & ~31;
+    p.tiles = ((N + WG_ROWS - 1) / WG_ROWS) * p.ntok;
     p.nkb = (K + KB - 1) / KB;
-    const size_t wblk = (size_t)p.rows8 * 128, xb = (size_t)p.npad * 128;
-    const size_t kblk = (dual ? 2 : 1) * wblk + xb;
-    p.ks = kblk <= 24 * 1024 && p.nkb >= 2 ? 2 : 1;
-    p.nks = (p.nkb + p.ks - 1) / p.ks;
-    p.stage = (size_t)p.ks * kblk;
-    // accumulator chunks of about 16 K blocks, as many as tensor memory holds (256 columns when the
-    // accumulators fit them, all 512 otherwise), double-buffered when a CTA has two ranges
-    const int acc_cols = p.npad * (dual ? 2 : 1), bufs = p.T > 1 ? 2 : 1;
-    int chunks = (p.nkb + 15) / 16;
-    const int room = (acc_cols * bufs <= 256 ? 256 : 512) / (acc_cols * bufs);
-    if (chunks > room) chunks = room;
-    if (chunks > p.nks / pk) chunks = p.nks / pk;
-    p.chunks = chunks;                       // 0: the accumulators do not fit tensor memory
-    p.tmem_cols = 32;
-    while (p.tmem_cols < acc_cols * bufs * (chunks > 0 ? chunks : 1)) p.tmem_cols *= 2;
-    const size_t reach = 16384 > wblk + xb ? 16384 - wblk - xb : 0;
-    size_t tail = (sizeof(WgCtrl) + 127) & ~(size_t)127;
-    if (tail < reach) tail = reach;
-    p.stages = (int)((WG_SMEM_MAX - 1024 - tail) / p.stage);
+    p.stage = (size_t)STAGE_BYTES * (dual ? 2 : 1) + (size_t)p.nt * 128;
+    p.stages = (int)((WG_SMEM_MAX - 1024 - WG_STAGING - sizeof(WgCtrl)) / p.stage);
     if (p.stages > WG_MAX_STAGES) p.stages = WG_MAX_STAGES;
-    p.smem = (size_t)p.stages * p.stage + tail + 1024;
+    p.smem = (size_t)p.stages * p.stage + 1024 + WG_STAGING + sizeof(WgCtrl);
+    p.pk = 1; p.gran = 1;
+    const int ratio = P / p.tiles;
+    if (!dual && (N & 7) == 0 && ratio >= 3 && p.nkb >= 16) {
+        p.pk = ratio < 8 ? ratio : 8;
+        if (p.pk > p.nkb / 8) p.pk = p.nkb / 8;
+        p.pairs = p.tiles * p.pk;
+        return p;
+    }
+    const double kb = (double)p.nkb, fix = 8.0;
+    const double whole = (double)((p.tiles + P - 1) / P) * kb, shares = (double)p.tiles * kb / P + fix;
+    if (whole <= shares) {
+        p.gran = p.nkb;
+        p.pairs = p.tiles < P ? p.tiles : P;
+    } else {
+        const long long units = (long long)p.tiles * p.nkb;
+        p.pairs = units / 4 < P ? (int)(units / 4 > 0 ? units / 4 : 1) : P;
+    }
     return p;
 }
 
 bool wide_supported(int m, int N, int K, bool dual) {
+    (void)dual;
     if (m < 1 || m > CSD_WIDE_ROWS || N < 1 || K < 64 || (K & 7)) return false;
     if ((long long)N * K < (1LL << 20)) return false;
-    const WgPlan p = wg_plan(m, N, K, dual);
-    return p.stages >= 2 && p.box >= 8 && p.chunks >= 1 && p.tmem_cols <= 512;
+    const long long tiles = (long long)((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128);
+    return tiles * ((K + KB - 1) / KB) * (tc_sm_count() + 1) < (1LL << 31);
 }
 
 int wide_ssq_pieces(int m, int N, int K, bool dual) {
-    if (wide_pk(m, N, K, dual) > 1) return wide_split_pieces(N);      // written by the kernel that adds the partial planes
     const WgPlan p = wg_plan(m, N, K, dual);
-    return p.V * p.qp;
-}
-size_t wide_partial_bytes(int m, int N, int K, bool dual) {
-    const int pk = wide_pk(m, N, K, dual);
-    return pk > 1 ? align_up((size_t)pk * m * N * sizeof(float), 256) : 0;
+    return p.pk > 1 ? wide_split_pieces(N) : 2 * ((N + WG_ROWS - 1) / WG_ROWS);
 }
 int wide_ssq_capacity(int N) {
-    const int sms = tc_sm_count(), per = (N + sms - 1) / sms, T = (per + 127) / 128;
-    const int a = sms * T * 4, b = wide_split_pieces(N) + 1;     // GEMM epilogue pieces, split-kernel pieces
+    const int a = 2 * ((N + WG_ROWS - 1) / WG_ROWS), b = wide_split_pieces(N);
     return a > b ? a : b;
 }
+// planes of at most one tile per pair, or one parked tile (of both matrices of a gated pair) per pair
+size_t wide_partial_bytes(int m) {
+    const int cols = m < 128 ? 2 * ((m + 31) & ~31) : 256;
+    return (size_t)(tc_sm_count() / 2) * WG_ROWS * cols * sizeof(float);
+}
+int wide_ticket_count(int m, int N) { return 2 * ((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128); }
 
 struct WgParams {
-    float* Y; int* status;
+    float* Y; float* partial; unsigned* tickets; int* status;
     const float* ssq_in; int ssq_cnt;
     __nv_bfloat16* out_xs; const __nv_bfloat16* out_gain; float* out_ssq; int out_ld;
-    int m, mpad, npad, N, K, ldy, nks, ks, T, V, box, rows8, stages, qp, chunks, tmem_cols, epilogue, pk;
-    size_t plane;                       // floats between the partial planes of a K-partitioned launch
+    int m, mpad, nt, ntok, tiles, nkb, pk, gran, N, K, ldy, stages, epilogue;
+    int vec_y;                          // Y takes 16-byte accesses
+    size_t plane;                       // floats between the partial planes (pk > 1)
     float eps;
 };
 
@@ -134,211 +146,386 @@ __device__ __forceinline__ void split2f(float x, uint16_t& hi, uint16_t& lo) {
     lo = float_to_bf16_bits(x - bf16_bits_to_float(hi));
 }
 
+// ---- the pair's forms of the tensor-core instructions ---------------------------------------------
+// a copy into this CTA's shared memory that completes on the barrier at cluster address `bar`
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
+                 ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
+    asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
+}
+// arrives at the barrier of this offset in both CTAs once the MMAs issued before have finished
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+// 1D copy from global into this CTA's shared memory (16-byte aligned on both sides, a multiple of 16 bytes)
+__device__ __forceinline__ void bulk_to_smem(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+// first unit of pair c: equal shares of `gran` units each
+__device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigned pairs, unsigned gran) {
+    return unit_begin(c, units / gran, pairs) * gran;
+}
+
 template <bool DUAL>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmX, const WgParams p) {
     constexpr int NT = DUAL ? 2 : 1;
-    const int NPAD = p.npad, ACC_COLS = NPAD * NT;
-    const uint32_t XBYTES = (uint32_t)NPAD * 128u;
-    const uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NPAD >> 3) << 17) |
-                           ((uint32_t)(TILE_N >> 4) << 24);   // f32 accumulate, bf16 x bf16, K-major both
+    constexpr uint32_t WB = NT * STAGE_BYTES;                 // weight bytes per stage and CTA
+    constexpr int CH = DUAL ? 4 : 8;                          // 16-token chunks an epilogue warp holds at most
+    const int nt = p.nt, htok = nt >> 1;
+    const uint32_t xterm = (uint32_t)htok * 128u;             // one term of this CTA's half of the tokens
+    const uint32_t stage_bytes = WB + 2u * xterm;
+    const uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) |
+                           ((uint32_t)(WG_ROWS >> 4) << 24);  // f32 accumulate, bf16 x bf16, K-major both
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const uint32_t wblk = (uint32_t)p.rows8 * 128u;
-    const uint32_t kblk = NT * wblk + XBYTES;                 // one K block of a stage: weights, then the rows' terms
-    const uint32_t stage_bytes = (uint32_t)p.ks * kblk;
-    WgCtrl* ctl = (WgCtrl*)(ring + (size_t)p.stages * stage_bytes);
+    float* staging = (float*)(ring + (size_t)p.stages * stage_bytes);
+    WgCtrl* ctl = (WgCtrl*)((unsigned char*)staging + WG_STAGING);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int kslice = p.pk > 1 ? (int)blockIdx.x % p.pk : 0;       // this CTA's part of the K extent ...
-    const int cta = p.pk > 1 ? (int)blockIdx.x / p.pk : (int)blockIdx.x;   // ... and its row ranges
-    const int ks0 = kslice * p.nks / p.pk, nloc = (kslice + 1) * p.nks / p.pk - ks0;
-    const int items = p.T * nloc;
-    const int koff = (int)(((long long)blockIdx.x * nloc) / gridDim.x);   // every CTA starts at its own K stage
-    const uint32_t tx_bytes = (uint32_t)p.ks * (NT * (uint32_t)p.box * 128u + XBYTES);
+    const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
+    const unsigned units = (unsigned)p.tiles * (unsigned)p.nkb;
+    unsigned u0, u1;
+    if (p.pk > 1) {
+        const unsigned t = (unsigned)(pair / p.pk) * (unsigned)p.nkb, part = (unsigned)(pair % p.pk);
+        u0 = t + part * (unsigned)p.nkb / (unsigned)p.pk;
+        u1 = t + (part + 1) * (unsigned)p.nkb / (unsigned)p.pk;
+    } else {
+        u0 = wg_begin(pair, units, pairs, p.gran);
+        u1 = wg_begin(pair + 1, units, pairs, p.gran);
+    }
+    const int items = (int)(u1 - u0);
 
     if (tid == 0) {
+#pragma unroll 1
         for (int s = 0; s < WG_MAX_STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&ctl->acc_full[b], 1); mbar_init(&ctl->acc_empty[b], 8); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&ctl->acc_full[b], 1); mbar_init(&ctl->acc_empty[b], 16); }
+        mbar_init(&ctl->part_full, 1);
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&ctl->tmem_base)), "r"((uint32_t)p.tmem_cols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&ctl->tmem_base)), "r"((uint32_t)(2 * WG_SET)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
+    cluster_barrier();               // nobody signals a barrier of the other CTA before it is initialised
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort_flag = &ctl->abort_flag;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (warp == 0) {
-        if (lane == 0) {
-            struct Cursor { int t, j, kq, row0; };
-            auto range_row = [&](int t) { return (int)(((long long)(cta * p.T + t) * p.N) / p.V); };
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(WG_REGS_CTL));
+        if (warp == 0 && lane == 0) {
+            // ---- TMA producer of this CTA; all copies of the pair complete on the first CTA's barriers
+            struct Cursor { int kb, row, tok; };              // K block, row tile, token tile
             auto step = [&](Cursor& c) {
-                if (++c.kq == ks0 + nloc) c.kq = ks0;
-                if (++c.j == nloc) { c.j = 0; ++c.t; c.row0 = range_row(c.t); }
+                if (++c.kb == p.nkb) { c.kb = 0; if (++c.tok == p.ntok) { c.tok = 0; ++c.row; } }
             };
-            auto load_w = [&](const Cursor& c, int s) {
+            const int tile0 = (int)(u0 / p.nkb);
+            Cursor cw{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
+            Cursor cx = cw;
+            auto load_w = [&](int s) {
                 unsigned char* dst = ring + (size_t)s * stage_bytes;
-                int x = c.kq * p.ks * KB;
-                mbar_expect_tx(&ctl->full[s], tx_bytes);
-                for (int h = 0; h < p.ks; ++h, x += KB, dst += kblk) {
-                    tma_load_2d(dst, &tmW, &ctl->full[s], x, c.row0);
-                    if (DUAL) tma_load_2d(dst + wblk, &tmW2, &ctl->full[s], x, c.row0);
-                }
+                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+                if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
+                tma_load_2d_pair(dst, &tmW, bar, cw.kb * KB, cw.row * WG_ROWS + rank * TILE_N);
+                if (DUAL) tma_load_2d_pair(dst + STAGE_BYTES, &tmW2, bar, cw.kb * KB, cw.row * WG_ROWS + rank * TILE_N);
+                step(cw);
             };
-            auto load_x = [&](const Cursor& c, int s) {
-                unsigned char* dst = ring + (size_t)s * stage_bytes + NT * wblk;
-                int x = c.kq * p.ks * KB;
-                for (int h = 0; h < p.ks; ++h, x += KB, dst += kblk) tma_load_2d(dst, &tmX, &ctl->full[s], x, 0);
+            auto load_x = [&](int s) {
+                unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
+                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+                const int r = cx.tok * nt + rank * htok;
+                tma_load_2d_pair(dst, &tmX, bar, cx.kb * KB, r);
+                tma_load_2d_pair(dst + xterm, &tmX, bar, cx.kb * KB, p.mpad + r);
+                step(cx);
             };
             const int pre = items < p.stages ? items : p.stages;
-            Cursor cw{0, 0, ks0 + koff, range_row(0)};
-            Cursor cx = cw;
-            for (int i = 0; i < pre; ++i) { load_w(cw, i); step(cw); }
+#pragma unroll 1
+            for (int i = 0; i < pre; ++i) load_w(i);
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            for (int i = 0; i < pre; ++i) { load_x(cx, i); step(cx); }
+#pragma unroll 1
+            for (int i = 0; i < pre; ++i) load_x(i);
             int s = 0;
             uint32_t ph = 0;
+#pragma unroll 1
             for (int i = pre; i < items && !*abort_flag; ++i) {
                 if (!mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
-                load_w(cw, s);
-                load_x(cw, s);
-                step(cw);
+                load_w(s);
+                load_x(s);
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            int s = 0;
+        } else if (warp == 1 && rank == 0 && lane == 0) {
+            // ---- MMA issuer of the pair
+            int s = 0, i = 0;
             uint32_t ph = 0;
+            int kb_begin = (int)(u0 % p.nkb);
+            unsigned g = 0;                                   // accumulator sets filled so far
             const uint64_t desc0 = smem_desc_sw128(smem_u32(ring));
-            for (int t = 0; t < p.T && !*abort_flag; ++t) {
-                const int b = t & 1;
-                if (!mbar_wait(&ctl->acc_empty[b], ((t >> 1) & 1) ^ 1)) { *abort_flag = 1; break; }
-                tc_fence_after();
-                uint32_t d0 = tmem + (uint32_t)(b * p.chunks * ACC_COLS);
-                int rem = 0;
-                bool fresh = true;
-                for (int j = 0; j < nloc; ++j) {
-                    if (!mbar_wait(&ctl->full[s], ph)) { *abort_flag = 1; break; }
+#pragma unroll 1
+            while (i < items && !*abort_flag) {
+                int left = min(p.nkb - kb_begin, items - i);  // K blocks of this segment
+                kb_begin = 0;
+#pragma unroll 1
+                while (left > 0) {
+                    const int b = g & 1, cnt = min(left, WG_DRAIN);
+                    if (!mbar_wait(&ctl->acc_empty[b], ((g >> 1) & 1) ^ 1)) { *abort_flag = 1; break; }
                     tc_fence_after();
-                    uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
-                    for (int h = 0; h < p.ks; ++h, ad += kblk >> 4) {
-                        const uint64_t bd = ad + ((NT * wblk) >> 4);
+                    const uint32_t d0 = tmem + (uint32_t)(b * WG_SET);
+#pragma unroll 1
+                    for (int j = 0; j < cnt; ++j, ++i) {
+                        if (!mbar_wait(&ctl->full[s], ph)) { *abort_flag = 1; break; }
+                        tc_fence_after();
+                        const uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * stage_bytes) >> 4);
+                        const uint64_t bh = ad + (WB >> 4), bl = bh + (xterm >> 4);
 #pragma unroll
                         for (int k = 0; k < KB / 16; ++k) {
-                            const uint32_t acc = (fresh && (h | k) == 0) ? 0u : 1u;
-                            tc_mma(d0, ad + 2 * k, bd + 2 * k, IDESC, acc);
-                            if (DUAL) tc_mma(d0 + NPAD, ad + (wblk >> 4) + 2 * k, bd + 2 * k, IDESC, acc);
+                            const uint32_t acc = (j | k) != 0;
+                            tc_mma_pair(d0, ad + 2 * k, bh + 2 * k, IDESC, acc);
+                            tc_mma_pair(d0, ad + 2 * k, bl + 2 * k, IDESC, 1u);
+                            if (DUAL) {
+                                tc_mma_pair(d0 + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bh + 2 * k, IDESC, acc);
+                                tc_mma_pair(d0 + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bl + 2 * k, IDESC, 1u);
+                            }
                         }
+                        tc_commit_pair(&ctl->empty[s]);
+                        if (++s == p.stages) { s = 0; ph ^= 1u; }
                     }
-                    tc_commit(&ctl->empty[s]);
-                    if (++s == p.stages) { s = 0; ph ^= 1u; }
-                    rem += p.chunks;
-                    fresh = rem >= nloc;
-                    if (fresh) { rem -= nloc; d0 += ACC_COLS; }
+                    if (*abort_flag) break;
+                    tc_commit_pair(&ctl->acc_full[b]);
+                    left -= cnt;
+                    ++g;
                 }
-                if (*abort_flag) break;
-                tc_commit(&ctl->acc_full[b]);
             }
         }
     } else {
-        // ---- epilogue warps: quadrant q of tensor memory holds weight rows q*32 .. q*32+31 of the range;
-        //      the two warps of a quadrant take the 16-row chunks of the block in turn
-        const int q = warp & 3, ew = warp - 2, half = ew >> 2, m = p.m, mpad = p.mpad;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(WG_REGS_EPI));
+        // ---- epilogue warps: quadrant q of tensor memory holds weight rows q*32 .. q*32+31 of this CTA's 128;
+        //      warp half `half` takes tokens half*htok .. of the tile, 16 at a time
+        const int q = warp & 3, ew = warp - 4, half = ew >> 2, et = tid - 128, m = p.m;
+        const int nch = nt >> 5;                              // 16-token chunks of this warp
+        const uint32_t part_bytes = (uint32_t)(TILE_N * NT * sizeof(float)) * (uint32_t)nt;
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        for (int r = ew; r < m; r += 8) {
-            float sc = 1.f;
-            if (p.ssq_in) {
+        const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0u);
+        float* stage_mem = staging + half * (2 * 16 * TILE_N);
+        unsigned g = 0, chunks_done = 0;
+#pragma unroll 1
+        for (int i = 0; i < items;) {
+            const int tile = (int)((u0 + i) / p.nkb), kb_begin = (int)((u0 + i) % p.nkb);
+            const int seg = min(p.nkb - kb_begin, items - i);
+            i += seg;
+            const int row_tile = tile / p.ntok, tok0 = (tile % p.ntok) * nt;
+            asm volatile("bar.sync 1, 256;" ::: "memory");    // everyone is past the previous tile's scale factors
+            if (p.ssq_in && p.pk == 1 && et < nt && tok0 + et < m) {
                 float sq = 0.f;
-                for (int c = lane; c < p.ssq_cnt; c += 32) sq += __ldcg(p.ssq_in + (size_t)c * m + r);
-                sq = warp_sum(sq);
-                sc = 1.f / sqrtf(sq / (float)p.K + p.eps);
+                const float* src = p.ssq_in + tok0 + et;
+#pragma unroll 8
+                for (int c = 0; c < p.ssq_cnt; ++c) sq += __ldcg(src + (size_t)c * m);
+                ctl->scale[et] = 1.f / sqrtf(sq / (float)p.K + p.eps);
             }
-            if (lane == 0) ctl->scale[r] = sc;
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        for (int t = 0; t < p.T; ++t) {
-            const int b = t & 1, v = cta * p.T + t;
-            const int row0 = (int)(((long long)v * p.N) / p.V), row1 = (int)(((long long)(v + 1) * p.N) / p.V);
-            const int n = row0 + q * 32 + lane;
-            const bool mine = n < row1;
-            float out_g = 1.f;
-            if (mine && p.out_xs && p.out_gain) out_g = __bfloat162float(p.out_gain[n]);
-            if (!mbar_wait(&ctl->acc_full[b], (t >> 1) & 1)) { *abort_flag = 1; break; }
-            tc_fence_after();
-            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * p.chunks * ACC_COLS);
-            const int nchunk = (m + 15) / 16, my_last = ((nchunk - 1 - half) / 2) * 2 + half;   // this warp's last chunk
-            if (half >= nchunk) {                // nothing to read: release the accumulators at once
-                if (lane == 0) mbar_arrive(&ctl->acc_empty[b]);
-                continue;
-            }
-            for (int r0 = 16 * half; r0 < m; r0 += 32) {
-                float val[16], up[16], lo[16], lo2[16], yold[16];
+            float acc[NT * CH * 16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) { val[i] = 0.f; up[i] = 0.f; lo[i] = 0.f; lo2[i] = 0.f; yold[i] = 0.f; }
-                if (p.epilogue == EPI_ADD && mine) {   // the residual rows of this chunk, all requested at once
+            for (int e = 0; e < NT * CH * 16; ++e) acc[e] = 0.f;
+            bool ok = true;
+#pragma unroll 1
+            for (int left = seg; left > 0; left -= WG_DRAIN, ++g) {
+                const int b = g & 1;
+                ok = mbar_wait(&ctl->acc_full[b], (g >> 1) & 1);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * WG_SET + half * htok);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (r0 + i < m) yold[i] = __ldcg(p.Y + (size_t)kslice * p.plane + (size_t)(r0 + i) * p.ldy + n);
+                for (int u = 0; u < NT; ++u)
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch)
+                        if (ch < nch) {
+                            float v[16];
+                            tc_ld16(taddr + (uint32_t)(u * nt + ch * 16), v);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) acc[(u * CH + ch) * 16 + e] += v[e];
+                        }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (rank == 0) mbar_arrive(&ctl->acc_empty[b]);
+                    else remote_arrive(empty_bar + (uint32_t)(b * sizeof(uint64_t)));
                 }
-                for (int ch = 0; ch < p.chunks; ++ch) {
-                    float a[16];
-                    tc_ld16(taddr + (uint32_t)(ch * ACC_COLS + r0), a);
+            }
+            if (!ok) { *abort_flag = 1; break; }              // (the same outcome in all eight warps)
+            if (p.pk == 1 && seg < p.nkb) {
+                // part of a tile: later contributors park and go on, the first one adds the parts in pair order.
+                // Parked layout [warp][chunk][quarter of 16][lane][4]: 512 contiguous bytes per warp access.
+                const int c_lo = cta_of_unit((unsigned)tile * p.nkb, units, pairs);
+                const int c_hi = cta_of_unit((unsigned)(tile + 1) * p.nkb - 1, units, pairs);
+                const uint32_t at = (uint32_t)(ew * nch * NT * 512 + lane * 4);
+                if (pair != c_lo) {
+                    float* dst = p.partial + (size_t)blockIdx.x * TILE_N * nt * NT + at;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) val[i] += a[i];
-                    tc_ld16(taddr + (uint32_t)(ch * ACC_COLS + mpad + r0), a);
+                    for (int u = 0; u < NT; ++u)
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) lo[i] += a[i];
-                    if (DUAL) {
-                        tc_ld16(taddr + (uint32_t)(ch * ACC_COLS + NPAD + r0), a);
+                        for (int ch = 0; ch < CH; ++ch)
+                            if (ch < nch) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) up[i] += a[i];
-                        tc_ld16(taddr + (uint32_t)(ch * ACC_COLS + NPAD + mpad + r0), a);
+                                for (int e = 0; e < 4; ++e) {
+                                    const float* a = acc + (u * CH + ch) * 16 + 4 * e;
+                                    __stcg(reinterpret_cast<float4*>(dst + (u * nch + ch) * 512 + e * 128), make_float4(a[0], a[1], a[2], a[3]));
+                                }
+                            }
+                    __threadfence();
+                    asm volatile("bar.sync 1, 256;" ::: "memory");
+                    if (et == 0) atomicAdd(&p.tickets[2 * tile + rank], 1u);
+                    continue;
+                }
+                // The first contributor's part is the last thing of its share: all MMAs are done, the ring is free,
+                // and a parked part (at most 128 KB) comes into it by one bulk copy (through registers, few
+                // loads in flight beside the accumulators, it took 8 us).
+                if (et == 0) {
+                    const unsigned want = (unsigned)(c_hi - c_lo);
+                    int spins = 0;
+#pragma unroll 1
+                    while (ld_acquire_gpu(&p.tickets[2 * tile + rank]) < want)
+                        if (++spins > SPIN_LIMIT) { *abort_flag = 1; break; }
+                    p.tickets[2 * tile + rank] = 0u;          // everyone has arrived: ready for the next launch
+                    __threadfence();
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                }
+                const float* mine = reinterpret_cast<const float*>(ring) + at;
+#pragma unroll 1
+                for (int c = c_lo + 1; c <= c_hi; ++c) {
+                    if (et == 0) {
+                        mbar_expect_tx(&ctl->part_full, part_bytes);
+                        bulk_to_smem(ring, p.partial + (size_t)(2 * c + rank) * TILE_N * nt * NT, part_bytes, &ctl->part_full);
+                    }
+                    if (!mbar_wait(&ctl->part_full, (uint32_t)(c - c_lo - 1) & 1u)) *abort_flag = 1;
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) lo2[i] += a[i];
+                    for (int u = 0; u < NT; ++u)
+#pragma unroll
+                        for (int ch = 0; ch < CH; ++ch)
+                            if (ch < nch) {
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const float4 v = *reinterpret_cast<const float4*>(mine + (u * nch + ch) * 512 + e * 128);
+                                    float* a = acc + (u * CH + ch) * 16 + 4 * e;
+                                    a[0] += v.x; a[1] += v.y; a[2] += v.z; a[3] += v.w;
+                                }
+                            }
+                    asm volatile("bar.sync 1, 256;" ::: "memory");    // the ring may be overwritten
+                }
+            } else {
+                asm volatile("bar.sync 1, 256;" ::: "memory");    // the tile's scale factors are written
+            }
+            // ---- finish, 16 tokens at a time: accumulators -> staging -> this warp's 4 tokens of the chunk, of which
+            //      a lane holds 4 neighbouring weight rows
+            const bool scaled = p.ssq_in && p.pk == 1;
+            const int n0 = row_tile * WG_ROWS + rank * TILE_N, n = n0 + lane * 4;
+            const int have = min(4, p.N - n);                 // weight rows of this lane inside the matrix
+            const bool vec = have == 4 && p.vec_y;
+            float gain[4] = {1.f, 1.f, 1.f, 1.f};
+            if (p.out_xs && p.out_gain) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j < have) gain[j] = __bfloat162float(p.out_gain[n + j]);
+            }
+            float* Y = p.Y ? p.Y + (p.pk > 1 ? (size_t)(pair % p.pk) * p.plane : 0) + n : nullptr;
+#pragma unroll 1
+            for (int ch = 0; ch < nch; ++ch) {
+                const int c0 = half * htok + ch * 16, r0 = tok0 + c0;     // column in the tile, token
+                if (r0 >= m) break;                           // (the same for the four warps of a half)
+                // (one matrix: two buffers in turn, one barrier; the pair: both matrices in one buffer, two barriers)
+                float* buf = stage_mem + (DUAL ? 0 : (chunks_done & 1) * (16 * TILE_N));
+                if (DUAL && chunks_done > 0) asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
+                ++chunks_done;
+                float* put = buf + q * 32 + lane;
+                // Registers have no index: one short copy per chunk, everything else is a loop over the chunks.  Unrolled
+                // over the chunks (100 KB of instructions, pushed out of the caches by the weight stream before every
+                // use) it ran at the speed of instruction fetch: up to 3 us a chunk, all SMs in step, against 1 us.
+#define WG_PUT(C)                                                                                                       \
+    case C:                                                                                                             \
+        if (C < CH) {                                                                                                   \
+            _Pragma("unroll") for (int e = 0; e < 16; ++e) {                                                            \
+                put[e * TILE_N] = acc[(C < CH ? C : 0) * 16 + e];                                                       \
+                if (DUAL) put[(16 + e) * TILE_N] = acc[((NT - 1) * CH + (C < CH ? C : 0)) * 16 + e];                    \
+            }                                                                                                           \
+        }                                                                                                               \
+        break;
+                switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
+#undef WG_PUT
+                asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
+                const int rw = r0 + q * 4;                    // this warp's tokens
+                float x[4][4], old[4][4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    old[k][0] = old[k][1] = old[k][2] = old[k][3] = 0.f;
+                    if (p.epilogue == EPI_ADD && rw + k < m) {            // their residual rows, requested together
+                        const float* y = Y + (size_t)(rw + k) * p.ldy;
+                        if (vec) {
+                            const float4 v = __ldcg(reinterpret_cast<const float4*>(y));
+                            old[k][0] = v.x; old[k][1] = v.y; old[k][2] = v.z; old[k][3] = v.w;
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (j < have) old[k][j] = __ldcg(y + j);
+                        }
                     }
                 }
-                if (r0 == 16 * my_last) {         // this warp's last read of the accumulator set
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->acc_empty[b]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int e = q * 4 + k;
+                    const float4 v = *reinterpret_cast<const float4*>(buf + e * TILE_N + lane * 4);
+                    const float sc = scaled ? ctl->scale[c0 + e] : 1.f;
+                    x[k][0] = v.x * sc; x[k][1] = v.y * sc; x[k][2] = v.z * sc; x[k][3] = v.w * sc;
+                    if (DUAL) {
+                        const float4 u4 = *reinterpret_cast<const float4*>(buf + (16 + e) * TILE_N + lane * 4);
+                        const float u[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            x[k][j] = (p.epilogue == EPI_GEGLU ? wg_gelu(x[k][j]) : wg_silu(x[k][j])) * (u[j] * sc);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) x[k][j] += old[k][j];
                 }
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int r = r0 + i;
-                    if (r < m) {                  // (uniform across the warp)
-                        const float scale = ctl->scale[r];
-                        float x = (val[i] + lo[i]) * scale;
-                        if (DUAL) {
-                            const float u = (up[i] + lo2[i]) * scale;
-                            x = (p.epilogue == EPI_GEGLU ? wg_gelu(x) : wg_silu(x)) * u;
+                for (int k = 0; k < 4; ++k) {
+                    const int r = rw + k;
+                    if (r >= m) break;
+                    if (Y) {
+                        float* y = Y + (size_t)r * p.ldy;
+                        if (vec) *reinterpret_cast<float4*>(y) = make_float4(x[k][0], x[k][1], x[k][2], x[k][3]);
+                        else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (j < have) y[j] = x[k][j];
                         }
-                        if (mine) {
-                            float* y = p.Y + (size_t)kslice * p.plane + (size_t)r * p.ldy + n;
-                            x += yold[i];
-                            *y = x;
+                    }
+                    if (p.out_ssq) {                          // (rows past the matrix came out as zeros)
+                        const float sq = warp_sum((x[k][0] * x[k][0] + x[k][1] * x[k][1]) + (x[k][2] * x[k][2] + x[k][3] * x[k][3]));
+                        if (lane == 0) p.out_ssq[(size_t)(row_tile * 2 + rank) * m + r] = sq;
+                    }
+                    if (p.out_xs && have > 0) {
+                        uint16_t h[4], l[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) split2f(x[k][j] * gain[j], h[j], l[j]);
+                        uint16_t* oh = reinterpret_cast<uint16_t*>(p.out_xs) + (size_t)r * p.out_ld + n;
+                        uint16_t* ol = oh + (size_t)p.mpad * p.out_ld;
+                        if (have == 4 && (p.out_ld & 3) == 0) {
+                            *reinterpret_cast<uint2*>(oh) = make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
+                            *reinterpret_cast<uint2*>(ol) = make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
                         } else {
-                            x = 0.f;              // lanes past the range carry garbage
-                        }
-                        if (p.out_ssq && q < p.qp) {
-                            const float sq = warp_sum(x * x);
-                            if (lane == 0) p.out_ssq[(size_t)(v * p.qp + q) * m + r] = sq;
-                        }
-                        if (p.out_xs && mine) {
-                            uint16_t h1, l1;
-                            split2f(x * out_g, h1, l1);
-                            uint16_t* o = reinterpret_cast<uint16_t*>(p.out_xs) + n;
-                            o[(size_t)r * p.out_ld] = h1;
-                            o[(size_t)(mpad + r) * p.out_ld] = l1;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (j < have) { oh[j] = h[j]; ol[j] = l[j]; }
                         }
                     }
                 }
@@ -351,9 +538,10 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
+    cluster_barrier();               // neither CTA leaves while the other's MMAs or arrivals may reach it
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)p.tmem_cols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * WG_SET)) : "memory");
     }
 }
 
@@ -399,17 +587,22 @@ split2_rows_kernel(const float* __restrict__ X, int ldx, int K, int m, int mpad,
     if (threadIdx.x == 0 && ssq && r < m) ssq[(size_t)blockIdx.x * m + r] = (part[0] + part[1]) + (part[2] + part[3]);
 }
 
-// Adds the partial planes of a K-partitioned launch in plane order, then the epilogue: optional
-// residual add into Y, optional two-term split (times a gain) and sum-of-squares pieces.
+// Adds the partial planes of a K-partitioned launch in plane order, then the epilogue: optional rms-norm
+// factor, residual add into Y, two-term split (times a gain) and sum-of-squares pieces.
 // grid = (N / 1024 rounded up, m); N a multiple of 8.
 __global__ void __launch_bounds__(128)
-wide_reduce_kernel(const float* __restrict__ P, int pk, size_t plane, int N, int m, int mpad, float* __restrict__ Y, int ldy,
-                   int add, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ xs, int out_ld,
+wide_reduce_kernel(const float* __restrict__ P, int pk, size_t plane, int N, int m, int mpad, const float* __restrict__ ssq_in,
+                   int ssq_cnt, int K, float eps, float* __restrict__ Y, int ldy, int add, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ xs, int out_ld,
                    float* __restrict__ ssq) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = blockIdx.y, k = (blockIdx.x * 128 + threadIdx.x) * 8;
-    float sq = 0.f;
+    float sq = 0.f, scale = 1.f;
+    if (ssq_in) {
+        float s = 0.f;
+        for (int c = (int)(threadIdx.x & 31); c < ssq_cnt; c += 32) s += __ldcg(ssq_in + (size_t)c * m + r);
+        scale = 1.f / sqrtf(warp_sum(s) / (float)K + eps);
+    }
     if (k < N) {
         float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int j = 0; j < pk; ++j) {
@@ -417,6 +610,8 @@ wide_reduce_kernel(const float* __restrict__ P, int pk, size_t plane, int N, int
             const float4 a = __ldcg(reinterpret_cast<const float4*>(src)), b = __ldcg(reinterpret_cast<const float4*>(src + 4));
             v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
         }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] *= scale;
         float* y = Y + (size_t)r * ldy + k;
         if (add) {
             const float4 a = *reinterpret_cast<const float4*>(y), b = *reinterpret_cast<const float4*>(y + 4);
@@ -471,42 +666,49 @@ static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const
         CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM_MAX));
         attr_set = true;
     }
-    PdlLaunch L(dim3((unsigned)pl.grid), dim3(WG_THREADS), pl.smem, st);
-    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, kern, tw, tw2, tx, wp));
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cudaLaunchAttribute attr[2];
+    cfg.gridDim = dim3((unsigned)(2 * pl.pairs)); cfg.blockDim = dim3(WG_THREADS); cfg.dynamicSmemBytes = pl.smem; cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    CSD_CUDA(cudaLaunchKernelEx(&cfg, kern, tw, tw2, tx, wp));
     count_launch();
     return CSD_OK;
 }
 
 csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     const bool dual = a.W2 != nullptr;
-    if (!a.W || !a.Y || !a.xs || (((uintptr_t)a.xs) & 15)) return CSD_ERR_INVALID_ARG;
+    if (!a.W || !a.xs || (((uintptr_t)a.xs) & 15) || !a.partial || !a.tickets) return CSD_ERR_INVALID_ARG;
+    if (!a.Y && (!dual || !a.out_xs)) return CSD_ERR_INVALID_ARG;
     if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU)) return CSD_ERR_INVALID_ARG;
     if (!wide_supported(a.m, a.N, a.K, dual)) return CSD_ERR_UNSUPPORTED;
-    int pk = a.ssq ? 1 : wide_pk(a.m, a.N, a.K, dual);
-    if (pk > 1 && (!a.partial || (a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) return CSD_ERR_INVALID_ARG;
-    const WgPlan pl = wg_plan(a.m, a.N, a.K, dual, pk);
-    if (pk > 1 && (pl.box > TILE_N || pl.chunks < 1 || pl.stages < 2)) return CSD_ERR_UNSUPPORTED;
+    const WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
+    if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) return CSD_ERR_INVALID_ARG;
     CUtensorMap tw, tw2, tx;
-    if (!tensor_map_2d(a.W, a.N, a.K, pl.box, &tw)) return CSD_ERR_UNSUPPORTED;
+    if (!tensor_map_2d(a.W, a.N, a.K, TILE_N, &tw)) return CSD_ERR_UNSUPPORTED;
     tw2 = tw;
-    if (dual && !tensor_map_2d(a.W2, a.N, a.K, pl.box, &tw2)) return CSD_ERR_UNSUPPORTED;
-    if (!tensor_map_2d(a.xs, pl.npad, a.K, pl.npad, &tx)) return CSD_ERR_UNSUPPORTED;
+    if (dual && !tensor_map_2d(a.W2, a.N, a.K, TILE_N, &tw2)) return CSD_ERR_UNSUPPORTED;
+    if (!tensor_map_2d(a.xs, 2 * pl.mpad, a.K, pl.nt / 2, &tx)) return CSD_ERR_UNSUPPORTED;
     WgParams wp;
-    wp.Y = a.Y; wp.status = status_word_device();
+    wp.Y = a.Y; wp.partial = a.partial; wp.tickets = a.tickets; wp.status = status_word_device();
     wp.ssq_in = a.ssq; wp.ssq_cnt = a.ssq_cnt;
     wp.out_xs = a.out_xs; wp.out_gain = a.out_gain; wp.out_ssq = a.out_ssq; wp.out_ld = a.out_ld;
-    wp.m = a.m; wp.mpad = pl.mpad; wp.npad = pl.npad; wp.N = a.N; wp.K = a.K; wp.ldy = a.ldy; wp.nks = pl.nks; wp.ks = pl.ks;
-    wp.T = pl.T; wp.V = pl.V; wp.box = pl.box; wp.rows8 = pl.rows8; wp.stages = pl.stages; wp.qp = pl.qp;
-    wp.chunks = pl.chunks; wp.tmem_cols = pl.tmem_cols; wp.epilogue = a.epilogue; wp.eps = a.eps;
-    wp.pk = pk; wp.plane = 0;
-    if (pk > 1) {                        // partial planes now, sums and epilogue in the small kernel after
+    wp.m = a.m; wp.mpad = pl.mpad; wp.nt = pl.nt; wp.ntok = pl.ntok; wp.tiles = pl.tiles; wp.nkb = pl.nkb; wp.pk = pl.pk;
+    wp.gran = pl.gran; wp.N = a.N; wp.K = a.K; wp.ldy = a.ldy; wp.stages = pl.stages; wp.epilogue = a.epilogue; wp.eps = a.eps;
+    wp.plane = 0;
+    wp.vec_y = (a.ldy & 3) == 0 && (((uintptr_t)a.Y) & 15) == 0;
+    if (pl.pk > 1) {                     // partial planes now, sums and epilogue in the small kernel after
         wp.Y = a.partial; wp.ldy = a.N; wp.plane = (size_t)a.m * a.N; wp.epilogue = EPI_STORE;
-        wp.out_xs = nullptr; wp.out_ssq = nullptr; wp.out_gain = nullptr;
+        wp.out_xs = nullptr; wp.out_ssq = nullptr; wp.out_gain = nullptr; wp.vec_y = 1;
         const csd_status s = launch_wg<false>(tw, tw2, tx, wp, pl, st);
         if (s != CSD_OK) return s;
         PdlLaunch L(dim3((unsigned)wide_split_pieces(a.N), (unsigned)a.m), dim3(128), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&L.cfg, wide_reduce_kernel, (const float*)a.partial, pk, wp.plane, a.N, a.m, pl.mpad, a.Y,
-                                    a.ldy, a.epilogue == EPI_ADD ? 1 : 0, a.out_gain, a.out_xs, a.out_ld, a.out_ssq));
+        CSD_CUDA(cudaLaunchKernelEx(&L.cfg, wide_reduce_kernel, (const float*)a.partial, pl.pk, wp.plane, a.N, a.m, pl.mpad, a.ssq,
+                                    a.ssq_cnt, a.K, a.eps, a.Y, a.ldy, a.epilogue == EPI_ADD ? 1 : 0, a.out_gain, a.out_xs,
+                                    a.out_ld, a.out_ssq));
         count_launch();
         return CSD_OK;
     }

@@ -184,12 +184,26 @@ static size_t walk_blob(const csd_model_config& c, const __nv_bfloat16* base, cs
 struct WsLayout {
     size_t kcache, vcache, xk, xv, ek, ev, x, qkv, attn, act, xenc, qkv_enc, rope_c, rope_s, dec_bias, enc_bias,
         buckets, gemm_partial, gemm_tickets, xs_tmp, ssq_tmp, xs_x, xs_attn, xs_act, ssq_x,
-        wx, wqkv, wattn, wact, wxs_x, wxs_attn, wxs_act, wssq, wpart, total;
+        wx, wqkv, wattn, wxs_x, wxs_attn, wxs_act, wssq, wpart, total;
     bool wide;
+    int wide_rows;
     size_t layer_kv, layer_x;
 };
 
-// The wide-block path serves a model when each of its layer matrices takes the wide kernel at 128 rows.
+// Rows of a wide pass: enough for the longest prompt or source, at most CSD_WIDE_ROWS.
+static int wide_rows_for(const csd_model_config& c) {
+    const int most = c.arch == 1 && c.max_enc_len > c.max_seq ? c.max_enc_len : c.max_seq;
+    const int r = (most + 127) / 128 * 128;
+    return r > CSD_WIDE_ROWS ? CSD_WIDE_ROWS : r;
+}
+
+// Rows of the next pass when `left` are to go: equal passes, none of them a small remainder.
+static int wide_pass(int left, int most) {
+    const int passes = (left + most - 1) / most;
+    return (left + passes - 1) / passes;
+}
+
+// The wide-block path serves a model when each of its layer matrices takes the wide kernel.
 static bool wide_capable(const csd_model_config& c) {
     const int d = c.d_model, di = c.n_heads * c.d_head, ff = c.d_ff, R = CSD_WIDE_ROWS;
     return wide_supported(R, di, d, false) && wide_supported(R, 3 * di, d, false) && wide_supported(R, d, di, false) &&
@@ -227,16 +241,15 @@ static WsLayout ws_layout(const csd_model_config& c) {
     L.ssq_x = put((size_t)linear_ssq_capacity((int)d) * R * 4);
     L.wide = wide_capable(c);
     if (L.wide) {
-        const size_t WR = CSD_WIDE_ROWS;
-        L.wx = put(WR * d * 4); L.wqkv = put(WR * 3 * di * 4); L.wattn = put(WR * di * 4); L.wact = put(WR * ff * 4);
+        L.wide_rows = wide_rows_for(c);
+        const size_t WR = (size_t)L.wide_rows;
+        L.wx = put(WR * d * 4); L.wqkv = put(WR * 3 * di * 4); L.wattn = put(WR * di * 4);
         L.wxs_x = put(2 * WR * d * 2); L.wxs_attn = put(2 * WR * di * 2); L.wxs_act = put(2 * WR * ff * 2);
         const size_t kmax_w = d > di ? (d > ff ? d : ff) : (di > ff ? di : ff);
         size_t pieces = (size_t)wide_ssq_capacity((int)d);
         if ((size_t)wide_split_pieces((int)kmax_w) > pieces) pieces = (size_t)wide_split_pieces((int)kmax_w);
         L.wssq = put(pieces * WR * 4);
-        size_t pb = wide_partial_bytes((int)WR, (int)d, (int)di, false);
-        if (wide_partial_bytes((int)WR, (int)d, (int)ff, false) > pb) pb = wide_partial_bytes((int)WR, (int)d, (int)ff, false);
-        L.wpart = put(pb > 0 ? pb : 256);
+        L.wpart = put(wide_partial_bytes((int)WR));
     }
     if (c.arch == 0) {
         L.rope_c = put((size_t)c.max_seq * (Dh / 2) * 4);
@@ -350,7 +363,7 @@ static csd_status feed_forward(csd_model* M, const LayerW& y, float* X, int m, c
 }
 
 // ---------------------------------------------------------------------------------------------
-// wide blocks: one pass of the decoder over up to CSD_WIDE_ROWS rows that only fills the cache
+// wide blocks: one pass of the decoder over up to M->wide_rows rows that only fills the cache
 // ---------------------------------------------------------------------------------------------
 static csd_status wide_linear(csd_model* M, const __nv_bfloat16* W, const __nv_bfloat16* W2, int N, int K, int m,
                               const __nv_bfloat16* xs, const float* ssq, int ssq_cnt, float* Y, int ldy, int epi,
@@ -359,13 +372,13 @@ static csd_status wide_linear(csd_model* M, const __nv_bfloat16* W, const __nv_b
     WideArgs a;
     a.W = W; a.W2 = W2; a.N = N; a.K = K; a.m = m; a.xs = xs; a.ssq = ssq; a.ssq_cnt = ssq_cnt; a.eps = M->cfg.norm_eps;
     a.Y = Y; a.ldy = ldy; a.epilogue = epi; a.out_xs = out_xs; a.out_ld = out_ld; a.out_gain = out_gain; a.out_ssq = out_ssq;
-    a.partial = M->wpart;
+    a.partial = M->wpart; a.tickets = M->gemm_tickets;
     ProfScope ps(M, 0, st);
     if (M->prof) M->prof_gemm_bytes += (double)N * K * 2.0 * (W2 ? 2.0 : 1.0);
     return launch_linear_wide(a, st);
 }
 
-// Attention of `m` <= CSD_WIDE_ROWS rows over K/V that are already in the cache: row r sees keys
+// Attention of `m` <= M->wide_rows rows over K/V that are already in the cache: row r sees keys
 // [0, n_keys0 + r) when causal, all n_keys0 otherwise.
 static csd_status wide_attention(csd_model* M, const float* q, int ldq, int m, __nv_bfloat16* Kc, __nv_bfloat16* Vc, int cap,
                                  int n_keys0, bool causal, const float* bias, int bias_len, int bias_zero, int q_pos0,
@@ -381,7 +394,7 @@ static csd_status wide_attention(csd_model* M, const float* q, int ldq, int m, _
     return attention(M, a, st);
 }
 
-// Decoder pass over m <= CSD_WIDE_ROWS rows at positions kv_len .. kv_len+m-1: K/V of every layer are
+// Decoder pass over m <= M->wide_rows rows at positions kv_len .. kv_len+m-1: K/V of every layer are
 // appended, nothing else is kept.
 static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, int kv_len, cudaStream_t st) {
     const csd_model_config& c = M->cfg;
@@ -433,7 +446,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
                                 M->wssq, st));
             cnt = wide_ssq_pieces(m, d, di, false);
         }
-        CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, cnt, M->wact, ff,
+        CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, cnt, nullptr, ff,
                             c.arch == 0 ? EPI_SWIGLU : EPI_GEGLU, M->wxs_act, ff, nullptr, nullptr, st));
         CSD_TRY(wide_linear(M, y.wdown, nullptr, d, ff, m, M->wxs_act, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d,
                             M->dec[l + 1].norm1, M->wssq, st));
@@ -448,7 +461,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
 // K/V of every decoder layer.
 static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
     const csd_model_config& c = M->cfg;
-    const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, ff = c.d_ff, E = c.max_enc_len, WR = CSD_WIDE_ROWS;
+    const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, ff = c.d_ff, E = c.max_enc_len, WR = wide_pass(n, M->wide_rows);
     for (int l = 0; l < c.n_enc_layers; ++l) {
         const LayerW& y = M->enc[l];
         const bool fused = y.wk == y.wq + (size_t)di * d && y.wv == y.wk + (size_t)di * d;
@@ -477,7 +490,7 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
             CSD_TRY(launch_wide_split(M->wattn, di, di, m, nullptr, M->wxs_attn, nullptr, st));
             CSD_TRY(wide_linear(M, y.wo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, xr, d, EPI_ADD, M->wxs_x, d, y.norm2,
                                 M->wssq, st));
-            CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, wide_ssq_pieces(m, d, di, false), M->wact, ff,
+            CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, wide_ssq_pieces(m, d, di, false), nullptr, ff,
                                 EPI_GEGLU, M->wxs_act, ff, nullptr, nullptr, st));
             CSD_TRY(wide_linear(M, y.wdown, nullptr, d, ff, m, M->wxs_act, nullptr, 0, xr, d, EPI_ADD, nullptr, 0, nullptr,
                                 nullptr, st));
@@ -563,10 +576,10 @@ extern "C" csd_status csd_model_create(const csd_model_config* cfg, const void* 
     M->xs_x = (__nv_bfloat16*)(ws + L.xs_x); M->xs_attn = (__nv_bfloat16*)(ws + L.xs_attn);
     M->xs_act = (__nv_bfloat16*)(ws + L.xs_act); M->ssq_x = (float*)(ws + L.ssq_x);
     M->status = status;
-    M->wide = L.wide;
+    M->wide = L.wide; M->wide_rows = L.wide_rows;
     if (L.wide) {
         M->wx = (float*)(ws + L.wx); M->wqkv = (float*)(ws + L.wqkv); M->wattn = (float*)(ws + L.wattn);
-        M->wact = (float*)(ws + L.wact); M->wxs_x = (__nv_bfloat16*)(ws + L.wxs_x);
+        M->wxs_x = (__nv_bfloat16*)(ws + L.wxs_x);
         M->wxs_attn = (__nv_bfloat16*)(ws + L.wxs_attn); M->wxs_act = (__nv_bfloat16*)(ws + L.wxs_act);
         M->wssq = (float*)(ws + L.wssq); M->wpart = (float*)(ws + L.wpart);
     }
@@ -706,7 +719,7 @@ extern "C" csd_status csd_prefill(csd_model* M, const int32_t* tokens_dev, int n
         int cnt = n - from;
         // wide passes while more than one review block is left, review-sized blocks otherwise
         if (M->wide && gemm_path() != 1 && cnt > small) {
-            if (cnt > CSD_WIDE_ROWS) cnt = CSD_WIDE_ROWS;
+            cnt = wide_pass(cnt, M->wide_rows);
             CSD_TRY(wide_decoder_pass(M, tokens_dev + from, cnt, kv_len + from, st));
         } else {
             if (cnt > small) cnt = small;

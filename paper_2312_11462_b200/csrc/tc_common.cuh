@@ -74,6 +74,36 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
     return d;
 }
 
+// Units of work are (tile, 64-wide K block) pairs in tile-major order; CTA (or CTA pair) c
+// owns the contiguous range [unit_begin(c), unit_begin(c+1)), so every SM streams the same
+// number of weight bytes whatever N and K are.
+// (units * ctas fits 32 bits: the planners refuse shapes where it would not)
+__device__ __forceinline__ unsigned unit_begin(unsigned c, unsigned units, unsigned ctas) { return c * units / ctas; }
+__device__ __forceinline__ int cta_of_unit(unsigned u, unsigned units, unsigned ctas) {
+    unsigned c = ((u + 1) * ctas - 1) / units;
+    while (c + 1 < ctas && unit_begin(c + 1, units, ctas) <= u) ++c;
+    while (c > 0 && unit_begin(c, units, ctas) > u) --c;
+    return (int)c;
+}
 
+// ---- clusters: addresses and barriers of the other CTAs
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 }  // namespace csd

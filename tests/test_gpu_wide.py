@@ -1,0 +1,66 @@
+"""Wide blocks at the edges of their tiles: prompts of 18 to over 1024 tokens (token tiles of 32 to 256
+columns, one to several of them, two passes) and encoder passes, each followed by a review that reads
+every cached position, against the oracle's plain forward."""
+import numpy as np
+import pytest
+
+import workloads
+from workloads import llama_shape, t5_shape
+from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, rel_l2, require_gpu, to_dev_i32
+
+pytestmark = pytest.mark.gpu
+
+# matrices just large enough for the wide kernel; 3 * d_inner is 12 row tiles, d_ff = 1416 ends inside one
+LLAMA = llama_shape(2, 1024, 16, 1416, 500, 1200)
+T5 = t5_shape(2, 1, 1024, 16, 64, 1416, 500, 32, 300)
+
+
+@pytest.fixture(scope="module")
+def b():
+    require_gpu()
+    from paper_2312_11462_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def llama_refs(orc):
+    """Oracle logits of 3-row reviews behind prompts of the lengths below, from one pass over the text."""
+    from paper_2312_11462_b200 import binding as b  # noqa: F401  (GPU tests only)
+    blob = workloads.make_weights(LLAMA, seed=41, device="cpu", gain_std=0.2)
+    toks = workloads.make_prompt(LLAMA.vocab, LLAMA.max_seq, seed=6)
+    om = orc.Model(LLAMA, orc.blob_to_u16(blob))
+    refs, pos = {}, 0
+    for n in LENGTHS:
+        if n > pos:
+            om.review_forward(toks[pos:n], pos)
+            pos = n
+        refs[n] = om.review_forward(toks[n:n + 3], n)     # (rows n .. n+2 are written again by the next stretch)
+    return blob, toks, refs
+
+
+LENGTHS = (18, 31, 32, 33, 64, 127, 128, 129, 255, 256, 257, 300, 513, 700, 1023, 1024, 1025, 1190)
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_prompt_lengths(b, llama_refs, n):
+    blob, toks, refs = llama_refs
+    m = b.Model(LLAMA, blob.cuda())
+    m.csd_prefill(to_dev_i32(toks[:n]), 0)
+    g = m.csd_review_forward(to_dev_i32(toks[n:n + 3]), n).cpu().numpy()
+    assert b.csd_device_status() == 0
+    assert rel_l2(g, refs[n]) <= LOGIT_REL_L2, rel_l2(g, refs[n])
+    assert np.abs(g - refs[n]).max() <= LOGIT_MAX_ABS
+
+
+@pytest.mark.parametrize("n", [18, 33, 129, 256, 300])
+def test_source_lengths(b, orc, n):
+    blob = workloads.make_weights(T5, seed=42, device="cpu", std=0.01, gain_std=0.2)
+    enc = workloads.make_prompt(T5.vocab, n, seed=n)
+    om, gm = orc.Model(T5, orc.blob_to_u16(blob)), b.Model(T5, blob.cuda())
+    om.encoder_forward(enc)
+    gm.csd_encoder_forward(to_dev_i32(enc))
+    blk = np.array([0, 5, 9], dtype=np.int32)
+    g, r = gm.csd_review_forward(to_dev_i32(blk), 0).cpu().numpy(), om.review_forward(blk, 0)
+    assert b.csd_device_status() == 0
+    assert rel_l2(g, r) <= LOGIT_REL_L2, rel_l2(g, r)
+    assert np.abs(g - r).max() <= LOGIT_MAX_ABS
