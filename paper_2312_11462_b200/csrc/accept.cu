@@ -1,5 +1,5 @@
-// Review rule of speculative sampling (Section 2; lenience / greedy: Section 3.1) as three
-// kernels over the vocabulary:
+// Review rule of speculative sampling (Section 2; lenience / greedy: Section 3.1): one kernel while the
+// rows are resident at once (accept_row_kernel), else three kernels over the vocabulary:
 //   stats    one streaming pass over all (2k+1) logit vectors of every row: per 8192-logit piece
 //            the max, arg-max and sum of exponentials (fp32).  This is the HBM-bound part: a
 //            warp owns a piece, keeps 8 x 16 bytes per lane in flight with the next 8 already
@@ -676,6 +676,304 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
     if (threadIdx.x == 0) out_tok[row] = s_pick != 0x7fffffff ? s_pick : (s_last >= 0 ? s_last : 0);
 }
 
+// ---------------------------------------------------------------------------------------------
+// The whole call in one kernel, for calls whose rows are resident at once: a row is a cluster of C CTAs of
+// 1024 threads, a CTA owns the slice [rank * S, rank * S + S) of the vocabulary in every vector.
+//   stats     a warp per piece of a vector's slice, as in the stats pass; the CTAs' results are exchanged
+//             through distributed shared memory and every CTA merges them and runs the accept tests itself
+//   resample  a warp owns S / 32 neighbouring entries of position n, lanes side by side; their fp64
+//             exponentials stay in registers; normalisers and masses are exchanged the same way, and the warp
+//             whose stretch holds u2 * S walks it 32 entries at a time.
+// These calls are bound by the chain of dependent steps, not by bytes: one row, k = 4, V = 32000 (1.15 MB)
+// took 23.3 us as stats (36 busy warps), decide and resample kernels, 17.2 us as one.  Sums have a fixed order.
+// ---------------------------------------------------------------------------------------------
+constexpr int AR_THREADS = 1024, AR_WARPS = AR_THREADS / 32, AR_MAXC = 16;
+constexpr int AR_TASKS = 2 * MAX_K + 1 + AR_WARPS;
+
+__device__ __forceinline__ StatPartial cluster_read_stat(const StatPartial* local, uint32_t rank) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
+    uint32_t r, w0, w1, w2, w3;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3) : "r"(r) : "memory");
+    StatPartial p;
+    p.mx = __uint_as_float(w0); p.sum = __uint_as_float(w1); p.arg = (int)w2; p.pad = (int)w3;
+    return p;
+}
+// a later piece (larger indices) joins the running (max, sum, arg-max)
+__device__ __forceinline__ void merge_stat(float& mx, float& z, int& arg, const StatPartial& q, float invT) {
+    if (q.mx > mx) {
+        z = (mx > -INFINITY ? z * __expf((mx - q.mx) * invT) : 0.f) + q.sum;
+        mx = q.mx; arg = q.arg;
+    } else if (q.mx > -INFINITY) {
+        z += q.sum * __expf((q.mx - mx) * invT);
+    }
+}
+
+// ordered sum of the warps' values; valid in every thread
+__device__ __forceinline__ double ar_block_sum(double v, double* s_warp) {
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return warp_sum(s_warp[threadIdx.x & 31]);
+}
+
+template <bool VEC, int PER>
+__global__ void __launch_bounds__(AR_THREADS, 1)
+accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, const int* __restrict__ onehot,
+                  const int* __restrict__ tokens, int rows, int k, int V, float temperature, float lenience, uint64_t seed,
+                  uint64_t step, int csize, int S, int pieces, int* __restrict__ n_acc, int* __restrict__ out_tok, int* status) {
+    __shared__ StatPartial s_task[AR_TASKS];
+    __shared__ StatPartial s_own[2 * MAX_K + 1];       // this CTA's slice of every vector
+    __shared__ float s_mx[2 * MAX_K + 1], s_z[2 * MAX_K + 1];
+    __shared__ int s_arg[2 * MAX_K + 1], s_acc[MAX_K + 1], s_point[MAX_K + 1], s_x[MAX_K + 1];
+    __shared__ double s_u2[MAX_K + 1], s_ex[5], s_warp[AR_WARPS], s_tab[64];
+    const int row = blockIdx.x / csize, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank();
+    const bool greedy = temperature == 0.f;
+    const float invT = greedy ? 1.f : 1.f / temperature;
+    if (!greedy && tid < 64) s_tab[tid] = c_exp2_table[tid];
+    pdl_wait();
+    pdl_trigger();
+    const int nvec = dl ? 2 * k + 1 : k + 1;
+    const float* trow = tl + (long long)row * (k + 1) * V;
+    const float* drow = dl ? dl + (long long)row * k * V : nullptr;
+    // what the accept tests need besides the statistics travels while those are formed (thread i: position i)
+    int x = 0;
+    bool bad = false, point = true;
+    float tx = 0.f, dx = 0.f;
+    if (tid < k) {
+        x = tokens[(long long)row * k + tid];
+        bad = x < 0 || x >= V;
+        point = !dl || (onehot && onehot[(long long)row * k + tid] != 0);
+        if (!greedy && !bad) {
+            tx = trow[(long long)tid * V + x];
+            if (!point) dx = drow[(long long)tid * V + x];
+        }
+    }
+    // ---- statistics of this CTA's slice
+    const int lo = rank * S, hi = min(V, lo + S);
+    const int plen = (S + pieces * 128 - 1) / (pieces * 128) * 128;
+#pragma unroll 1
+    for (int task = warp; task < nvec * pieces; task += AR_WARPS) {
+        const int vec = task / pieces, from = lo + (task % pieces) * plen, to = min(hi, from + plen);
+        const float* src = vec <= k ? trow + (long long)vec * V : drow + (long long)(vec - k - 1) * V;
+        float mx = -INFINITY, sum = 0.f;
+        int arg = 0x7fffffff;
+#pragma unroll 1
+        for (int e0 = from; e0 < to; e0 += ST_SUB) {
+            float cur[32];
+            load_sub<VEC>(src, e0, to, lane, cur);
+            float bm = -INFINITY;
+            int ba = 0x7fffffff;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (cur[j] > bm) { bm = cur[j]; ba = sub_index<VEC>(e0, lane, j); }
+            if (bm > mx) {
+                sum = mx > -INFINITY ? sum * __expf((mx - bm) * invT) : 0.f;
+                mx = bm; arg = ba;
+            }
+            if (!greedy && mx > -INFINITY) {
+                float a = 0.f;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) a += __expf((cur[j] - mx) * invT);
+                sum += a;
+            }
+        }
+        float wm = mx;
+        int wa = arg;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, wm, o);
+            const int oa = __shfl_xor_sync(0xffffffffu, wa, o);
+            if (om > wm || (om == wm && oa < wa)) { wm = om; wa = oa; }
+        }
+        float scaled = (!greedy && mx > -INFINITY) ? sum * __expf((mx - wm) * invT) : 0.f;
+        scaled = warp_sum(scaled);
+        if (lane == 0) { StatPartial q; q.mx = wm; q.sum = scaled; q.arg = wa; q.pad = 0; s_task[task] = q; }
+    }
+    __syncthreads();
+    if (tid < nvec) {
+        float mx = -INFINITY, z = 0.f;
+        int arg = 0x7fffffff;
+        for (int c = 0; c < pieces; ++c) merge_stat(mx, z, arg, s_task[tid * pieces + c], invT);
+        StatPartial q; q.mx = mx; q.sum = z; q.arg = arg; q.pad = 0;
+        s_own[tid] = q;
+    }
+    cluster_sync_all();
+    if (tid < nvec) {
+        StatPartial q[AR_MAXC];
+#pragma unroll
+        for (int c = 0; c < AR_MAXC; ++c)
+            if (c < csize) q[c] = cluster_read_stat(&s_own[tid], (uint32_t)c);
+        float mx = -INFINITY, z = 0.f;
+        int arg = 0x7fffffff;
+#pragma unroll
+        for (int c = 0; c < AR_MAXC; ++c)
+            if (c < csize) merge_stat(mx, z, arg, q[c], invT);
+        s_mx[tid] = mx; s_z[tid] = z; s_arg[tid] = arg;
+    }
+    __syncthreads();
+    // ---- the accept tests of all positions at once
+    if (tid <= k) {
+        bool accept = false;
+        double u2 = 0.0;
+        if (greedy) {
+            accept = tid < k && x == s_arg[tid];
+        } else {
+            const Philox4 r = philox4x32_10((uint32_t)tid, (uint32_t)row, (uint32_t)step, (uint32_t)(step >> 32), (uint32_t)seed,
+                                            (uint32_t)(seed >> 32));
+            u2 = word_uniform(r.w[1]);
+            if (tid < k && !bad) {
+                const double T = (double)temperature;
+                const double px = exp(((double)tx - (double)s_mx[tid]) / T) / (double)s_z[tid];
+                const double qx = point ? 1.0 : exp(((double)dx - (double)s_mx[k + 1 + tid]) / T) / (double)s_z[k + 1 + tid];
+                accept = word_uniform(r.w[0]) * qx < (point ? 1.0 : (double)lenience) * px;   // no lenience for the statistical drafter's tokens (Appendix B)
+            }
+        }
+        if (tid < k && bad && rank == 0) set_status(status, CSD_ERR_BAD_TOKEN);
+        s_acc[tid] = accept ? 1 : 0; s_point[tid] = point ? 1 : 0; s_x[tid] = bad ? 0 : x; s_u2[tid] = u2;
+    }
+    __syncthreads();
+    int n = 0;
+    while (n < k && s_acc[n]) ++n;
+    if (rank == 0 && tid == 0) {
+        n_acc[row] = n;
+        if (greedy) out_tok[row] = s_arg[n];
+    }
+    if (greedy) {
+        cluster_sync_all();                            // no CTA leaves while another may still read its statistics
+        return;
+    }
+    // ---- resample at position n
+    const double inv_temp = 1.0 / (double)temperature, max_t = (double)s_mx[n];
+    int mode = n == k ? MODE_TARGET_ONLY : (s_point[n] ? MODE_RESID_POINT : MODE_RESID_LOGITS);
+    const double max_q = mode == MODE_RESID_LOGITS ? (double)s_mx[k + 1 + n] : 0.0, u2 = s_u2[n];
+    const int xn = s_x[n];
+    const float* t = trow + (long long)n * V;
+    const float* d = mode == MODE_RESID_LOGITS ? drow + (long long)n * V : nullptr;
+    const int e0 = lo + warp * (PER * 32) + lane;      // entries e0 + 32 j
+    double et[PER], ed[PER];
+    {
+        float tv[PER], dv[PER];
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int e = e0 + 32 * j;
+            tv[j] = e < hi ? t[e] : -INFINITY;
+            dv[j] = d && e < hi ? d[e] : -INFINITY;
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            et[j] = exp_neg(((double)tv[j] - max_t) * inv_temp, s_tab);       // -inf (past the slice) gives 0
+            ed[j] = d ? exp_neg(((double)dv[j] - max_q) * inv_temp, s_tab) : 0.0;
+        }
+    }
+    double sp = 0.0, sq = 0.0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) { sp += et[j]; sq += ed[j]; }
+    sp = ar_block_sum(sp, s_warp);
+    if (d) sq = ar_block_sum(sq, s_warp);
+    if (tid == 0) { s_ex[0] = sp; s_ex[1] = sq; }
+    cluster_sync_all();
+    double Zp = 0.0, Zq = 0.0;
+    {
+        const double a = lane < csize ? cluster_read_f64(&s_ex[0], (uint32_t)lane) : 0.0;
+        const double c = lane < csize ? cluster_read_f64(&s_ex[1], (uint32_t)lane) : 0.0;
+        Zp = warp_sum(a); Zq = warp_sum(c);
+    }
+    const double inv_zt = 1.0 / Zp, inv_zq = Zq > 0.0 ? 1.0 / Zq : 0.0;
+    auto resid = [&](int j) -> double {
+        if (e0 + 32 * j >= hi) return 0.0;
+        const double pv = et[j] * inv_zt;
+        if (mode == MODE_TARGET_ONLY) return pv;
+        const double qv = mode == MODE_RESID_POINT ? (e0 + 32 * j == xn ? 1.0 : 0.0) : ed[j] * inv_zq;
+        return pv > qv ? pv - qv : 0.0;
+    };
+    double mass_w = 0.0, before = 0.0, total = 0.0;    // this warp's mass, the mass before its stretch, the row's
+    int last_rank = 0;
+    // (a second time with the target law itself if the residual is empty)
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        double local = 0.0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) local += resid(j);
+        mass_w = warp_sum(local);
+        __syncthreads();
+        if (lane == 0) s_warp[warp] = mass_w;
+        __syncthreads();
+        double run = s_warp[lane];                     // inclusive prefix over the warps
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double up = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += up;
+        }
+        if (tid == AR_THREADS - 1) s_ex[2 + pass] = run;
+        before = warp > 0 ? __shfl_sync(0xffffffffu, run, (warp + 31) & 31) : 0.0;
+        cluster_sync_all();
+        double m = lane < csize ? cluster_read_f64(&s_ex[2 + pass], (uint32_t)lane) : 0.0, incl = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        total = __shfl_sync(0xffffffffu, incl, csize - 1);
+        if (!(total > 0.0) || !isfinite(total)) {
+            if (pass == 0 && mode != MODE_TARGET_ONLY) { mode = MODE_TARGET_ONLY; continue; }
+        }
+        const double head = __shfl_sync(0xffffffffu, incl - m, rank);         // mass before this CTA
+        const unsigned some = __ballot_sync(0xffffffffu, m > 0.0);
+        last_rank = some ? 31 - __clz(some) : 0;
+        before += head;
+        break;
+    }
+    // ---- the entry: smallest index whose cumulative mass exceeds u2 * total; rounding may leave none, then the
+    //      last entry that carries mass
+    const double target = u2 * total;
+    __shared__ int s_pick, s_last;
+    if (tid == 0) { s_pick = 0x7fffffff; s_last = -1; s_ex[4] = 0.0; }
+    __syncthreads();
+    // (only the stretches around the target are walked: the warp whose prefix interval holds it, and its neighbours
+    // in case rounding moved the boundary)
+    if (before <= target * (1.0 + 1e-12) && before + mass_w >= target * (1.0 - 1e-12)) {
+        double cum = before;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const double r = resid(j);
+            double incl = r;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double up = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += up;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, r > 0.0 && cum + incl > target);
+            if (hit) {
+                if (lane == 0) atomicMin(&s_pick, lo + warp * (PER * 32) + 32 * j + __ffs(hit) - 1);
+                break;
+            }
+            cum += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    if (rank == last_rank) {
+        int mine = -1;
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            if (resid(j) > 0.0) mine = e0 + 32 * j;
+        mine = __reduce_max_sync(0xffffffffu, mine);
+        if (lane == 0 && mine >= 0) atomicMax(&s_last, mine);
+    }
+    __syncthreads();
+    if (tid == 0) s_ex[4] = s_pick != 0x7fffffff ? (double)s_pick : -1.0 - (double)max(s_last, 0);
+    cluster_sync_all();
+    if (rank == 0 && warp == 0) {
+        // the first CTA (vocabulary order) that found an entry has it
+        const double v = lane < csize ? cluster_read_f64(&s_ex[4], (uint32_t)lane) : -1.0;
+        const unsigned found = __ballot_sync(0xffffffffu, lane < csize && v >= 0.0);
+        const double pick = __shfl_sync(0xffffffffu, v, found ? __ffs(found) - 1 : last_rank);
+        if (lane == 0) out_tok[row] = found ? (int)pick : (int)(-1.0 - pick);
+    }
+    cluster_sync_all();                                // no CTA leaves while its results may still be read
+}
+
 struct AcceptLayout {
     size_t part_off, info_off, z_off, zsum_off, r_off, ticket_off, total;
     int nchunk_a, nchunk_r;
@@ -750,6 +1048,54 @@ static bool fused_resample_ok(int csize) {
     return state[csize] == 1;
 }
 
+// Clusters of `csize` CTAs of the one-kernel form that are resident at once (0: none); asked once per size.
+template <bool VEC, int PER>
+static int row_clusters(int csize) {
+    static int known[AR_MAXC + 1];              // 0 unknown, else 1 + the answer
+    if (known[csize] == 0) {
+        int n = 0;
+        bool ok = true;
+        if (csize > 8)
+            ok = cudaFuncSetAttribute(accept_row_kernel<VEC, PER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (ok) {
+            cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+            cudaLaunchAttribute attr[1];
+            cfg.gridDim = dim3((unsigned)csize); cfg.blockDim = dim3(AR_THREADS);
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            ok = cudaOccupancyMaxActiveClusters(&n, accept_row_kernel<VEC, PER>, &cfg) == cudaSuccess;
+        }
+        if (!ok) { (void)cudaGetLastError(); n = 0; }
+        known[csize] = 1 + n;
+    }
+    return known[csize] - 1;
+}
+
+template <bool VEC, int PER>
+static csd_status launch_accept_row(const float* tl, const float* dl, const int* onehot, const int* tokens, int rows, int k,
+                                    int V, float temperature, float lenience, uint64_t seed, uint64_t step, int csize,
+                                    int* n_acc, int* out_tok, int* status, cudaStream_t st, bool* done) {
+    *done = false;
+    if (row_clusters<VEC, PER>(csize) < rows) return CSD_OK;
+    const int S = ((V + csize - 1) / csize + 3) & ~3, nvec = dl ? 2 * k + 1 : k + 1;
+    int pieces = (AR_WARPS + nvec - 1) / nvec;           // enough pieces for every warp, of at least 1024 logits
+    if (pieces > (S + ST_SUB - 1) / ST_SUB) pieces = (S + ST_SUB - 1) / ST_SUB;
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cudaLaunchAttribute attr[2];
+    cfg.gridDim = dim3((unsigned)(rows * csize)); cfg.blockDim = dim3(AR_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    CSD_CUDA(cudaLaunchKernelEx(&cfg, accept_row_kernel<VEC, PER>, tl, dl, onehot, tokens, rows, k, V, temperature, lenience,
+                                seed, step, csize, S, pieces, n_acc, out_tok, status));
+    count_launch();
+    *done = true;
+    return CSD_OK;
+}
+
 // The three passes on scratch `ws` (accept_layout bytes).  Every word a pass reads is written by an
 // earlier pass of the same call (the decide pass clears the resample tickets), so the scratch
 // needs no initialisation.
@@ -771,6 +1117,28 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     const long long nvec = n_tvec + (use_d ? (long long)rows * k : 0);
     if (nvec > 0x7fffffffLL) return CSD_ERR_UNSUPPORTED;
     const bool vec_ok = (V % 4 == 0) && (((uintptr_t)tl & 15) == 0) && (!use_d || ((uintptr_t)dl & 15) == 0);
+    // One kernel while its clusters are all resident; smallest power of two that leaves a CTA at most
+    // 4096 entries (8192 beyond 32768), doubled while that leaves it 512 and the rows still fit.
+    if (V <= AR_MAXC * 8192) {
+        if (!greedy) {
+            const csd_status ts = exp_table_ready();
+            if (ts != CSD_OK) return ts;
+        }
+        int csize = 1;
+        while (csize < 8 && (V + csize - 1) / csize > 4096) csize *= 2;
+        if (V > 8 * 8192) csize = 16;
+        const bool wide = ((V + csize - 1) / csize + 3) / 4 * 4 > 4096;
+        while (csize < 8 && rows * csize * 2 <= accept_sm_count() && V / (csize * 2) >= 512) csize *= 2;
+        bool done = false;
+        csd_status s;
+        if (vec_ok)
+            s = wide ? launch_accept_row<true, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done)
+                     : launch_accept_row<true, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done);
+        else
+            s = wide ? launch_accept_row<false, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done)
+                     : launch_accept_row<false, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done);
+        if (s != CSD_OK || done) return s;
+    }
     const long long items = nvec * L.nchunk_a;
     long long ctas = (items + ST_THREADS / 32 - 1) / (ST_THREADS / 32);
     const long long cap = (long long)accept_sm_count() * 2;       // two resident CTAs per SM, grid-stride beyond
