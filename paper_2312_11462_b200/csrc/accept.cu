@@ -10,10 +10,8 @@
 //            does not depend on summation order or on fp32 rounding: first the per-chunk sums
 //            of the exponentials (the normalisers), then per chunk the mass of the residual
 //            max(0, p - q) (or of p after k acceptances); the CTA that finishes a row last takes
-//            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (argument
-//            reduction by ln 2 and a degree-11 Taylor polynomial, relative error below 1e-13 on
-//            the arguments that occur, x <= 0), and every division is a multiplication by a
-//            reciprocal formed once.
+//            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
+//            law is normalised: every comparison is made on products instead of quotients.
 #include "common.cuh"
 #include "philox.cuh"
 #include <math.h>
@@ -138,93 +136,146 @@ accept_stats_kernel(const float* __restrict__ tl, const float* __restrict__ dl, 
 // ---------------------------------------------------------------------------------------------
 constexpr int MAX_K = 64;
 
-__global__ void __launch_bounds__(128)
+// exp(x) for x <= 0 in fp64 by table and polynomial: x = (64 m + j) ln2/64 + r with |r| <= ln2/128,
+// exp(x) = 2^m * 2^(j/64) * e^r; the 64 table entries are correctly rounded doubles made on the host,
+// e^r is its Taylor series to r^5 (remainder below 4e-17), 2^m goes through the exponent field.
+// Relative error about 3e-16.  Below -708 the result is 0 (under the smallest normal number).
+__constant__ double c_exp2_table[64];
+__device__ __forceinline__ void exp_table_to_shared(double* s_tab) {
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) s_tab[i] = c_exp2_table[i];
+    __syncthreads();
+}
+// The rounding to n goes through the magic constant 1.5 * 2^52 (n is the low word of the sum): rint and the
+// conversion to int run at a quarter of the fp64 rate and bounded the resample passes.
+__device__ __forceinline__ double exp_neg(double x, const double* __restrict__ s_tab) {
+    const double magic = 6755399441055744.0;
+    const double t = fma(x, 92.33248261689366, magic);        // 64 / ln 2
+    const double nf = t - magic;
+    const int n = __double2loint(t);
+    double r = fma(-nf, 0.01083042468962958, x);              // ln 2 / 64, high part (low 22 bits clear: nf * high is exact)
+    r = fma(-nf, 6.619564634077006e-12, r);                   // ln 2 / 64, low part
+    double p = 1.0 / 120.0;
+    p = fma(p, r, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(p, r, 1.0);
+    p *= r;                                                   // e^r - 1
+    const double tj = s_tab[n & 63];
+    const double v = fma(tj, p, tj);
+    const int hi = __double2hiint(v) + ((n >> 6) << 20);      // m >= -1022: stays a normal number
+    return x > -708.0 ? __hiloint2double(hi, __double2loint(v)) : 0.0;
+}
+
+// u q(x) < l p(x) without a division; no lenience for the statistical drafter's tokens (Appendix B)
+__device__ __forceinline__ bool accept_test(double u, float tx, float mt, float zt, bool point, float dx, float mq, float zq,
+                                            double inv_temp, float lenience, const double* __restrict__ s_tab) {
+    const double ep = exp_neg(((double)tx - (double)mt) * inv_temp, s_tab);
+    if (point) return u * (double)zt < ep;
+    const double eq = exp_neg(((double)dx - (double)mq) * inv_temp, s_tab);
+    return u * eq * (double)zt < (double)lenience * ep * (double)zq;
+}
+
+// a later piece (larger indices) joins the running (max, sum, arg-max)
+__device__ __forceinline__ void merge_stat(float& mx, float& z, int& arg, const StatPartial& q, float invT) {
+    if (q.mx > mx) {
+        z = (mx > -INFINITY ? z * __expf((mx - q.mx) * invT) : 0.f) + q.sum;
+        mx = q.mx; arg = q.arg;
+    } else if (q.mx > -INFINITY) {
+        z += q.sum * __expf((q.mx - mx) * invT);
+    }
+}
+
+// the pieces held by G neighbouring lanes, in index order, into the first of them
+template <int G>
+__device__ __forceinline__ void merge_stat_lanes(StatPartial& a, float invT) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        StatPartial q;
+        q.mx = __shfl_down_sync(0xffffffffu, a.mx, o); q.sum = __shfl_down_sync(0xffffffffu, a.sum, o);
+        q.arg = __shfl_down_sync(0xffffffffu, a.arg, o); q.pad = 0;
+        if (((int)threadIdx.x & (2 * o - 1)) == 0) merge_stat(a.mx, a.sum, a.arg, q, invT);
+    }
+}
+
+constexpr int DC_THREADS = 512, DC_LANES = 16;   // lanes that merge one vector's pieces
+
+__global__ void __launch_bounds__(DC_THREADS)
 accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl, const int* __restrict__ onehot,
                      const int* __restrict__ tokens, int rows, int k, int V, float temperature, float lenience,
                      uint64_t seed, uint64_t step, const StatPartial* __restrict__ part, int nchunk,
                      int* __restrict__ n_acc, int* __restrict__ out_tok, RowInfo* __restrict__ info,
                      unsigned* __restrict__ tickets, int* status) {
-    pdl_wait();
-    pdl_trigger();
-    const int row = blockIdx.x;
+    const int row = blockIdx.x, tid = threadIdx.x;
     __shared__ float s_mx[2 * MAX_K + 1];
     __shared__ float s_z[2 * MAX_K + 1];
     __shared__ int s_arg[2 * MAX_K + 1];
     __shared__ int s_acc[MAX_K], s_x[MAX_K], s_point[MAX_K];
-    __shared__ double s_u2[MAX_K];
+    __shared__ double s_u2[MAX_K], s_tab[64];
     const bool greedy = temperature == 0.f;
     const float invT = greedy ? 1.f : 1.f / temperature;
+    if (!greedy && tid < 64) s_tab[tid] = c_exp2_table[tid];
+    pdl_wait();
+    pdl_trigger();
     const int nvec_row = dl ? 2 * k + 1 : k + 1;
     const long long n_tvec = (long long)rows * (k + 1);
-    // ---- merge the pieces of every vector of this row (one thread per vector, one pass)
-    for (int i = threadIdx.x; i < nvec_row; i += blockDim.x) {
-        const long long vec = i <= k ? (long long)row * (k + 1) + i : n_tvec + (long long)row * k + (i - k - 1);
-        const StatPartial* p = part + vec * nchunk;
-        float mx = -INFINITY, z = 0.f;
-        int arg = 0x7fffffff;
-#pragma unroll 4
-        for (int c = 0; c < nchunk; ++c) {
-            const StatPartial q = p[c];
-            if (q.mx > mx) {        // pieces come in index order, so ">" keeps the earliest arg-max
-                z = mx > -INFINITY ? z * __expf((mx - q.mx) * invT) : 0.f;
-                mx = q.mx; arg = q.arg;
-                z += q.sum;
-            } else if (q.mx > -INFINITY) {
-                z += q.sum * __expf((q.mx - mx) * invT);
-            }
+    // what the accept tests need besides the statistics travels while those are merged (thread i: position i)
+    int x = 0;
+    bool bad = false, point = true;
+    float tx = 0.f, dx = 0.f;
+    if (tid < k) {
+        x = tokens[(long long)row * k + tid];
+        bad = x < 0 || x >= V;
+        point = dl == nullptr || (onehot && onehot[(long long)row * k + tid] != 0);
+        if (!greedy && !bad) {
+            tx = tl[((long long)row * (k + 1) + tid) * V + x];
+            if (!point) dx = dl[((long long)row * k + tid) * V + x];
         }
-        s_mx[i] = mx; s_z[i] = greedy ? 0.f : z; s_arg[i] = arg;
     }
-    if (threadIdx.x == 0 && tickets) { tickets[row] = 0u; tickets[rows + row] = 0u; }   // for the two resample passes
+    // ---- merge the pieces of every vector of this row: 16 lanes a vector, so that a piece per lane is requested at
+    //      once (one thread per vector walked 16 pieces of V = 128256 in four round trips)
+    for (int i0 = 0; i0 < nvec_row; i0 += DC_THREADS / DC_LANES) {
+        const int i = i0 + tid / DC_LANES, l = tid % DC_LANES;
+        StatPartial a;
+        a.mx = -INFINITY; a.sum = 0.f; a.arg = 0x7fffffff; a.pad = 0;
+        if (i < nvec_row) {
+            const long long vec = i <= k ? (long long)row * (k + 1) + i : n_tvec + (long long)row * k + (i - k - 1);
+            const StatPartial* p = part + vec * nchunk;
+            const int each = (nchunk + DC_LANES - 1) / DC_LANES;      // a lane's pieces are neighbours, in index order
+            for (int c = l * each; c < min(nchunk, (l + 1) * each); ++c) merge_stat(a.mx, a.sum, a.arg, p[c], invT);
+        }
+        merge_stat_lanes<DC_LANES>(a, invT);
+        if (i < nvec_row && l == 0) { s_mx[i] = a.mx; s_z[i] = a.sum; s_arg[i] = a.arg; }
+    }
+    if (tid == 0 && tickets) { tickets[row] = 0u; tickets[rows + row] = 0u; }   // for the two resample passes
     __syncthreads();
-    const int* tok = tokens + (long long)row * k;
     RowInfo ri;
     ri.n = k; ri.mode = MODE_DONE; ri.x = 0; ri.pad = 0; ri.max_t = 0; ri.max_q = 0; ri.u2 = 0;
-    if (greedy) {
-        if (threadIdx.x != 0) return;
-        int n = 0;
-        while (n < k && tok[n] == s_arg[n]) ++n;
-        for (int i = 0; i < k; ++i)             // a drafted id outside the vocabulary is rejected and recorded
-            if (tok[i] < 0 || tok[i] >= V) set_status(status, CSD_ERR_BAD_TOKEN);
-        n_acc[row] = n;
-        out_tok[row] = s_arg[n];
-        ri.n = n;
-        info[row] = ri;
-        return;
+    if (tid < k) {                              // a drafted id outside the vocabulary is rejected and recorded
+        if (bad) set_status(status, CSD_ERR_BAD_TOKEN);
+        s_x[tid] = bad ? 0 : x; s_point[tid] = point ? 1 : 0;
+        if (greedy) s_acc[tid] = x == s_arg[tid];
     }
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     const uint32_t c2 = (uint32_t)step, c3 = (uint32_t)(step >> 32);
-    const double T = (double)temperature;
     // ---- the accept tests of all positions at once (thread i: position i)
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-        int x = tok[i];
-        const Philox4 r = philox4x32_10((uint32_t)i, (uint32_t)row, c2, c3, k0, k1);
-        const bool point = dl == nullptr || (onehot && onehot[(long long)row * k + i] != 0);
-        bool accept = false;
-        if (x < 0 || x >= V) {
-            set_status(status, CSD_ERR_BAD_TOKEN);
-            x = 0;
-        } else {
-            const double u = word_uniform(r.w[0]);
-            const double px = exp(((double)tl[((long long)row * (k + 1) + i) * V + x] - (double)s_mx[i]) / T) / (double)s_z[i];
-            double qx = 1.0;
-            if (!point)
-                qx = exp(((double)dl[((long long)row * k + i) * V + x] - (double)s_mx[k + 1 + i]) / T) /
-                     (double)s_z[k + 1 + i];
-            accept = u * qx < (point ? 1.0 : (double)lenience) * px;   // no lenience for the statistical drafter's tokens (Appendix B)
-        }
-        s_acc[i] = accept ? 1 : 0; s_x[i] = x; s_point[i] = point ? 1 : 0; s_u2[i] = word_uniform(r.w[1]);
+    if (!greedy && tid < k) {
+        const Philox4 r = philox4x32_10((uint32_t)tid, (uint32_t)row, c2, c3, k0, k1);
+        const double inv_temp = 1.0 / (double)temperature;
+        s_acc[tid] = !bad && accept_test(word_uniform(r.w[0]), tx, s_mx[tid], s_z[tid], point, dx, point ? 0.f : s_mx[k + 1 + tid],
+                                         point ? 1.f : s_z[k + 1 + tid], inv_temp, lenience, s_tab);
+        s_u2[tid] = word_uniform(r.w[1]);
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (tid != 0) return;
     int n = 0;
     while (n < k && s_acc[n]) ++n;
-    if (n < k) {
-        const bool point = s_point[n] != 0;
-        ri.mode = point ? MODE_RESID_POINT : MODE_RESID_LOGITS;
+    if (greedy) {
+        out_tok[row] = s_arg[n];
+    } else if (n < k) {
+        ri.mode = s_point[n] ? MODE_RESID_POINT : MODE_RESID_LOGITS;
         ri.x = s_x[n];
         ri.max_t = (double)s_mx[n];
-        ri.max_q = point ? 0.0 : (double)s_mx[k + 1 + n];
+        ri.max_q = s_point[n] ? 0.0 : (double)s_mx[k + 1 + n];
         ri.u2 = s_u2[n];
     } else {
         const Philox4 r = philox4x32_10((uint32_t)k, (uint32_t)row, c2, c3, k0, k1);
@@ -252,33 +303,6 @@ __device__ __forceinline__ double block_sum_ordered(double v, double* s_warp) {
     return tot;
 }
 
-// exp(x) for x <= 0 in fp64 by table and polynomial: x = (64 m + j) ln2/64 + r with |r| <= ln2/128,
-// exp(x) = 2^m * 2^(j/64) * e^r; the 64 table entries are correctly rounded doubles made on the host,
-// e^r is its Taylor series to r^5 (remainder below 4e-17), 2^m goes through the exponent field.
-// Relative error about 3e-16.  Below -708 the result is 0 (under the smallest normal number).
-__constant__ double c_exp2_table[64];
-__device__ __forceinline__ void exp_table_to_shared(double* s_tab) {
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) s_tab[i] = c_exp2_table[i];
-    __syncthreads();
-}
-__device__ __forceinline__ double exp_neg(double x, const double* __restrict__ s_tab) {
-    if (!(x > -708.0)) return 0.0;
-    const double nf = rint(x * 92.33248261689366);           // 64 / ln 2
-    double r = fma(-nf, 0.01083042468962958, x);              // ln 2 / 64, high part (low 22 bits clear: nf * high is exact)
-    r = fma(-nf, 6.619564634077006e-12, r);                   // ln 2 / 64, low part
-    const int n = (int)nf;
-    double p = 1.0 / 120.0;
-    p = fma(p, r, 1.0 / 24.0);
-    p = fma(p, r, 1.0 / 6.0);
-    p = fma(p, r, 0.5);
-    p = fma(p, r, 1.0);
-    p *= r;                                                   // e^r - 1
-    const double tj = s_tab[n & 63];
-    const double v = fma(tj, p, tj);
-    const long long bits = __double_as_longlong(v) + ((long long)(n >> 6) << 52);   // m >= -1022: stays a normal number
-    return __longlong_as_double(bits);
-}
-
 // eight consecutive logits of a vector (two 16-byte loads when the vector allows it); past V: -inf
 __device__ __forceinline__ void load8(const float* __restrict__ src, int e0, int V, bool vec, float (&v)[8]) {
     if (vec && e0 + 7 < V) {
@@ -291,27 +315,25 @@ __device__ __forceinline__ void load8(const float* __restrict__ src, int e0, int
     }
 }
 
-struct ResidualCtx {
-    const float* t; const float* d; const double* tab;
-    double max_t, max_q, invT, inv_zt, inv_zq;
-    int mode, x;
-};
-__device__ __forceinline__ double residual_at(const ResidualCtx& c, int e) {
-    const double p = exp_neg(((double)c.t[e] - c.max_t) * c.invT, c.tab) * c.inv_zt;
-    if (c.mode == MODE_TARGET_ONLY) return p;
-    const double q = c.mode == MODE_RESID_POINT ? (e == c.x ? 1.0 : 0.0)
-                                                : exp_neg(((double)c.d[e] - c.max_q) * c.invT, c.tab) * c.inv_zq;
-    const double r = p - q;
-    return r > 0.0 ? r : 0.0;
+// The residual max(0, p - q) of an entry up to a positive factor that is the same for the whole row (the pick
+// compares sums with u2 times their total): Zp Zq (et / Zp - ed / Zq) for two laws, Zp (et / Zp - [e == x]) against
+// a point mass, et for the target law itself.  et and ed are exp((logit - max) / T).
+__device__ __forceinline__ double residual_from(int mode, double et, double ed, double Zp, double Zq, bool at_x) {
+    if (mode == MODE_TARGET_ONLY) return et;
+    const double a = mode == MODE_RESID_POINT ? et : et * Zq;
+    const double b = mode == MODE_RESID_POINT ? (at_x ? Zp : 0.0) : ed * Zp;
+    return a > b ? a - b : 0.0;
 }
 
+struct ResidualCtx {
+    const float* t; const float* d; const double* tab;
+    double max_t, max_q, invT, Zp, Zq;
+    int mode, x;
+};
 __device__ __forceinline__ double residual_of(const ResidualCtx& c, int e, float tv, float dv) {
-    const double p = exp_neg(((double)tv - c.max_t) * c.invT, c.tab) * c.inv_zt;
-    if (c.mode == MODE_TARGET_ONLY) return p;
-    const double q = c.mode == MODE_RESID_POINT ? (e == c.x ? 1.0 : 0.0)
-                                                : exp_neg(((double)dv - c.max_q) * c.invT, c.tab) * c.inv_zq;
-    const double r = p - q;
-    return r > 0.0 ? r : 0.0;
+    const double et = exp_neg(((double)tv - c.max_t) * c.invT, c.tab);
+    const double ed = c.mode == MODE_RESID_LOGITS ? exp_neg(((double)dv - c.max_q) * c.invT, c.tab) : 0.0;
+    return residual_from(c.mode, et, ed, c.Zp, c.Zq, e == c.x);
 }
 
 // pass 1: per-chunk sums of exp((t - max_t)/T) and exp((d - max_q)/T)
@@ -395,7 +417,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
     c.t = tl + ((long long)row * (k + 1) + ri.n) * V;
     c.d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
     c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature;
-    c.inv_zt = 1.0 / Zp; c.inv_zq = Zq > 0.0 ? 1.0 / Zq : 0.0;
+    c.Zp = Zp; c.Zq = Zq;
     c.mode = ri.mode; c.x = ri.x; c.tab = s_tab;
     {
         const int e0 = chunk * RS_CHUNK + threadIdx.x * RS_PER_THREAD;
@@ -432,7 +454,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         for (int c0 = 0; c0 < nchunk; c0 += RS_THREADS) {
             const int ch = c0 + threadIdx.x;
             double mval = 0.0;
-            if (ch < nchunk) mval = empty ? zrow[ch].x * c.inv_zt : __ldcg(rrow + ch);
+            if (ch < nchunk) mval = empty ? zrow[ch].x : __ldcg(rrow + ch);
             s_mass[threadIdx.x] = mval;
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -453,7 +475,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
                 s_empty = is_empty ? 1 : 0;
                 if (is_empty) {   // empty residual: fall back to the target law itself
                     acc = 0.0;
-                    for (int ch = 0; ch < nchunk; ++ch) acc += zrow[ch].x * c.inv_zt;
+                    for (int ch = 0; ch < nchunk; ++ch) acc += zrow[ch].x;
                 }
                 s_S = acc;
             } else {
@@ -478,7 +500,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         const int e = e0 + j;
         r[j] = 0.0;
         if (e < V) {
-            r[j] = residual_at(c, e);
+            r[j] = residual_of(c, e, c.t[e], c.d ? c.d[e] : 0.f);
             if (r[j] > 0.0) my_last = e;
         }
         local += r[j];
@@ -607,16 +629,9 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
     double Zp = 0.0, Zq = 0.0;
     for (int c = 0; c < csize; ++c) { Zp += cluster_read_f64(&s_ex[0], (uint32_t)c); Zq += cluster_read_f64(&s_ex[1], (uint32_t)c); }
     cluster_sync_all();                               // everyone has read before s_ex is reused
-    ResidualCtx cx;
-    cx.t = nullptr; cx.d = nullptr; cx.tab = s_tab; cx.max_t = ri.max_t; cx.max_q = ri.max_q; cx.invT = invT;
-    cx.inv_zt = 1.0 / Zp; cx.inv_zq = Zq > 0.0 ? 1.0 / Zq : 0.0; cx.mode = ri.mode; cx.x = ri.x;
+    const int xn = ri.x;
     auto resid = [&](int j, int mode) -> double {
-        if (e0 + j >= V) return 0.0;
-        const double p = et[j] * cx.inv_zt;
-        if (mode == MODE_TARGET_ONLY) return p;
-        const double q = mode == MODE_RESID_POINT ? (e0 + j == cx.x ? 1.0 : 0.0) : ed[j] * cx.inv_zq;
-        const double r = p - q;
-        return r > 0.0 ? r : 0.0;
+        return e0 + j < V ? residual_from(mode, et[j], ed[j], Zp, Zq, e0 + j == xn) : 0.0;
     };
     // ---- second exchange: masses (a second time with the target law itself if the residual is empty)
     int mode = ri.mode;
@@ -685,7 +700,7 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
 //             exponentials stay in registers; normalisers and masses are exchanged the same way, and the warp
 //             whose stretch holds u2 * S walks it 32 entries at a time.
 // These calls are bound by the chain of dependent steps, not by bytes: one row, k = 4, V = 32000 (1.15 MB)
-// took 23.3 us as stats (36 busy warps), decide and resample kernels, 17.2 us as one.  Sums have a fixed order.
+// took 23.3 us as stats (36 busy warps), decide and resample kernels, 14.2 us as one (statistics 5, exchange and tests 3, resample 5).  Sums have a fixed order.
 // ---------------------------------------------------------------------------------------------
 constexpr int AR_THREADS = 1024, AR_WARPS = AR_THREADS / 32, AR_MAXC = 16;
 constexpr int AR_TASKS = 2 * MAX_K + 1 + AR_WARPS;
@@ -699,25 +714,6 @@ __device__ __forceinline__ StatPartial cluster_read_stat(const StatPartial* loca
     p.mx = __uint_as_float(w0); p.sum = __uint_as_float(w1); p.arg = (int)w2; p.pad = (int)w3;
     return p;
 }
-// a later piece (larger indices) joins the running (max, sum, arg-max)
-__device__ __forceinline__ void merge_stat(float& mx, float& z, int& arg, const StatPartial& q, float invT) {
-    if (q.mx > mx) {
-        z = (mx > -INFINITY ? z * __expf((mx - q.mx) * invT) : 0.f) + q.sum;
-        mx = q.mx; arg = q.arg;
-    } else if (q.mx > -INFINITY) {
-        z += q.sum * __expf((q.mx - mx) * invT);
-    }
-}
-
-// ordered sum of the warps' values; valid in every thread
-__device__ __forceinline__ double ar_block_sum(double v, double* s_warp) {
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
-    __syncthreads();
-    return warp_sum(s_warp[threadIdx.x & 31]);
-}
-
 template <bool VEC, int PER>
 __global__ void __launch_bounds__(AR_THREADS, 1)
 accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, const int* __restrict__ onehot,
@@ -727,7 +723,7 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
     __shared__ StatPartial s_own[2 * MAX_K + 1];       // this CTA's slice of every vector
     __shared__ float s_mx[2 * MAX_K + 1], s_z[2 * MAX_K + 1];
     __shared__ int s_arg[2 * MAX_K + 1], s_acc[MAX_K + 1], s_point[MAX_K + 1], s_x[MAX_K + 1];
-    __shared__ double s_u2[MAX_K + 1], s_ex[5], s_warp[AR_WARPS], s_tab[64];
+    __shared__ double s_u2[MAX_K + 1], s_ex[4], s_warp[AR_WARPS], s_warp2[AR_WARPS], s_tab[64];
     const int row = blockIdx.x / csize, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank();
     const bool greedy = temperature == 0.f;
@@ -801,20 +797,19 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
         s_own[tid] = q;
     }
     cluster_sync_all();
-    if (tid < nvec) {
-        StatPartial q[AR_MAXC];
-#pragma unroll
-        for (int c = 0; c < AR_MAXC; ++c)
-            if (c < csize) q[c] = cluster_read_stat(&s_own[tid], (uint32_t)c);
-        float mx = -INFINITY, z = 0.f;
-        int arg = 0x7fffffff;
-#pragma unroll
-        for (int c = 0; c < AR_MAXC; ++c)
-            if (c < csize) merge_stat(mx, z, arg, q[c], invT);
-        s_mx[tid] = mx; s_z[tid] = z; s_arg[tid] = arg;
+    // (16 lanes a vector, one CTA's result each: a thread that walked the CTAs took 0.9 us longer)
+#pragma unroll 1
+    for (int i0 = 0; i0 < nvec; i0 += AR_THREADS / AR_MAXC) {
+        const int i = i0 + tid / AR_MAXC, l = tid % AR_MAXC;
+        StatPartial a;
+        a.mx = -INFINITY; a.sum = 0.f; a.arg = 0x7fffffff; a.pad = 0;
+        if (i < nvec && l < csize) a = cluster_read_stat(&s_own[i], (uint32_t)l);
+        merge_stat_lanes<AR_MAXC>(a, invT);
+        if (i < nvec && l == 0) { s_mx[i] = a.mx; s_z[i] = a.sum; s_arg[i] = a.arg; }
     }
     __syncthreads();
     // ---- the accept tests of all positions at once
+    const double inv_temp = 1.0 / (double)temperature;
     if (tid <= k) {
         bool accept = false;
         double u2 = 0.0;
@@ -824,12 +819,8 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
             const Philox4 r = philox4x32_10((uint32_t)tid, (uint32_t)row, (uint32_t)step, (uint32_t)(step >> 32), (uint32_t)seed,
                                             (uint32_t)(seed >> 32));
             u2 = word_uniform(r.w[1]);
-            if (tid < k && !bad) {
-                const double T = (double)temperature;
-                const double px = exp(((double)tx - (double)s_mx[tid]) / T) / (double)s_z[tid];
-                const double qx = point ? 1.0 : exp(((double)dx - (double)s_mx[k + 1 + tid]) / T) / (double)s_z[k + 1 + tid];
-                accept = word_uniform(r.w[0]) * qx < (point ? 1.0 : (double)lenience) * px;   // no lenience for the statistical drafter's tokens (Appendix B)
-            }
+            if (tid < k && !bad) accept = accept_test(word_uniform(r.w[0]), tx, s_mx[tid], s_z[tid], point, dx, point ? 0.f : s_mx[k + 1 + tid],
+                                                      point ? 1.f : s_z[k + 1 + tid], inv_temp, lenience, s_tab);
         }
         if (tid < k && bad && rank == 0) set_status(status, CSD_ERR_BAD_TOKEN);
         s_acc[tid] = accept ? 1 : 0; s_point[tid] = point ? 1 : 0; s_x[tid] = bad ? 0 : x; s_u2[tid] = u2;
@@ -846,7 +837,7 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
         return;
     }
     // ---- resample at position n
-    const double inv_temp = 1.0 / (double)temperature, max_t = (double)s_mx[n];
+    const double max_t = (double)s_mx[n];
     int mode = n == k ? MODE_TARGET_ONLY : (s_point[n] ? MODE_RESID_POINT : MODE_RESID_LOGITS);
     const double max_q = mode == MODE_RESID_LOGITS ? (double)s_mx[k + 1 + n] : 0.0, u2 = s_u2[n];
     const int xn = s_x[n];
@@ -871,26 +862,28 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
     double sp = 0.0, sq = 0.0;
 #pragma unroll
     for (int j = 0; j < PER; ++j) { sp += et[j]; sq += ed[j]; }
-    sp = ar_block_sum(sp, s_warp);
-    if (d) sq = ar_block_sum(sq, s_warp);
-    if (tid == 0) { s_ex[0] = sp; s_ex[1] = sq; }
+    sp = warp_sum(sp); sq = warp_sum(sq);
+    if (lane == 0) { s_warp[warp] = sp; s_warp2[warp] = sq; }
+    __syncthreads();
+    if (warp == 0) {
+        sp = warp_sum(s_warp[lane]); sq = warp_sum(s_warp2[lane]);
+        if (lane == 0) { s_ex[0] = sp; s_ex[1] = sq; }
+    }
     cluster_sync_all();
     double Zp = 0.0, Zq = 0.0;
     {
-        const double a = lane < csize ? cluster_read_f64(&s_ex[0], (uint32_t)lane) : 0.0;
-        const double c = lane < csize ? cluster_read_f64(&s_ex[1], (uint32_t)lane) : 0.0;
-        Zp = warp_sum(a); Zq = warp_sum(c);
+        // (lanes 0-15 read the CTAs' Zp, lanes 16-31 their Zq)
+        double a = lane % AR_MAXC < csize ? cluster_read_f64(&s_ex[lane / AR_MAXC], (uint32_t)(lane % AR_MAXC)) : 0.0;
+#pragma unroll
+        for (int o = AR_MAXC / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        Zp = __shfl_sync(0xffffffffu, a, 0); Zq = __shfl_sync(0xffffffffu, a, AR_MAXC);
     }
-    const double inv_zt = 1.0 / Zp, inv_zq = Zq > 0.0 ? 1.0 / Zq : 0.0;
     auto resid = [&](int j) -> double {
-        if (e0 + 32 * j >= hi) return 0.0;
-        const double pv = et[j] * inv_zt;
-        if (mode == MODE_TARGET_ONLY) return pv;
-        const double qv = mode == MODE_RESID_POINT ? (e0 + 32 * j == xn ? 1.0 : 0.0) : ed[j] * inv_zq;
-        return pv > qv ? pv - qv : 0.0;
+        return e0 + 32 * j < hi ? residual_from(mode, et[j], ed[j], Zp, Zq, e0 + 32 * j == xn) : 0.0;
     };
-    double mass_w = 0.0, before = 0.0, total = 0.0;    // this warp's mass, the mass before its stretch, the row's
-    int last_rank = 0;
+    double mass_w = 0.0, run = 0.0, head = 0.0, total = 0.0;   // this warp's mass, the masses up to its end, before this CTA, all
+    int owner = 0, forced = 0;
+    double target = 0.0;
     // (a second time with the target law itself if the residual is empty)
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
@@ -901,77 +894,62 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
         __syncthreads();
         if (lane == 0) s_warp[warp] = mass_w;
         __syncthreads();
-        double run = s_warp[lane];                     // inclusive prefix over the warps
+        run = s_warp[lane];                            // inclusive prefix over the warps, lane = warp
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const double up = __shfl_up_sync(0xffffffffu, run, o);
             if (lane >= o) run += up;
         }
         if (tid == AR_THREADS - 1) s_ex[2 + pass] = run;
-        before = warp > 0 ? __shfl_sync(0xffffffffu, run, (warp + 31) & 31) : 0.0;
         cluster_sync_all();
-        double m = lane < csize ? cluster_read_f64(&s_ex[2 + pass], (uint32_t)lane) : 0.0, incl = m;
+        const double m = lane < csize ? cluster_read_f64(&s_ex[2 + pass], (uint32_t)lane) : 0.0;
+        double incl = m;                               // inclusive prefix over the CTAs, lane = CTA
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const double up = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += up;
         }
         total = __shfl_sync(0xffffffffu, incl, csize - 1);
-        if (!(total > 0.0) || !isfinite(total)) {
-            if (pass == 0 && mode != MODE_TARGET_ONLY) { mode = MODE_TARGET_ONLY; continue; }
-        }
-        const double head = __shfl_sync(0xffffffffu, incl - m, rank);         // mass before this CTA
+        if (pass == 0 && mode != MODE_TARGET_ONLY && (!(total > 0.0) || !isfinite(total))) { mode = MODE_TARGET_ONLY; continue; }
+        // the CTA whose masses reach past u2 * total; rounding may leave none, then the last one that carries mass
+        target = u2 * total;
+        const unsigned past = __ballot_sync(0xffffffffu, lane < csize && incl > target);
         const unsigned some = __ballot_sync(0xffffffffu, m > 0.0);
-        last_rank = some ? 31 - __clz(some) : 0;
-        before += head;
+        forced = past == 0;
+        owner = past ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
+        head = __shfl_sync(0xffffffffu, incl - m, rank);
         break;
     }
-    // ---- the entry: smallest index whose cumulative mass exceeds u2 * total; rounding may leave none, then the
-    //      last entry that carries mass
-    const double target = u2 * total;
-    __shared__ int s_pick, s_last;
-    if (tid == 0) { s_pick = 0x7fffffff; s_last = -1; s_ex[4] = 0.0; }
-    __syncthreads();
-    // (only the stretches around the target are walked: the warp whose prefix interval holds it, and its neighbours
-    // in case rounding moved the boundary)
-    if (before <= target * (1.0 + 1e-12) && before + mass_w >= target * (1.0 - 1e-12)) {
-        double cum = before;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has read what it needs of the others
+    if (rank == owner) {
+        // ---- in it the warp (all lanes of all warps know the prefix), then the smallest index whose cumulative mass
+        //      exceeds the target; forced, or where rounding leaves none: the last entry that carries mass
+        const unsigned past = __ballot_sync(0xffffffffu, head + run > target);
+        const unsigned some = __ballot_sync(0xffffffffu, s_warp[lane] > 0.0);
+        const int wpick = past && !forced ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
+        if (warp == wpick) {
+            double cum = head + __shfl_sync(0xffffffffu, run, (wpick + 31) & 31) * (wpick > 0 ? 1.0 : 0.0);
+            int pick = -1, last = -1;
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const double r = resid(j);
-            double incl = r;
+            for (int j = 0; j < PER; ++j) {
+                const double r = resid(j);
+                double incl = r;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const double up = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += up;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const double up = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += up;
+                }
+                const unsigned hit = __ballot_sync(0xffffffffu, r > 0.0 && cum + incl > target);
+                const unsigned mass = __ballot_sync(0xffffffffu, r > 0.0);
+                const int first = lo + warp * (PER * 32) + 32 * j;
+                if (pick < 0 && hit && !forced) pick = first + __ffs(hit) - 1;
+                if (mass) last = first + 31 - __clz(mass);
+                cum += __shfl_sync(0xffffffffu, incl, 31);
             }
-            const unsigned hit = __ballot_sync(0xffffffffu, r > 0.0 && cum + incl > target);
-            if (hit) {
-                if (lane == 0) atomicMin(&s_pick, lo + warp * (PER * 32) + 32 * j + __ffs(hit) - 1);
-                break;
-            }
-            cum += __shfl_sync(0xffffffffu, incl, 31);
+            if (lane == 0) out_tok[row] = pick >= 0 ? pick : max(last, 0);
         }
     }
-    if (rank == last_rank) {
-        int mine = -1;
-#pragma unroll
-        for (int j = 0; j < PER; ++j)
-            if (resid(j) > 0.0) mine = e0 + 32 * j;
-        mine = __reduce_max_sync(0xffffffffu, mine);
-        if (lane == 0 && mine >= 0) atomicMax(&s_last, mine);
-    }
-    __syncthreads();
-    if (tid == 0) s_ex[4] = s_pick != 0x7fffffff ? (double)s_pick : -1.0 - (double)max(s_last, 0);
-    cluster_sync_all();
-    if (rank == 0 && warp == 0) {
-        // the first CTA (vocabulary order) that found an entry has it
-        const double v = lane < csize ? cluster_read_f64(&s_ex[4], (uint32_t)lane) : -1.0;
-        const unsigned found = __ballot_sync(0xffffffffu, lane < csize && v >= 0.0);
-        const double pick = __shfl_sync(0xffffffffu, v, found ? __ffs(found) - 1 : last_rank);
-        if (lane == 0) out_tok[row] = found ? (int)pick : (int)(-1.0 - pick);
-    }
-    cluster_sync_all();                                // no CTA leaves while its results may still be read
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
 }
 
 struct AcceptLayout {
@@ -1077,8 +1055,10 @@ static csd_status launch_accept_row(const float* tl, const float* dl, const int*
                                     int V, float temperature, float lenience, uint64_t seed, uint64_t step, int csize,
                                     int* n_acc, int* out_tok, int* status, cudaStream_t st, bool* done) {
     *done = false;
-    if (row_clusters<VEC, PER>(csize) < rows) return CSD_OK;
     const int S = ((V + csize - 1) / csize + 3) & ~3, nvec = dl ? 2 * k + 1 : k + 1;
+    // (a CTA takes in about 40 GB/s here: beyond about 320 KB of slices the stats pass over all SMs is faster; one row,
+    // V = 128256: k = 4, 289 KB, 29.6 us against 34.3; k = 8, 545 KB, 35.0 against 34.3)
+    if ((long long)nvec * S * 4 > 320 * 1024 || row_clusters<VEC, PER>(csize) < rows) return CSD_OK;
     int pieces = (AR_WARPS + nvec - 1) / nvec;           // enough pieces for every warp, of at least 1024 logits
     if (pieces > (S + ST_SUB - 1) / ST_SUB) pieces = (S + ST_SUB - 1) / ST_SUB;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
@@ -1119,11 +1099,11 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     const bool vec_ok = (V % 4 == 0) && (((uintptr_t)tl & 15) == 0) && (!use_d || ((uintptr_t)dl & 15) == 0);
     // One kernel while its clusters are all resident; smallest power of two that leaves a CTA at most
     // 4096 entries (8192 beyond 32768), doubled while that leaves it 512 and the rows still fit.
+    if (!greedy) {
+        const csd_status ts = exp_table_ready();
+        if (ts != CSD_OK) return ts;
+    }
     if (V <= AR_MAXC * 8192) {
-        if (!greedy) {
-            const csd_status ts = exp_table_ready();
-            if (ts != CSD_OK) return ts;
-        }
         int csize = 1;
         while (csize < 8 && (V + csize - 1) / csize > 4096) csize *= 2;
         if (V > 8 * 8192) csize = 16;
@@ -1152,17 +1132,13 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
             CSD_CUDA(cudaLaunchKernelEx(&ls.cfg, accept_stats_kernel<true>, tl, dl, n_tvec, V, invT, greedy_i, part, L.nchunk_a, items));
         else
             CSD_CUDA(cudaLaunchKernelEx(&ls.cfg, accept_stats_kernel<false>, tl, dl, n_tvec, V, invT, greedy_i, part, L.nchunk_a, items));
-        PdlLaunch ld(dim3((unsigned)rows), dim3(128), 0, st);
+        PdlLaunch ld(dim3((unsigned)rows), dim3(DC_THREADS), 0, st);
         CSD_CUDA(cudaLaunchKernelEx(&ld.cfg, accept_decide_kernel, tl, dl, (const int*)onehot, (const int*)tokens, rows, k, V,
                                     temperature, lenience, seed, step, (const StatPartial*)part, L.nchunk_a, (int*)n_acc,
                                     (int*)out_tok, info, tickets, status));
     }
     count_launch(2);
     const int csize = (V + RF_SLICE - 1) / RF_SLICE;
-    if (!greedy) {
-        const csd_status ts = exp_table_ready();
-        if (ts != CSD_OK) return ts;
-    }
     if (!greedy && fused_resample_ok(csize)) {  // a row fits one cluster: the fused resample kernel
         cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
         cudaLaunchAttribute attr[2];
