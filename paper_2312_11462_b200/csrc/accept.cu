@@ -23,8 +23,7 @@ constexpr int ST_THREADS = 256;
 constexpr int ST_CHUNK = 8192;   // logits per warp item of the stats pass
 constexpr int ST_SUB = 1024;     // logits a warp has in registers at a time (8 x float4 per lane)
 constexpr int RS_THREADS = 256;
-constexpr int RS_PER_THREAD = 8;
-constexpr int RS_CHUNK = RS_THREADS * RS_PER_THREAD;  // logits per CTA of the resample pass
+constexpr int RS_CHUNK = 512;    // logits per warp of the resample passes: 8 neighbours a lane, twice
 
 struct __align__(16) StatPartial {
     float mx;
@@ -289,20 +288,13 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 }
 
 // ---------------------------------------------------------------------------------------------
-// resample passes (fp64).  grid = (rows, chunks).  Every sum has one fixed order: lanes by
-// xor-shuffle, warps in index order, chunks in index order.
+// resample passes (fp64).  A WARP owns a chunk of 512 logits of a row (8 neighbours a lane, twice, all
+// requested at once); no block-wide synchronisation.  The fp64 pipe (about 13
+// instructions an exponential) needs 12 us a pass at 64 rows and V = 128256, the table reads from shared memory as
+// much; measured 30 and 46 us (a block of 256 threads per chunk with barriers: 38 and 54 us; 2048 logits a warp: 43
+// and 58; persistent blocks with a conflict-free copy of the table per lane: 35 and 91, the picks wait).
+// Every sum has one fixed order: a lane's entries, lanes by xor-shuffle or prefix scan, chunks in index order.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ double block_sum_ordered(double v, double* s_warp) {
-    v = warp_sum(v);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) s_warp[warp] = v;
-    __syncthreads();
-    double tot = 0.0;
-    for (int w = 0; w < RS_THREADS / 32; ++w) tot += s_warp[w];
-    return tot;
-}
-
 // eight consecutive logits of a vector (two 16-byte loads when the vector allows it); past V: -inf
 __device__ __forceinline__ void load8(const float* __restrict__ src, int e0, int V, bool vec, float (&v)[8]) {
     if (vec && e0 + 7 < V) {
@@ -336,200 +328,183 @@ __device__ __forceinline__ double residual_of(const ResidualCtx& c, int e, float
     return residual_from(c.mode, et, ed, c.Zp, c.Zq, e == c.x);
 }
 
-// pass 1: per-chunk sums of exp((t - max_t)/T) and exp((d - max_q)/T)
-__global__ void __launch_bounds__(RS_THREADS)
-resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int k, int V, float temperature,
+__device__ __forceinline__ double warp_scan(double v, int lane) {      // inclusive prefix
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double up = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += up;
+    }
+    return v;
+}
+// one warp of a row's chunks has finished: true in the whole warp for the last of them
+__device__ __forceinline__ bool last_of_row(unsigned* ticket, int nchunk, int lane) {
+    unsigned old = 0;
+    if (lane == 0) {
+        __threadfence();
+        old = atomicAdd(ticket, 1u);
+    }
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (old != (unsigned)nchunk - 1u) return false;
+    __threadfence();
+    return true;
+}
+
+// pass 1: per-chunk sums of exp((t - max_t)/T) and exp((d - max_q)/T), and their totals
+__global__ void __launch_bounds__(RS_THREADS, 3)
+resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
                   const RowInfo* __restrict__ info, double2* __restrict__ zpart, double2* __restrict__ zsum,
                   unsigned* __restrict__ tickets, int nchunk) {
-    const int row = blockIdx.x, chunk = blockIdx.y;
-    __shared__ double s_warp[RS_THREADS / 32];
     __shared__ double s_tab[64];
     exp_table_to_shared(s_tab);
     pdl_wait();            // the row records come from the decide pass
     pdl_trigger();
+    const int lane = threadIdx.x & 31;
+    const long long item = (long long)blockIdx.x * (RS_THREADS / 32) + (threadIdx.x >> 5);
+    const int row = (int)(item / nchunk), chunk = (int)(item % nchunk);
+    if (row >= rows) return;
     const RowInfo ri = info[row];
-    if (ri.mode == MODE_DONE) return;
     const double invT = 1.0 / (double)temperature;
     const float* t = tl + ((long long)row * (k + 1) + ri.n) * V;
     const float* d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
-    const int e0 = chunk * RS_CHUNK + threadIdx.x * RS_PER_THREAD;
+    const bool vec = (V % 4 == 0) && ((((uintptr_t)t) & 15) == 0) && (!d || (((uintptr_t)d) & 15) == 0);
+    const int e0 = chunk * RS_CHUNK + lane * 8;
     double sp = 0.0, sq = 0.0;
-    {
-        static_assert(RS_PER_THREAD == 8, "load8 covers a thread's entries");
-        const bool vec = (V % 4 == 0) && ((((uintptr_t)t) & 15) == 0) && (!d || (((uintptr_t)d) & 15) == 0);
-        float tv[8], dv[8];
-        load8(t, e0, V, vec, tv);
-        if (d) load8(d, e0, V, vec, dv);
+    float tv[2][8], dv[2][8];
 #pragma unroll
-        for (int j = 0; j < RS_PER_THREAD; ++j) {
-            sp += exp_neg(((double)tv[j] - ri.max_t) * invT, s_tab);      // -inf (past V) gives 0
-            if (d) sq += exp_neg(((double)dv[j] - ri.max_q) * invT, s_tab);
-        }
+    for (int h = 0; h < 2; ++h) {
+        load8(t, e0 + h * 256, V, vec, tv[h]);
+        if (d) load8(d, e0 + h * 256, V, vec, dv[h]);
     }
-    sp = block_sum_ordered(sp, s_warp);
-    sq = block_sum_ordered(sq, s_warp);
-    __shared__ int s_is_last;
-    __shared__ double2 s_z[RS_THREADS];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sp += exp_neg(((double)tv[h][j] - ri.max_t) * invT, s_tab);      // -inf (past V) gives 0
+    if (d) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sq += exp_neg(((double)dv[h][j] - ri.max_q) * invT, s_tab);
+    }
+    sp = warp_sum(sp);
+    sq = warp_sum(sq);
     double2* zrow = zpart + (long long)row * nchunk;
-    if (threadIdx.x == 0) {
-        zrow[chunk] = make_double2(sp, sq);
-        __threadfence();
-        s_is_last = atomicAdd(&tickets[row], 1u) == (unsigned)nchunk - 1u;
-    }
-    __syncthreads();
-    if (!s_is_last) return;
-    // last chunk of the row: the totals, summed in chunk order (loads in parallel, adds by one thread)
-    __threadfence();
-    double Zp = 0.0, Zq = 0.0;
-    for (int c0 = 0; c0 < nchunk; c0 += RS_THREADS) {
-        const int c = c0 + threadIdx.x;
-        s_z[threadIdx.x] = c < nchunk ? make_double2(__ldcg(&zrow[c].x), __ldcg(&zrow[c].y)) : make_double2(0.0, 0.0);
-        __syncthreads();
-        if (threadIdx.x == 0)
-            for (int i = 0; i < RS_THREADS && c0 + i < nchunk; ++i) { Zp += s_z[i].x; Zq += s_z[i].y; }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) zsum[row] = make_double2(Zp, Zq);
+    if (lane == 0) zrow[chunk] = make_double2(sp, sq);
+    if (!last_of_row(&tickets[row], nchunk, lane)) return;
+    sp = sq = 0.0;
+    for (int c = lane; c < nchunk; c += 32) { sp += __ldcg(&zrow[c].x); sq += __ldcg(&zrow[c].y); }
+    sp = warp_sum(sp);
+    sq = warp_sum(sq);
+    if (lane == 0) zsum[row] = make_double2(sp, sq);
 }
 
-// pass 2: per-chunk mass of the residual; the CTA that arrives last at the row's ticket picks the token
-__global__ void __launch_bounds__(RS_THREADS)
-resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int k, int V, float temperature,
+// pass 2: per-chunk mass of the residual; the warp that arrives last at the row's ticket picks the token
+__global__ void __launch_bounds__(RS_THREADS, 3)
+resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
                      const RowInfo* __restrict__ info, const double2* __restrict__ zpart,
                      const double2* __restrict__ zsum, double* __restrict__ rpart, unsigned* __restrict__ tickets,
                      int nchunk, int* __restrict__ out_tok) {
-    const int row = blockIdx.x, chunk = blockIdx.y;
-    pdl_wait();            // the normalisers come from the pass before this one
-    pdl_trigger();
-    const RowInfo ri = info[row];
-    if (ri.mode == MODE_DONE) return;
-    __shared__ double s_warp[RS_THREADS / 32];
-    __shared__ double s_scan[RS_THREADS / 32];
-    __shared__ double s_d[2];    // target, base
-    __shared__ int s_i[3];       // chunk, mode, forced-last flag
-    __shared__ int s_pick, s_last, s_is_last;
     __shared__ double s_tab[64];
     exp_table_to_shared(s_tab);
+    pdl_wait();            // the normalisers come from the pass before this one
+    pdl_trigger();
+    const int lane = threadIdx.x & 31;
+    const long long item = (long long)blockIdx.x * (RS_THREADS / 32) + (threadIdx.x >> 5);
+    const int row = (int)(item / nchunk), chunk = (int)(item % nchunk);
+    if (row >= rows) return;
+    const RowInfo ri = info[row];
     const double2* zrow = zpart + (long long)row * nchunk;
     double* rrow = rpart + (long long)row * nchunk;
-    const double Zp = zsum[row].x, Zq = zsum[row].y;
     ResidualCtx c;
     c.t = tl + ((long long)row * (k + 1) + ri.n) * V;
     c.d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
     c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature;
-    c.Zp = Zp; c.Zq = Zq;
+    c.Zp = zsum[row].x; c.Zq = zsum[row].y;
     c.mode = ri.mode; c.x = ri.x; c.tab = s_tab;
+    const bool vec = (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
     {
-        const int e0 = chunk * RS_CHUNK + threadIdx.x * RS_PER_THREAD;
-        const bool vec = (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
-        float tv[8], dv[8];
-        load8(c.t, e0, V, vec, tv);
-        if (c.d) load8(c.d, e0, V, vec, dv);
+        const int e0 = chunk * RS_CHUNK + lane * 8;
         double sr = 0.0;
+        float tv[2][8], dv[2][8];
 #pragma unroll
-        for (int j = 0; j < RS_PER_THREAD; ++j)
-            if (e0 + j < V) sr += residual_of(c, e0 + j, tv[j], c.d ? dv[j] : 0.f);
-        sr = block_sum_ordered(sr, s_warp);
-        if (threadIdx.x == 0) {
-            rrow[chunk] = sr;
-            __threadfence();
-            s_is_last = atomicAdd(&tickets[row], 1u) == (unsigned)nchunk - 1u;
+        for (int h = 0; h < 2; ++h) {
+            load8(c.t, e0 + h * 256, V, vec, tv[h]);
+            if (c.d) load8(c.d, e0 + h * 256, V, vec, dv[h]);
         }
-        __syncthreads();
-        if (!s_is_last) return;
-        __threadfence();
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sr += residual_of(c, e0 + h * 256 + j, tv[h][j], c.d ? dv[h][j] : 0.f);   // past V: et is 0
+        sr = warp_sum(sr);
+        if (lane == 0) rrow[chunk] = sr;
     }
-    // ---- last CTA of the row: which chunk holds u2 * S, then the entry inside it.  Chunk masses are
-    //      fetched by all threads into shared memory; one thread adds them in chunk order.
-    __shared__ double s_mass[RS_THREADS];
-    __shared__ double s_S;
-    __shared__ int s_empty;
+    if (!last_of_row(&tickets[row], nchunk, lane)) return;
+    // ---- which chunk holds u2 * S: a lane owns neighbouring chunks; a second time with the target law itself if the
+    //      residual is empty.  Rounding may leave none, then the last chunk that carries mass.
+    const int each = (nchunk + 31) / 32, c_lo = min(nchunk, lane * each), c_hi = min(nchunk, c_lo + each);
+    double mine = 0.0, incl = 0.0, S = 0.0;
+    auto mass_of = [&](int ch) -> double { return c.mode == MODE_TARGET_ONLY ? __ldcg(&zrow[ch].x) : __ldcg(rrow + ch); };
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-        // pass 0: total mass S (and whether the residual is empty); pass 1: the chunk that holds u2 * S
-        const bool empty = pass == 1 && s_empty;
-        double acc = 0.0, target = 0.0;
-        int pick_chunk = -1, last_pos = 0;
-        double base = 0.0;
-        if (pass == 1) target = ri.u2 * s_S;
-        for (int c0 = 0; c0 < nchunk; c0 += RS_THREADS) {
-            const int ch = c0 + threadIdx.x;
-            double mval = 0.0;
-            if (ch < nchunk) mval = empty ? zrow[ch].x : __ldcg(rrow + ch);
-            s_mass[threadIdx.x] = mval;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                for (int i = 0; i < RS_THREADS && c0 + i < nchunk; ++i) {
-                    const double mass = s_mass[i];
-                    if (pass == 0) { acc += mass; continue; }
-                    if (pick_chunk >= 0) break;
-                    if (mass > 0.0) last_pos = c0 + i;
-                    if (acc + mass > target) { pick_chunk = c0 + i; base = acc; break; }
-                    acc += mass;
-                }
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            if (pass == 0) {
-                const bool is_empty = !(acc > 0.0) || !isfinite(acc);
-                s_empty = is_empty ? 1 : 0;
-                if (is_empty) {   // empty residual: fall back to the target law itself
-                    acc = 0.0;
-                    for (int ch = 0; ch < nchunk; ++ch) acc += zrow[ch].x;
-                }
-                s_S = acc;
-            } else {
-                int forced = 0;
-                if (pick_chunk < 0) { pick_chunk = last_pos; forced = 1; }
-                s_d[0] = target; s_d[1] = base;
-                s_i[0] = pick_chunk; s_i[1] = s_empty ? (int)MODE_TARGET_ONLY : ri.mode; s_i[2] = forced;
-                s_pick = 0x7fffffff; s_last = -1;
-            }
-        }
-        __syncthreads();
+        mine = 0.0;
+        for (int ch = c_lo; ch < c_hi; ++ch) mine += mass_of(ch);
+        incl = warp_scan(mine, lane);
+        S = __shfl_sync(0xffffffffu, incl, 31);
+        if (pass == 0 && c.mode != MODE_TARGET_ONLY && (!(S > 0.0) || !isfinite(S))) { c.mode = MODE_TARGET_ONLY; continue; }
+        break;
     }
-    const double target = s_d[0], base = s_d[1];
-    const int pick_chunk = s_i[0], forced = s_i[2];
-    c.mode = s_i[1];
-    const int e0 = pick_chunk * RS_CHUNK + threadIdx.x * RS_PER_THREAD;
-    double r[RS_PER_THREAD];
-    double local = 0.0;
-    int my_last = -1;
+    const double target = ri.u2 * S;
+    const unsigned past = __ballot_sync(0xffffffffu, incl > target), some = __ballot_sync(0xffffffffu, mine > 0.0);
+    const bool forced = past == 0;
+    const int src = past ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
+    double cum = incl - mine;
+    int pick_chunk = c_lo;
+    if (lane == src) {
+        int last_pos = c_lo, hit = -1;
+        for (int ch = c_lo; ch < c_hi; ++ch) {
+            const double m = mass_of(ch);
+            if (m > 0.0) last_pos = ch;
+            if (!forced && cum + m > target) { hit = ch; break; }
+            cum += m;
+        }
+        if (hit < 0) {                                  // the last chunk with mass, from its own start
+            hit = last_pos;
+            cum = incl - mine;
+            for (int ch = c_lo; ch < last_pos; ++ch) cum += mass_of(ch);
+        }
+        pick_chunk = hit;
+    }
+    pick_chunk = __shfl_sync(0xffffffffu, pick_chunk, src);
+    cum = __shfl_sync(0xffffffffu, cum, src);
+    // ---- the entry: smallest index whose cumulative mass exceeds the target, else the last that carries mass
+    int pick = -1, last = -1;
+#pragma unroll 1
+    for (int e = pick_chunk * RS_CHUNK; e < min(V, (pick_chunk + 1) * RS_CHUNK) && pick < 0; e += 256) {
+        const int at = e + lane * 8;
+        float tv[8], dv[8];
+        load8(c.t, at, V, vec, tv);
+        if (c.mode == MODE_RESID_LOGITS) load8(c.d, at, V, vec, dv);
+        double r[8], local = 0.0;
+        int my_last = -1;
 #pragma unroll
-    for (int j = 0; j < RS_PER_THREAD; ++j) {
-        const int e = e0 + j;
-        r[j] = 0.0;
-        if (e < V) {
-            r[j] = residual_of(c, e, c.t[e], c.d ? c.d[e] : 0.f);
-            if (r[j] > 0.0) my_last = e;
+        for (int j = 0; j < 8; ++j) {
+            r[j] = residual_of(c, at + j, tv[j], c.mode == MODE_RESID_LOGITS ? dv[j] : 0.f);
+            if (r[j] > 0.0) my_last = at + j;
+            local += r[j];
         }
-        local += r[j];
-    }
-    // exclusive prefix of the per-thread sums, in thread order
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double incl = local;
+        const double in = warp_scan(local, lane);
+        double run = cum + (in - local);
+        int found = 0x7fffffff;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    double woff = 0.0;
-    for (int w = 0; w < warp; ++w) woff += s_scan[w];
-    double cum = base + woff + (incl - local);
-    int found = 0x7fffffff;
-    if (!forced) {
-#pragma unroll
-        for (int j = 0; j < RS_PER_THREAD; ++j) {
-            cum += r[j];
-            if (found == 0x7fffffff && r[j] > 0.0 && cum > target) found = e0 + j;
+        for (int j = 0; j < 8; ++j) {
+            run += r[j];
+            if (!forced && found == 0x7fffffff && r[j] > 0.0 && run > target) found = at + j;
         }
+        found = __reduce_min_sync(0xffffffffu, found);
+        if (found != 0x7fffffff) pick = found;
+        last = max(last, __reduce_max_sync(0xffffffffu, my_last));
+        cum += __shfl_sync(0xffffffffu, in, 31);
     }
-    if (found != 0x7fffffff) atomicMin(&s_pick, found);
-    if (my_last >= 0) atomicMax(&s_last, my_last);
-    __syncthreads();
-    if (threadIdx.x == 0) out_tok[row] = s_pick != 0x7fffffff ? s_pick : (s_last >= 0 ? s_last : 0);
+    if (lane == 0) out_tok[row] = pick >= 0 ? pick : max(last, 0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1152,12 +1127,12 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
                                     (int*)out_tok));
         count_launch();
     } else if (!greedy) {
-        dim3 g2((unsigned)rows, (unsigned)L.nchunk_r);
+        const dim3 g2((unsigned)(((long long)rows * L.nchunk_r + RS_THREADS / 32 - 1) / (RS_THREADS / 32)));
         PdlLaunch lz(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lz.cfg, resample_z_kernel, tl, dl, k, V, temperature, (const RowInfo*)info, zpart, zsum, tickets,
-                                    L.nchunk_r));
+        CSD_CUDA(cudaLaunchKernelEx(&lz.cfg, resample_z_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, zpart, zsum,
+                                    tickets, L.nchunk_r));
         PdlLaunch lp(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, resample_pick_kernel, tl, dl, k, V, temperature, (const RowInfo*)info,
+        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, resample_pick_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info,
                                     (const double2*)zpart, (const double2*)zsum, rpart, tickets + rows, L.nchunk_r, (int*)out_tok));
         count_launch(2);
     }
