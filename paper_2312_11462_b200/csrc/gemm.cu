@@ -20,6 +20,7 @@ constexpr int GW = GT / 32;      // warps per CTA
 constexpr int KSTEP = 256;       // K elements one warp covers per step (32 lanes x 8 bf16)
 constexpr int CTAS_PER_SM = 2;
 constexpr long long AUTO_TC_MIN_WEIGHTS = 1 << 20;   // automatic choice: matrices at least this large go to the tensor-core kernel
+constexpr long long AUTO_ROW_MAX_WORK = 150 << 20;      // weights x rows up to which blocks of up to 8 rows take the row kernel
 constexpr size_t SMEM_BUDGET = 110 * 1024;   // per CTA, so that two CTAs share an SM
 
 template <int M, bool DUAL>
@@ -328,8 +329,19 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual) {
 
 int linear_ticket_count(int N) { return N + 1; }   // one ticket per row group, at least one row each (the wide kernel needs fewer)
 
+// The row kernel (automatic choice only).  Measured back to back, us for row / tensor-core / split-K CUDA-core kernel:
+// 2304 x 768 at 1, 5, 8 rows 1.9 / 7.4 / 2.4, 3.2 / 8.1 / 3.5, 4.1 / 7.6 / 4.2; 768 x 3072 2.4 / 7.6 / 6.2, 4.9 / 8.2 / 8.2,
+// 6.7 / 8.3 / 7.9; 32000 x 768 8.4 / 14.2 / 10.8, 12.0 / 14.3 / 13.9, 17.6 / 14.9 / 17.5 (fp32 FMA and the rows' shared-memory
+// reads bound it from there on); at 17 rows 7.0 / 8.4 / 5.7, 12.3 / 10.6 / 9.6, 36 / 16 / 37, and a 68M-shaped forward
+// is faster on the tensor cores, whose kernels hand each other the rows (108 us against 128 on the CUDA cores).
+static bool linear_uses_rows(int m, int N, int K, bool dual) {
+    return gemm_path() == 0 && m <= 8 && row_supported(m, N, K, dual) &&
+           (long long)N * K * (dual ? 2 : 1) * m <= AUTO_ROW_MAX_WORK;
+}
+
 bool linear_uses_tensor_cores(int m, int N, int K, bool dual) {
     const int path = gemm_path();
+    if (linear_uses_rows(m, N, K, dual)) return false;
     // measured on the 7B layer shapes the tensor-core kernel wins at every m (a 5-row review forward
     // takes 4.0 ms against 5.2 ms, a 17-row one 5.5 ms against 15 ms); tiny matrices stay on the simpler kernel
     return path != 1 && tc_supported(m, N, K, dual) && (path == 2 || (long long)N * K >= AUTO_TC_MIN_WEIGHTS);
@@ -367,6 +379,7 @@ csd_status launch_linear(const LinearArgs& a, cudaStream_t st) {
     if (a.xs && linear_uses_row_ranges(a.m, a.N, a.K, dual)) return launch_linear_rs(a, st);
     if (a.xs && linear_uses_tensor_cores(a.m, a.N, a.K, dual)) return launch_linear_tc(a, st);
     if ((((uintptr_t)a.X) & 15) || (a.ldx & 3)) return CSD_ERR_INVALID_ARG;
+    if (linear_uses_rows(a.m, a.N, a.K, dual) && !a.out_xs && !a.out_ssq) return launch_linear_row(a, st);
     const LinearPlan pl = plan_linear(a.m, a.N, a.K, dual);
     if (pl.kslices > 1 && (!a.partial || !a.tickets)) return CSD_ERR_INVALID_ARG;
     GemmParams gp;

@@ -11,6 +11,10 @@ int tc_ticket_count(int N);
 csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st);
 csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st);   // a.X (times a.gain) -> a.xs, a.ssq
 
+// whole weight rows per warp on the CUDA cores (gemm_row.cu), for the matrices of draft models
+bool row_supported(int m, int N, int K, bool dual);
+csd_status launch_linear_row(const LinearArgs& a, cudaStream_t st);
+
 // row-range variant (gemm_rs.cu): every CTA owns whole output columns, nothing is shared between CTAs
 bool rs_supported(int m, int N, int K, bool dual);
 int rs_ssq_pieces(int m, int N, int K, bool dual);     // sum-of-squares pieces its epilogue writes

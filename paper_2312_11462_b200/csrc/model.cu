@@ -12,18 +12,31 @@ namespace csd {
 // ---------------------------------------------------------------------------------------------
 // small kernels
 // ---------------------------------------------------------------------------------------------
-__global__ void embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict__ E, int V, int d,
+__global__ void __launch_bounds__(128)
+embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict__ E, int V, int d,
                              float* __restrict__ x, int* status) {
     pdl_wait();
     pdl_trigger();
-    const int r = blockIdx.x;
+    const int r = blockIdx.y;
     int t = tokens[r];
     if (t < 0 || t >= V) {
-        if (threadIdx.x == 0) set_status(status, CSD_ERR_BAD_TOKEN);
+        if (threadIdx.x == 0 && blockIdx.x == 0) set_status(status, CSD_ERR_BAD_TOKEN);
         t = 0;
     }
-    const __nv_bfloat16* e = E + (size_t)t * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)r * d + i] = __bfloat162float(e[i]);
+    const int k = (blockIdx.x * 128 + threadIdx.x) * 8;
+    if (k >= d) return;
+    const uint4 e = *reinterpret_cast<const uint4*>(E + (size_t)t * d + k);
+    float* dst = x + (size_t)r * d + k;
+    *reinterpret_cast<float4*>(dst) = make_float4(bf16lo(e.x), bf16hi(e.x), bf16lo(e.y), bf16hi(e.y));
+    *reinterpret_cast<float4*>(dst + 4) = make_float4(bf16lo(e.z), bf16hi(e.z), bf16lo(e.w), bf16hi(e.w));
+}
+
+static csd_status launch_embed(const int32_t* tokens, const __nv_bfloat16* E, int V, int d, int m, float* x, int* status,
+                               cudaStream_t st) {
+    PdlLaunch L(dim3((unsigned)((d + 1023) / 1024), (unsigned)m), dim3(128), 0, st);
+    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_kernel, tokens, E, V, d, x, status));
+    count_launch();
+    return CSD_OK;
 }
 
 // The same gather for a forward whose first projection runs on the tensor cores: besides the fp32 rows it
@@ -401,8 +414,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
     const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, ff = c.d_ff;
     {
         ProfScope ps(M, 2, st);
-        embed_kernel<<<m, 128, 0, st>>>(tokens, M->embed, c.vocab, d, M->wx, M->status);
-        count_launch();
+        CSD_TRY(launch_embed(tokens, M->embed, c.vocab, d, m, M->wx, M->status, st));
     }
     int cnt = 0;                       // pieces in wssq that describe the rows in wxs_x (0: wxs_x not current)
     for (int l = 0; l < c.n_layers; ++l) {
@@ -661,8 +673,7 @@ extern "C" csd_status csd_encoder_forward(csd_model* M, const int32_t* enc_token
     cudaStream_t st = (cudaStream_t)stream;
     const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, E = c.max_enc_len;
     const int CH = 16;
-    embed_kernel<<<n, 128, 0, st>>>(enc_tokens_dev, M->embed, c.vocab, d, M->xenc, M->status);
-    count_launch();
+    CSD_TRY(launch_embed(enc_tokens_dev, M->embed, c.vocab, d, n, M->xenc, M->status, st));
     if (M->wide && gemm_path() != 1 && n > CSD_MAX_ROWS) {      // large model: wide blocks
         CSD_TRY(wide_encoder(M, n, st));
         M->enc_len = n;
@@ -809,10 +820,10 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
                 block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x, M->ssq_x, M->status);
             M->ssq_x_cnt = split_ssq_entries(d);
             x_ready = true;
+            count_launch();
         } else {
-            embed_kernel<<<m, 128, 0, st>>>(block_tokens_dev, M->embed, V, d, M->x, M->status);
+            CSD_TRY(launch_embed(block_tokens_dev, M->embed, V, d, m, M->x, M->status, st));
         }
-        count_launch();
     }
     const int ff = c.d_ff;
     const bool tc_o = linear_uses_tensor_cores(m, d, di, false);
