@@ -327,7 +327,7 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual) {
     return align_up(worst, 256);
 }
 
-int linear_ticket_count(int N) { return N + 1; }   // one ticket per row group, at least one row each (the wide kernel needs fewer)
+int linear_ticket_count(int N) { return N + 8; }   // one per row group of at least one row; four per 128-row tile; the wide kernel needs fewer
 
 // The row kernel (automatic choice only).  Measured back to back, us for row / tensor-core / split-K CUDA-core kernel:
 // 2304 x 768 at 1, 5, 8 rows 1.9 / 7.4 / 2.4, 3.2 / 8.1 / 3.5, 4.1 / 7.6 / 4.2; 768 x 3072 2.4 / 7.6 / 6.2, 4.9 / 8.2 / 8.2,

@@ -7,7 +7,6 @@ namespace csd {
 int tc_sm_count();
 bool tc_supported(int m, int N, int K, bool dual);
 size_t tc_scratch_bytes(int m, int N, int K, bool dual);
-int tc_ticket_count(int N);
 csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st);
 csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st);   // a.X (times a.gain) -> a.xs, a.ssq
 
