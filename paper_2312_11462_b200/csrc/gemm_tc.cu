@@ -12,8 +12,8 @@
 // Work is cut into (tile, K block) units and every CTA (one per SM) owns an equal contiguous share
 // of them, so all SMs stream the same number of bytes; a tile that straddles CTAs is finished by
 // the first of them (for which it comes last), adding the parts the others parked in CTA order
-// (deterministic).  Roles inside a CTA (192 threads): warp 0 lane 0 issues TMA, warp 1 lane 0
-// issues MMA, warps 2-5 read the accumulators from tensor memory (one quadrant each) and run the
+// (deterministic).  Roles inside a CTA (192 or 320 threads): warp 0 lane 0 issues TMA, warp 1
+// lane 0 issues MMA, the others read the accumulators from tensor memory (a quadrant each) and run the
 // epilogue: rms-norm factor, residual add or gated activation, and optionally the three-term
 // split and sum-of-squares pieces of the result for the next GEMM.  The first ring-full of weight
 // tiles is requested before the programmatic-dependent-launch wait.  Every mbarrier wait is
@@ -25,6 +25,10 @@
 
 namespace csd {
 
+// Epilogue warps: one per tensor-memory quadrant, two (half of the rows each) for blocks of more than 9 rows, whose
+// finish one warp per quadrant takes 3.4 us over at 17 rows.  16 layers of the 7B shape with one / two: 5 rows 1560 /
+// 1577 us, 9 rows 1667 / 1683, 13 rows 1835 / 1803, 17 rows 2060 / 1971.
+template <int M> struct EpilogueWarps { static constexpr int value = M > 9 ? 8 : 4; };
 constexpr size_t TC_SMEM_MAX = 111 * 1024;              // two CTAs (of consecutive kernels) fit one SM
 
 static int g_path = 0;
@@ -184,11 +188,12 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 }
 
 template <int M, bool DUAL>
-__global__ void __launch_bounds__(TC_THREADS, 2)
+__global__ void __launch_bounds__(64 + 32 * EpilogueWarps<M>::value, 2)
 skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                       const __grid_constant__ CUtensorMap tmX, const TcParams p) {
     constexpr int NPAD = 3 * M <= 16 ? 16 : (3 * M <= 32 ? 32 : (3 * M <= 48 ? 48 : 64));
     constexpr int NT = DUAL ? 2 : 1;
+    constexpr int EW = EpilogueWarps<M>::value;
     constexpr int ACC_ONE = NPAD * NT;                        // tensor-memory columns of one accumulator
     // The tensor core's fp32 accumulation loses a little with every add of a long chain, so the K blocks
     // of a segment go round-robin to NACC accumulators (as many as fit 256 columns twice over, at most
@@ -196,10 +201,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
     constexpr int NACC = 2 * ACC_ONE * 4 <= 256 ? 4 : (2 * ACC_ONE * 2 <= 256 ? 2 : 1);
     constexpr int ACC_COLS = ACC_ONE * NACC;                  // columns per accumulator set (one segment)
     constexpr int TMEM_COLS = 2 * ACC_COLS <= 32 ? 32 : (2 * ACC_COLS <= 64 ? 64 : (2 * ACC_COLS <= 128 ? 128 : 256));
-    constexpr int XBYTES = NPAD * 128;                        // the rows' terms for one K block
+    constexpr int XBYTES = NPAD * 128;                        // room of the rows' terms for one K block; 3 M rows are copied:
+                                                              // what the pad holds reaches only columns nobody reads
     constexpr int KS = (!DUAL && NPAD <= 16) ? 2 : 1;         // K blocks per stage
     constexpr int WB = (DUAL ? 2 : KS) * STAGE_BYTES;         // weight bytes per stage
     constexpr int STAGE = WB + KS * XBYTES;
+    constexpr uint32_t TX_BYTES = WB + KS * 3 * M * 128;      // bytes that arrive per stage
     constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NPAD >> 3) << 17) |
                                ((uint32_t)(TILE_N >> 4) << 24);   // f32 accumulate, bf16 x bf16, K-major both
 
@@ -221,9 +228,9 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 
     if (tid == 0) {
         for (int s = 0; s < 12; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&ctl->acc_full[b], 1); mbar_init(&ctl->acc_empty[b], 4); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&ctl->acc_full[b], 1); mbar_init(&ctl->acc_empty[b], EW); }
         mbar_init(&ctl->red_ready, 1);
-        mbar_init(&ctl->red_done, 4 * 3);               // one arrival per epilogue warp of the three other CTAs
+        mbar_init(&ctl->red_done, EW * 3);               // one arrival per epilogue warp of the three other CTAs
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -258,7 +265,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             const int kb0 = kb;
             for (int i = 0; i < pre; ++i) {
                 unsigned char* dst = ring + (size_t)i * STAGE;
-                mbar_expect_tx(&ctl->full[i], (uint32_t)STAGE);
+                mbar_expect_tx(&ctl->full[i], TX_BYTES);
                 tma_load_2d(dst, &tmW, &ctl->full[i], kb * KS * KB, tile * TILE_N);
                 if (DUAL) tma_load_2d(dst + STAGE_BYTES, &tmW2, &ctl->full[i], kb * KB, tile * TILE_N);
                 if (KS == 2) tma_load_2d(dst + STAGE_BYTES, &tmW, &ctl->full[i], (kb * KS + 1) * KB, tile * TILE_N);   // past K: zero fill
@@ -277,7 +284,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             for (int i = pre; i < items && !*abort_flag; ++i) {
                 if (!mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
                 unsigned char* dst = ring + (size_t)s * STAGE;
-                mbar_expect_tx(&ctl->full[s], (uint32_t)STAGE);
+                mbar_expect_tx(&ctl->full[s], TX_BYTES);
                 tma_load_2d(dst, &tmW, &ctl->full[s], kb * KS * KB, tile * TILE_N);
                 if (DUAL) tma_load_2d(dst + STAGE_BYTES, &tmW2, &ctl->full[s], kb * KB, tile * TILE_N);
                 if (KS == 2) tma_load_2d(dst + STAGE_BYTES, &tmW, &ctl->full[s], (kb * KS + 1) * KB, tile * TILE_N);
@@ -325,15 +332,18 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             }
         }
     } else {
-        // ---- epilogue warps: quadrant q of tensor memory holds weight rows q*32 .. q*32+31 of the tile
-        const int q = warp & 3, et = (warp - 2) * 32 + lane;
+        // ---- epilogue warps: quadrant q of tensor memory holds weight rows q*32 .. q*32+31 of the tile; with
+        //      eight warps a quadrant's two take half of the block's rows each
+        constexpr int MH = EW == 8 ? (M + 1) / 2 : M;
+        const int q = warp & 3, half = (warp - 2) >> 2, et = (warp - 2) * 32 + lane;
+        const int row0 = half * MH, nrow = half ? M - MH : MH;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         if (p.ssq_in && et < M) {               // rms-norm factor of every row from the pieces of its sum of squares
             float sq = 0.f;
             for (int c = 0; c < p.ssq_cnt; ++c) sq += __ldcg(p.ssq_in + (size_t)c * M + et);
             ctl->scale[et] = 1.f / sqrtf(sq / (float)p.K + p.eps);
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(EW * 32) : "memory");
         float* my_part = p.partial + (size_t)cta * 2 * NT * M * TILE_N;
         int i = 0;
         for (int seg = 0; i < items; ++seg) {
@@ -342,7 +352,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             const int seg_len = min(p.nkb - kb_begin, items - i);
             i += seg_len;
             const int col = q * 32 + lane, n = tile * TILE_N + col;
-            constexpr int NV = NT * M;
+            constexpr int NV = NT * MH;
             // Part of a tile.  Its contributors are consecutive CTAs; the first of them finishes it.
             // For the last contributor the tile is the FIRST thing it computes, so its partial sums
             // are parked in global memory (and its arrival counted) long before the first contributor,
@@ -360,21 +370,22 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             // the residual values, the gain, and the other parts as soon as they are parked.  (Fetched afterwards, behind
             // a block barrier and a device fence on both sides, the parts cost 4.5 us of a 35 us gate+up launch.)  A
             // warp parks, counts and fetches its own 32 columns: no block-wide step.
-            float yold[M], extra[NV];
+            float yold[MH], extra[NV];
             float out_g = 1.f;
 #pragma unroll
-            for (int r = 0; r < M; ++r) yold[r] = 0.f;
+            for (int r = 0; r < MH; ++r) yold[r] = 0.f;
 #pragma unroll
             for (int v = 0; v < NV; ++v) extra[v] = 0.f;
             if (finisher && n < p.N) {
                 if (p.epilogue == EPI_ADD) {
 #pragma unroll
-                    for (int r = 0; r < M; ++r) yold[r] = __ldcg(p.Y + (size_t)r * p.ldy + n);
+                    for (int r = 0; r < MH; ++r)
+                        if (r < nrow) yold[r] = __ldcg(p.Y + (size_t)(row0 + r) * p.ldy + n);
                 }
                 if (p.out_xs && p.out_gain) out_g = __bfloat162float(p.out_gain[n]);
             }
             if (finisher && c_hi > c_lo) {
-                unsigned* ticket = p.tickets + tile * 4 + q;
+                unsigned* ticket = p.tickets + tile * 8 + half * 4 + q;
                 if (lane == 0) {
                     const unsigned want = (unsigned)(c_hi - c_lo);
                     int spins = 0;
@@ -386,7 +397,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 }
                 __syncwarp();
                 // the other parts in CTA order (deterministic); as many contributors' loads in flight together as about
-                // 48 registers hold (all of them, in one round trip, for a 5-row block)
+                // 48 registers hold
                 constexpr int CH = NV <= 6 ? 8 : (48 / NV < 1 ? 1 : 48 / NV);
 #pragma unroll 1
                 for (int c = c_lo + 1; c <= c_hi; c += CH) {
@@ -394,9 +405,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 #pragma unroll
                     for (int h = 0; h < CH; ++h) {
                         const int cc = min(c + h, c_hi);
-                        const float* src = p.partial + ((size_t)cc * 2) * NT * M * TILE_N + col;
+                        const float* src = p.partial + (((size_t)cc * 2) * NT * M + row0) * TILE_N + col;
 #pragma unroll
-                        for (int v = 0; v < NV; ++v) part[h][v] = __ldcg(src + v * TILE_N);
+                        for (int u = 0; u < NT; ++u)
+#pragma unroll
+                            for (int r = 0; r < MH; ++r)
+                                part[h][u * MH + r] = r < nrow ? __ldcg(src + (u * M + r) * TILE_N) : 0.f;
                     }
 #pragma unroll
                     for (int h = 0; h < CH; ++h)
@@ -408,32 +422,28 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             }
             if (!mbar_wait(&ctl->acc_full[b], (seg >> 1) & 1)) { *abort_flag = 1; break; }   // same outcome in all four warps
             tc_fence_after();
-            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * ACC_COLS);
-            float sums[NT][M];
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * ACC_COLS + row0);
+            float sums[NT][MH];
 #pragma unroll
             for (int u = 0; u < NT; ++u) {
-                float third[M], second[M];
+                float third[MH], second[MH];
 #pragma unroll
-                for (int r = 0; r < M; ++r) { sums[u][r] = 0.f; second[r] = 0.f; third[r] = 0.f; }
+                for (int r = 0; r < MH; ++r) { sums[u][r] = 0.f; second[r] = 0.f; third[r] = 0.f; }
 #pragma unroll
                 for (int a = 0; a < NACC; ++a) {
                     if (a >= seg_len) break;            // a short segment used fewer accumulators
+                    float v[3][MH];                     // (with M odd, half 1 reads one column too many, inside NPAD, and drops it)
 #pragma unroll
-                    for (int c0 = 0; c0 < NPAD; c0 += 16) {
-                        if (c0 >= 3 * M) break;
-                        float v[16];
-                        tc_ld16(taddr + (uint32_t)(a * ACC_ONE + u * NPAD + c0), v);
+                    for (int t = 0; t < 3; ++t) tc_ld_cols<MH>(taddr + (uint32_t)(a * ACC_ONE + u * NPAD + t * M), v[t]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const int col = c0 + c;
-                            if (col < M) sums[u][col] += v[c];
-                            else if (col < 2 * M) second[col - M] += v[c];
-                            else if (col < 3 * M) third[col - 2 * M] += v[c];
-                        }
+                    for (int r = 0; r < MH; ++r) {
+                        asm volatile("" : "+f"(v[0][r]), "+f"(v[1][r]), "+f"(v[2][r]));   // not before the wait
+                        sums[u][r] += v[0][r]; second[r] += v[1][r]; third[r] += v[2][r];
                     }
                 }
 #pragma unroll
-                for (int r = 0; r < M; ++r) sums[u][r] += second[r] + third[r];   // small terms first
+                for (int r = 0; r < MH; ++r) sums[u][r] += second[r] + third[r];   // small terms first
             }
             tc_fence_before();
             __syncwarp();
@@ -443,7 +453,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 // finishes the tile; when its own MMAs are done its ring is free, it tells the others, they
                 // write their parts into it (distributed shared memory) and signal back, and it adds the
                 // parts in rank order.
-                float* buf = reinterpret_cast<float*>(ring);          // [3][NV][128]
+                float* buf = reinterpret_cast<float*>(ring);          // [3][NT * M][128]
                 if (crank == 0) {
                     if (et == 0)
                         for (int r = 1; r < p.csplit; ++r) remote_arrive(map_to_cta(smem_u32(&ctl->red_ready), (uint32_t)r));
@@ -453,15 +463,16 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 #pragma unroll
                         for (int u = 0; u < NT; ++u)
 #pragma unroll
-                            for (int rr = 0; rr < M; ++rr) sums[u][rr] += buf[((r - 1) * NV + u * M + rr) * TILE_N + col];
+                            for (int rr = 0; rr < MH; ++rr)
+                                if (rr < nrow) sums[u][rr] += buf[((r - 1) * NT * M + u * M + row0 + rr) * TILE_N + col];
                 } else {
                     if (!mbar_wait_cluster(&ctl->red_ready, 0)) *abort_flag = 1;
                     const uint32_t dst = map_to_cta(smem_u32(buf), 0u);
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
 #pragma unroll
-                        for (int rr = 0; rr < M; ++rr)
-                            remote_store(dst + (uint32_t)((((crank - 1) * NV + u * M + rr) * TILE_N + col) * 4), sums[u][rr]);
+                        for (int rr = 0; rr < MH; ++rr)
+                            if (rr < nrow) remote_store(dst + (uint32_t)((((crank - 1) * NT * M + u * M + row0 + rr) * TILE_N + col) * 4), sums[u][rr]);
                     __syncwarp();
                     if (lane == 0) remote_arrive(map_to_cta(smem_u32(&ctl->red_done), 0u));
                     continue;
@@ -471,51 +482,54 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 #pragma unroll
                 for (int u = 0; u < NT; ++u)
 #pragma unroll
-                    for (int r = 0; r < M; ++r) __stcg(mine + (u * M + r) * TILE_N + col, sums[u][r]);
+                    for (int r = 0; r < MH; ++r)
+                        if (r < nrow) __stcg(mine + (u * M + row0 + r) * TILE_N + col, sums[u][r]);
                 __syncwarp();
-                if (lane == 0) red_release_gpu(p.tickets + tile * 4 + q, 1u);
+                if (lane == 0) red_release_gpu(p.tickets + tile * 8 + half * 4 + q, 1u);
                 continue;
             }
 #pragma unroll
             for (int u = 0; u < NT; ++u)
 #pragma unroll
-                for (int r = 0; r < M; ++r) sums[u][r] += extra[u * M + r];
-            // ---- finish the tile: this thread owns output column n for all M rows
-            float outv[M];
+                for (int r = 0; r < MH; ++r) sums[u][r] += extra[u * MH + r];
+            // ---- finish the tile: this thread owns output column n for its half of the rows
+            float outv[MH];
 #pragma unroll
-            for (int r = 0; r < M; ++r) {
-                const float scale = p.ssq_in ? ctl->scale[r] : 1.f;
-                float val = sums[0][r] * scale;
-                if (DUAL) {
-                    const float up = sums[NT - 1][r] * scale;
-                    val = (p.epilogue == EPI_GEGLU ? tc_gelu(val) : tc_silu(val)) * up;
+            for (int r = 0; r < MH; ++r) {
+                outv[r] = 0.f;
+                if (r < nrow) {
+                    const float scale = p.ssq_in ? ctl->scale[row0 + r] : 1.f;
+                    float val = sums[0][r] * scale;
+                    if (DUAL) {
+                        const float up = sums[NT - 1][r] * scale;
+                        val = (p.epilogue == EPI_GEGLU ? tc_gelu(val) : tc_silu(val)) * up;
+                    }
+                    if (n < p.N) {
+                        if (p.epilogue == EPI_ADD) val += yold[r];
+                        p.Y[(size_t)(row0 + r) * p.ldy + n] = val;
+                        outv[r] = val;
+                    }
                 }
-                if (n < p.N) {
-                    float* y = p.Y + (size_t)r * p.ldy + n;
-                    if (p.epilogue == EPI_ADD) val += yold[r];
-                    *y = val;
-                } else {
-                    val = 0.f;
-                }
-                outv[r] = val;
             }
             if (p.out_ssq) {                      // pieces of the rows' sums of squares, one per 32 columns
 #pragma unroll
-                for (int r = 0; r < M; ++r) {
-                    const float sq = warp_sum(outv[r] * outv[r]);
-                    if (lane == 0) p.out_ssq[(size_t)(tile * 4 + q) * M + r] = sq;
-                }
+                for (int r = 0; r < MH; ++r)
+                    if (r < nrow) {
+                        const float sq = warp_sum(outv[r] * outv[r]);
+                        if (lane == 0) p.out_ssq[(size_t)(tile * 4 + q) * M + row0 + r] = sq;
+                    }
             }
             if (p.out_xs && n < p.N) {            // the rows as three bf16 terms for the GEMM that reads them next
 #pragma unroll
-                for (int r = 0; r < M; ++r) {
-                    uint16_t b1, b2, b3;
-                    split3(outv[r] * out_g, b1, b2, b3);
-                    uint16_t* o = reinterpret_cast<uint16_t*>(p.out_xs) + n;
-                    o[(size_t)r * p.out_ld] = b1;
-                    o[(size_t)(M + r) * p.out_ld] = b2;
-                    o[(size_t)(2 * M + r) * p.out_ld] = b3;
-                }
+                for (int r = 0; r < MH; ++r)
+                    if (r < nrow) {
+                        uint16_t b1, b2, b3;
+                        split3(outv[r] * out_g, b1, b2, b3);
+                        uint16_t* o = reinterpret_cast<uint16_t*>(p.out_xs) + n;
+                        o[(size_t)(row0 + r) * p.out_ld] = b1;
+                        o[(size_t)(M + row0 + r) * p.out_ld] = b2;
+                        o[(size_t)(2 * M + row0 + r) * p.out_ld] = b3;
+                    }
             }
         }
     }
@@ -609,7 +623,7 @@ static csd_status launch_tc(const CUtensorMap& tw, const CUtensorMap& tw2, const
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    pdl_config(cfg, attr, dim3((unsigned)pl.grid), dim3(TC_THREADS), pl.smem + 1024, st);
+    pdl_config(cfg, attr, dim3((unsigned)pl.grid), dim3(64 + 32 * EpilogueWarps<M>::value), pl.smem + 1024, st);
     if (pl.csplit > 1) {
         attr[1].id = cudaLaunchAttributeClusterDimension;
         attr[1].val.clusterDim.x = (unsigned)pl.csplit; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
@@ -630,7 +644,7 @@ csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st) {
     if (!tensor_map_2d(a.W, a.N, a.K, TILE_N, &tw)) return CSD_ERR_UNSUPPORTED;
     tw2 = tw;
     if (dual && !tensor_map_2d(a.W2, a.N, a.K, TILE_N, &tw2)) return CSD_ERR_UNSUPPORTED;
-    if (!tensor_map_2d(a.xs, 3 * a.m, a.K, pl.npad, &tx)) return CSD_ERR_UNSUPPORTED;
+    if (!tensor_map_2d(a.xs, 3 * a.m, a.K, 3 * a.m, &tx)) return CSD_ERR_UNSUPPORTED;
     int ssq_cnt = a.ssq_cnt;
     if (!a.xs_ready) {
         const csd_status s = launch_split_rows(a, st);
