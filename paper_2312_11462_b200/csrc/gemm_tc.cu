@@ -263,12 +263,13 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             const int pre = items < p.stages ? items : p.stages;
             int tile = (int)(u0 / p.nkb), kb = (int)(u0 % p.nkb);
             const int kb0 = kb;
+            const uint64_t once = policy_evict_first();
             for (int i = 0; i < pre; ++i) {
                 unsigned char* dst = ring + (size_t)i * STAGE;
                 mbar_expect_tx(&ctl->full[i], TX_BYTES);
-                tma_load_2d(dst, &tmW, &ctl->full[i], kb * KS * KB, tile * TILE_N);
-                if (DUAL) tma_load_2d(dst + STAGE_BYTES, &tmW2, &ctl->full[i], kb * KB, tile * TILE_N);
-                if (KS == 2) tma_load_2d(dst + STAGE_BYTES, &tmW, &ctl->full[i], (kb * KS + 1) * KB, tile * TILE_N);   // past K: zero fill
+                tma_load_2d_once(dst, &tmW, &ctl->full[i], kb * KS * KB, tile * TILE_N, once);
+                if (DUAL) tma_load_2d_once(dst + STAGE_BYTES, &tmW2, &ctl->full[i], kb * KB, tile * TILE_N, once);
+                if (KS == 2) tma_load_2d_once(dst + STAGE_BYTES, &tmW, &ctl->full[i], (kb * KS + 1) * KB, tile * TILE_N, once);   // past K: zero fill
                 if (++kb == p.nkb) { kb = 0; ++tile; }
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -285,9 +286,9 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 if (!mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
                 unsigned char* dst = ring + (size_t)s * STAGE;
                 mbar_expect_tx(&ctl->full[s], TX_BYTES);
-                tma_load_2d(dst, &tmW, &ctl->full[s], kb * KS * KB, tile * TILE_N);
-                if (DUAL) tma_load_2d(dst + STAGE_BYTES, &tmW2, &ctl->full[s], kb * KB, tile * TILE_N);
-                if (KS == 2) tma_load_2d(dst + STAGE_BYTES, &tmW, &ctl->full[s], (kb * KS + 1) * KB, tile * TILE_N);
+                tma_load_2d_once(dst, &tmW, &ctl->full[s], kb * KS * KB, tile * TILE_N, once);
+                if (DUAL) tma_load_2d_once(dst + STAGE_BYTES, &tmW2, &ctl->full[s], kb * KB, tile * TILE_N, once);
+                if (KS == 2) tma_load_2d_once(dst + STAGE_BYTES, &tmW, &ctl->full[s], (kb * KS + 1) * KB, tile * TILE_N, once);
 #pragma unroll
                 for (int j = 0; j < KS; ++j)
                     tma_load_2d(dst + WB + j * XBYTES, &tmX, &ctl->full[s], (kb * KS + j) * KB, 0);
