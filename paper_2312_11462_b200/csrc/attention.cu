@@ -11,15 +11,14 @@
 // Rows see keys [0, n_keys + r) when causal, all n_keys otherwise (cross-attention, encoder).
 #include <cooperative_groups.h>
 #include "attention.cuh"
+#include "attention_mma.cuh"
 #include "gemm_tc.cuh"
-#include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace csd {
 
 constexpr int AT = 256;
-constexpr int TILE = 64;
 constexpr int MAXM = CSD_MAX_ROWS;
 constexpr int MAX_SPLITS = 8;          // portable cluster size
 constexpr int STAGES = 2;
@@ -43,7 +42,6 @@ struct AttnParams {
     __nv_bfloat16* out_xs; int out_xs_ld;
     int xs_m, xs_r0;        // three-term output: rows per term of the whole buffer, row of this block's first row
     int* status;
-    int sub_rows;           // > 0: grid.z sub-blocks of this many rows each, over a cache that already holds every row
     int ldq, ld_new, m, cap, H, n_keys, n_old, early_loads, causal, bias_len, bias_zero, q_pos0, ldo, nsplit, split_len;
     float scale;
     // tree-shaped block: row r sees block row j only if bit j of tmask[r] is set (its ancestors and
@@ -75,8 +73,7 @@ __device__ __forceinline__ void store_split(__nv_bfloat16* xs, int ld, int m, in
 // first fetches everything it needs from all splits in one batch of independent remote loads.
 template <int DH, int REC>
 __device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* rec, const AttnParams& p, int h, int split,
-                                             int m, int r0) {
-    // m rows of this CTA's records; they are rows r0 .. r0+m-1 of the launch's output
+                                             int m) {
     for (int i = split * AT + threadIdx.x; i < m * DH; i += p.nsplit * AT) {
         const int r = i / DH, d = i % DH;
         float ms[MAX_SPLITS], ls[MAX_SPLITS], vs[MAX_SPLITS];
@@ -100,14 +97,14 @@ __device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* 
                 den = fmaf(ls[s], w, den);
             }
         const float ov = den > 0.f ? num / den : 0.f;
-        p.out[(size_t)(r0 + r) * p.ldo + h * DH + d] = ov;
+        p.out[(size_t)r * p.ldo + h * DH + d] = ov;
         if (p.out_xs) {
             uint16_t b1, b2, b3;
             split3(ov, b1, b2, b3);
             uint16_t* xs = reinterpret_cast<uint16_t*>(p.out_xs) + h * DH + d;
-            xs[(size_t)(p.xs_r0 + r0 + r) * p.out_xs_ld] = b1;
-            xs[(size_t)(p.xs_m + p.xs_r0 + r0 + r) * p.out_xs_ld] = b2;
-            xs[(size_t)(2 * p.xs_m + p.xs_r0 + r0 + r) * p.out_xs_ld] = b3;
+            xs[(size_t)(p.xs_r0 + r) * p.out_xs_ld] = b1;
+            xs[(size_t)(p.xs_m + p.xs_r0 + r) * p.out_xs_ld] = b2;
+            xs[(size_t)(2 * p.xs_m + p.xs_r0 + r) * p.out_xs_ld] = b3;
         }
     }
 }
@@ -352,7 +349,7 @@ block_attention_kernel(const AttnParams p) {
     }
     if (tid < m) { rec[tid * C::REC + DH] = row_m[tid]; rec[tid * C::REC + DH + 1] = row_l[tid]; }
     cluster.sync();
-    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m, 0);
+    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m);
     cluster.sync();       // no CTA leaves while another may still read its record
 }
 
@@ -365,25 +362,6 @@ block_attention_kernel(const AttnParams p) {
 // bf16 in the cache, are exact.  Warp w owns keys 8w..8w+7 of the tile in q.K^T and output
 // dimensions 16w..16w+15 in P.V; rows 16..31 (a 17-row block) are a second m16 tile.
 // -------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// value = hi + lo with hi = bf16(value), lo = bf16(value - hi)
-__device__ __forceinline__ void split2(float v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-    hi = __float2bfloat16_rn(v);
-    lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
-
 template <int DH> struct MmaCfg {
     static constexpr int QP = DH * 2 + 16;                   // bytes per q row: bf16 plus one 16-byte skew
     static constexpr int PP = TILE * 2 + 16;                 // bytes per row of softmax weights
@@ -396,11 +374,6 @@ template <int DH> struct MmaCfg {
                2 * (size_t)MAXM * DH * 2 + 3 * 32 * 4 + 64;
     }
 };
-// byte offset of 16-byte chunk c (8 dimensions) of key row j inside a swizzled tile
-template <int DH> __device__ __forceinline__ uint32_t kv_off(int j, int c) {
-    return (uint32_t)((c >> 3) * (TILE * 128) + j * 128 + (((c & 7) ^ (j & 7)) << 4));
-}
-
 template <int DH, int MT>
 __global__ void __launch_bounds__(AT)
 block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -426,12 +399,9 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h = blockIdx.x, split = blockIdx.y;
-    // sub-block mode (sub_rows > 0, no append): blockIdx.z picks rows r0 .. r0+m-1 of a block of p.m rows
-    const int r0 = p.sub_rows ? (int)blockIdx.z * p.sub_rows : 0;
-    const int m = p.sub_rows ? min(p.sub_rows, p.m - r0) : p.m, half = DH / 2;
-    const int n_keys = p.n_keys + (p.causal ? r0 : 0);          // keys visible to this CTA's first row
+    const int m = p.m, half = DH / 2, n_keys = p.n_keys;
     const int total = p.causal ? n_keys + m - 1 : n_keys;
-    const int n_old = p.sub_rows ? total : p.n_old;
+    const int n_old = p.n_old;
     const int s_begin = split * p.split_len;
     const int s_end = min(total, s_begin + p.split_len);
     const int n_tiles = s_end > s_begin ? (s_end - s_begin + TILE - 1) / TILE : 0;
@@ -487,7 +457,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
             const int i = tid + e * AT;
             if (i < m * half) {
                 const int r = i / half, d = i % half;
-                const float* qr = p.q + (size_t)(r0 + r) * p.ldq + h * DH;
+                const float* qr = p.q + (size_t)r * p.ldq + h * DH;
                 qv[e][0] = qr[d]; qv[e][1] = qr[d + half];
                 if (p.k_new) {
                     const float* kr = p.k_new + (size_t)r * p.ld_new + h * DH;
@@ -627,7 +597,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
                         if (vis) {
                             s = ((sacc2[g][1][0][e] + sacc2[g][1][1][e]) + (sacc2[g][0][0][e] + sacc2[g][0][1][e])) * p.scale;
                             if (bias_h) {
-                                int bi = key - (p.q_pos0 + r0 + r) + p.bias_zero;
+                                int bi = key - (p.q_pos0 + r) + p.bias_zero;
                                 bi = max(0, min(p.bias_len - 1, bi));
                                 s += bias_h[bi];
                             }
@@ -741,9 +711,9 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
                         const int d = 16 * warp + 8 * t + 2 * (lane & 3);
-                        float* dst = p.out + (size_t)(r0 + r) * p.ldo + h * DH + d;
+                        float* dst = p.out + (size_t)r * p.ldo + h * DH + d;
                         dst[0] = o[mt][t][2 * hr] * inv; dst[1] = o[mt][t][2 * hr + 1] * inv;
-                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, p.xs_r0 + r0 + r, h * DH + d, dst[0], dst[1]);
+                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, p.xs_r0 + r, h * DH + d, dst[0], dst[1]);
                     }
                 }
         }
@@ -767,7 +737,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
     }
     if (tid < m) { rec[tid * C::REC + DH] = row_m[tid]; rec[tid * C::REC + DH + 1] = row_l[tid]; }
     cluster.sync();
-    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m, r0);
+    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m);
     cluster.sync();       // no CTA leaves while another may still read its record
 }
 // One 64-key tile per CTA while that keeps the splits of a head inside one portable cluster (8)
@@ -775,6 +745,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
 // tiles in flight at once; long caches walk several tiles per CTA, two requests ahead.
 static bool g_attn_cuda_cores = false;
 void set_attention_cuda_cores(bool on) { g_attn_cuda_cores = on; }
+bool row_attention_supported(int Dh) { return (Dh == 64 || Dh == 128) && !g_attn_cuda_cores; }
 
 int attn_splits(int total_keys, int H) {
     int by_sm = (2 * 148 + H - 1) / H;
@@ -788,8 +759,7 @@ int attn_splits(int total_keys, int H) {
 static void attn_launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const AttnParams& ap, size_t smem,
                                cudaStream_t st) {
     cfg = cudaLaunchConfig_t{};
-    cfg.gridDim = dim3((unsigned)ap.H, (unsigned)ap.nsplit,
-                       (unsigned)(ap.sub_rows > 0 ? (ap.m + ap.sub_rows - 1) / ap.sub_rows : 1));
+    cfg.gridDim = dim3((unsigned)ap.H, (unsigned)ap.nsplit);
     cfg.blockDim = dim3(AT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -834,34 +804,27 @@ static csd_status launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const
     return CSD_OK;
 }
 
-// Blocks of more than MAXM rows over a cache that already holds their keys (wide prefill, encoder):
-// one launch whose grid.z walks sub-blocks of 32 rows on the tensor-core kernel; elsewhere one
-// launch per MAXM rows.
-static csd_status launch_attention_rows(const AttnArgs& a, cudaStream_t st);
-static csd_status launch_attention_block(const AttnArgs& a, int sub_rows, cudaStream_t st);
+static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st);
 
+// Blocks of more than MAXM rows over a cache that already holds their keys (wide passes whose head dimension has no
+// launch_row_attention): one launch per MAXM rows.
 csd_status launch_attention(const AttnArgs& a, cudaStream_t st) {
-    if (a.m > MAXM) return launch_attention_rows(a, st);
-    return launch_attention_block(a, 0, st);
-}
-
-static csd_status launch_attention_rows(const AttnArgs& a, cudaStream_t st) {
+    if (a.m <= MAXM) return launch_attention_block(a, st);
     if (a.k_new || a.tree_mask || a.out_xs || a.m > CSD_WIDE_ROWS) return CSD_ERR_INVALID_ARG;
-    if ((a.Dh == 64 || a.Dh == 128) && !g_attn_cuda_cores) return launch_attention_block(a, 32, st);
     for (int r0 = 0; r0 < a.m; r0 += MAXM) {
         AttnArgs s = a;
         s.q = a.q + (size_t)r0 * a.ldq; s.m = a.m - r0 < MAXM ? a.m - r0 : MAXM;
         s.n_keys = a.causal ? a.n_keys + r0 : a.n_keys;
         s.q_pos0 = a.q_pos0 + r0;
         s.out = a.out + (size_t)r0 * a.ldo;
-        const csd_status rc = launch_attention_block(s, 0, st);
+        const csd_status rc = launch_attention_block(s, st);
         if (rc != CSD_OK) return rc;
     }
     return CSD_OK;
 }
 
-static csd_status launch_attention_block(const AttnArgs& a, int sub_rows, cudaStream_t st) {
-    if (!a.q || !a.Kc || !a.Vc || !a.out || a.m < 1 || (sub_rows == 0 && a.m > MAXM) || a.H < 1 || a.n_keys < 0)
+static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st) {
+    if (!a.q || !a.Kc || !a.Vc || !a.out || a.m < 1 || a.m > MAXM || a.H < 1 || a.n_keys < 0)
         return CSD_ERR_INVALID_ARG;
     const bool append = a.k_new != nullptr;
     if (append && (!a.v_new || !a.causal || a.n_keys < 1)) return CSD_ERR_INVALID_ARG;
@@ -885,18 +848,7 @@ static csd_status launch_attention_block(const AttnArgs& a, int sub_rows, cudaSt
         ap.tree = 1;
         for (int r = 0; r < MAXM; ++r) { ap.tmask[r] = r < a.m ? a.tree_mask[r] : 0u; ap.tdepth[r] = r < a.m ? (unsigned char)a.tree_depth[r] : 0; }
     }
-    ap.sub_rows = sub_rows;
-    // sub-blocks: each (head, sub-block) pair is a cluster of its own; the split length follows the
-    // last sub-block, which sees the most keys (earlier ones leave their last splits empty)
-    ap.nsplit = attn_splits(total, sub_rows > 0 ? a.H * ((a.m + sub_rows - 1) / sub_rows) : a.H);
-    if (sub_rows > 0) {
-        // these launches are throughput-bound: as many splits as keep the whole grid resident at once
-        // (two CTAs per SM), rather than one more that spills into a second wave
-        const int pairs = a.H * ((a.m + sub_rows - 1) / sub_rows);
-        int fit = 2 * 148 / pairs;
-        if (fit < 1) fit = 1;
-        if (ap.nsplit > fit) ap.nsplit = fit;
-    }
+    ap.nsplit = attn_splits(total, a.H);
     int len = (total + ap.nsplit - 1) / ap.nsplit;
     ap.split_len = (len + TILE - 1) / TILE * TILE;
     ap.nsplit = (total + ap.split_len - 1) / ap.split_len;
@@ -904,12 +856,11 @@ static csd_status launch_attention_block(const AttnArgs& a, int sub_rows, cudaSt
     if ((a.Dh == 64 || a.Dh == 128) && !g_attn_cuda_cores) {
         CUtensorMap tk, tv;
         if (tensor_map_2d(a.Kc, a.H * a.cap, a.Dh, TILE, &tk) && tensor_map_2d(a.Vc, a.H * a.cap, a.Dh, TILE, &tv)) {
-            const bool one_tile = sub_rows == 0 && a.m <= 16;
+            const bool one_tile = a.m <= 16;
             if (a.Dh == 64) return one_tile ? launch_mma<64, 1>(tk, tv, ap, st) : launch_mma<64, 2>(tk, tv, ap, st);
             return one_tile ? launch_mma<128, 1>(tk, tv, ap, st) : launch_mma<128, 2>(tk, tv, ap, st);
         }
     }
-    if (sub_rows > 0) return CSD_ERR_UNSUPPORTED;     // sub-blocks exist on the tensor-core kernel only
     switch (a.Dh) {
         case 32: return launch_dh<32>(ap, st);
         case 64: return launch_dh<64>(ap, st);

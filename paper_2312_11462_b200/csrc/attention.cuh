@@ -22,6 +22,11 @@ struct AttnArgs {
     int out_xs_ld = 0;
     int out_xs_rows = 0;                  // rows per term of the out_xs buffer (0: m) and this block's first row in it
     int out_xs_row0 = 0;
+    // Many rows (launch_row_attention): rotation of q by these tables at positions q_pos0 + r, and the output as two bf16
+    // terms, row = term * out_xs_rows + r, instead of fp32 rows
+    const float* q_rope_cos = nullptr;
+    const float* q_rope_sin = nullptr;
+    __nv_bfloat16* out_xs2 = nullptr;
     // Self-attention of a drafted block (causal, n_keys = committed keys + 1): the block's own key
     // and value rows are still fp32 projections [m, ld_new]; the kernel rotates q and k (when
     // rope tables [pos][Dh/2] are given), rounds k and v to bf16, appends them to the cache at
@@ -45,5 +50,8 @@ struct AttnArgs {
 int attn_splits(int total_keys, int H);
 void set_attention_cuda_cores(bool on);   // true: always the CUDA-core kernel (for comparison runs)
 csd_status launch_attention(const AttnArgs& a, cudaStream_t st);
+// Whether the rows of a wide pass take launch_row_attention: head dimension 64 or 128, comparison switch off.
+bool row_attention_supported(int Dh);
+csd_status launch_row_attention(const AttnArgs& a, cudaStream_t st);
 
 }  // namespace csd

@@ -105,35 +105,58 @@ __global__ void bias_table_kernel(const __nv_bfloat16* __restrict__ rel_bias, co
     table[idx] = __bfloat162float(rel_bias[(size_t)bucket[i] * H + h]);
 }
 
-// Rotates q (in place) and k of the block's rows, then appends k and v to the cache as bf16.
-// grid = (rows, heads); src is the fused projection output [rows, ld] with q|k|v column blocks.
-__global__ void rope_append_kernel(float* __restrict__ src, int ld, int q_off, int k_off, int v_off, int Dh,
-                                   int pos0, int cap, const float* __restrict__ cs, const float* __restrict__ sn,
-                                   __nv_bfloat16* __restrict__ Kc, __nv_bfloat16* __restrict__ Vc) {
+// Rotates k (and q in place where q_off >= 0), then appends k and v to the cache as bf16; src is the projection output
+// [rows, ld] with q|k|v column blocks.  A thread takes four rotation pairs of one (row, head), heads fastest, so a warp reads
+// whole lines of a row and writes whole 128-byte halves of cache rows (1000 rows x 32 heads x 128:
+// 8.7 us; 48 us with a block per (row, head) that also rotated q).
+__global__ void __launch_bounds__(256)
+rope_append_kernel(float* __restrict__ src, int ld, int rows, int H, int q_off, int k_off, int v_off, int Dh,
+                   int pos0, int cap, const float* __restrict__ cs, const float* __restrict__ sn,
+                   __nv_bfloat16* __restrict__ Kc, __nv_bfloat16* __restrict__ Vc) {
     pdl_wait();
     pdl_trigger();
-    const int r = blockIdx.x, h = blockIdx.y, pos = pos0 + r, half = Dh / 2;
-    float* row = src + (size_t)r * ld;
-    __nv_bfloat16* kdst = Kc + ((size_t)h * cap + pos) * Dh;
-    __nv_bfloat16* vdst = Vc + ((size_t)h * cap + pos) * Dh;
-    for (int i = threadIdx.x; i < half; i += blockDim.x) {
-        float k0 = row[k_off + h * Dh + i], k1 = row[k_off + h * Dh + i + half];
-        if (cs) {
-            const float c = cs[(size_t)pos * half + i], s = sn[(size_t)pos * half + i];
-            if (q_off >= 0) {
-                float* q = row + q_off + h * Dh;
-                const float q0 = q[i], q1 = q[i + half];
-                q[i] = q0 * c - q1 * s;
-                q[i + half] = q0 * s + q1 * c;
-            }
-            const float a = k0 * c - k1 * s, b = k0 * s + k1 * c;
-            k0 = a; k1 = b;
+    const int half = Dh / 2, per = half / 4, idx = blockIdx.x * 256 + threadIdx.x;
+    const int i = idx % per * 4, h = idx / per % H, r = idx / (per * H), pos = pos0 + r;
+    if (r >= rows) return;
+    float* row = src + (size_t)r * ld + h * Dh + i;
+    __nv_bfloat16* kdst = Kc + ((size_t)h * cap + pos) * Dh + i;
+    __nv_bfloat16* vdst = Vc + ((size_t)h * cap + pos) * Dh + i;
+    float4 k0 = *reinterpret_cast<const float4*>(row + k_off), k1 = *reinterpret_cast<const float4*>(row + k_off + half);
+    const float4 v0 = *reinterpret_cast<const float4*>(row + v_off), v1 = *reinterpret_cast<const float4*>(row + v_off + half);
+    if (cs) {
+        const float4 c = *reinterpret_cast<const float4*>(cs + (size_t)pos * half + i);
+        const float4 s = *reinterpret_cast<const float4*>(sn + (size_t)pos * half + i);
+        auto turn = [&](float4& a, float4& b) {
+            const float4 x = a, y = b;
+            a = make_float4(x.x * c.x - y.x * s.x, x.y * c.y - y.y * s.y, x.z * c.z - y.z * s.z, x.w * c.w - y.w * s.w);
+            b = make_float4(x.x * s.x + y.x * c.x, x.y * s.y + y.y * c.y, x.z * s.z + y.z * c.z, x.w * s.w + y.w * c.w);
+        };
+        if (q_off >= 0) {
+            float4 q0 = *reinterpret_cast<const float4*>(row + q_off), q1 = *reinterpret_cast<const float4*>(row + q_off + half);
+            turn(q0, q1);
+            *reinterpret_cast<float4*>(row + q_off) = q0;
+            *reinterpret_cast<float4*>(row + q_off + half) = q1;
         }
-        kdst[i] = __float2bfloat16_rn(k0);
-        kdst[i + half] = __float2bfloat16_rn(k1);
-        vdst[i] = __float2bfloat16_rn(row[v_off + h * Dh + i]);
-        vdst[i + half] = __float2bfloat16_rn(row[v_off + h * Dh + i + half]);
+        turn(k0, k1);
     }
+    auto put = [](__nv_bfloat16* dst, const float4& v) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    };
+    put(kdst, k0);
+    put(kdst + half, k1);
+    put(vdst, v0);
+    put(vdst + half, v1);
+}
+
+static csd_status launch_rope_append(float* src, int ld, int rows, int H, int q_off, int k_off, int v_off, int Dh, int pos0,
+                                     int cap, const float* cs, const float* sn, __nv_bfloat16* Kc, __nv_bfloat16* Vc,
+                                     cudaStream_t st) {
+    const size_t threads = (size_t)rows * H * (Dh / 8);
+    PdlLaunch L(dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st);
+    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, rope_append_kernel, src, ld, rows, H, q_off, k_off, v_off, Dh, pos0, cap, cs, sn, Kc, Vc));
+    count_launch();
+    return CSD_OK;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -392,19 +415,28 @@ static csd_status wide_linear(csd_model* M, const __nv_bfloat16* W, const __nv_b
 }
 
 // Attention of `m` <= M->wide_rows rows over K/V that are already in the cache: row r sees keys
-// [0, n_keys0 + r) when causal, all n_keys0 otherwise.
+// [0, n_keys0 + r) when causal, all n_keys0 otherwise.  The result is left in two-term form in wxs_attn.
+// rope: q is still to be rotated where launch_row_attention does that itself.
 static csd_status wide_attention(csd_model* M, const float* q, int ldq, int m, __nv_bfloat16* Kc, __nv_bfloat16* Vc, int cap,
-                                 int n_keys0, bool causal, const float* bias, int bias_len, int bias_zero, int q_pos0,
-                                 float* out, cudaStream_t st) {
+                                 int n_keys0, bool causal, bool rope, const float* bias, int bias_len, int bias_zero, int q_pos0,
+                                 cudaStream_t st) {
     const csd_model_config& c = M->cfg;
-    AttnArgs a;       // one launch over all rows where the tensor-core kernel applies (sub-blocks in its grid)
+    const int di = M->di;
+    AttnArgs a;
     a.q = q; a.ldq = ldq; a.m = m;
     a.Kc = Kc; a.Vc = Vc; a.cap = cap; a.H = c.n_heads; a.Dh = c.d_head;
     a.n_keys = n_keys0; a.causal = causal ? 1 : 0;
     a.scale = c.arch == 0 ? 1.f / sqrtf((float)c.d_head) : 1.f;
     a.bias = bias; a.bias_len = bias_len; a.bias_zero = bias_zero; a.q_pos0 = q_pos0;
-    a.out = out; a.ldo = M->di;
-    return attention(M, a, st);
+    if (row_attention_supported(c.d_head)) {
+        if (rope) { a.q_rope_cos = M->rope_c; a.q_rope_sin = M->rope_s; }
+        a.out_xs2 = M->wxs_attn; a.out_xs_ld = di; a.out_xs_rows = (m + 15) & ~15;
+        ProfScope ps(M, 1, st);
+        return launch_row_attention(a, st);
+    }
+    a.out = M->wattn; a.ldo = di;
+    CSD_TRY(attention(M, a, st));
+    return launch_wide_split(M->wattn, di, di, m, nullptr, M->wxs_attn, nullptr, st);
 }
 
 // Decoder pass over m <= M->wide_rows rows at positions kv_len .. kv_len+m-1: K/V of every layer are
@@ -436,14 +468,12 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
         }
         {   // rotate q and k, append k and v of all rows; the sub-blocks below then only read the cache
             ProfScope ps(M, 2, st);
-            rope_append_kernel<<<dim3(m, H), 64, 0, st>>>(M->wqkv, 3 * di, c.arch == 0 ? 0 : -1, di, 2 * di, Dh, kv_len, c.max_seq,
-                                                          c.arch == 0 ? M->rope_c : nullptr, c.arch == 0 ? M->rope_s : nullptr, Kl, Vl);
-            count_launch();
+            CSD_TRY(launch_rope_append(M->wqkv, 3 * di, m, H, c.arch == 0 && !row_attention_supported(Dh) ? 0 : -1, di, 2 * di, Dh, kv_len,
+                                       c.max_seq, c.arch == 0 ? M->rope_c : nullptr, c.arch == 0 ? M->rope_s : nullptr, Kl, Vl, st));
         }
         if (l + 1 == c.n_layers) break;    // the cache is complete; the rest of the last layer feeds nothing
-        CSD_TRY(wide_attention(M, M->wqkv, 3 * di, m, Kl, Vl, c.max_seq, kv_len + 1, true,
-                               c.arch == 1 ? M->dec_bias : nullptr, c.max_seq, c.max_seq - 1, kv_len, M->wattn, st));
-        CSD_TRY(launch_wide_split(M->wattn, di, di, m, nullptr, M->wxs_attn, nullptr, st));
+        CSD_TRY(wide_attention(M, M->wqkv, 3 * di, m, Kl, Vl, c.max_seq, kv_len + 1, true, c.arch == 0,
+                               c.arch == 1 ? M->dec_bias : nullptr, c.max_seq, c.max_seq - 1, kv_len, st));
         const __nv_bfloat16* after_o = c.arch == 1 ? y.norm_x : y.norm2;
         CSD_TRY(wide_linear(M, y.wo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d, after_o,
                             M->wssq, st));
@@ -452,8 +482,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
             CSD_TRY(wide_linear(M, y.xq, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, M->wqkv, 3 * di, EPI_STORE, nullptr, 0,
                                 nullptr, nullptr, st));
             CSD_TRY(wide_attention(M, M->wqkv, 3 * di, m, M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x,
-                                   c.max_enc_len, M->enc_len, false, nullptr, 0, 0, 0, M->wattn, st));
-            CSD_TRY(launch_wide_split(M->wattn, di, di, m, nullptr, M->wxs_attn, nullptr, st));
+                                   c.max_enc_len, M->enc_len, false, false, nullptr, 0, 0, 0, st));
             CSD_TRY(wide_linear(M, y.xo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d, y.norm2,
                                 M->wssq, st));
             cnt = wide_ssq_pieces(m, d, di, false);
@@ -492,14 +521,12 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
                                         EPI_STORE, nullptr, 0, nullptr, nullptr, st));
             }
         }
-        rope_append_kernel<<<dim3(n, H), 64, 0, st>>>(M->qkv_enc, 3 * di, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->ek, M->ev);
-        count_launch();
+        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->ek, M->ev, st));
         for (int r0 = 0; r0 < n; r0 += WR) {
             const int m = n - r0 < WR ? n - r0 : WR;
             float* xr = M->xenc + (size_t)r0 * d;
-            CSD_TRY(wide_attention(M, M->qkv_enc + (size_t)r0 * 3 * di, 3 * di, m, M->ek, M->ev, E, n, false, M->enc_bias,
-                                   2 * E - 1, E - 1, r0, M->wattn, st));
-            CSD_TRY(launch_wide_split(M->wattn, di, di, m, nullptr, M->wxs_attn, nullptr, st));
+            CSD_TRY(wide_attention(M, M->qkv_enc + (size_t)r0 * 3 * di, 3 * di, m, M->ek, M->ev, E, n, false, false, M->enc_bias,
+                                   2 * E - 1, E - 1, r0, st));
             CSD_TRY(wide_linear(M, y.wo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, xr, d, EPI_ADD, M->wxs_x, d, y.norm2,
                                 M->wssq, st));
             CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, wide_ssq_pieces(m, d, di, false), nullptr, ff,
@@ -520,9 +547,7 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
             CSD_TRY(wide_linear(M, y.xv, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, out + 2 * di, 3 * di, EPI_STORE, nullptr, 0,
                                 nullptr, nullptr, st));
         }
-        rope_append_kernel<<<dim3(n, H), 64, 0, st>>>(M->qkv_enc, 3 * di, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr,
-                                                      M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x);
-        count_launch();
+        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x, st));
     }
     CSD_CUDA(cudaGetLastError());
     return CSD_OK;
@@ -685,9 +710,7 @@ extern "C" csd_status csd_encoder_forward(csd_model* M, const int32_t* enc_token
             const int m = n - r0 < CH ? n - r0 : CH;
             CSD_TRY(project_qkv(M, y, M->xenc + (size_t)r0 * d, m, M->qkv_enc + (size_t)r0 * 3 * di, st));
         }
-        rope_append_kernel<<<dim3(n, H), 64, 0, st>>>(M->qkv_enc, 3 * di, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr,
-                                                      M->ek, M->ev);
-        count_launch();
+        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->ek, M->ev, st));
         for (int r0 = 0; r0 < n; r0 += CH) {
             const int m = n - r0 < CH ? n - r0 : CH;
             AttnArgs a;
@@ -710,9 +733,7 @@ extern "C" csd_status csd_encoder_forward(csd_model* M, const int32_t* enc_token
             CSD_TRY(linear(M, y.xk, nullptr, di, d, xr, d, m, M->enc_final_norm, o + di, 3 * di, EPI_STORE, st));
             CSD_TRY(linear(M, y.xv, nullptr, di, d, xr, d, m, M->enc_final_norm, o + 2 * di, 3 * di, EPI_STORE, st));
         }
-        rope_append_kernel<<<dim3(n, H), 64, 0, st>>>(M->qkv_enc, 3 * di, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr,
-                                                      M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x);
-        count_launch();
+        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x, st));
     }
     CSD_CUDA(cudaGetLastError());
     M->enc_len = n;
