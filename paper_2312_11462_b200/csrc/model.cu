@@ -824,7 +824,8 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
     if (!segs) { segs = &whole; nseg = 1; }
     const csd_model_config& c = M->cfg;
     if (m < 1 || m > c.max_rows || kv_len < 0) return CSD_ERR_INVALID_ARG;
-    if (kv_len + m > c.max_seq) return CSD_ERR_CAPACITY;
+    for (int g = 0; g < nseg; ++g)                 // (of a batch, each block behind its own sequence's cache)
+        if (segs[g].kv_len + segs[g].rows > c.max_seq) return CSD_ERR_CAPACITY;
     if (c.arch == 1 && M->enc_len < 1) return CSD_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, V = c.vocab;

@@ -71,3 +71,18 @@ def test_batch_argument_errors(b):
         b.csd_review_forward_batch([m1, m2], [t[:9], t[:9]], [0, 0])        # 18 rows
     out = b.csd_review_forward_batch([m1, m2], [t[:8], t[:9]], [0, 0])
     assert out[0].shape[0] == 8 and out[1].shape[0] == 9
+
+
+def test_first_sequence_fills_its_cache(b, orc):
+    shape = SHAPES["tiny_target"]
+    blob = workloads.make_weights(shape, seed=22, device="cuda", std=0.05, gain_std=0.1)
+    seqs = [workloads.make_prompt(shape.vocab, shape.max_seq, seed=50 + i) for i in range(2)]
+    kv, rows = [shape.max_seq - 2, 9], [2, 5]
+    gms, oms = [b.Model(shape, blob) for _ in kv], [orc.Model(shape, orc.blob_to_u16(blob)) for _ in kv]
+    for i in range(2):
+        gms[i].csd_prefill(to_dev_i32(seqs[i][:kv[i]]), 0)
+        oms[i].review_forward(seqs[i][:kv[i]], 0)
+    got = b.csd_review_forward_batch(gms, [to_dev_i32(seqs[i][kv[i]:kv[i] + rows[i]]) for i in range(2)], kv)
+    for i in range(2):
+        ref = oms[i].review_forward(seqs[i][kv[i]:kv[i] + rows[i]], kv[i])
+        assert rel_l2(got[i].cpu().numpy(), ref) <= LOGIT_REL_L2
