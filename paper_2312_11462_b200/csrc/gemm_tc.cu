@@ -295,6 +295,13 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 if (++kb == p.nkb) { kb = 0; ++tile; }
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
+            // Cluster split: the slot that no load needs any more takes the other ranks' parts (see the epilogue), and they
+            // may write once its MMAs are done, a ring before the last.  (Asked for after the last MMA it cost the four
+            // CTAs a round trip: 16 layers of the 7B shape at 5 rows 1469 us, 1448 so.)
+            if (p.csplit > 1 && crank == 0 && !*abort_flag) {
+                if (items >= p.stages && !mbar_wait(&ctl->empty[s], ph)) *abort_flag = 1;
+                for (int r = 1; r < p.csplit; ++r) remote_arrive(map_to_cta(smem_u32(&ctl->red_ready), (uint32_t)r));
+            }
         }
     } else if (warp == 1) {
         // ---- MMA issuer: one accumulator set per segment (the part of a tile inside this CTA's range)
@@ -451,13 +458,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             if (lane == 0) mbar_arrive(&ctl->acc_empty[b]);
             if (p.csplit > 1) {
                 // Cluster split: the four CTAs of the cluster hold the four K ranges of this tile.  Rank 0
-                // finishes the tile; when its own MMAs are done its ring is free, it tells the others, they
+                // finishes the tile: its producer has told the others which of its ring slots is free, they
                 // write their parts into it (distributed shared memory) and signal back, and it adds the
                 // parts in rank order.
-                float* buf = reinterpret_cast<float*>(ring);          // [3][NT * M][128]
+                const unsigned len0 = (unsigned)p.nkb / (unsigned)p.csplit, slots = (unsigned)p.stages;   // rank 0's items
+                float* buf = reinterpret_cast<float*>(ring + (size_t)(len0 >= slots ? len0 % slots : len0) * STAGE);   // [3][NT * M][128]
                 if (crank == 0) {
-                    if (et == 0)
-                        for (int r = 1; r < p.csplit; ++r) remote_arrive(map_to_cta(smem_u32(&ctl->red_ready), (uint32_t)r));
                     if (!mbar_wait_cluster(&ctl->red_done, 0)) *abort_flag = 1;
 #pragma unroll
                     for (int r = 1; r < 4; ++r)
