@@ -740,20 +740,25 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
     merge_splits<DH, C::REC>(cluster, rec, p, h, split, m);
     cluster.sync();       // no CTA leaves while another may still read its record
 }
-// One 64-key tile per CTA while that keeps the splits of a head inside one portable cluster (8)
-// and the grid near two CTAs per SM: short caches are latency-bound, and more splits mean more
-// tiles in flight at once; long caches walk several tiles per CTA, two requests ahead.
 static bool g_attn_cuda_cores = false;
 void set_attention_cuda_cores(bool on) { g_attn_cuda_cores = on; }
 bool row_attention_supported(int Dh) { return (Dh == 64 || Dh == 128) && !g_attn_cuda_cores; }
 
-int attn_splits(int total_keys, int H) {
-    int by_sm = (2 * 148 + H - 1) / H;
-    int by_len = (total_keys + TILE - 1) / TILE;
-    int n = by_sm < by_len ? by_sm : by_len;
-    if (n < 1) n = 1;
+// Splits per head: one 64-key tile per CTA while that keeps the splits of a head inside one portable cluster (8) and the
+// grid near two CTAs per SM (short caches are latency-bound, and more splits mean more tiles in flight at once); long
+// caches walk several tiles per CTA, two requests ahead.  At head dimension 128 one CTA fits beside a GEMM's on an SM, and
+// how many more than the SMs there are pays depends on the output projection behind it (8 layers of the 7B shape):
+//   up to 5 rows it leaves SMs free.  Caches of 5 to 8 tiles do with a CTA per SM, each walking two (5 rows, 300 keys: 774 us
+//   with 5 splits, 761 with 3); longer ones gain from all 8 (1000 keys: 800 us, 806 with 7).
+//   larger blocks fill every SM with it, and the last CTAs of clusters of 8 start only when it is through (9 rows, 1000 keys:
+//   882 us with 8, 845 with 7; 17 rows, 1500 keys: 1105, 1031), so 7 at most.
+int attn_splits(int total_keys, int H, int Dh, int gemm_rows) {
+    const int by_sm = (2 * 148 + H - 1) / H, tiles = (total_keys + TILE - 1) / TILE;
+    int n = by_sm < tiles ? by_sm : tiles;
     if (n > MAX_SPLITS) n = MAX_SPLITS;
-    return n;
+    if (Dh == 128 && gemm_rows > 5 && n == MAX_SPLITS) n = MAX_SPLITS - 1;
+    if (Dh == 128 && gemm_rows <= 5 && n == tiles && tiles > 4 && H * tiles > 148) n = (tiles + 1) / 2;
+    return n < 1 ? 1 : n;
 }
 
 static void attn_launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, const AttnParams& ap, size_t smem,
@@ -848,7 +853,7 @@ static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st) {
         ap.tree = 1;
         for (int r = 0; r < MAXM; ++r) { ap.tmask[r] = r < a.m ? a.tree_mask[r] : 0u; ap.tdepth[r] = r < a.m ? (unsigned char)a.tree_depth[r] : 0; }
     }
-    ap.nsplit = attn_splits(total, a.H);
+    ap.nsplit = attn_splits(total, a.H, a.Dh, a.out_xs_rows > 0 ? a.out_xs_rows : a.m);
     int len = (total + ap.nsplit - 1) / ap.nsplit;
     ap.split_len = (len + TILE - 1) / TILE * TILE;
     ap.nsplit = (total + ap.split_len - 1) / ap.split_len;

@@ -47,7 +47,7 @@ struct AttnArgs {
     const int* tree_depth = nullptr;
 };
 
-int attn_splits(int total_keys, int H);
+int attn_splits(int total_keys, int H, int Dh, int gemm_rows);   // gemm_rows: rows of the projection that follows
 void set_attention_cuda_cores(bool on);   // true: always the CUDA-core kernel (for comparison runs)
 csd_status launch_attention(const AttnArgs& a, cudaStream_t st);
 // Whether the rows of a wide pass take launch_row_attention: head dimension 64 or 128, comparison switch off.
