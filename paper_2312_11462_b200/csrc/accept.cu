@@ -12,7 +12,7 @@
 //            max(0, p - q) (or of p after k acceptances); the CTA that finishes a row last takes
 //            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
-#include "common.cuh"
+#include "model.cuh"
 #include "philox.cuh"
 #include <math.h>
 #include <mutex>
@@ -692,8 +692,9 @@ __device__ __forceinline__ StatPartial cluster_read_stat(const StatPartial* loca
 template <bool VEC, int PER>
 __global__ void __launch_bounds__(AR_THREADS, 1)
 accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, const int* __restrict__ onehot,
-                  const int* __restrict__ tokens, int rows, int k, int V, float temperature, float lenience, uint64_t seed,
-                  uint64_t step, int csize, int S, int pieces, int* __restrict__ n_acc, int* __restrict__ out_tok, int* status) {
+                  const int* tokens, int rows, int k, int V, float temperature, float lenience, uint64_t seed,
+                  uint64_t step, int csize, int S, int pieces, int* __restrict__ n_acc, int* __restrict__ out_tok, int* seq,
+                  int* status) {
     __shared__ StatPartial s_task[AR_TASKS];
     __shared__ StatPartial s_own[2 * MAX_K + 1];       // this CTA's slice of every vector
     __shared__ float s_mx[2 * MAX_K + 1], s_z[2 * MAX_K + 1];
@@ -804,8 +805,11 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
     int n = 0;
     while (n < k && s_acc[n]) ++n;
     if (rank == 0 && tid == 0) {
+        if (greedy) {
+            if (seq) seq[n] = s_arg[n];                // (`seq` may be `tokens`: every CTA has read those by now)
+            out_tok[row] = s_arg[n];
+        }
         n_acc[row] = n;
-        if (greedy) out_tok[row] = s_arg[n];
     }
     if (greedy) {
         cluster_sync_all();                            // no CTA leaves while another may still read its statistics
@@ -921,7 +925,11 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
                 if (mass) last = first + 31 - __clz(mass);
                 cum += __shfl_sync(0xffffffffu, incl, 31);
             }
-            if (lane == 0) out_tok[row] = pick >= 0 ? pick : max(last, 0);
+            if (lane == 0) {
+                const int y = pick >= 0 ? pick : max(last, 0);
+                if (seq) seq[n] = y;
+                out_tok[row] = y;
+            }
         }
     }
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
@@ -1028,7 +1036,7 @@ static int row_clusters(int csize) {
 template <bool VEC, int PER>
 static csd_status launch_accept_row(const float* tl, const float* dl, const int* onehot, const int* tokens, int rows, int k,
                                     int V, float temperature, float lenience, uint64_t seed, uint64_t step, int csize,
-                                    int* n_acc, int* out_tok, int* status, cudaStream_t st, bool* done) {
+                                    int* n_acc, int* out_tok, int* seq, int* status, cudaStream_t st, bool* done) {
     *done = false;
     const int S = ((V + csize - 1) / csize + 3) & ~3, nvec = dl ? 2 * k + 1 : k + 1;
     // (a CTA takes in about 40 GB/s here: beyond about 320 KB of slices the stats pass over all SMs is faster; one row,
@@ -1045,7 +1053,7 @@ static csd_status launch_accept_row(const float* tl, const float* dl, const int*
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
     CSD_CUDA(cudaLaunchKernelEx(&cfg, accept_row_kernel<VEC, PER>, tl, dl, onehot, tokens, rows, k, V, temperature, lenience,
-                                seed, step, csize, S, pieces, n_acc, out_tok, status));
+                                seed, step, csize, S, pieces, n_acc, out_tok, seq, status));
     count_launch();
     *done = true;
     return CSD_OK;
@@ -1057,7 +1065,7 @@ static csd_status launch_accept_row(const float* tl, const float* dl, const int*
 static csd_status run_accept(const float* tl, const float* dl_in, const int32_t* onehot, const int32_t* tokens, int rows,
                              int k, int V, float temperature, float lenience, uint64_t seed, uint64_t step,
                              int32_t* n_acc, int32_t* out_tok, char* ws, const AcceptLayout& L, int* status,
-                             cudaStream_t st) {
+                             cudaStream_t st, int32_t* seq = nullptr, bool* seq_written = nullptr) {
     StatPartial* part = (StatPartial*)(ws + L.part_off);
     RowInfo* info = (RowInfo*)(ws + L.info_off);
     double2* zpart = (double2*)(ws + L.z_off);
@@ -1087,11 +1095,12 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
         bool done = false;
         csd_status s;
         if (vec_ok)
-            s = wide ? launch_accept_row<true, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done)
-                     : launch_accept_row<true, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done);
+            s = wide ? launch_accept_row<true, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
+                     : launch_accept_row<true, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
         else
-            s = wide ? launch_accept_row<false, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done)
-                     : launch_accept_row<false, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, status, st, &done);
+            s = wide ? launch_accept_row<false, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
+                     : launch_accept_row<false, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
+        if (seq_written) *seq_written = done && seq;
         if (s != CSD_OK || done) return s;
     }
     const long long items = nvec * L.nchunk_a;
@@ -1149,11 +1158,11 @@ extern "C" size_t csd_spec_accept_workspace_bytes(int rows, int k, int V) {
     return accept_layout(rows, k, V).total;
 }
 
-extern "C" csd_status csd_spec_accept(const float* target_logits_dev, const float* draft_logits_dev,
-                                      const int32_t* onehot_dev, const int32_t* draft_tokens_dev, int rows, int k,
-                                      int V, float temperature, float lenience, uint64_t seed, uint64_t step,
-                                      int32_t* n_accepted_dev, int32_t* out_token_dev, void* workspace_dev,
-                                      size_t workspace_bytes, void* stream) {
+namespace csd {
+csd_status accept_into(const float* target_logits_dev, const float* draft_logits_dev, const int32_t* onehot_dev,
+                       const int32_t* draft_tokens_dev, int rows, int k, int V, float temperature, float lenience, uint64_t seed,
+                       uint64_t step, int32_t* n_accepted_dev, int32_t* out_token_dev, void* workspace_dev,
+                       size_t workspace_bytes, void* stream, int32_t* seq, bool* seq_written) {
     if (rows < 0 || k < 0 || k > MAX_K || V < 1 || !(temperature >= 0.f) || !(lenience >= 1.f))
         return CSD_ERR_INVALID_ARG;
     if (rows == 0) return CSD_OK;
@@ -1166,7 +1175,18 @@ extern "C" csd_status csd_spec_accept(const float* target_logits_dev, const floa
     int* status = status_word_device();
     if (!status) return CSD_ERR_CUDA;
     return run_accept(target_logits_dev, draft_logits_dev, onehot_dev, draft_tokens_dev, rows, k, V, temperature, lenience,
-                      seed, step, n_accepted_dev, out_token_dev, (char*)workspace_dev, L, status, (cudaStream_t)stream);
+                      seed, step, n_accepted_dev, out_token_dev, (char*)workspace_dev, L, status, (cudaStream_t)stream, seq,
+                      seq_written);
+}
+}  // namespace csd
+
+extern "C" csd_status csd_spec_accept(const float* target_logits_dev, const float* draft_logits_dev,
+                                      const int32_t* onehot_dev, const int32_t* draft_tokens_dev, int rows, int k,
+                                      int V, float temperature, float lenience, uint64_t seed, uint64_t step,
+                                      int32_t* n_accepted_dev, int32_t* out_token_dev, void* workspace_dev,
+                                      size_t workspace_bytes, void* stream) {
+    return accept_into(target_logits_dev, draft_logits_dev, onehot_dev, draft_tokens_dev, rows, k, V, temperature, lenience, seed,
+                       step, n_accepted_dev, out_token_dev, workspace_dev, workspace_bytes, stream, nullptr, nullptr);
 }
 
 

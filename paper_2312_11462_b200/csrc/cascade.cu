@@ -149,8 +149,9 @@ static csd_status review(Gen& g, int r, int P, int nd) {
     const float len_r = r == 0 ? 1.f : g.lenience;   // lenience never applies when the target reviews
     volatile int32_t* res = g.pinned;
     res[0] = -1; res[1] = -1;                        // the kernels overwrite both with values >= 0
-    csd_status s = csd_spec_accept(target, dl, onehot, g.seq + P, 1, nd, V, g.temperature, len_r, g.seed, g.step++,
-                                   g.result_map, g.result_map + 1, g.accept_ws, g.accept_bytes, g.stream);
+    bool placed = false;                             // the kernel has put the output token into the sequence
+    csd_status s = accept_into(target, dl, onehot, g.seq + P, 1, nd, V, g.temperature, len_r, g.seed, g.step++, g.result_map,
+                               g.result_map + 1, g.accept_ws, g.accept_bytes, g.stream, g.seq + P, &placed);
     if (s != CSD_OK) return s;
     // The accept kernels write (n_acc, out token) straight into mapped pinned host memory.  The host
     // watches the two words instead of sleeping in a stream synchronisation (whose wake-up costs more
@@ -165,8 +166,10 @@ static csd_status review(Gen& g, int r, int P, int nd) {
     if (res[0] < 0 || res[1] < 0) CSD_CUDA(cudaStreamSynchronize(g.stream));
     const int n_acc = g.pinned[0];
     if (n_acc < 0 || n_acc > nd) return CSD_ERR_CUDA;
-    g.pinned[CSD_MAX_ROWS + 8] = g.pinned[1];     // (a slot the next review does not overwrite while this copy is in flight)
-    CSD_CUDA(cudaMemcpyAsync(g.seq + P + n_acc, g.pinned + CSD_MAX_ROWS + 8, 4, cudaMemcpyHostToDevice, g.stream));
+    if (!placed) {
+        g.pinned[CSD_MAX_ROWS + 8] = g.pinned[1];     // (a slot the next review does not overwrite while this copy is in flight)
+        CSD_CUDA(cudaMemcpyAsync(g.seq + P + n_acc, g.pinned + CSD_MAX_ROWS + 8, 4, cudaMemcpyHostToDevice, g.stream));
+    }
     g.st->reviews[r] += 1;
     g.st->drafted[r] += nd;
     g.st->accepted[r] += n_acc;

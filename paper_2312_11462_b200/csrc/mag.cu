@@ -76,6 +76,7 @@ __global__ void mag_build_kernel(const int32_t* __restrict__ hay, int L, int max
 }
 
 constexpr int MAG_MAX_N = 64;
+constexpr int AHEAD = 4;
 
 __global__ void __launch_bounds__(32)
 mag_draft_kernel(const int32_t* __restrict__ hay, int L, const int32_t* __restrict__ bigram, int V,
@@ -90,58 +91,94 @@ mag_draft_kernel(const int32_t* __restrict__ hay, int L, const int32_t* __restri
     __shared__ int32_t tail[CSD_MAG_MAX_ORDER + MAG_MAX_N];
     const int lane = threadIdx.x;
     const int keep = T < max_order ? T : max_order;
+    // (the kernel after this one may set itself up now; it waits before it reads what is written here)
+    pdl_trigger();
+    pdl_wait();
     for (int i = lane; i < keep; i += 32) tail[i] = seq[T - keep + i];
     __syncwarp();
     int len = keep;       // valid tokens in tail
     int total = T;        // length of the (virtual) full sequence
     int made = 0;
     while (made < n) {
-        const int limit = min(min(total, max_order), len);
+        // Without a hit the next tokens are the bigram chain from the last one.  Follow it for up to AHEAD tokens at once
+        // and request the table entries of all the suffixes that result together: one round trip instead of one (table,
+        // then bigram) per token.  Four tokens without a hit: MAG_MEASURED.
+        const int steps = G > 0 ? 1 : min(AHEAD, n - made);
+        int32_t nx[AHEAD];
+        bool bad[AHEAD];
+        {
+            int32_t last = tail[len - 1];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) {
+                bad[j] = last < 0 || last >= V;
+                nx[j] = j < steps && !bad[j] ? bigram[last] : 0;
+                last = nx[j];
+                if (j < steps && lane == 0) tail[len + j] = nx[j];
+            }
+        }
+        __syncwarp();
         const int order = lane + 1;
-        int hit = -1;
-        if (order <= limit && slots > 0) {
-            const int32_t* g = tail + len - order;
-            uint32_t h = gram_hash(g, order) & (uint32_t)(slots - 1);
-            for (int probe = 0; probe < slots; ++probe) {
-                int cur = table[h];
-                if (cur == EMPTY_SLOT) break;
+        int first[AHEAD];
+        uint32_t at[AHEAD];
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            first[j] = EMPTY_SLOT;
+            at[j] = 0;
+            if (j < steps && slots > 0 && order <= min(min(total + j, max_order), len + j)) {
+                at[j] = gram_hash(tail + len + j - order, order) & (uint32_t)(slots - 1);
+                first[j] = table[at[j]];
+            }
+        }
+        bool copied = false;
+        int taken = 0;
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            if (j >= steps || copied) break;
+            const int limit = min(min(total + j, max_order), len + j);
+            const int32_t* g = tail + len + j - order;
+            int hit = -1, cur = first[j];
+            uint32_t h = at[j];
+            for (int probe = 0; cur != EMPTY_SLOT && probe < slots; ++probe) {
                 if ((cur & 63) == order && same_gram(hay + (cur >> 6), g, order)) { hit = cur >> 6; break; }
                 h = (h + 1) & (uint32_t)(slots - 1);
+                cur = table[h];
             }
-        }
-        if (G > 0) {
-            // ends e in [L-1, LJ-2]: the occurrence's follower e+1 exists and is generated text
-            best_end[lane + 1] = 0x7fffffff;
-            __syncwarp();
-            for (int e = max(L - 1, 0) + lane; e <= LJ - 2; e += 32) {
-                int agree = 0;
-                while (agree < limit && agree <= e && joined(e - agree) == tail[len - 1 - agree]) ++agree;
-                for (int o = 1; o <= agree; ++o) atomicMin(&best_end[o], e);
+            if (G > 0) {
+                // ends e in [L-1, LJ-2]: the occurrence's follower e+1 exists and is generated text
+                best_end[lane + 1] = 0x7fffffff;
+                __syncwarp();
+                for (int e = max(L - 1, 0) + lane; e <= LJ - 2; e += 32) {
+                    int agree = 0;
+                    while (agree < limit && agree <= e && joined(e - agree) == tail[len - 1 - agree]) ++agree;
+                    for (int o = 1; o <= agree; ++o) atomicMin(&best_end[o], e);
+                }
+                __syncwarp();
+                if (hit < 0 && order <= limit && best_end[order] != 0x7fffffff) hit = best_end[order] - order + 1;
+                __syncwarp();
             }
-            __syncwarp();
-            if (hit < 0 && order <= limit && best_end[order] != 0x7fffffff) hit = best_end[order] - order + 1;
-            __syncwarp();
-        }
-        const unsigned ballot = __ballot_sync(0xffffffffu, hit >= 0);
-        if (ballot == 0) {
-            int32_t last = tail[len - 1];
-            int32_t nx = 0;
-            if (last >= 0 && last < V) nx = bigram[last];
-            else if (lane == 0) set_status(status, CSD_ERR_BAD_TOKEN);
-            if (lane == 0) { tail[len] = nx; out[made] = nx; }
-            len += 1; total += 1; made += 1;
-        } else {
+            const unsigned ballot = __ballot_sync(0xffffffffu, hit >= 0);
+            if (ballot == 0) {
+                if (lane == 0) {
+                    out[made + j] = nx[j];
+                    if (bad[j]) set_status(status, CSD_ERR_BAD_TOKEN);
+                }
+                taken = j + 1;
+                continue;
+            }
             const int best = 31 - __clz(ballot);              // lane of the longest order that hit
             const int start = __shfl_sync(0xffffffffu, hit, best);
-            int idx = start + best + 1;                      // haystack index of the next token
-            int cnt = min(n - made, LJ - idx);
+            const int idx = start + best + 1;                 // haystack index of the next token
+            const int cnt = min(n - made - j, LJ - idx);
+            __syncwarp();
             for (int i = lane; i < cnt; i += 32) {
-                int32_t t = joined(idx + i);
-                tail[len + i] = t;
-                out[made + i] = t;
+                const int32_t t = joined(idx + i);
+                tail[len + j + i] = t;
+                out[made + j + i] = t;
             }
-            len += cnt; total += cnt; made += cnt;
+            taken = j + cnt;
+            copied = true;
         }
+        len += taken; total += taken; made += taken;
         __syncwarp();
     }
 }
@@ -209,10 +246,10 @@ static csd_status mag_draft(csd_mag* g, const int32_t* seq_dev, int T, int gen_f
     if (n < 1 || n > MAG_MAX_N) return CSD_ERR_INVALID_ARG;
     int* status = status_word_device();
     if (!status) return CSD_ERR_CUDA;
-    mag_draft_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(g->hay, g->L, g->bigram, g->V, g->table, g->slots,
-                                                          g->max_order, seq_dev, T, gen_from, n, out_tokens_dev, status);
+    PdlLaunch pl(dim3(1), dim3(32), 0, (cudaStream_t)stream);
+    CSD_CUDA(cudaLaunchKernelEx(&pl.cfg, mag_draft_kernel, g->hay, g->L, g->bigram, g->V, (const int*)g->table, g->slots,
+                                g->max_order, seq_dev, T, gen_from, n, out_tokens_dev, status));
     count_launch();
-    CSD_CUDA(cudaGetLastError());
     return CSD_OK;
 }
 

@@ -838,8 +838,9 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
         const LayerW& y0 = M->dec[0];
         const bool fused_qkv = y0.wk == y0.wq + (size_t)di * d && y0.wv == y0.wk + (size_t)di * d;
         if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
-            embed_split_kernel<<<dim3((unsigned)split_ssq_entries(d), (unsigned)m), 128, 0, st>>>(
-                block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x, M->ssq_x, M->status);
+            PdlLaunch L(dim3((unsigned)split_ssq_entries(d), (unsigned)m), dim3(128), 0, st);
+            CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_split_kernel, block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x,
+                                        M->ssq_x, M->status));
             M->ssq_x_cnt = split_ssq_entries(d);
             x_ready = true;
             count_launch();

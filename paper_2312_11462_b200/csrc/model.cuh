@@ -51,6 +51,13 @@ struct csd_model {
 };
 
 namespace csd {
+// csd_spec_accept that also puts the output token at seq[number accepted] where it runs as one kernel (*seq_written says
+// whether it did); one row; seq may be the draft tokens themselves.
+csd_status accept_into(const float* target_logits_dev, const float* draft_logits_dev, const int32_t* onehot_dev,
+                       const int32_t* draft_tokens_dev, int rows, int k, int V, float temperature, float lenience, uint64_t seed,
+                       uint64_t step, int32_t* n_accepted_dev, int32_t* out_token_dev, void* workspace_dev,
+                       size_t workspace_bytes, void* stream, int32_t* seq, bool* seq_written);
+
 // Records an event pair around the launches made during its lifetime when profiling is on.
 struct ProfScope {
     csd_model* M; cudaStream_t st; bool on;
