@@ -47,10 +47,11 @@ struct __align__(8) WgCtrl {
     int abort_flag;
     float scale[256];                        // rms-norm factors of the tile's tokens
 };
-// Epilogue staging: per token half two buffers of 16 tokens x 128 weight rows.  An accumulator thread owns one
-// weight row, memory wants the rows of a token side by side: through these buffers a warp gets 4 whole
-// 128-row stretches per chunk and moves 16 bytes per lane.
-constexpr size_t WG_STAGING = 2 * 2 * 16 * TILE_N * sizeof(float);
+// Epilogue staging: a warp's 32 weight rows x 16 tokens (of both matrices of a gated pair).  An accumulator thread owns one
+// weight row, memory wants the rows of a token side by side.  A single matrix's second half holds the pieces of the
+// sums of squares (one float per quadrant and token).
+constexpr size_t WG_STAGING = 2 * 8 * 16 * 32 * sizeof(float);
+static_assert(8 * 16 * 32 + 4 * WG_SET <= 2 * 8 * 16 * 32, "sums of squares fit behind the staging of a single matrix");
 
 // How a launch is divided.  tiles = row tiles x token tiles, tokens fastest, so that pairs running at the
 // same time share weight rows in L2.  Three ways:
@@ -319,8 +320,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const uint32_t part_bytes = (uint32_t)(TILE_N * NT * sizeof(float)) * (uint32_t)nt;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0u);
-        float* stage_mem = staging + half * (2 * 16 * TILE_N);
-        unsigned g = 0, chunks_done = 0;
+        unsigned g = 0;
 #pragma unroll 1
         for (int i = 0; i < items;) {
             const int tile = (int)((u0 + i) / p.nkb), kb_begin = (int)((u0 + i) % p.nkb);
@@ -426,12 +426,15 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             } else {
                 asm volatile("bar.sync 1, 256;" ::: "memory");    // the tile's scale factors are written
             }
-            // ---- finish, 16 tokens at a time: accumulators -> staging -> this warp's 4 tokens of the chunk, of which
-            //      a lane holds 4 neighbouring weight rows
+            // ---- finish, 16 tokens at a time, each warp for itself: its 32 weight rows x 16 tokens go through its own
+            //      staging so that a lane then holds 4 neighbouring rows of a token, 8 lanes a token's whole 128 bytes.
+            //      (Staged by four warps for 128 rows, a chunk waited at two barriers: T5-xxl-shaped source of
+            //      256 tokens 7.5 ms, 6.8 so.)
             const bool scaled = p.ssq_in && p.pk == 1;
-            const int n0 = row_tile * WG_ROWS + rank * TILE_N, n = n0 + lane * 4;
+            const int c = (lane & 7) * 4, e0 = lane >> 3;     // this lane's rows of the warp's 32, first of its tokens (every 4th)
+            const int n = row_tile * WG_ROWS + rank * TILE_N + q * 32 + c;
             const int have = min(4, p.N - n);                 // weight rows of this lane inside the matrix
-            const bool vec = have == 4 && p.vec_y;
+            const bool vec = have == 4 && p.vec_y, add = p.epilogue == EPI_ADD;
             float gain[4] = {1.f, 1.f, 1.f, 1.f};
             if (p.out_xs && p.out_gain) {
 #pragma unroll
@@ -439,37 +442,14 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     if (j < have) gain[j] = __bfloat162float(p.out_gain[n + j]);
             }
             float* Y = p.Y ? p.Y + (p.pk > 1 ? (size_t)(pair % p.pk) * p.plane : 0) + n : nullptr;
-#pragma unroll 1
-            for (int ch = 0; ch < nch; ++ch) {
-                const int c0 = half * htok + ch * 16, r0 = tok0 + c0;     // column in the tile, token
-                if (r0 >= m) break;                           // (the same for the four warps of a half)
-                // (one matrix: two buffers in turn, one barrier; the pair: both matrices in one buffer, two barriers)
-                float* buf = stage_mem + (DUAL ? 0 : (chunks_done & 1) * (16 * TILE_N));
-                if (DUAL && chunks_done > 0) asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
-                ++chunks_done;
-                float* put = buf + q * 32 + lane;
-                // Registers have no index: one short copy per chunk, everything else is a loop over the chunks.  Unrolled
-                // over the chunks (100 KB of instructions, pushed out of the caches by the weight stream before every
-                // use) it ran at the speed of instruction fetch: up to 3 us a chunk, all SMs in step, against 1 us.
-#define WG_PUT(C)                                                                                                       \
-    case C:                                                                                                             \
-        if (C < CH) {                                                                                                   \
-            _Pragma("unroll") for (int e = 0; e < 16; ++e) {                                                            \
-                put[e * TILE_N] = acc[(C < CH ? C : 0) * 16 + e];                                                       \
-                if (DUAL) put[(16 + e) * TILE_N] = acc[((NT - 1) * CH + (C < CH ? C : 0)) * 16 + e];                    \
-            }                                                                                                           \
-        }                                                                                                               \
-        break;
-                switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
-#undef WG_PUT
-                asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
-                const int rw = r0 + q * 4;                    // this warp's tokens
-                float x[4][4], old[4][4];
+            float old[4][4];                                  // residual values of a chunk, requested a chunk ahead
+            auto load_old = [&](int ch) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
+                    const int r = tok0 + half * htok + ch * 16 + 4 * k + e0;
                     old[k][0] = old[k][1] = old[k][2] = old[k][3] = 0.f;
-                    if (p.epilogue == EPI_ADD && rw + k < m) {            // their residual rows, requested together
-                        const float* y = Y + (size_t)(rw + k) * p.ldy;
+                    if (add && ch < nch && r < m) {
+                        const float* y = Y + (size_t)r * p.ldy;
                         if (vec) {
                             const float4 v = __ldcg(reinterpret_cast<const float4*>(y));
                             old[k][0] = v.x; old[k][1] = v.y; old[k][2] = v.z; old[k][3] = v.w;
@@ -480,14 +460,40 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         }
                     }
                 }
+            };
+            load_old(0);
+            float* buf = staging + ew * (NT * 16 * 32);
+            float* sums = staging + 8 * 16 * 32;              // [quadrant][token]: sums of squares over a warp's 32 rows
+#pragma unroll 1
+            for (int ch = 0; ch < nch; ++ch) {
+                const int c0 = half * htok + ch * 16, r0 = tok0 + c0;     // column in the tile, token
+                if (r0 >= m) break;                           // (the same for the four warps of a half)
+                float* put = buf + lane;
+                // Registers have no index: one short copy per chunk, everything else is a loop over the chunks.  Unrolled
+                // over the chunks (100 KB of instructions, pushed out of the caches by the weight stream before every
+                // use) it ran at the speed of instruction fetch: up to 3 us a chunk, all SMs in step, against 1 us.
+                __syncwarp();                                 // the chunk before has been read
+#define WG_PUT(C)                                                                                                       \
+    case C:                                                                                                             \
+        if (C < CH) {                                                                                                   \
+            _Pragma("unroll") for (int e = 0; e < 16; ++e) {                                                            \
+                put[e * 32] = acc[(C < CH ? C : 0) * 16 + e];                                                           \
+                if (DUAL) put[(16 + e) * 32] = acc[((NT - 1) * CH + (C < CH ? C : 0)) * 16 + e];                        \
+            }                                                                                                           \
+        }                                                                                                               \
+        break;
+                switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
+#undef WG_PUT
+                __syncwarp();
+                float x[4][4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int e = q * 4 + k;
-                    const float4 v = *reinterpret_cast<const float4*>(buf + e * TILE_N + lane * 4);
+                    const int e = 4 * k + e0;
+                    const float4 v = *reinterpret_cast<const float4*>(buf + e * 32 + c);
                     const float sc = scaled ? ctl->scale[c0 + e] : 1.f;
                     x[k][0] = v.x * sc; x[k][1] = v.y * sc; x[k][2] = v.z * sc; x[k][3] = v.w * sc;
                     if (DUAL) {
-                        const float4 u4 = *reinterpret_cast<const float4*>(buf + (16 + e) * TILE_N + lane * 4);
+                        const float4 u4 = *reinterpret_cast<const float4*>(buf + (16 + e) * 32 + c);
                         const float u[4] = {u4.x, u4.y, u4.z, u4.w};
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
@@ -496,10 +502,20 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll
                     for (int j = 0; j < 4; ++j) x[k][j] += old[k][j];
                 }
+                if (add) load_old(ch + 1);
+                if (!DUAL && p.out_ssq) {                     // (rows past the matrix came out as zeros)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        float sq = (x[k][0] * x[k][0] + x[k][1] * x[k][1]) + (x[k][2] * x[k][2] + x[k][3] * x[k][3]);
+#pragma unroll
+                        for (int o = 1; o < 8; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                        if ((lane & 7) == 0) sums[q * WG_SET + c0 + 4 * k + e0] = sq;
+                    }
+                }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int r = rw + k;
-                    if (r >= m) break;
+                    const int r = r0 + 4 * k + e0;
+                    if (r >= m) continue;
                     if (Y) {
                         float* y = Y + (size_t)r * p.ldy;
                         if (vec) *reinterpret_cast<float4*>(y) = make_float4(x[k][0], x[k][1], x[k][2], x[k][3]);
@@ -508,10 +524,6 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                             for (int j = 0; j < 4; ++j)
                                 if (j < have) y[j] = x[k][j];
                         }
-                    }
-                    if (p.out_ssq) {                          // (rows past the matrix came out as zeros)
-                        const float sq = warp_sum((x[k][0] * x[k][0] + x[k][1] * x[k][1]) + (x[k][2] * x[k][2] + x[k][3] * x[k][3]));
-                        if (lane == 0) p.out_ssq[(size_t)(row_tile * 2 + rank) * m + r] = sq;
                     }
                     if (p.out_xs && have > 0) {
                         uint16_t h[4], l[4];
@@ -529,6 +541,13 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         }
                     }
                 }
+            }
+            if (!DUAL && p.out_ssq) {                         // one piece per token and CTA: its 128 rows
+                asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
+                const int col = half * htok + (et & 127);
+                if ((et & 127) < htok && tok0 + col < m)
+                    p.out_ssq[(size_t)(row_tile * 2 + rank) * m + tok0 + col] =
+                        (sums[col] + sums[WG_SET + col]) + (sums[2 * WG_SET + col] + sums[3 * WG_SET + col]);
             }
         }
     }
@@ -683,7 +702,7 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     const bool dual = a.W2 != nullptr;
     if (!a.W || !a.xs || (((uintptr_t)a.xs) & 15) || !a.partial || !a.tickets) return CSD_ERR_INVALID_ARG;
     if (!a.Y && (!dual || !a.out_xs)) return CSD_ERR_INVALID_ARG;
-    if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU)) return CSD_ERR_INVALID_ARG;
+    if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU) || (dual && a.out_ssq)) return CSD_ERR_INVALID_ARG;
     if (!wide_supported(a.m, a.N, a.K, dual)) return CSD_ERR_UNSUPPORTED;
     const WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
     if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) return CSD_ERR_INVALID_ARG;

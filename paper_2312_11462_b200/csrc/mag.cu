@@ -102,7 +102,7 @@ mag_draft_kernel(const int32_t* __restrict__ hay, int L, const int32_t* __restri
     while (made < n) {
         // Without a hit the next tokens are the bigram chain from the last one.  Follow it for up to AHEAD tokens at once
         // and request the table entries of all the suffixes that result together: one round trip instead of one (table,
-        // then bigram) per token.  Four tokens without a hit: MAG_MEASURED.
+        // then bigram) per token.
         const int steps = G > 0 ? 1 : min(AHEAD, n - made);
         int32_t nx[AHEAD];
         bool bad[AHEAD];

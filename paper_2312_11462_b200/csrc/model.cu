@@ -538,16 +538,19 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& y = M->dec[l];
         for (int r0 = 0; r0 < n; r0 += WR) {
-            const int m = n - r0 < WR ? n - r0 : WR;
-            CSD_TRY(launch_wide_split(M->xenc + (size_t)r0 * d, d, d, m, M->enc_final_norm, M->wxs_x, M->wssq, st));
-            const int cnt = wide_split_pieces(d);
+            const int m = n - r0 < WR ? n - r0 : WR, cnt = wide_split_pieces(d);
+            if (l == 0 || n > WR)            // (one block of rows: their terms serve all layers)
+                CSD_TRY(launch_wide_split(M->xenc + (size_t)r0 * d, d, d, m, M->enc_final_norm, M->wxs_x, M->wssq, st));
             float* out = M->qkv_enc + (size_t)r0 * 3 * di;
-            CSD_TRY(wide_linear(M, y.xk, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, out + di, 3 * di, EPI_STORE, nullptr, 0, nullptr,
-                                nullptr, st));
-            CSD_TRY(wide_linear(M, y.xv, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, out + 2 * di, 3 * di, EPI_STORE, nullptr, 0,
-                                nullptr, nullptr, st));
+            const bool fused = y.xv == y.xk + (size_t)di * d;
+            CSD_TRY(wide_linear(M, y.xk, nullptr, fused ? 2 * di : di, d, m, M->wxs_x, M->wssq, cnt, out + di, 3 * di, EPI_STORE,
+                                nullptr, 0, nullptr, nullptr, st));
+            if (!fused)
+                CSD_TRY(wide_linear(M, y.xv, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, out + 2 * di, 3 * di, EPI_STORE, nullptr, 0,
+                                    nullptr, nullptr, st));
         }
-        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr, M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x, st));
+        CSD_TRY(launch_rope_append(M->qkv_enc, 3 * di, n, H, -1, di, 2 * di, Dh, 0, E, nullptr, nullptr,
+                                   M->xk + (size_t)l * M->layer_x, M->xv + (size_t)l * M->layer_x, st));
     }
     CSD_CUDA(cudaGetLastError());
     return CSD_OK;
