@@ -3,8 +3,8 @@
 // one run (Section 2) and the weights should stream once per pass.
 //
 // Each fp32 value of X enters as TWO bf16 terms x = hi + lo (16 mantissa bits, relative error
-// 2^-17), laid out as [2][mpad][K].  A tile is 256 weight rows x nt tokens (the gated pair: 256 rows
-// of both matrices x nt tokens; nt <= 256, <= 128 for the pair) and belongs to a PAIR of CTAs on
+// 2^-17), laid out as [2][mpad][K].  A tile is 256 weight rows x nt <= 256 tokens (the gated pair:
+// 128 rows of each matrix, or up to 128 tokens 256 rows of each) and belongs to a PAIR of CTAs on
 // neighbouring SMs: tcgen05.mma with cta_group::2, 128 weight rows and half of the tokens staged by
 // each CTA, both terms accumulated into the same fp32 columns.
 //
@@ -66,6 +66,7 @@ static_assert(8 * 16 * 32 + 4 * WG_SET <= 2 * 8 * 16 * 32, "sums of squares fit 
 // of a full tile (0.55 us each).
 struct WgPlan {
     int mpad, nt, ntok, tiles, nkb, pairs, pk, gran, stages;
+    bool mixed;                              // gated pair: a tile's weight rows are half gate, half up
     size_t stage, smem;
 };
 
@@ -73,13 +74,15 @@ int wide_split_pieces(int K) { return (K + 1023) / 1024; }
 
 static WgPlan wg_plan(int m, int N, int K, bool dual) {
     WgPlan p{};
-    const int P = tc_sm_count() / 2, most = dual ? 128 : 256;
+    const int P = tc_sm_count() / 2, most = dual && m <= 128 ? 128 : 256;
+    p.mixed = dual && m > 128;
+    const int rows = p.mixed ? WG_ROWS / 2 : WG_ROWS;
     p.mpad = (m + 15) & ~15;
     p.ntok = (m + most - 1) / most;
     p.nt = ((m + p.ntok - 1) / p.ntok + 31) & ~31;
-    p.tiles = ((N + WG_ROWS - 1) / WG_ROWS) * p.ntok;
+    p.tiles = ((N + rows - 1) / rows) * p.ntok;
     p.nkb = (K + KB - 1) / KB;
-    p.stage = (size_t)STAGE_BYTES * (dual ? 2 : 1) + (size_t)p.nt * 128;
+    p.stage = (size_t)STAGE_BYTES * (dual && !p.mixed ? 2 : 1) + (size_t)p.nt * 128;
     p.stages = (int)((WG_SMEM_MAX - 1024 - WG_STAGING - sizeof(WgCtrl)) / p.stage);
     if (p.stages > WG_MAX_STAGES) p.stages = WG_MAX_STAGES;
     p.smem = (size_t)p.stages * p.stage + 1024 + WG_STAGING + sizeof(WgCtrl);
@@ -107,7 +110,7 @@ bool wide_supported(int m, int N, int K, bool dual) {
     (void)dual;
     if (m < 1 || m > CSD_WIDE_ROWS || N < 1 || K < 64 || (K & 7)) return false;
     if ((long long)N * K < (1LL << 20)) return false;
-    const long long tiles = (long long)((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128);
+    const long long tiles = (long long)((N + WG_ROWS / 2 - 1) / (WG_ROWS / 2)) * ((m + 127) / 128);
     return tiles * ((K + KB - 1) / KB) * (tc_sm_count() + 1) < (1LL << 31);
 }
 
@@ -124,7 +127,11 @@ size_t wide_partial_bytes(int m) {
     const int cols = m < 128 ? 2 * ((m + 31) & ~31) : 256;
     return (size_t)(tc_sm_count() / 2) * WG_ROWS * cols * sizeof(float);
 }
-int wide_ticket_count(int m, int N) { return 2 * ((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128); }
+int wide_ticket_count(int m, int N) {
+    const int half = WG_ROWS / 2;
+    const int a = ((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128), b = ((N + half - 1) / half) * ((m + 255) / 256);
+    return 2 * (a > b ? a : b);
+}
 
 struct WgParams {
     float* Y; float* partial; unsigned* tickets; int* status;
@@ -173,11 +180,18 @@ __device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigne
     return unit_begin(c, units / gran, pairs) * gran;
 }
 
-template <bool DUAL>
+// MODE 0: one matrix; 1: a gated pair, both matrices' 256 rows in a stage (up to 128 tokens); 2: a gated pair, the CTA's
+// 128 rows are 64 of the gate and the same 64 of the up matrix, so that the MMAs are 256 tokens wide.  (At N = 128 an MMA reads
+// its 128 weight rows from shared memory for half the work, and those reads, not the tensor pipe, set the pace: gate and up of
+// the 7B shape at 1000 tokens 323 us in mode 1, 277 in mode 2; of the T5-xxl shape at 256 tokens 92 and 82.
+// Up to 128 tokens mode 1 moves fewer bytes: its tile is 256 outputs wide.)
+template <int MODE>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmX, const WgParams p) {
+    constexpr bool DUAL = MODE == 1, MIXED = MODE == 2;
     constexpr int NT = DUAL ? 2 : 1;
+    constexpr int OUT_ROWS = MIXED ? WG_ROWS / 2 : WG_ROWS;   // outputs of a tile
     constexpr uint32_t WB = NT * STAGE_BYTES;                 // weight bytes per stage and CTA
     constexpr int CH = DUAL ? 4 : 8;                          // 16-token chunks an epilogue warp holds at most
     const int nt = p.nt, htok = nt >> 1;
@@ -241,8 +255,10 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 unsigned char* dst = ring + (size_t)s * stage_bytes;
                 const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
                 if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
-                tma_load_2d_pair(dst, &tmW, bar, cw.kb * KB, cw.row * WG_ROWS + rank * TILE_N);
-                if (DUAL) tma_load_2d_pair(dst + STAGE_BYTES, &tmW2, bar, cw.kb * KB, cw.row * WG_ROWS + rank * TILE_N);
+                const int row = cw.row * OUT_ROWS + rank * (OUT_ROWS / 2);
+                tma_load_2d_pair(dst, &tmW, bar, cw.kb * KB, row);
+                if (DUAL) tma_load_2d_pair(dst + STAGE_BYTES, &tmW2, bar, cw.kb * KB, row);
+                if (MIXED) tma_load_2d_pair(dst + STAGE_BYTES / 2, &tmW2, bar, cw.kb * KB, row);
                 step(cw);
             };
             auto load_x = [&](int s) {
@@ -432,9 +448,9 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             //      256 tokens 7.5 ms, 6.8 so.)
             const bool scaled = p.ssq_in && p.pk == 1;
             const int c = (lane & 7) * 4, e0 = lane >> 3;     // this lane's rows of the warp's 32, first of its tokens (every 4th)
-            const int n = row_tile * WG_ROWS + rank * TILE_N + q * 32 + c;
+            const int n = row_tile * OUT_ROWS + rank * (OUT_ROWS / 2) + (MIXED ? q & 1 : q) * 32 + c;
             const int have = min(4, p.N - n);                 // weight rows of this lane inside the matrix
-            const bool vec = have == 4 && p.vec_y, add = p.epilogue == EPI_ADD;
+            const bool vec = have == 4 && p.vec_y, add = MODE == 0 && p.epilogue == EPI_ADD;
             float gain[4] = {1.f, 1.f, 1.f, 1.f};
             if (p.out_xs && p.out_gain) {
 #pragma unroll
@@ -462,17 +478,22 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 }
             };
             load_old(0);
-            float* buf = staging + ew * (NT * 16 * 32);
+            // (mixed: warps q and q + 2 hold gate and up of the same outputs; each finishes half of the chunk's tokens from
+            //  both stagings, of which there are two in turn, so that one barrier of the two warps per chunk will do)
+            float* buf = staging + ew * ((MIXED ? 2 : NT) * 16 * 32);
+            const float* gate = staging + (half * 4 + (q & 1)) * (2 * 16 * 32);
+            constexpr int KC = MIXED ? 2 : 4;                 // tokens of a chunk that a lane finishes
+            const int k0 = MIXED ? (q >> 1) * 2 : 0;
             float* sums = staging + 8 * 16 * 32;              // [quadrant][token]: sums of squares over a warp's 32 rows
 #pragma unroll 1
             for (int ch = 0; ch < nch; ++ch) {
                 const int c0 = half * htok + ch * 16, r0 = tok0 + c0;     // column in the tile, token
                 if (r0 >= m) break;                           // (the same for the four warps of a half)
-                float* put = buf + lane;
+                float* put = buf + lane + (MIXED ? (ch & 1) * (16 * 32) : 0);
                 // Registers have no index: one short copy per chunk, everything else is a loop over the chunks.  Unrolled
                 // over the chunks (100 KB of instructions, pushed out of the caches by the weight stream before every
                 // use) it ran at the speed of instruction fetch: up to 3 us a chunk, all SMs in step, against 1 us.
-                __syncwarp();                                 // the chunk before has been read
+                if (!MIXED) __syncwarp();                     // the chunk before has been read
 #define WG_PUT(C)                                                                                                       \
     case C:                                                                                                             \
         if (C < CH) {                                                                                                   \
@@ -484,26 +505,29 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         break;
                 switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
 #undef WG_PUT
-                __syncwarp();
+                if (MIXED) asm volatile("bar.sync %0, 64;" ::"r"(4 + half * 2 + (q & 1)) : "memory");
+                else __syncwarp();
                 float x[4][4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int e = 4 * k + e0;
-                    const float4 v = *reinterpret_cast<const float4*>(buf + e * 32 + c);
+                for (int k = 0; k < KC; ++k) {
+                    const int e = 4 * (k0 + k) + e0;
+                    const float* from = MIXED ? gate + (ch & 1) * (16 * 32) : buf;
+                    const float4 v = *reinterpret_cast<const float4*>(from + e * 32 + c);
                     const float sc = scaled ? ctl->scale[c0 + e] : 1.f;
                     x[k][0] = v.x * sc; x[k][1] = v.y * sc; x[k][2] = v.z * sc; x[k][3] = v.w * sc;
-                    if (DUAL) {
-                        const float4 u4 = *reinterpret_cast<const float4*>(buf + (16 + e) * 32 + c);
+                    if (DUAL || MIXED) {
+                        const float4 u4 = *reinterpret_cast<const float4*>(from + (MIXED ? 2 * 2 * 16 + e : 16 + e) * 32 + c);
                         const float u[4] = {u4.x, u4.y, u4.z, u4.w};
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
                             x[k][j] = (p.epilogue == EPI_GEGLU ? wg_gelu(x[k][j]) : wg_silu(x[k][j])) * (u[j] * sc);
                     }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) x[k][j] += old[k][j];
+                    for (int j = 0; j < 4; ++j)
+                        if (MODE == 0) x[k][j] += old[k][j];
                 }
                 if (add) load_old(ch + 1);
-                if (!DUAL && p.out_ssq) {                     // (rows past the matrix came out as zeros)
+                if (MODE == 0 && p.out_ssq) {                     // (rows past the matrix came out as zeros)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         float sq = (x[k][0] * x[k][0] + x[k][1] * x[k][1]) + (x[k][2] * x[k][2] + x[k][3] * x[k][3]);
@@ -513,8 +537,8 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int r = r0 + 4 * k + e0;
+                for (int k = 0; k < KC; ++k) {
+                    const int r = r0 + 4 * (k0 + k) + e0;
                     if (r >= m) continue;
                     if (Y) {
                         float* y = Y + (size_t)r * p.ldy;
@@ -542,7 +566,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     }
                 }
             }
-            if (!DUAL && p.out_ssq) {                         // one piece per token and CTA: its 128 rows
+            if (MODE == 0 && p.out_ssq) {                         // one piece per token and CTA: its 128 rows
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
                 const int col = half * htok + (et & 127);
                 if ((et & 127) < htok && tok0 + col < m)
@@ -676,10 +700,10 @@ csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_b
     return CSD_OK;
 }
 
-template <bool DUAL>
+template <int MODE>
 static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const WgParams& wp,
                             const WgPlan& pl, cudaStream_t st) {
-    auto kern = wide_gemm_kernel<DUAL>;
+    auto kern = wide_gemm_kernel<MODE>;
     static bool attr_set = false;
     if (!attr_set) {
         CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM_MAX));
@@ -707,9 +731,10 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     const WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
     if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) return CSD_ERR_INVALID_ARG;
     CUtensorMap tw, tw2, tx;
-    if (!tensor_map_2d(a.W, a.N, a.K, TILE_N, &tw)) return CSD_ERR_UNSUPPORTED;
+    const int box = pl.mixed ? TILE_N / 2 : TILE_N;
+    if (!tensor_map_2d(a.W, a.N, a.K, box, &tw)) return CSD_ERR_UNSUPPORTED;
     tw2 = tw;
-    if (dual && !tensor_map_2d(a.W2, a.N, a.K, TILE_N, &tw2)) return CSD_ERR_UNSUPPORTED;
+    if (dual && !tensor_map_2d(a.W2, a.N, a.K, box, &tw2)) return CSD_ERR_UNSUPPORTED;
     if (!tensor_map_2d(a.xs, 2 * pl.mpad, a.K, pl.nt / 2, &tx)) return CSD_ERR_UNSUPPORTED;
     WgParams wp;
     wp.Y = a.Y; wp.partial = a.partial; wp.tickets = a.tickets; wp.status = status_word_device();
@@ -722,7 +747,7 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     if (pl.pk > 1) {                     // partial planes now, sums and epilogue in the small kernel after
         wp.Y = a.partial; wp.ldy = a.N; wp.plane = (size_t)a.m * a.N; wp.epilogue = EPI_STORE;
         wp.out_xs = nullptr; wp.out_ssq = nullptr; wp.out_gain = nullptr; wp.vec_y = 1;
-        const csd_status s = launch_wg<false>(tw, tw2, tx, wp, pl, st);
+        const csd_status s = launch_wg<0>(tw, tw2, tx, wp, pl, st);
         if (s != CSD_OK) return s;
         PdlLaunch L(dim3((unsigned)wide_split_pieces(a.N), (unsigned)a.m), dim3(128), 0, st);
         CSD_CUDA(cudaLaunchKernelEx(&L.cfg, wide_reduce_kernel, (const float*)a.partial, pl.pk, wp.plane, a.N, a.m, pl.mpad, a.ssq,
@@ -731,7 +756,8 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
         count_launch();
         return CSD_OK;
     }
-    return dual ? launch_wg<true>(tw, tw2, tx, wp, pl, st) : launch_wg<false>(tw, tw2, tx, wp, pl, st);
+    if (pl.mixed) return launch_wg<2>(tw, tw2, tx, wp, pl, st);
+    return dual ? launch_wg<1>(tw, tw2, tx, wp, pl, st) : launch_wg<0>(tw, tw2, tx, wp, pl, st);
 }
 
 }  // namespace csd
