@@ -25,11 +25,25 @@
 
 namespace csd {
 
-// Epilogue warps: one per tensor-memory quadrant, two (half of the rows each) for blocks of more than 9 rows, whose
-// finish one warp per quadrant takes 3.4 us over at 17 rows.  16 layers of the 7B shape with one / two: 5 rows 1560 /
-// 1577 us, 9 rows 1667 / 1683, 13 rows 1835 / 1803, 17 rows 2060 / 1971.
-template <int M> struct EpilogueWarps { static constexpr int value = M > 9 ? 8 : 4; };
+// Epilogue warps: one per tensor-memory quadrant, or two (half of the rows each) for larger blocks on smaller matrices, where
+// the finish is much of the launch.  With four / eight warps, 16 layers of the 7B shape (matrices of 45 M elements and more, one of
+// 17 M): 11 rows 1586 / 1630 us, 13 rows 1625 / 1661, 17 rows 1768 / 1800; T5-xxl-shaped decoder (three of 17 M): 17 rows
+// 3350 / 3316; 68M-shaped draft (at most 25 M): 12 rows 97 / 95, 17 rows 116 / 108.
+static int epilogue_warps(int m, int N, int K) { return m > 9 && (long long)N * K < (1LL << 25) ? 8 : 4; }
 constexpr size_t TC_SMEM_MAX = 111 * 1024;              // two CTAs (of consecutive kernels) fit one SM
+
+// K blocks of a stage: two for a single matrix on a block of up to 8 rows (32 KB of weights per barrier round trip, like the
+// gated pair; 3-5 % faster per forward than one), one otherwise.
+__host__ __device__ constexpr int stage_kblocks(int m, bool dual) { return !dual && m <= 8 ? 2 : 1; }
+
+// Where stages of weights and row terms together would leave few of them, the row terms (two stages' worth) live beside 96 KB of
+// weight boxes:
+//   the gated pair on blocks of more than 10 rows: a common stage takes 38 to 40 KB, two fit, 32 to 64 KB of weights
+//     are in flight per SM; as six single boxes, each with a barrier, 16 layers of the 7B shape go from 1703 to 1627 us at 11
+//     rows, 1840 to 1783 at 17.  (Boxes with a barrier each, and one more for the row terms, at every size: 12 % slower.)
+//   a single matrix on 6 to 8 rows: three stages of two K blocks (of row terms too): 6 rows 1491 -> 1475 us, 8 rows 1535 -> 1526.
+__host__ __device__ constexpr bool split_rings(int m, bool dual) { return dual ? m > 10 : m > 5 && m <= 8; }
+__host__ __device__ constexpr int split_xslot(int m) { return (3 * m * 128 + 1023) / 1024 * 1024; }
 
 static int g_path = 0;
 void set_gemm_path(int path) { g_path = path; }
@@ -59,10 +73,7 @@ static TcPlan tc_plan(int m, int N, int K, bool dual) {
     p.npad = npad_for(m);
     p.tiles = (N + TILE_N - 1) / TILE_N;
     p.kblocks = (K + KB - 1) / KB;
-    // single-matrix GEMM on a block of up to 5 rows: a stage holds two K blocks (32 KB of weights per barrier
-    // round trip, like the gated pair; measured 3-5 % faster per forward).  Larger blocks keep one K block per
-    // stage, or too few stages would fit.
-    const int ks = (!dual && p.npad <= 16) ? 2 : 1;
+    const int ks = stage_kblocks(m, dual);
     p.kblocks = (p.kblocks + ks - 1) / ks;
     const long long units = (long long)p.tiles * p.kblocks;
     long long grid = units / 4;                           // at least four units per CTA
@@ -83,6 +94,7 @@ static TcPlan tc_plan(int m, int N, int K, bool dual) {
     p.stages = (int)((TC_SMEM_MAX - 1024) / stage);
     if (p.stages > 12) p.stages = 12;
     p.smem = (size_t)p.stages * stage + 1024;
+    if (split_rings(m, dual)) p.smem = (size_t)6 * STAGE_BYTES + (size_t)2 * ks * split_xslot(m) + 1024;
     p.scratch_floats = (size_t)p.grid * 2 * (dual ? 2 : 1) * m * TILE_N;
     return p;
 }
@@ -187,13 +199,12 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     return false;
 }
 
-template <int M, bool DUAL>
-__global__ void __launch_bounds__(64 + 32 * EpilogueWarps<M>::value, 2)
+template <int M, bool DUAL, int EW>
+__global__ void __launch_bounds__(64 + 32 * EW, 2)
 skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                       const __grid_constant__ CUtensorMap tmX, const TcParams p) {
     constexpr int NPAD = 3 * M <= 16 ? 16 : (3 * M <= 32 ? 32 : (3 * M <= 48 ? 48 : 64));
     constexpr int NT = DUAL ? 2 : 1;
-    constexpr int EW = EpilogueWarps<M>::value;
     constexpr int ACC_ONE = NPAD * NT;                        // tensor-memory columns of one accumulator
     // The tensor core's fp32 accumulation loses a little with every add of a long chain, so the K blocks
     // of a segment go round-robin to NACC accumulators (as many as fit 256 columns twice over, at most
@@ -203,7 +214,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
     constexpr int TMEM_COLS = 2 * ACC_COLS <= 32 ? 32 : (2 * ACC_COLS <= 64 ? 64 : (2 * ACC_COLS <= 128 ? 128 : 256));
     constexpr int XBYTES = NPAD * 128;                        // room of the rows' terms for one K block; 3 M rows are copied:
                                                               // what the pad holds reaches only columns nobody reads
-    constexpr int KS = (!DUAL && NPAD <= 16) ? 2 : 1;         // K blocks per stage
+    constexpr int KS = stage_kblocks(M, DUAL);
     constexpr int WB = (DUAL ? 2 : KS) * STAGE_BYTES;         // weight bytes per stage
     constexpr int STAGE = WB + KS * XBYTES;
     constexpr uint32_t TX_BYTES = WB + KS * 3 * M * 128;      // bytes that arrive per stage
@@ -212,7 +223,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    TcCtrl* ctl = (TcCtrl*)(ring + (size_t)p.stages * STAGE);
+    // Separate rings: `ring` holds the row terms of two items (an item: KS K blocks), `wring` the weights, WPI slots an item.
+    constexpr bool SPLIT = split_rings(M, DUAL);
+    constexpr int XSLOT = split_xslot(M);                     // (MMAs read up to NPAD rows: past a slot lies the next, then the weights)
+    constexpr int WPI = DUAL ? 2 : 1, WSLOT = STAGE_BYTES * KS, WSLOTS = 6 / KS;
+    unsigned char* wring = ring + (SPLIT ? 2 * KS * XSLOT : 0);
+    TcCtrl* ctl = (TcCtrl*)(SPLIT ? wring + (size_t)WSLOTS * WSLOT : ring + (size_t)p.stages * STAGE);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x, ctas = gridDim.x;
@@ -264,6 +280,43 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             int tile = (int)(u0 / p.nkb), kb = (int)(u0 % p.nkb);
             const int kb0 = kb;
             const uint64_t once = policy_evict_first();
+            if constexpr (SPLIT) {
+                // the terms of an item complete on the barrier of its first slot of weights
+                int xk = kb, x_next = 0, ws = 0;
+                auto load_w = [&](int u) {
+                    const int t = u % WPI;
+                    unsigned char* dst = wring + (size_t)ws * WSLOT;
+                    mbar_expect_tx(&ctl->full[ws], WSLOT + (t ? 0 : KS * 3 * M * 128));
+#pragma unroll
+                    for (int h = 0; h < KS; ++h)              // past K: zero fill
+                        tma_load_2d_once(dst + h * STAGE_BYTES, t ? &tmW2 : &tmW, &ctl->full[ws], (kb * KS + h) * KB, tile * TILE_N, once);
+                    if (t == WPI - 1 && ++kb == p.nkb) { kb = 0; ++tile; }
+                    if (++ws == WSLOTS) ws = 0;
+                };
+                auto load_x = [&]() {
+#pragma unroll
+                    for (int h = 0; h < KS; ++h)
+                        tma_load_2d(ring + ((x_next & 1) * KS + h) * XSLOT, &tmX, &ctl->full[WPI * x_next % WSLOTS], (xk * KS + h) * KB, 0);
+                    if (++xk == p.nkb) xk = 0;
+                    ++x_next;
+                };
+                const int slots = WPI * items;
+                int u = 0;
+                for (; u < WSLOTS && u < slots; ++u) load_w(u);
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                for (int i = 0; i < 2 && i < items; ++i) load_x();
+                int es = 0;
+                uint32_t eph = 0;
+                while (x_next < items && !*abort_flag) {      // an item is through: its slots of weights, its terms
+#pragma unroll
+                    for (int t = 0; t < WPI; ++t, ++u) {
+                        if (!mbar_wait(&ctl->empty[es], eph)) { *abort_flag = 1; break; }
+                        if (u < slots) load_w(u);
+                        if (++es == WSLOTS) { es = 0; eph ^= 1u; }
+                    }
+                    if (!*abort_flag) load_x();
+                }
+            } else {
             for (int i = 0; i < pre; ++i) {
                 unsigned char* dst = ring + (size_t)i * STAGE;
                 mbar_expect_tx(&ctl->full[i], TX_BYTES);
@@ -302,6 +355,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 if (items >= p.stages && !mbar_wait(&ctl->empty[s], ph)) *abort_flag = 1;
                 for (int r = 1; r < p.csplit; ++r) remote_arrive(map_to_cta(smem_u32(&ctl->red_ready), (uint32_t)r));
             }
+            }
         }
     } else if (warp == 1) {
         // ---- MMA issuer: one accumulator set per segment (the part of a tile inside this CTA's range)
@@ -310,6 +364,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             uint32_t ph = 0;                      // parity of the phase of full[s] that fills slot s next
             int kb_begin = (int)(u0 % p.nkb);
             const uint64_t desc0 = smem_desc_sw128(smem_u32(ring));   // descriptors differ in the address field only
+            const uint64_t descw = smem_desc_sw128(smem_u32(wring));
             for (int seg = 0; i < items && !*abort_flag; ++seg) {
                 const int b = seg & 1;
                 const int seg_len = min(p.nkb - kb_begin, items - i);
@@ -320,6 +375,24 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 for (int j = 0; j < seg_len; ++j, ++i) {
                     const uint32_t d0 = dset + (uint32_t)((j % NACC) * ACC_ONE);
                     const int first = j < NACC ? 0 : 1;       // an accumulator's first K block overwrites it
+                    if constexpr (SPLIT) {
+                        const uint64_t bd = desc0 + (uint64_t)((uint32_t)((i & 1) * KS * XSLOT) >> 4);
+#pragma unroll
+                        for (int t = 0; t < WPI; ++t) {
+                            if (!mbar_wait(&ctl->full[s], ph)) { *abort_flag = 1; break; }
+                            tc_fence_after();
+                            const uint64_t ad = descw + (uint64_t)(((uint32_t)s * (uint32_t)WSLOT) >> 4);
+#pragma unroll
+                            for (int h = 0; h < KS; ++h)
+#pragma unroll
+                                for (int k = 0; k < KB / 16; ++k)
+                                    tc_mma(d0 + t * NPAD, ad + ((h * STAGE_BYTES) >> 4) + 2 * k, bd + ((h * XSLOT) >> 4) + 2 * k, IDESC, (first | h | k) != 0);
+                            tc_commit(&ctl->empty[s]);
+                            if (++s == WSLOTS) { s = 0; ph ^= 1u; }
+                        }
+                        if (*abort_flag) break;
+                        continue;
+                    }
                     if (!mbar_wait(&ctl->full[s], ph)) { *abort_flag = 1; break; }
                     tc_fence_after();
                     const uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * (uint32_t)STAGE) >> 4);
@@ -617,10 +690,10 @@ csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st) {
     return CSD_OK;
 }
 
-template <int M, bool DUAL>
+template <int M, bool DUAL, int EW>
 static csd_status launch_tc(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const TcParams& tp,
                             const TcPlan& pl, cudaStream_t st) {
-    auto kern = skinny_gemm_tc_kernel<M, DUAL>;
+    auto kern = skinny_gemm_tc_kernel<M, DUAL, EW>;
     static bool attr_set = false;
     if (!attr_set) {
         CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX + 1024));
@@ -630,7 +703,7 @@ static csd_status launch_tc(const CUtensorMap& tw, const CUtensorMap& tw2, const
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    pdl_config(cfg, attr, dim3((unsigned)pl.grid), dim3(64 + 32 * EpilogueWarps<M>::value), pl.smem + 1024, st);
+    pdl_config(cfg, attr, dim3((unsigned)pl.grid), dim3(64 + 32 * EW), pl.smem + 1024, st);
     if (pl.csplit > 1) {
         attr[1].id = cudaLaunchAttributeClusterDimension;
         attr[1].val.clusterDim.x = (unsigned)pl.csplit; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
@@ -664,8 +737,13 @@ csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st) {
     tp.out_xs = a.out_xs; tp.out_gain = a.out_gain; tp.out_ssq = a.out_ssq; tp.out_ld = a.out_ld;
     tp.N = a.N; tp.K = a.K; tp.ldy = a.ldy; tp.nkb = pl.kblocks; tp.tiles = pl.tiles; tp.stages = pl.stages; tp.csplit = pl.csplit;
     tp.epilogue = a.epilogue; tp.eps = a.eps;
-#define CSD_TC_CASE(MM) \
-    case MM: return dual ? launch_tc<MM, true>(tw, tw2, tx, tp, pl, st) : launch_tc<MM, false>(tw, tw2, tx, tp, pl, st);
+    const bool more = epilogue_warps(a.m, a.N, a.K) == 8;
+#define CSD_TC_CASE(MM)                                                                                             \
+    case MM:                                                                                                        \
+        if (MM > 9 && more)                                                                                         \
+            return dual ? launch_tc<MM, true, (MM > 9 ? 8 : 4)>(tw, tw2, tx, tp, pl, st)                              \
+                        : launch_tc<MM, false, (MM > 9 ? 8 : 4)>(tw, tw2, tx, tp, pl, st);                            \
+        return dual ? launch_tc<MM, true, 4>(tw, tw2, tx, tp, pl, st) : launch_tc<MM, false, 4>(tw, tw2, tx, tp, pl, st);
     switch (a.m) {
         CSD_TC_CASE(1) CSD_TC_CASE(2) CSD_TC_CASE(3) CSD_TC_CASE(4) CSD_TC_CASE(5) CSD_TC_CASE(6) CSD_TC_CASE(7)
         CSD_TC_CASE(8) CSD_TC_CASE(9) CSD_TC_CASE(10) CSD_TC_CASE(11) CSD_TC_CASE(12) CSD_TC_CASE(13)
