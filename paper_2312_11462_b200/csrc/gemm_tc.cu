@@ -613,12 +613,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             }
         }
     }
-    if (*abort_flag) {
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {              // (looked at behind the barrier: any warp may have given up last)
         if (tid == 0) set_status(p.status, CSD_ERR_TIMEOUT);
         __nanosleep(2000000);          // let copies already in flight land before the CTA's memory is released
     }
-    tc_fence_before();
-    __syncthreads();
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");

@@ -575,12 +575,12 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             }
         }
     }
-    if (*abort_flag) {
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {              // (looked at behind the barrier: any warp may have given up last)
         if (tid == 0) set_status(p.status, CSD_ERR_TIMEOUT);
         __nanosleep(2000000);
     }
-    tc_fence_before();
-    __syncthreads();
     cluster_barrier();               // neither CTA leaves while the other's MMAs or arrivals may reach it
     if (warp == 1) {
         tc_fence_after();
