@@ -53,6 +53,7 @@ static int npad_for(int m) { int c = 3 * m; return c <= 16 ? 16 : (c <= 32 ? 32 
 
 struct TcPlan {
     int npad, tiles, kblocks, grid, stages, csplit;    // kblocks: stages of work per tile (one or two 64-wide K blocks each)
+    int outer, single;                                 // three CTAs per two tiles: units of an outer CTA, of the first of an odd last tile's
     size_t smem, scratch_floats;
 };
 
@@ -80,15 +81,31 @@ static TcPlan tc_plan(int m, int N, int K, bool dual) {
     if (grid < 1) grid = 1;
     if (grid > tc_sm_count()) grid = tc_sm_count();
     p.grid = (int)grid;
-    // A single-matrix GEMM with few tiles (N = 4096: 32) on a block of up to 5 rows is cut the other way:
+    // A single-matrix GEMM with few tiles (N = 4096: 32) on a block of up to 8 rows is cut the other way:
     // every tile goes to a cluster of four CTAs that share its K range and add their parts up through
     // distributed shared memory, on chip, instead of parking them in global memory.  4 x 32 = 128 streaming
-    // SMs still draw the full bandwidth.  (Measured: 0.8 % faster per 7B forward at 5 rows, no gain at 9,
-    // 1 % slower at 17, hence the row limit.)
+    // SMs still draw the full bandwidth.  (16 layers of the 7B shape: 8 rows 1515 -> 1498 us; T5-xxl-shaped decoder, three
+    // such matrices a layer, 6 rows 2822 -> 2731.  With one K block a stage, from 9 rows on: no gain at 9, 1 % slower at 17.)
     p.csplit = 1;
-    if (!dual && p.npad <= 16 && p.tiles * 4 <= tc_sm_count() && p.tiles * 4 >= 96 && p.kblocks >= 8) {
+    if (!dual && ks == 2 && p.tiles * 4 <= tc_sm_count() && p.tiles * 4 >= 96 && p.kblocks >= 8) {
         p.csplit = 4;
         p.grid = p.tiles * 4;
+    }
+    p.outer = p.single = 0;
+    // Three CTAs per two tiles where that is between 3/4 of the SMs and all of them (q|k|v and gate+up of the 7B and T5-xxl shapes),
+    // blocks of up to 10 rows.  In equal shares of all units about every third CTA lies inside one tile and parks when it ends,
+    // just when the tile's finisher has ended as well and must wait for it.  Here the outer CTAs of a group finish a tile each
+    // and the middle one, which parks for both, has 6 stages of 32 KB less than they, about what parking takes: 16 layers of
+    // the 7B shape at 5 rows 1434 -> 1419 us (1470 with three equal shares, 1432 with 10 less), 10 rows 1587 -> 1570; from
+    // 11 rows on level, and 12 rows of the T5-xxl shape, whose gate+up gets 120 CTAs, 3050 -> 3071.
+    if (m <= 10 && p.csplit == 1 && p.kblocks >= 32) {
+        const int ctas = p.tiles / 2 * 3 + (p.tiles & 1) * 2;
+        if (ctas <= tc_sm_count() && ctas >= tc_sm_count() * 3 / 4) {
+            const int less = dual || ks == 2 ? 6 : 12;
+            p.grid = ctas;
+            p.outer = (2 * p.kblocks + less + 1) / 3;
+            p.single = (p.kblocks + less) / 2;
+        }
     }
     const size_t stage = (size_t)STAGE_BYTES * (dual ? 2 : ks) + (size_t)p.npad * 128 * ks;
     p.stages = (int)((TC_SMEM_MAX - 1024) / stage);
@@ -167,7 +184,7 @@ struct TcParams {
     float* Y; float* partial; unsigned* tickets; int* status;
     const float* ssq_in; int ssq_cnt;                      // rms-norm: sum of squares of the input rows, in pieces
     __nv_bfloat16* out_xs; const __nv_bfloat16* out_gain; float* out_ssq; int out_ld;
-    int N, K, ldy, nkb, tiles, stages, epilogue, csplit;
+    int N, K, ldy, nkb, tiles, stages, epilogue, csplit, outer, single;
     float eps;
 };
 
@@ -239,6 +256,18 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
         const unsigned t = (unsigned)(cta / p.csplit) * (unsigned)p.nkb;
         u0 = t + (unsigned)crank * (unsigned)p.nkb / (unsigned)p.csplit;
         u1 = t + (unsigned)(crank + 1) * (unsigned)p.nkb / (unsigned)p.csplit;
+    }
+    const bool outer = M <= 10 && p.outer > 0;                // three CTAs per two tiles
+    if (outer) {
+        const int g = cta / 3, j = cta - 3 * g;
+        const unsigned t = (unsigned)(2 * g) * (unsigned)p.nkb, two = 2u * (unsigned)p.nkb;
+        if (2 * g + 1 == p.tiles) {
+            u0 = t + (j ? (unsigned)p.single : 0u);
+            u1 = t + (j ? (unsigned)p.nkb : (unsigned)p.single);
+        } else {
+            u0 = t + (j == 0 ? 0u : (j == 1 ? (unsigned)p.outer : two - (unsigned)p.outer));
+            u1 = t + (j == 0 ? (unsigned)p.outer : (j == 1 ? two - (unsigned)p.outer : two));
+        }
     }
     const int items = (int)(u1 - u0);
 
@@ -316,6 +345,9 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                     }
                     if (!*abort_flag) load_x();
                 }
+                // (every slot but the last two items' has been handed back by now)
+                if (p.csplit > 1 && crank == 0 && !*abort_flag)
+                    for (int r = 1; r < p.csplit; ++r) remote_arrive(map_to_cta(smem_u32(&ctl->red_ready), (uint32_t)r));
             } else {
             for (int i = 0; i < pre; ++i) {
                 unsigned char* dst = ring + (size_t)i * STAGE;
@@ -441,8 +473,13 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
             // the tile parks at the end, and the finisher waits for it (bounded).  Measured against
             // "whoever arrives last finishes": 1.7 % faster per forward at 5 rows, 4 % at 17.
             const bool part_of_tile = p.csplit == 1 && seg_len < p.nkb;
-            int c_lo = cta, c_hi = cta;
-            if (part_of_tile) {
+            int c_lo = cta, c_hi = cta, slot = 0;               // the finisher; the others are c_lo + 1 .. c_hi, parked in `slot`
+            if (part_of_tile && outer) {
+                const int mid = tile / 2 * 3 + 1;
+                slot = tile & 1;
+                c_lo = mid - 1; c_hi = mid;
+                if (slot) { c_lo = cta == mid + 1 ? cta : mid + 1; c_hi = mid; }
+            } else if (part_of_tile) {
                 c_lo = cta_of_unit((unsigned)tile * p.nkb, units, ctas);
                 c_hi = cta_of_unit((unsigned)(tile + 1) * p.nkb - 1, units, ctas);
             }
@@ -465,10 +502,11 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 }
                 if (p.out_xs && p.out_gain) out_g = __bfloat162float(p.out_gain[n]);
             }
-            if (finisher && c_hi > c_lo) {
+            const int others = outer ? (part_of_tile ? 1 : 0) : c_hi - c_lo;
+            if (finisher && others > 0) {
                 unsigned* ticket = p.tickets + tile * 8 + half * 4 + q;
                 if (lane == 0) {
-                    const unsigned want = (unsigned)(c_hi - c_lo);
+                    const unsigned want = (unsigned)others;
                     int spins = 0;
 #pragma unroll 1
                     while (ld_acquire_gpu(ticket) < want) {
@@ -481,12 +519,12 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 // 48 registers hold
                 constexpr int CH = NV <= 6 ? 8 : (48 / NV < 1 ? 1 : 48 / NV);
 #pragma unroll 1
-                for (int c = c_lo + 1; c <= c_hi; c += CH) {
+                for (int c = outer ? c_hi : c_lo + 1; c <= c_hi; c += CH) {
                     float part[CH][NV];
 #pragma unroll
                     for (int h = 0; h < CH; ++h) {
                         const int cc = min(c + h, c_hi);
-                        const float* src = p.partial + (((size_t)cc * 2) * NT * M + row0) * TILE_N + col;
+                        const float* src = p.partial + (((size_t)cc * 2 + slot) * NT * M + row0) * TILE_N + col;
 #pragma unroll
                         for (int u = 0; u < NT; ++u)
 #pragma unroll
@@ -534,8 +572,9 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 // finishes the tile: its producer has told the others which of its ring slots is free, they
                 // write their parts into it (distributed shared memory) and signal back, and it adds the
                 // parts in rank order.
-                const unsigned len0 = (unsigned)p.nkb / (unsigned)p.csplit, slots = (unsigned)p.stages;   // rank 0's items
-                float* buf = reinterpret_cast<float*>(ring + (size_t)(len0 >= slots ? len0 % slots : len0) * STAGE);   // [3][NT * M][128]
+                const unsigned len0 = (unsigned)p.nkb / (unsigned)p.csplit;           // rank 0's items
+                const unsigned slots = SPLIT ? (unsigned)WSLOTS : (unsigned)p.stages, free_slot = len0 >= slots ? len0 % slots : len0;
+                float* buf = reinterpret_cast<float*>(SPLIT ? wring + (size_t)free_slot * WSLOT : ring + (size_t)free_slot * STAGE);   // [3][NT * M][128]
                 if (crank == 0) {
                     if (!mbar_wait_cluster(&ctl->red_done, 0)) *abort_flag = 1;
 #pragma unroll
@@ -558,7 +597,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                     continue;
                 }
             } else if (!finisher) {
-                float* mine = my_part;                  // (a later contributor's part opens its share: slot 0)
+                float* mine = my_part + (size_t)slot * NT * M * TILE_N;   // (a later contributor's part opens its share: slot 0)
 #pragma unroll
                 for (int u = 0; u < NT; ++u)
 #pragma unroll
@@ -735,7 +774,7 @@ csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st) {
     tp.Y = a.Y; tp.partial = a.partial; tp.tickets = a.tickets; tp.status = status_word_device();
     tp.ssq_in = a.gain ? a.ssq : nullptr; tp.ssq_cnt = ssq_cnt;
     tp.out_xs = a.out_xs; tp.out_gain = a.out_gain; tp.out_ssq = a.out_ssq; tp.out_ld = a.out_ld;
-    tp.N = a.N; tp.K = a.K; tp.ldy = a.ldy; tp.nkb = pl.kblocks; tp.tiles = pl.tiles; tp.stages = pl.stages; tp.csplit = pl.csplit;
+    tp.N = a.N; tp.K = a.K; tp.ldy = a.ldy; tp.nkb = pl.kblocks; tp.tiles = pl.tiles; tp.stages = pl.stages; tp.outer = pl.outer; tp.single = pl.single; tp.csplit = pl.csplit;
     tp.epilogue = a.epilogue; tp.eps = a.eps;
     const bool more = epilogue_warps(a.m, a.N, a.K) == 8;
 #define CSD_TC_CASE(MM)                                                                                             \
