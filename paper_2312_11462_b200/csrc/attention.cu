@@ -51,6 +51,15 @@ struct AttnParams {
     unsigned char tdepth[MAXM];
 };
 
+// What differs between the sequences of a batched review: grid.z of the tensor-core kernel picks one.  (A launch per
+// sequence: three blocks of 5, 3 and 5 rows of the 7B shape 3569 us, 3347 so.)
+constexpr int MAX_SEGS = 4;
+struct AttnSeg {
+    const float* q; const float* k_new; const float* v_new; __nv_bfloat16* Kc; __nv_bfloat16* Vc; float* out;
+    int m, n_keys, n_old, split_len, q_pos0, xs_r0;
+};
+struct AttnSegs { CUtensorMap k[MAX_SEGS], v[MAX_SEGS]; AttnSeg seg[MAX_SEGS]; };
+
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
@@ -72,8 +81,8 @@ __device__ __forceinline__ void store_split(__nv_bfloat16* xs, int ld, int m, in
 // distributed shared memory: the CTAs of a head share out the m*DH output elements; each thread
 // first fetches everything it needs from all splits in one batch of independent remote loads.
 template <int DH, int REC>
-__device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* rec, const AttnParams& p, int h, int split,
-                                             int m) {
+__device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* rec, const AttnParams& p, float* out, int xs_r0,
+                                             int h, int split, int m) {
     for (int i = split * AT + threadIdx.x; i < m * DH; i += p.nsplit * AT) {
         const int r = i / DH, d = i % DH;
         float ms[MAX_SPLITS], ls[MAX_SPLITS], vs[MAX_SPLITS];
@@ -97,14 +106,14 @@ __device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* 
                 den = fmaf(ls[s], w, den);
             }
         const float ov = den > 0.f ? num / den : 0.f;
-        p.out[(size_t)r * p.ldo + h * DH + d] = ov;
+        out[(size_t)r * p.ldo + h * DH + d] = ov;
         if (p.out_xs) {
             uint16_t b1, b2, b3;
             split3(ov, b1, b2, b3);
             uint16_t* xs = reinterpret_cast<uint16_t*>(p.out_xs) + h * DH + d;
-            xs[(size_t)(p.xs_r0 + r) * p.out_xs_ld] = b1;
-            xs[(size_t)(p.xs_m + p.xs_r0 + r) * p.out_xs_ld] = b2;
-            xs[(size_t)(2 * p.xs_m + p.xs_r0 + r) * p.out_xs_ld] = b3;
+            xs[(size_t)(xs_r0 + r) * p.out_xs_ld] = b1;
+            xs[(size_t)(p.xs_m + xs_r0 + r) * p.out_xs_ld] = b2;
+            xs[(size_t)(2 * p.xs_m + xs_r0 + r) * p.out_xs_ld] = b3;
         }
     }
 }
@@ -349,7 +358,7 @@ block_attention_kernel(const AttnParams p) {
     }
     if (tid < m) { rec[tid * C::REC + DH] = row_m[tid]; rec[tid * C::REC + DH + 1] = row_l[tid]; }
     cluster.sync();
-    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m);
+    merge_splits<DH, C::REC>(cluster, rec, p, p.out, p.xs_r0, h, split, m);
     cluster.sync();       // no CTA leaves while another may still read its record
 }
 
@@ -376,9 +385,9 @@ template <int DH> struct MmaCfg {
 };
 template <int DH, int MT>
 __global__ void __launch_bounds__(AT)
-block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                           const AttnParams p) {
+block_attention_mma_kernel(const __grid_constant__ AttnSegs segs, const AttnParams p) {
     using C = MmaCfg<DH>;
+    const AttnSeg& sg = segs.seg[blockIdx.z];
     constexpr int R = MT * 16;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
@@ -399,14 +408,14 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h = blockIdx.x, split = blockIdx.y;
-    const int m = p.m, half = DH / 2, n_keys = p.n_keys;
+    const int m = sg.m, half = DH / 2, n_keys = sg.n_keys;
     const int total = p.causal ? n_keys + m - 1 : n_keys;
-    const int n_old = p.n_old;
-    const int s_begin = split * p.split_len;
-    const int s_end = min(total, s_begin + p.split_len);
+    const int n_old = sg.n_old;
+    const int s_begin = split * sg.split_len;
+    const int s_end = min(total, s_begin + sg.split_len);
     const int n_tiles = s_end > s_begin ? (s_end - s_begin + TILE - 1) / TILE : 0;
-    __nv_bfloat16* Kh = p.Kc + (size_t)h * p.cap * DH;
-    __nv_bfloat16* Vh = p.Vc + (size_t)h * p.cap * DH;
+    __nv_bfloat16* Kh = sg.Kc + (size_t)h * p.cap * DH;
+    __nv_bfloat16* Vh = sg.Vc + (size_t)h * p.cap * DH;
     const float* bias_h = p.bias ? p.bias + (size_t)h * p.bias_len : nullptr;
 
     if (tid == 0) {
@@ -424,8 +433,8 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
         mbar_expect_tx(&full[st], 2 * (uint32_t)C::TILE_BYTES);
 #pragma unroll
         for (int b = 0; b < C::NBOX; ++b) {
-            tma_load_2d(Ks + st * C::TILE_BYTES + b * (TILE * 128), &tmK, &full[st], b * 64, row0);
-            tma_load_2d(Vs + st * C::TILE_BYTES + b * (TILE * 128), &tmV, &full[st], b * 64, row0);
+            tma_load_2d(Ks + st * C::TILE_BYTES + b * (TILE * 128), &segs.k[blockIdx.z], &full[st], b * 64, row0);
+            tma_load_2d(Vs + st * C::TILE_BYTES + b * (TILE * 128), &segs.v[blockIdx.z], &full[st], b * 64, row0);
         }
     };
     // (see the CUDA-core kernel above for why the requests may precede the dependency wait)
@@ -457,11 +466,11 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
             const int i = tid + e * AT;
             if (i < m * half) {
                 const int r = i / half, d = i % half;
-                const float* qr = p.q + (size_t)r * p.ldq + h * DH;
+                const float* qr = sg.q + (size_t)r * p.ldq + h * DH;
                 qv[e][0] = qr[d]; qv[e][1] = qr[d + half];
-                if (p.k_new) {
-                    const float* kr = p.k_new + (size_t)r * p.ld_new + h * DH;
-                    const float* vr = p.v_new + (size_t)r * p.ld_new + h * DH;
+                if (sg.k_new) {
+                    const float* kr = sg.k_new + (size_t)r * p.ld_new + h * DH;
+                    const float* vr = sg.v_new + (size_t)r * p.ld_new + h * DH;
                     kv[e][0] = kr[d]; kv[e][1] = kr[d + half];
                     vv[e][0] = vr[d]; vv[e][1] = vr[d + half];
                 }
@@ -479,7 +488,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
                 __nv_bfloat16* qhr = reinterpret_cast<__nv_bfloat16*>(qh + r * C::QP);
                 __nv_bfloat16* qlr = reinterpret_cast<__nv_bfloat16*>(ql + r * C::QP);
                 qhr[d] = h0; qhr[d + half] = h1; qlr[d] = l0; qlr[d + half] = l1;
-                if (p.k_new) {
+                if (sg.k_new) {
                     const __nv_bfloat16 ka = __float2bfloat16_rn(kv[e][0] * c - kv[e][1] * s);
                     const __nv_bfloat16 kb = __float2bfloat16_rn(kv[e][0] * s + kv[e][1] * c);
                     const __nv_bfloat16 va = __float2bfloat16_rn(vv[e][0]), vb = __float2bfloat16_rn(vv[e][1]);
@@ -597,7 +606,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
                         if (vis) {
                             s = ((sacc2[g][1][0][e] + sacc2[g][1][1][e]) + (sacc2[g][0][0][e] + sacc2[g][0][1][e])) * p.scale;
                             if (bias_h) {
-                                int bi = key - (p.q_pos0 + r) + p.bias_zero;
+                                int bi = key - (sg.q_pos0 + r) + p.bias_zero;
                                 bi = max(0, min(p.bias_len - 1, bi));
                                 s += bias_h[bi];
                             }
@@ -711,9 +720,9 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
                         const int d = 16 * warp + 8 * t + 2 * (lane & 3);
-                        float* dst = p.out + (size_t)r * p.ldo + h * DH + d;
+                        float* dst = sg.out + (size_t)r * p.ldo + h * DH + d;
                         dst[0] = o[mt][t][2 * hr] * inv; dst[1] = o[mt][t][2 * hr + 1] * inv;
-                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, p.xs_r0 + r, h * DH + d, dst[0], dst[1]);
+                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, sg.xs_r0 + r, h * DH + d, dst[0], dst[1]);
                     }
                 }
         }
@@ -737,7 +746,7 @@ block_attention_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid
     }
     if (tid < m) { rec[tid * C::REC + DH] = row_m[tid]; rec[tid * C::REC + DH + 1] = row_l[tid]; }
     cluster.sync();
-    merge_splits<DH, C::REC>(cluster, rec, p, h, split, m);
+    merge_splits<DH, C::REC>(cluster, rec, p, sg.out, sg.xs_r0, h, split, m);
     cluster.sync();       // no CTA leaves while another may still read its record
 }
 static bool g_attn_cuda_cores = false;
@@ -793,7 +802,7 @@ static csd_status launch_dh(const AttnParams& ap, cudaStream_t st) {
 }
 
 template <int DH, int MT>
-static csd_status launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& ap, cudaStream_t st) {
+static csd_status launch_mma(const AttnSegs& segs, int nseg, const AttnParams& ap, cudaStream_t st) {
     auto kern = block_attention_mma_kernel<DH, MT>;
     static bool attr_set = false;
     const size_t smem = MmaCfg<DH>::smem(MT * 16);
@@ -804,17 +813,18 @@ static csd_status launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     attn_launch_config(cfg, attr, ap, smem, st);
-    CSD_CUDA(cudaLaunchKernelEx(&cfg, kern, tk, tv, ap));
+    cfg.gridDim.z = (unsigned)nseg;
+    CSD_CUDA(cudaLaunchKernelEx(&cfg, kern, segs, ap));
     count_launch();
     return CSD_OK;
 }
 
-static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st);
+static csd_status launch_attention_block(const AttnArgs* a, int n, cudaStream_t st);
 
 // Blocks of more than MAXM rows over a cache that already holds their keys (wide passes whose head dimension has no
 // launch_row_attention): one launch per MAXM rows.
 csd_status launch_attention(const AttnArgs& a, cudaStream_t st) {
-    if (a.m <= MAXM) return launch_attention_block(a, st);
+    if (a.m <= MAXM) return launch_attention_block(&a, 1, st);
     if (a.k_new || a.tree_mask || a.out_xs || a.m > CSD_WIDE_ROWS) return CSD_ERR_INVALID_ARG;
     for (int r0 = 0; r0 < a.m; r0 += MAXM) {
         AttnArgs s = a;
@@ -822,27 +832,48 @@ csd_status launch_attention(const AttnArgs& a, cudaStream_t st) {
         s.n_keys = a.causal ? a.n_keys + r0 : a.n_keys;
         s.q_pos0 = a.q_pos0 + r0;
         s.out = a.out + (size_t)r0 * a.ldo;
-        const csd_status rc = launch_attention_block(s, st);
+        const csd_status rc = launch_attention_block(&s, 1, st);
         if (rc != CSD_OK) return rc;
     }
     return CSD_OK;
 }
 
-static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st) {
-    if (!a.q || !a.Kc || !a.Vc || !a.out || a.m < 1 || a.m > MAXM || a.H < 1 || a.n_keys < 0)
-        return CSD_ERR_INVALID_ARG;
+csd_status launch_attention_batch(const AttnArgs* a, int n, cudaStream_t st) {
+    const bool together = n > 0 && (a[0].Dh == 64 || a[0].Dh == 128) && !g_attn_cuda_cores;
+    for (int i = 0; i < n;) {
+        int cnt = together ? (n - i < MAX_SEGS ? n - i : MAX_SEGS) : 1;
+        for (int j = i; j < i + cnt; ++j)
+            if (a[j].tree_mask || a[j].m > 16) cnt = 1;
+        const csd_status rc = launch_attention_block(a + i, cnt, st);
+        if (rc != CSD_OK) return rc;
+        i += cnt;
+    }
+    return CSD_OK;
+}
+
+// The blocks of n sequences of one model (n <= MAX_SEGS; more than one on the tensor-core kernel only, without a tree).
+static csd_status launch_attention_block(const AttnArgs* args, int n, cudaStream_t st) {
+    const AttnArgs& a = args[0];
+    int longest = 0, rows = 0, totals[MAX_SEGS];
+    for (int i = 0; i < n; ++i) {
+        const AttnArgs& b = args[i];
+        if (!b.q || !b.Kc || !b.Vc || !b.out || b.m < 1 || b.m > MAXM || b.H < 1 || b.n_keys < 0) return CSD_ERR_INVALID_ARG;
+        const bool append = b.k_new != nullptr;
+        if (append && (!b.v_new || !b.causal || b.n_keys < 1)) return CSD_ERR_INVALID_ARG;
+        if ((b.rope_cos != nullptr) != (b.rope_sin != nullptr) || (b.rope_cos && !append)) return CSD_ERR_INVALID_ARG;
+        if ((((uintptr_t)b.Kc) & 15) || (((uintptr_t)b.Vc) & 15)) return CSD_ERR_INVALID_ARG;
+        totals[i] = b.causal ? b.n_keys + b.m - 1 : b.n_keys;
+        if (totals[i] < 1 || totals[i] > b.cap) return CSD_ERR_CAPACITY;
+        if (totals[i] > longest) longest = totals[i];
+        if (b.m > rows) rows = b.m;
+    }
     const bool append = a.k_new != nullptr;
-    if (append && (!a.v_new || !a.causal || a.n_keys < 1)) return CSD_ERR_INVALID_ARG;
-    if ((a.rope_cos != nullptr) != (a.rope_sin != nullptr) || (a.rope_cos && !append)) return CSD_ERR_INVALID_ARG;
-    if ((((uintptr_t)a.Kc) & 15) || (((uintptr_t)a.Vc) & 15)) return CSD_ERR_INVALID_ARG;
-    const int total = a.causal ? a.n_keys + a.m - 1 : a.n_keys;
-    if (total < 1 || total > a.cap) return CSD_ERR_CAPACITY;
     AttnParams ap;
     ap.q = a.q; ap.k_new = a.k_new; ap.v_new = a.v_new; ap.ld_new = a.ld_new; ap.rope_cos = a.rope_cos;
     ap.rope_sin = a.rope_sin; ap.Kc = a.Kc; ap.Vc = a.Vc; ap.bias = a.bias; ap.out = a.out;
     ap.status = status_word_device();
     ap.ldq = a.ldq; ap.m = a.m; ap.cap = a.cap; ap.H = a.H; ap.n_keys = a.n_keys;
-    ap.n_old = append ? a.n_keys - 1 : total;
+    ap.n_old = append ? a.n_keys - 1 : totals[0];
     ap.early_loads = a.kv_settled ? 1 : 0;
     ap.causal = a.causal; ap.bias_len = a.bias_len; ap.bias_zero = a.bias_zero; ap.q_pos0 = a.q_pos0;
     ap.ldo = a.ldo; ap.scale = a.scale; ap.out_xs = a.out_xs; ap.out_xs_ld = a.out_xs_ld;
@@ -853,19 +884,27 @@ static csd_status launch_attention_block(const AttnArgs& a, cudaStream_t st) {
         ap.tree = 1;
         for (int r = 0; r < MAXM; ++r) { ap.tmask[r] = r < a.m ? a.tree_mask[r] : 0u; ap.tdepth[r] = r < a.m ? (unsigned char)a.tree_depth[r] : 0; }
     }
-    ap.nsplit = attn_splits(total, a.H, a.Dh, a.out_xs_rows > 0 ? a.out_xs_rows : a.m);
-    int len = (total + ap.nsplit - 1) / ap.nsplit;
-    ap.split_len = (len + TILE - 1) / TILE * TILE;
-    ap.nsplit = (total + ap.split_len - 1) / ap.split_len;
+    // every sequence's splits share one cluster shape, set by the longest cache; shorter ones leave their last splits empty
+    ap.nsplit = attn_splits(longest, a.H * n, a.Dh, a.out_xs_rows > 0 ? a.out_xs_rows : a.m);
+    auto split_len = [&](int total) { return ((total + ap.nsplit - 1) / ap.nsplit + TILE - 1) / TILE * TILE; };
+    ap.nsplit = (longest + split_len(longest) - 1) / split_len(longest);
+    ap.split_len = split_len(totals[0]);
     // head dimensions 64 and 128 run on the tensor cores; the caches then need tensor maps (rows = all heads' positions)
     if ((a.Dh == 64 || a.Dh == 128) && !g_attn_cuda_cores) {
-        CUtensorMap tk, tv;
-        if (tensor_map_2d(a.Kc, a.H * a.cap, a.Dh, TILE, &tk) && tensor_map_2d(a.Vc, a.H * a.cap, a.Dh, TILE, &tv)) {
-            const bool one_tile = a.m <= 16;
-            if (a.Dh == 64) return one_tile ? launch_mma<64, 1>(tk, tv, ap, st) : launch_mma<64, 2>(tk, tv, ap, st);
-            return one_tile ? launch_mma<128, 1>(tk, tv, ap, st) : launch_mma<128, 2>(tk, tv, ap, st);
+        AttnSegs segs;
+        bool maps = true;
+        for (int i = 0; i < n; ++i) {
+            const AttnArgs& b = args[i];
+            maps = maps && tensor_map_2d(b.Kc, b.H * b.cap, b.Dh, TILE, &segs.k[i]) && tensor_map_2d(b.Vc, b.H * b.cap, b.Dh, TILE, &segs.v[i]);
+            segs.seg[i] = AttnSeg{b.q, b.k_new, b.v_new, b.Kc, b.Vc, b.out, b.m, b.n_keys, b.k_new ? b.n_keys - 1 : totals[i],
+                                  split_len(totals[i]), b.q_pos0, b.out_xs_row0};
+        }
+        if (maps) {
+            if (a.Dh == 64) return rows <= 16 ? launch_mma<64, 1>(segs, n, ap, st) : launch_mma<64, 2>(segs, n, ap, st);
+            return rows <= 16 ? launch_mma<128, 1>(segs, n, ap, st) : launch_mma<128, 2>(segs, n, ap, st);
         }
     }
+    if (n > 1) return CSD_ERR_UNSUPPORTED;
     switch (a.Dh) {
         case 32: return launch_dh<32>(ap, st);
         case 64: return launch_dh<64>(ap, st);

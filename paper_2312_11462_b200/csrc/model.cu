@@ -363,6 +363,10 @@ static csd_status attention(csd_model* M, const AttnArgs& a, cudaStream_t st) {
     ProfScope ps(M, 1, st);
     return launch_attention(a, st);
 }
+static csd_status attention(csd_model* M, const AttnArgs* blocks, int n, cudaStream_t st) {
+    ProfScope ps(M, 1, st);
+    return n == 1 ? launch_attention(blocks[0], st) : launch_attention_batch(blocks, n, st);
+}
 
 // q|k|v projections of `m` rows with the norm fused; one GEMM when the three matrices are
 // contiguous in the blob (they are whenever d_inner * d_model is a multiple of 128).
@@ -862,9 +866,10 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
             if (x_ready) { qo.xs_in = M->xs_x; qo.ssq_in = M->ssq_x; qo.ssq_cnt = M->ssq_x_cnt; }
             CSD_TRY(project_qkv(M, y, M->x, m, M->qkv, st, &qo));
         }
+        AttnArgs blocks[CSD_MAX_ROWS];
         for (int g = 0; g < nseg; ++g) {
             const Segment& sg = segs[g];
-            AttnArgs a;
+            AttnArgs& a = blocks[g];
             a.q = M->qkv + (size_t)sg.row0 * 3 * di; a.ldq = 3 * di; a.m = sg.rows;
             a.Kc = sg.S->kcache + (size_t)l * sg.S->layer_kv; a.Vc = sg.S->vcache + (size_t)l * sg.S->layer_kv;
             a.cap = c.max_seq; a.H = H; a.Dh = Dh;
@@ -877,8 +882,8 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
             if (c.arch == 0) { a.rope_cos = M->rope_c; a.rope_sin = M->rope_s; }
             a.tree_mask = tree_mask; a.tree_depth = tree_depth;
             if (tc_o) { a.out_xs = M->xs_attn; a.out_xs_ld = di; a.out_xs_rows = m; a.out_xs_row0 = sg.row0; }
-            CSD_TRY(attention(M, a, st));
         }
+        CSD_TRY(attention(M, blocks, nseg, st));
         // output projection into the residual rows; hands them on to the norm that follows
         LinOpt oo;
         if (tc_o) oo.xs_in = M->xs_attn;
@@ -892,15 +897,16 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
             CSD_TRY(linear(M, y.xq, nullptr, di, d, M->x, d, m, y.norm_x, M->qkv, 3 * di, EPI_STORE, st, &xq));
             for (int g = 0; g < nseg; ++g) {
                 const Segment& sg = segs[g];
-                AttnArgs x;
+                AttnArgs& x = blocks[g];
+                x = AttnArgs();
                 x.q = M->qkv + (size_t)sg.row0 * 3 * di; x.ldq = 3 * di; x.m = sg.rows;
                 x.Kc = sg.S->xk + (size_t)l * sg.S->layer_x; x.Vc = sg.S->xv + (size_t)l * sg.S->layer_x;
                 x.cap = c.max_enc_len; x.H = H; x.Dh = Dh; x.n_keys = sg.S->enc_len;
                 x.causal = 0; x.scale = 1.f; x.out = M->attn + (size_t)sg.row0 * di; x.ldo = di;
                 x.kv_settled = true;  // written once by the encoder pass
                 if (tc_o) { x.out_xs = M->xs_attn; x.out_xs_ld = di; x.out_xs_rows = m; x.out_xs_row0 = sg.row0; }
-                CSD_TRY(attention(M, x, st));
             }
+            CSD_TRY(attention(M, blocks, nseg, st));
             LinOpt xo;
             if (tc_o) xo.xs_in = M->xs_attn;
             x_ready = tc_o && linear_uses_tensor_cores(m, ff, d, true);

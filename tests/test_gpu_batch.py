@@ -86,3 +86,21 @@ def test_first_sequence_fills_its_cache(b, orc):
     for i in range(2):
         ref = oms[i].review_forward(seqs[i][kv[i]:kv[i] + rows[i]], kv[i])
         assert rel_l2(got[i].cpu().numpy(), ref) <= LOGIT_REL_L2
+
+
+@pytest.mark.parametrize("rows", [(3, 1, 4, 2, 6, 1), (16, 1), (1, 16), (4, 4, 4, 4, 1)])
+def test_more_sequences_than_one_launch_takes(b, orc, rows):
+    """Caches from empty to several key tiles, head dimension 128: sequences share a cluster shape, so some splits are empty."""
+    shape = llama_shape(1, 1024, 8, 512, 500, 420)
+    blob = workloads.make_weights(shape, seed=23, device="cuda", std=0.05, gain_std=0.1)
+    kv = [0, 400, 63, 128, 257, 9][:len(rows)]
+    seqs = [workloads.make_prompt(shape.vocab, shape.max_seq, seed=70 + i) for i in range(len(rows))]
+    gms, oms = [b.Model(shape, blob) for _ in rows], [orc.Model(shape, orc.blob_to_u16(blob)) for _ in rows]
+    for g, o, s, n in zip(gms, oms, seqs, kv):
+        if n:
+            g.csd_prefill(to_dev_i32(s[:n]), 0)
+            o.review_forward(s[:n], 0)
+    got = b.csd_review_forward_batch(gms, [to_dev_i32(s[n:n + r]) for s, n, r in zip(seqs, kv, rows)], kv)
+    assert b.csd_device_status() == 0
+    for i, (o, s, n, r) in enumerate(zip(oms, seqs, kv, rows)):
+        assert rel_l2(got[i].cpu().numpy(), o.review_forward(s[n:n + r], n)) <= LOGIT_REL_L2, i
