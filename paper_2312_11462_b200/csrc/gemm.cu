@@ -339,6 +339,8 @@ static bool linear_uses_rows(int m, int N, int K, bool dual) {
            (long long)N * K * (dual ? 2 : 1) * m <= AUTO_ROW_MAX_WORK;
 }
 
+bool linear_gathers(int m, int N, int K) { return linear_uses_rows(m, N, K, false); }
+
 bool linear_uses_tensor_cores(int m, int N, int K, bool dual) {
     const int path = gemm_path();
     if (linear_uses_rows(m, N, K, dual)) return false;
@@ -376,6 +378,7 @@ csd_status launch_linear(const LinearArgs& a, cudaStream_t st) {
     const bool dual = a.W2 != nullptr;
     if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU)) return CSD_ERR_INVALID_ARG;
     if ((((uintptr_t)a.W) & 15) || (dual && (((uintptr_t)a.W2) & 15))) return CSD_ERR_INVALID_ARG;
+    if (a.tokens && (!linear_gathers(a.m, a.N, a.K) || dual || !a.embed || !a.x_out || a.vocab < 1)) return CSD_ERR_INVALID_ARG;
     if (a.xs && linear_uses_row_ranges(a.m, a.N, a.K, dual)) return launch_linear_rs(a, st);
     if (a.xs && linear_uses_tensor_cores(a.m, a.N, a.K, dual)) return launch_linear_tc(a, st);
     if ((((uintptr_t)a.X) & 15) || (a.ldx & 3)) return CSD_ERR_INVALID_ARG;

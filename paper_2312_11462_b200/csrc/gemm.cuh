@@ -29,6 +29,12 @@ struct LinearArgs {
     int out_ld = 0;
     const __nv_bfloat16* out_gain = nullptr;
     float* out_ssq = nullptr;            // [linear_ssq_pieces(...)][m] pieces of the sums of squares of the rows of Y
+    // row kernel only (linear_gathers): X is gathered by the launch itself, row r = embed[tokens[r]] (K columns), and written to
+    // x_out [m, ldx] for the kernels after it
+    const int32_t* tokens = nullptr;
+    const __nv_bfloat16* embed = nullptr;
+    int vocab = 0;
+    float* x_out = nullptr;
 };
 
 int split_rows(int m);                   // 16, 32, 48 or 64 operand rows hold the 3m terms
@@ -38,6 +44,7 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual);
 int linear_ticket_count(int N);
 csd_status launch_linear(const LinearArgs& a, cudaStream_t st);
 bool linear_uses_tensor_cores(int m, int N, int K, bool dual);   // the kernel launch_linear would pick (given a.xs)
+bool linear_gathers(int m, int N, int K);                        // ... is the row kernel, which can gather its rows (one matrix)
 bool linear_uses_row_ranges(int m, int N, int K, bool dual);     // ... and which of the two tensor-core kernels
 int linear_ssq_pieces(int m, int N, int K, bool dual);           // out_ssq pieces that launch writes
 int linear_ssq_capacity(int N);                                  // upper bound of the above over m, K

@@ -330,6 +330,7 @@ static csd_status check_config(const csd_model_config* c) {
 struct LinOpt {
     const __nv_bfloat16* xs_in = nullptr; const float* ssq_in = nullptr; int ssq_cnt = 0;
     __nv_bfloat16* out_xs = nullptr; int out_ld = 0; const __nv_bfloat16* out_gain = nullptr; float* out_ssq = nullptr;
+    const int32_t* tokens = nullptr;       // the rows are still to be gathered (see LinearArgs), into M->x
 };
 
 // One linear layer of the forward; all of them share the model's split scratch.
@@ -345,6 +346,7 @@ static csd_status linear(csd_model* M, const __nv_bfloat16* W, const __nv_bfloat
             a.xs = const_cast<__nv_bfloat16*>(o->xs_in); a.xs_ready = true;
             a.ssq = const_cast<float*>(o->ssq_in); a.ssq_cnt = o->ssq_cnt;
         }
+        if (o->tokens) { a.tokens = o->tokens; a.embed = M->embed; a.vocab = M->cfg.vocab; a.x_out = M->x; }
         a.out_xs = o->out_xs; a.out_ld = o->out_ld; a.out_gain = o->out_gain; a.out_ssq = o->out_ssq;
         if (o->out_ssq == M->ssq_x) M->ssq_x_cnt = linear_ssq_pieces(m, N, K, W2 != nullptr);
     }
@@ -839,12 +841,14 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
     // x_ready: M->xs_x / M->ssq_x hold the residual rows (times the gain of the norm that reads them
     // next) in three-term form, written by the epilogue of the GEMM that produced the rows (for the
     // embedded rows: by the gather itself, when the first projection takes that form)
-    bool x_ready = false;
+    bool x_ready = false, gather = false;      // gather: the first projection fetches the embedded rows itself
     {
         ProfScope ps(M, 2, st);
         const LayerW& y0 = M->dec[0];
         const bool fused_qkv = y0.wk == y0.wq + (size_t)di * d && y0.wv == y0.wk + (size_t)di * d;
-        if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
+        gather = fused_qkv && linear_gathers(m, 3 * di, d) && !linear_uses_tensor_cores(m, 3 * di, d, false);
+        if (gather) {
+        } else if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
             PdlLaunch L(dim3((unsigned)split_ssq_entries(d), (unsigned)m), dim3(128), 0, st);
             CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_split_kernel, block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x,
                                         M->ssq_x, M->status));
@@ -864,6 +868,7 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
         {
             LinOpt qo;
             if (x_ready) { qo.xs_in = M->xs_x; qo.ssq_in = M->ssq_x; qo.ssq_cnt = M->ssq_x_cnt; }
+            if (gather && l == 0) qo.tokens = block_tokens_dev;
             CSD_TRY(project_qkv(M, y, M->x, m, M->qkv, st, &qo));
         }
         AttnArgs blocks[CSD_MAX_ROWS];
