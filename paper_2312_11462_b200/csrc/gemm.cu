@@ -421,7 +421,7 @@ static LinearWs linear_ws(int m, int N, int K) {
     w.partial = off;
     {
         size_t pb = linear_scratch_bytes(m > CSD_MAX_ROWS ? CSD_MAX_ROWS : m, N, K, false);
-        if (m > CSD_MAX_ROWS && wide_partial_bytes(m) > pb) pb = wide_partial_bytes(m);
+        if (m > CSD_MAX_ROWS && wide_supported(m, N, K, false) && wide_partial_bytes(m) > pb) pb = wide_partial_bytes(m);
         off += pb;
     }
     w.xs = off;      off += align_up((size_t)3 * rows * K * 2, 256);
