@@ -13,6 +13,7 @@
 //            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
 #include "model.cuh"
+#include "per_device.cuh"
 #include "philox.cuh"
 #include <math.h>
 #include <mutex>
@@ -969,11 +970,11 @@ static int accept_sm_count() {
 
 // The table of 2^(j/64), correctly rounded, goes to constant memory once per device.
 static csd_status exp_table_ready() {
-    static bool done[64];
+    static bool done[MAX_DEVICES];
     static std::mutex mu;
     int dev = 0;
     CSD_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return CSD_ERR_UNSUPPORTED;
+    if (dev < 0 || dev >= MAX_DEVICES) return CSD_ERR_UNSUPPORTED;
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
         double tab[64];
@@ -1009,11 +1010,14 @@ static bool fused_resample_ok(int csize) {
     return state[csize] == 1;
 }
 
-// Clusters of `csize` CTAs of the one-kernel form that are resident at once (0: none); asked once per size.
+// Clusters of `csize` CTAs of the one-kernel form that are resident at once on the current device (0: none).  The opt-in to
+// clusters above 8 is an attribute of the kernel on one device, so both are settled for each device.
 template <bool VEC, int PER>
 static int row_clusters(int csize) {
-    static int known[AR_MAXC + 1];              // 0 unknown, else 1 + the answer
-    if (known[csize] == 0) {
+    static PerDevice known[AR_MAXC + 1];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    return known[csize].get(dev, [csize] {
         int n = 0;
         bool ok = true;
         if (csize > 8)
@@ -1028,9 +1032,8 @@ static int row_clusters(int csize) {
             ok = cudaOccupancyMaxActiveClusters(&n, accept_row_kernel<VEC, PER>, &cfg) == cudaSuccess;
         }
         if (!ok) { (void)cudaGetLastError(); n = 0; }
-        known[csize] = 1 + n;
-    }
-    return known[csize] - 1;
+        return n;
+    });
 }
 
 template <bool VEC, int PER>
@@ -1052,8 +1055,13 @@ static csd_status launch_accept_row(const float* tl, const float* dl, const int*
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    CSD_CUDA(cudaLaunchKernelEx(&cfg, accept_row_kernel<VEC, PER>, tl, dl, onehot, tokens, rows, k, V, temperature, lenience,
-                                seed, step, csize, S, pieces, n_acc, out_tok, seq, status));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, accept_row_kernel<VEC, PER>, tl, dl, onehot, tokens, rows, k, V, temperature,
+                                             lenience, seed, step, csize, S, pieces, n_acc, out_tok, seq, status);
+    if (e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidClusterSize || e == cudaErrorLaunchOutOfResources) {
+        (void)cudaGetLastError();                        // a configuration the device does not take: left to the passes
+        return CSD_OK;
+    }
+    CSD_CUDA(e);
     count_launch();
     *done = true;
     return CSD_OK;
@@ -1283,7 +1291,6 @@ extern "C" csd_status csd_tree_accept_greedy(const float* target_logits_dev, con
 namespace csd {
 constexpr size_t STATIC_SCRATCH_BYTES = (size_t)2 << 20;   // 2 MiB, held by every GPU that loads the library
 static __device__ __align__(256) unsigned char g_accept_scratch[STATIC_SCRATCH_BYTES];
-constexpr int MAX_DEVICES = 64;
 static void* g_accept_scratch_ptr[MAX_DEVICES];             // device address of the array, per device
 static std::mutex g_accept_scratch_mu;
 }  // namespace csd
