@@ -13,7 +13,6 @@
 //            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
 #include "model.cuh"
-#include "per_device.cuh"
 #include "philox.cuh"
 #include <math.h>
 #include <mutex>
@@ -985,29 +984,24 @@ static csd_status exp_table_ready() {
     return CSD_OK;
 }
 
-// Whether clusters of `csize` CTAs of the fused resample kernel can run on this device (sizes above
-// 8 are an opt-in of the hardware); asked once per size.
+// Whether clusters of `csize` CTAs of the fused resample kernel can run on the current device.
 static bool fused_resample_ok(int csize) {
-    static int state[RF_MAXC + 1];              // 0 unknown, 1 yes, 2 no
+    static PerDevice known[RF_USE_MAXC + 1];
     if (csize < 1 || csize > RF_USE_MAXC) return false;
-    if (state[csize] == 0) {
-        bool ok = true;
-        if (csize > 8)
-            ok = cudaFuncSetAttribute(resample_fused_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-        if (ok) {
-            cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
-            cudaLaunchAttribute attr[1];
-            cfg.gridDim = dim3((unsigned)csize); cfg.blockDim = dim3(RF_THREADS);
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr; cfg.numAttrs = 1;
-            int n = 0;
-            ok = cudaOccupancyMaxActiveClusters(&n, resample_fused_kernel, &cfg) == cudaSuccess && n >= 1;
-        }
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return known[csize].get(dev, [csize] {
+        cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+        cudaLaunchAttribute attr[1];
+        cfg.gridDim = dim3((unsigned)csize); cfg.blockDim = dim3(RF_THREADS);
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        const bool ok = cudaOccupancyMaxActiveClusters(&n, resample_fused_kernel, &cfg) == cudaSuccess && n >= 1;
         if (!ok) (void)cudaGetLastError();
-        state[csize] = ok ? 1 : 2;
-    }
-    return state[csize] == 1;
+        return ok ? 1 : 0;
+    }) == 1;
 }
 
 // Clusters of `csize` CTAs of the one-kernel form that are resident at once on the current device (0: none).  The opt-in to

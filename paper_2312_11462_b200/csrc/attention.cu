@@ -788,11 +788,9 @@ static void attn_launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* att
 template <int DH>
 static csd_status launch_dh(const AttnParams& ap, cudaStream_t st) {
     auto kern = block_attention_kernel<DH>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnCfg<DH>::SMEM));
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const csd_status ok = allow_smem(ready, kern, AttnCfg<DH>::SMEM);
+    if (ok != CSD_OK) return ok;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     attn_launch_config(cfg, attr, ap, AttnCfg<DH>::SMEM, st);
@@ -804,12 +802,10 @@ static csd_status launch_dh(const AttnParams& ap, cudaStream_t st) {
 template <int DH, int MT>
 static csd_status launch_mma(const AttnSegs& segs, int nseg, const AttnParams& ap, cudaStream_t st) {
     auto kern = block_attention_mma_kernel<DH, MT>;
-    static bool attr_set = false;
+    static PerDevice ready;
     const size_t smem = MmaCfg<DH>::smem(MT * 16);
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr_set = true;
-    }
+    const csd_status ok = allow_smem(ready, kern, smem);
+    if (ok != CSD_OK) return ok;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     attn_launch_config(cfg, attr, ap, smem, st);

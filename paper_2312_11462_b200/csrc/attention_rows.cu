@@ -257,11 +257,9 @@ row_attention_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 template <int DH>
 static csd_status launch_rows(const CUtensorMap& tk, const CUtensorMap& tv, const RowsParams& rp, int H, cudaStream_t st) {
     auto kern = row_attention_kernel<DH>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RowsCfg<DH>::SMEM));
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const csd_status ok = allow_smem(ready, kern, RowsCfg<DH>::SMEM);
+    if (ok != CSD_OK) return ok;
     PdlLaunch L(dim3((unsigned)H, (unsigned)((rp.m + RROWS - 1) / RROWS)), dim3(32 * RW), RowsCfg<DH>::SMEM, st);
     CSD_CUDA(cudaLaunchKernelEx(&L.cfg, kern, tk, tv, rp));
     count_launch();

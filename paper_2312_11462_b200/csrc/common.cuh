@@ -5,6 +5,7 @@
 #include <stdint.h>
 #include <stddef.h>
 #include "../../include/csd.h"
+#include "per_device.cuh"
 
 namespace csd {
 
@@ -21,6 +22,21 @@ long long launches_so_far();
         cudaError_t e__ = (expr);                             \
         if (e__ != cudaSuccess) return csd::note_cuda(e__);   \
     } while (0)
+
+// Opts a kernel in to `bytes` of dynamic shared memory on the current device, once for each device (`ready`: one per kernel);
+// largest: also asks for the largest shared-memory carve-out, or a second CTA (the next kernel's) does not fit the SM.
+template <class Kernel>
+csd_status allow_smem(PerDevice& ready, Kernel* kern, size_t bytes, bool largest = false) {
+    int dev = -1;
+    CSD_CUDA(cudaGetDevice(&dev));
+    cudaError_t e = cudaSuccess;
+    ready.get(dev, [&] {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess && largest) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        return e == cudaSuccess ? 0 : -1;
+    });
+    return note_cuda(e);
+}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

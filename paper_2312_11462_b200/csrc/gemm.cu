@@ -295,11 +295,9 @@ skinny_gemm_kernel(const GemmParams p) {
 template <int M, bool DUAL>
 static csd_status launch_one(const GemmParams& gp, const LinearPlan& pl, cudaStream_t st) {
     auto kern = skinny_gemm_kernel<M, DUAL>;
-    static bool attr_set = false;   // per instantiation
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BUDGET + 4096));
-        attr_set = true;
-    }
+    static PerDevice ready;   // per instantiation
+    const csd_status ok = allow_smem(ready, kern, SMEM_BUDGET + 4096);
+    if (ok != CSD_OK) return ok;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)pl.grid);
     cfg.blockDim = dim3(GT);

@@ -227,11 +227,9 @@ row_gemm_kernel(const RowParams p) {
 template <int M, int R, int S, bool DUAL, bool GATHER>
 static csd_status launch_row_one(const RowParams& rp, cudaStream_t st) {
     auto kern = row_gemm_kernel<M, R, S, DUAL, GATHER>;
-    static bool attr_set = false;   // per instantiation
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RW_SMEM_MAX));
-        attr_set = true;
-    }
+    static PerDevice ready;   // per instantiation
+    const csd_status ok = allow_smem(ready, kern, RW_SMEM_MAX);
+    if (ok != CSD_OK) return ok;
     const int groups = (rp.N + R - 1) / R;
     int grid = (groups + RW_WARPS - 1) / RW_WARPS;
     if (grid > 2 * tc_sm_count()) grid = 2 * tc_sm_count();

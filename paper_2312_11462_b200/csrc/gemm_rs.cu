@@ -352,13 +352,9 @@ template <int M, bool DUAL>
 static csd_status launch_rs(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const RsParams& rp,
                             const RsPlan& pl, cudaStream_t st) {
     auto kern = skinny_gemm_rs_kernel<M, DUAL>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM_MAX));
-        // ask for the largest shared-memory carve-out, or the second CTA (the next kernel's) does not fit
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const csd_status ok = allow_smem(ready, kern, RS_SMEM_MAX, true);
+    if (ok != CSD_OK) return ok;
     PdlLaunch L(dim3((unsigned)pl.grid), dim3(TC_THREADS), pl.smem, st);
     CSD_CUDA(cudaLaunchKernelEx(&L.cfg, kern, tw, tw2, tx, rp));
     count_launch();

@@ -733,13 +733,9 @@ template <int M, bool DUAL, int EW>
 static csd_status launch_tc(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const TcParams& tp,
                             const TcPlan& pl, cudaStream_t st) {
     auto kern = skinny_gemm_tc_kernel<M, DUAL, EW>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX + 1024));
-        // ask for the largest shared-memory carve-out, or the second CTA (the next kernel's) does not fit
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const csd_status ok = allow_smem(ready, kern, TC_SMEM_MAX + 1024, true);
+    if (ok != CSD_OK) return ok;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     pdl_config(cfg, attr, dim3((unsigned)pl.grid), dim3(64 + 32 * EW), pl.smem + 1024, st);

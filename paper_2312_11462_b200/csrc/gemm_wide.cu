@@ -704,11 +704,9 @@ template <int MODE>
 static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const WgParams& wp,
                             const WgPlan& pl, cudaStream_t st) {
     auto kern = wide_gemm_kernel<MODE>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        CSD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM_MAX));
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const csd_status ok = allow_smem(ready, kern, WG_SMEM_MAX);
+    if (ok != CSD_OK) return ok;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
     cudaLaunchAttribute attr[2];
     cfg.gridDim = dim3((unsigned)(2 * pl.pairs)); cfg.blockDim = dim3(WG_THREADS); cfg.dynamicSmemBytes = pl.smem; cfg.stream = st;

@@ -45,8 +45,10 @@ def test_every_device_is_asked_once(tmp_path):
 
 
 def test_no_attribute_of_a_kernel_is_settled_for_the_first_device_only():
-    """Function attributes belong to a device: no launcher may keep one flag for all of them."""
+    """Attributes belong to a kernel on one device: whoever sets one goes through PerDevice."""
     csrc = os.path.join(ROOT, "paper_2312_11462_b200", "csrc")
-    text = open(os.path.join(csrc, "accept.cu")).read()
-    at = text.index("static int row_clusters")
-    assert "static int known" not in text[at:at + 400] and "PerDevice known" in text[at:at + 400]
+    for name in sorted(os.listdir(csrc)):
+        lines = open(os.path.join(csrc, name)).read().split("\n")
+        for i, line in enumerate(lines):
+            if "cudaFuncSetAttribute(" in line:
+                assert any(".get(dev," in before for before in lines[max(0, i - 8):i]), (name, i + 1)
