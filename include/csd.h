@@ -157,10 +157,11 @@ csd_status csd_tree_accept_greedy(const float* target_logits_dev, const int32_t*
 
 /* Prompt prefill: the model takes the input tokens in one run (Section 2).  Appends n tokens
  * (any n >= 1 with kv_len + n <= max_seq) at positions kv_len .. kv_len+n-1 to the cache of every
- * layer and produces no logits.  Models whose layer matrices are large enough for the tensor-core
- * kernels go through the weights once per 1024 tokens (wide blocks, two bf16 terms per fp32
- * activation); the rest, and a remainder of at most max_rows tokens, go through the review
- * kernels.  arch 1: decoder tokens, after csd_encoder_forward. */
+ * layer and produces no logits.  Models whose layer matrices have from 1037 rows (2^20 elements) to,
+ * for the gated pair, 18944 rows take prompts of more than max_rows tokens in equal wide passes of
+ * at most 1024 tokens each (at most max_seq rounded up to 128), two bf16 terms per fp32 activation;
+ * other models and shorter prompts go through the review kernels, which carry activations exactly.
+ * arch 1: decoder tokens, after csd_encoder_forward. */
 csd_status csd_prefill(csd_model* m, const int32_t* tokens_dev, int n, int kv_len, void* stream);
 
 /* Per-kernel-class timing of later forwards of this model (measurement aid; the paper's unit of

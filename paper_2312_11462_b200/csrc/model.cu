@@ -239,9 +239,15 @@ static int wide_pass(int left, int most) {
     return (left + passes - 1) / passes;
 }
 
-// The wide-block path serves a model when each of its layer matrices takes the wide kernel.
+// The wide-block path serves a model when each of its layer matrices takes the wide kernel and the model's prompts have gone by
+// two-term rows all along.  The review kernels carry rows exactly, in three terms, and that is what a model with a matrix of
+// fewer than 1037 rows (d_model 1024) or a feed-forward wider than 18944 keeps: rel-L2 from an fp64 forward behind prompts of 20,
+// 64 and 300 tokens, two layers, in review blocks / in wide passes: d_model 1024 2.7e-5, 8.1e-5, 3.5e-5 / 1.9e-4, 1.8e-4, 1.2e-4;
+// d_ff 20480 8.5e-5, 8.2e-5, 6.6e-5 / 2.3e-4, 1.5e-4, 1.5e-4.  (A 148-SM grid of 128-row ranges drew the lines: at least eight rows a
+// CTA, one range of the gated pair.)
 static bool wide_capable(const csd_model_config& c) {
     const int d = c.d_model, di = c.n_heads * c.d_head, ff = c.d_ff, R = CSD_WIDE_ROWS;
+    if (d <= 7 * 148 || di <= 7 * 148 || ff <= 7 * 148 || ff > 128 * 148) return false;
     return wide_supported(R, di, d, false) && wide_supported(R, 3 * di, d, false) && wide_supported(R, d, di, false) &&
            wide_supported(R, ff, d, true) && wide_supported(R, d, ff, false);
 }

@@ -10,7 +10,7 @@ from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, rel_l2, require_gpu, to_dev_i3
 
 pytestmark = pytest.mark.gpu
 
-LLAMA = llama_shape(2, 1024, 8, 1416, 500, 400)
+LLAMA = llama_shape(2, 1152, 9, 1416, 500, 400)
 
 
 @pytest.fixture(scope="module")

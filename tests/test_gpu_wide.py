@@ -3,6 +3,7 @@ columns, one to several of them, two passes) and encoder passes, each followed b
 every cached position, against the oracle's plain forward."""
 import numpy as np
 import pytest
+import torch
 
 import workloads
 from workloads import llama_shape, t5_shape
@@ -10,9 +11,9 @@ from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, rel_l2, require_gpu, to_dev_i3
 
 pytestmark = pytest.mark.gpu
 
-# matrices just large enough for the wide kernel; 3 * d_inner is 12 row tiles, d_ff = 1416 ends inside one
-LLAMA = llama_shape(2, 1024, 16, 1416, 500, 1200)
-T5 = t5_shape(2, 1, 1024, 16, 64, 1416, 500, 32, 300)
+# matrices just large enough for the wide passes; every one ends inside a row tile
+LLAMA = llama_shape(2, 1088, 17, 1416, 500, 1200)
+T5 = t5_shape(2, 1, 1088, 17, 64, 1416, 500, 32, 300)
 
 
 @pytest.fixture(scope="module")
@@ -64,3 +65,17 @@ def test_source_lengths(b, orc, n):
     assert b.csd_device_status() == 0
     assert rel_l2(g, r) <= LOGIT_REL_L2, rel_l2(g, r)
     assert np.abs(g - r).max() <= LOGIT_MAX_ABS
+
+
+@pytest.mark.parametrize("shape", [llama_shape(2, 1024, 16, 1416, 500, 200), llama_shape(1, 1088, 17, 18952, 500, 200)], ids=["d1024", "ff18952"])
+def test_models_outside_keep_exact_rows(b, shape):
+    """Models outside the sizes of the wide passes: a prompt is what its review-sized blocks are, bit for bit."""
+    blob = workloads.make_weights(shape, seed=43, device="cuda", gain_std=0.2)
+    toks = to_dev_i32(workloads.make_prompt(shape.vocab, 130, seed=3))
+    whole, blocks = b.Model(shape, blob), b.Model(shape, blob)
+    whole.csd_prefill(toks[:120].contiguous(), 0)
+    for p in range(0, 120, 17):
+        blocks.csd_review_forward(toks[p:min(p + 17, 120)].contiguous(), p, append_only=True)
+    rows = toks[120:125].contiguous()
+    assert torch.equal(whole.csd_review_forward(rows, 120), blocks.csd_review_forward(rows, 120))
+    assert b.csd_device_status() == 0
