@@ -185,7 +185,9 @@ csd_status csd_model_profile_read(csd_model* m, void* stream, csd_profile* out);
  * forward is made of (W bf16 row-major, X and Y fp32 row-major, fp32 accumulation).  Exposed
  * for kernel-level tests and roofline measurements.  K multiple of 8; 1 <= m <= 17 runs the review
  * kernels, 18 <= m <= 128 the wide-block kernel of the prefill (two bf16 terms per fp32 value, relative
- * error about 1e-5; needs N * K >= 2^20 and K >= 64, CSD_ERR_UNSUPPORTED otherwise). */
+ * error about 1e-5; needs N * K >= 2^20 and K >= 64, CSD_ERR_UNSUPPORTED otherwise).  For matrices of
+ * fewer than 2^20 elements and on path 1 the workspace has to be zero before its first call (every call
+ * leaves it ready for the next of the same shape); otherwise it may hold anything. */
 size_t csd_linear_workspace_bytes(int m, int N, int K);
 /* Which kernel the contraction uses, process-wide: 0 = automatic choice per shape, 1 = the
  * CUDA-core kernel (128-bit streaming loads, fp32 FMA), 2 = the tensor-core kernel (TMA-staged

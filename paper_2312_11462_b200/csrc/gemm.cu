@@ -325,7 +325,9 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual) {
     return align_up(worst, 256);
 }
 
-int linear_ticket_count(int N) { return N + 8; }   // one per row group of at least one row; four per 128-row tile; the wide kernel needs fewer
+// One per row group of at least one row (CUDA-core kernel); eight per 128-row tile (tensor-core kernel) are fewer.  The wide kernel's
+// (at most four per 128 rows and 256 tokens: wide_ticket_count) are looked after where its tickets are handed out.
+int linear_ticket_count(int N) { return N + 8; }
 
 // The row kernel (automatic choice only).  Measured back to back, us for row / tensor-core / split-K CUDA-core kernel:
 // 2304 x 768 at 1, 5, 8 rows 1.9 / 7.4 / 2.4, 3.2 / 8.1 / 3.5, 4.1 / 7.6 / 4.2; 768 x 3072 2.4 / 7.6 / 6.2, 4.9 / 8.2 / 8.2,
@@ -415,7 +417,9 @@ static LinearWs linear_ws(int m, int N, int K) {
     LinearWs w;
     size_t off = 0;
     const int rows = m > CSD_MAX_ROWS ? CSD_LINEAR_ROWS : CSD_MAX_ROWS;
-    w.tickets = off; off += align_up((size_t)linear_ticket_count(N) * sizeof(unsigned), 256);
+    int tickets = linear_ticket_count(N);
+    if (m > CSD_MAX_ROWS && wide_ticket_count(m, N) > tickets) tickets = wide_ticket_count(m, N);
+    w.tickets = off; off += align_up((size_t)tickets * sizeof(unsigned), 256);
     w.partial = off;
     {
         size_t pb = linear_scratch_bytes(m > CSD_MAX_ROWS ? CSD_MAX_ROWS : m, N, K, false);
@@ -433,8 +437,8 @@ extern "C" size_t csd_linear_workspace_bytes(int m, int N, int K) {
     return linear_ws(m, N, K).total;
 }
 
-// The workspace must be zero before the first call (the ticket words live in it); every launch
-// leaves the tickets zero again, so one cudaMemset after allocation is enough.
+// The tensor-core kernels' tickets are zeroed by the split in front of them, whatever the workspace holds.  The CUDA-core kernel
+// (small matrices) expects zeros and leaves zeros.
 extern "C" csd_status csd_linear(const void* W_bf16_dev, int N, int K, const float* X_dev, int m, float* Y_dev,
                                  void* workspace_dev, size_t workspace_bytes, void* stream) {
     if (m < 1 || m > CSD_LINEAR_ROWS || N < 1 || K < 8 || (K & 7)) return CSD_ERR_INVALID_ARG;
@@ -445,7 +449,8 @@ extern "C" csd_status csd_linear(const void* W_bf16_dev, int N, int K, const flo
     char* ws = (char*)workspace_dev;
     if (m > CSD_MAX_ROWS) {                  // wide block: two-term rows, the wide tensor-core kernel
         if (!wide_supported(m, N, K, false)) return CSD_ERR_UNSUPPORTED;
-        csd_status s = launch_wide_split(X_dev, K, K, m, nullptr, (__nv_bfloat16*)(ws + w.xs), nullptr, (cudaStream_t)stream);
+        csd_status s = launch_wide_split(X_dev, K, K, m, nullptr, (__nv_bfloat16*)(ws + w.xs), nullptr, (cudaStream_t)stream,
+                                         (unsigned*)(ws + w.tickets), wide_ticket_count(m, N));
         if (s != CSD_OK) return s;
         WideArgs wa;
         wa.W = (const __nv_bfloat16*)W_bf16_dev; wa.N = N; wa.K = K; wa.m = m; wa.xs = (const __nv_bfloat16*)(ws + w.xs);
@@ -457,6 +462,7 @@ extern "C" csd_status csd_linear(const void* W_bf16_dev, int N, int K, const flo
     a.W = (const __nv_bfloat16*)W_bf16_dev; a.N = N; a.K = K; a.X = X_dev; a.ldx = K; a.m = m;
     a.Y = Y_dev; a.ldy = N; a.epilogue = EPI_STORE;
     a.tickets = (unsigned*)(ws + w.tickets);
+    a.clear_tickets = true;
     a.partial = (float*)(ws + w.partial);
     a.xs = (__nv_bfloat16*)(ws + w.xs);
     a.ssq = (float*)(ws + w.ssq);

@@ -24,6 +24,7 @@ struct LinearArgs {
     bool xs_ready = false;               // false: launch_linear splits X (times gain) into xs first
     float* ssq = nullptr;                // [ssq_cnt][m] pieces of the sums of squares of the rows of X (gain != null)
     int ssq_cnt = 0;                     // entries valid in ssq when xs_ready
+    bool clear_tickets = false;          // the stand-alone split (xs_ready false) zeroes the tickets first: they may hold anything
     // optional extra outputs for the GEMM that consumes Y next
     __nv_bfloat16* out_xs = nullptr;     // three-term split of (Y * out_gain), [3m][out_ld]
     int out_ld = 0;

@@ -668,9 +668,10 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
 // each row's sum of squares.  grid = (K / 1024 rounded up, m).
 __global__ void __launch_bounds__(128)
 split_rows_kernel(const float* __restrict__ X, int ldx, int K, int m, const __nv_bfloat16* __restrict__ gain,
-                  __nv_bfloat16* __restrict__ xs, float* __restrict__ ssq) {
+                  __nv_bfloat16* __restrict__ xs, float* __restrict__ ssq, unsigned* __restrict__ clear, int clear_count) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    clear_words(clear, clear_count);
     const int r = blockIdx.y, k = (blockIdx.x * 128 + threadIdx.x) * 8;
     float sq = 0.f;
     if (k < K) {
@@ -724,7 +725,8 @@ csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st) {
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3((unsigned)split_ssq_entries(a.K), (unsigned)a.m), dim3(128), 0, st);
     CSD_CUDA(cudaLaunchKernelEx(&cfg, split_rows_kernel, a.X, a.ldx, a.K, a.m, a.gain, a.xs,
-                                a.gain ? a.ssq : (float*)nullptr));
+                                a.gain ? a.ssq : (float*)nullptr, a.clear_tickets ? a.tickets : (unsigned*)nullptr,
+                                a.clear_tickets ? (a.N + TILE_N - 1) / TILE_N * 8 : 0));
     count_launch();
     return CSD_OK;
 }

@@ -46,8 +46,9 @@ int wide_ssq_capacity(int N);
 size_t wide_partial_bytes(int m);
 int wide_ticket_count(int m, int N);
 int wide_split_pieces(int K);
+// clear, clear_count: ticket words zeroed on the way, for a launch_linear_wide whose tickets may hold anything
 csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_bfloat16* gain, __nv_bfloat16* xs,
-                             float* ssq, cudaStream_t st);
+                             float* ssq, cudaStream_t st, unsigned* clear = nullptr, int clear_count = 0);
 csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st);
 
 // 0 = automatic choice, 1 = CUDA-core kernel only, 2 = stream-K tensor-core kernel wherever it applies,

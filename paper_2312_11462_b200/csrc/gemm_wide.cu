@@ -592,9 +592,10 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 // pieces of each row's sum of squares.  grid = (K / 1024 rounded up, mpad).
 __global__ void __launch_bounds__(128)
 split2_rows_kernel(const float* __restrict__ X, int ldx, int K, int m, int mpad, const __nv_bfloat16* __restrict__ gain,
-                   __nv_bfloat16* __restrict__ xs, float* __restrict__ ssq) {
+                   __nv_bfloat16* __restrict__ xs, float* __restrict__ ssq, unsigned* __restrict__ clear, int clear_count) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    clear_words(clear, clear_count);
     const int r = blockIdx.y, k = (blockIdx.x * 128 + threadIdx.x) * 8;
     float sq = 0.f;
     if (k < K) {
@@ -691,11 +692,11 @@ wide_reduce_kernel(const float* __restrict__ P, int pk, size_t plane, int N, int
 }
 
 csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_bfloat16* gain, __nv_bfloat16* xs,
-                             float* ssq, cudaStream_t st) {
+                             float* ssq, cudaStream_t st, unsigned* clear, int clear_count) {
     if (!X || !xs || (((uintptr_t)X) & 15) || (ldx & 3) || (K & 7) || m < 1 || m > CSD_WIDE_ROWS) return CSD_ERR_INVALID_ARG;
     const int mpad = (m + 15) & ~15;
     PdlLaunch L(dim3((unsigned)wide_split_pieces(K), (unsigned)mpad), dim3(128), 0, st);
-    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, split2_rows_kernel, X, ldx, K, m, mpad, gain, xs, ssq));
+    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, split2_rows_kernel, X, ldx, K, m, mpad, gain, xs, ssq, clear, clear_count));
     count_launch();
     return CSD_OK;
 }

@@ -273,7 +273,12 @@ static WsLayout ws_layout(const csd_model_config& c) {
     };
     mat(3 * di, d, false); mat(di, d, false); mat(d, di, false); mat(ff, d, true); mat(d, ff, false); mat(V, d, false);
     L.gemm_partial = put(gp);
-    L.gemm_tickets = put((size_t)linear_ticket_count((int)nmax) * 4);
+    L.wide = wide_capable(c);
+    L.wide_rows = L.wide ? wide_rows_for(c) : 0;
+    size_t tickets = (size_t)linear_ticket_count((int)nmax);
+    const size_t widest = 3 * di > ff ? (3 * di > d ? 3 * di : d) : (ff > d ? ff : d);        // widest matrix of a wide pass
+    if (L.wide && (size_t)wide_ticket_count(L.wide_rows, (int)widest) > tickets) tickets = (size_t)wide_ticket_count(L.wide_rows, (int)widest);
+    L.gemm_tickets = put(tickets * 4);
     const size_t kmax = d > di ? (d > ff ? d : ff) : (di > ff ? di : ff);
     L.xs_tmp = put(3 * R * kmax * 2);
     L.ssq_tmp = put((size_t)split_ssq_entries((int)kmax) * R * 4);
@@ -281,9 +286,7 @@ static WsLayout ws_layout(const csd_model_config& c) {
     L.xs_attn = put(3 * R * di * 2);
     L.xs_act = put(3 * R * ff * 2);
     L.ssq_x = put((size_t)linear_ssq_capacity((int)d) * R * 4);
-    L.wide = wide_capable(c);
     if (L.wide) {
-        L.wide_rows = wide_rows_for(c);
         const size_t WR = (size_t)L.wide_rows;
         L.wx = put(WR * d * 4); L.wqkv = put(WR * 3 * di * 4); L.wattn = put(WR * di * 4);
         L.wxs_x = put(2 * WR * d * 2); L.wxs_attn = put(2 * WR * di * 2); L.wxs_act = put(2 * WR * ff * 2);

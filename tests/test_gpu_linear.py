@@ -85,3 +85,27 @@ def test_wide_blocks(orc):
         full = (X.double() @ W.double().T)
         assert float((Y.double() - full).norm() / full.norm()) < 3e-5
     assert b.csd_device_status() == 0
+
+
+def test_workspaces_that_hold_anything(orc):
+    """The tensor-core kernels count a tile's parts in words of the workspace: what an earlier call on another shape, or
+    whoever had the memory before, left there must not matter."""
+    require_gpu()
+    from paper_2312_11462_b200 import binding as b
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+
+    def check(m, N, K, ws, bound):
+        W = (0.05 * torch.randn(N, K, generator=g, device="cuda")).to(torch.bfloat16)
+        X = torch.randn(m, K, generator=g, device="cuda")
+        full = X.double() @ W.double().T
+        assert float((b.csd_linear(W, X, ws).double() - full).norm() / full.norm()) < bound, (m, N, K)
+
+    for m, N, K in ((18, 12288, 4096), (128, 20000, 1032), (40, 4096, 4096), (9, 12544, 2048), (17, 32000, 768), (1, 12288, 4096)):
+        ws = torch.full((b.lib.csd_linear_workspace_bytes(m, N, K),), 0x5a, dtype=torch.uint8, device="cuda")
+        check(m, N, K, ws, 3e-5 if m > 17 else 5e-6)
+    # a smaller matrix's partial sums lie where a larger one has its tickets
+    ws = b.csd_linear_workspace(17, 32000, 4096, "cuda")
+    for m, N, K in ((17, 1024, 4096), (17, 32000, 4096), (17, 2048, 4096), (5, 32000, 4096)):
+        check(m, N, K, ws, 5e-6)
+    assert b.csd_device_status() == 0
