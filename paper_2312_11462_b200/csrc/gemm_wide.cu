@@ -72,7 +72,8 @@ struct WgPlan {
 
 int wide_split_pieces(int K) { return (K + 1023) / 1024; }
 
-static WgPlan wg_plan(int m, int N, int K, bool dual) {
+// planes: whether the result may go through planes (their reduction stores 16 bytes at a time)
+static WgPlan wg_plan(int m, int N, int K, bool dual, bool planes = true) {
     WgPlan p{};
     const int P = tc_sm_count() / 2, most = dual && m <= 128 ? 128 : 256;
     p.mixed = dual && m > 128;
@@ -88,7 +89,7 @@ static WgPlan wg_plan(int m, int N, int K, bool dual) {
     p.smem = (size_t)p.stages * p.stage + 1024 + WG_STAGING + sizeof(WgCtrl);
     p.pk = 1; p.gran = 1;
     const int ratio = P / p.tiles;
-    if (!dual && (N & 7) == 0 && ratio >= 3 && p.nkb >= 16) {
+    if (planes && !dual && (N & 7) == 0 && ratio >= 3 && p.nkb >= 16) {
         p.pk = ratio < 8 ? ratio : 8;
         if (p.pk > p.nkb / 8) p.pk = p.nkb / 8;
         p.pairs = p.tiles * p.pk;
@@ -727,8 +728,11 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     if (!a.Y && (!dual || !a.out_xs)) return CSD_ERR_INVALID_ARG;
     if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU) || (dual && a.out_ssq)) return CSD_ERR_INVALID_ARG;
     if (!wide_supported(a.m, a.N, a.K, dual)) return CSD_ERR_UNSUPPORTED;
-    const WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
-    if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) return CSD_ERR_INVALID_ARG;
+    WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
+    if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) {
+        if (a.out_ssq) return CSD_ERR_INVALID_ARG;       // (its pieces are counted by the plan with planes)
+        pl = wg_plan(a.m, a.N, a.K, dual, false);
+    }
     CUtensorMap tw, tw2, tx;
     const int box = pl.mixed ? TILE_N / 2 : TILE_N;
     if (!tensor_map_2d(a.W, a.N, a.K, box, &tw)) return CSD_ERR_UNSUPPORTED;

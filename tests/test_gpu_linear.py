@@ -109,3 +109,22 @@ def test_workspaces_that_hold_anything(orc):
     for m, N, K in ((17, 1024, 4096), (17, 32000, 4096), (17, 2048, 4096), (5, 32000, 4096)):
         check(m, N, K, ws, 5e-6)
     assert b.csd_device_status() == 0
+
+
+@pytest.mark.parametrize("m,N,K", [(18, 1536, 1024), (128, 2304, 1536), (64, 4096, 4096), (33, 4099, 520)])
+def test_wide_blocks_into_any_address(m, N, K):
+    """A result that starts on a 4-byte boundary only (K parts then go through shares instead of planes)."""
+    require_gpu()
+    from paper_2312_11462_b200 import binding as b
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m)
+    W = (0.05 * torch.randn(N, K, generator=g, device="cuda")).to(torch.bfloat16)
+    X = torch.randn(m, K, generator=g, device="cuda")
+    full = X.double() @ W.double().T
+    room = torch.full((m * N + 8,), 7.0, device="cuda")
+    for off in (0, 1, 2, 3):
+        room.fill_(7.0)
+        Y = b.csd_linear(W, X, out=room[off:off + m * N].view(m, N))
+        assert float((Y.double() - full).norm() / full.norm()) < 3e-5, off
+        assert (room[:off] == 7.0).all() and (room[off + m * N:] == 7.0).all()
+    assert b.csd_device_status() == 0
