@@ -242,8 +242,8 @@ csd_status csd_spec_accept(const float* target_logits_dev, const float* draft_lo
  * library carries it until the process exits; csd_spec_accept_static_capacity returns the size).
  * The call allocates nothing, on the host or on the device, and takes the same inputs and gives
  * the same outputs as csd_spec_accept.  Differences:
- *   - problems whose scratch need (csd_spec_accept_workspace_bytes) exceeds the capacity are
- *     refused with CSD_ERR_CAPACITY; 64 rows x 16 drafted tokens x 128256 logits fits;
+ *   - problems whose scratch exceeds the capacity also when it is cut shortest are refused with
+ *     CSD_ERR_CAPACITY; 64 rows x 16 drafted tokens x 128256 logits fits;
  *   - a token id outside [0, V) is still treated as rejected, but is not recorded in the device
  *     status word (recording would need that word to exist, and creating it allocates);
  *   - the first call on each device looks up the device address of the array (with that device

@@ -350,6 +350,8 @@ __device__ __forceinline__ bool last_of_row(unsigned* ticket, int nchunk, int la
 }
 
 // pass 1: per-chunk sums of exp((t - max_t)/T) and exp((d - max_q)/T), and their totals
+// SETS: a chunk is SETS times 512 logits (1; 4 where the scratch at hand does not hold the sums of the short ones)
+template <int SETS>
 __global__ void __launch_bounds__(RS_THREADS, 3)
 resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
                   const RowInfo* __restrict__ info, double2* __restrict__ zpart, double2* __restrict__ zsum,
@@ -367,23 +369,26 @@ resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, in
     const float* t = tl + ((long long)row * (k + 1) + ri.n) * V;
     const float* d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
     const bool vec = (V % 4 == 0) && ((((uintptr_t)t) & 15) == 0) && (!d || (((uintptr_t)d) & 15) == 0);
-    const int e0 = chunk * RS_CHUNK + lane * 8;
     double sp = 0.0, sq = 0.0;
-    float tv[2][8], dv[2][8];
+#pragma unroll 1
+    for (int set = 0; set < SETS; ++set) {
+        const int e0 = (chunk * SETS + set) * RS_CHUNK + lane * 8;
+        float tv[2][8], dv[2][8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        load8(t, e0 + h * 256, V, vec, tv[h]);
-        if (d) load8(d, e0 + h * 256, V, vec, dv[h]);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sp += exp_neg(((double)tv[h][j] - ri.max_t) * invT, s_tab);      // -inf (past V) gives 0
-    if (d) {
+        for (int h = 0; h < 2; ++h) {
+            load8(t, e0 + h * 256, V, vec, tv[h]);
+            if (d) load8(d, e0 + h * 256, V, vec, dv[h]);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sq += exp_neg(((double)dv[h][j] - ri.max_q) * invT, s_tab);
+            for (int j = 0; j < 8; ++j) sp += exp_neg(((double)tv[h][j] - ri.max_t) * invT, s_tab);      // -inf (past V) gives 0
+        if (d) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) sq += exp_neg(((double)dv[h][j] - ri.max_q) * invT, s_tab);
+        }
     }
     sp = warp_sum(sp);
     sq = warp_sum(sq);
@@ -398,6 +403,7 @@ resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, in
 }
 
 // pass 2: per-chunk mass of the residual; the warp that arrives last at the row's ticket picks the token
+template <int SETS>
 __global__ void __launch_bounds__(RS_THREADS, 3)
 resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
                      const RowInfo* __restrict__ info, const double2* __restrict__ zpart,
@@ -422,18 +428,21 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
     c.mode = ri.mode; c.x = ri.x; c.tab = s_tab;
     const bool vec = (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
     {
-        const int e0 = chunk * RS_CHUNK + lane * 8;
         double sr = 0.0;
-        float tv[2][8], dv[2][8];
+#pragma unroll 1
+        for (int set = 0; set < SETS; ++set) {
+            const int e0 = (chunk * SETS + set) * RS_CHUNK + lane * 8;
+            float tv[2][8], dv[2][8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            load8(c.t, e0 + h * 256, V, vec, tv[h]);
-            if (c.d) load8(c.d, e0 + h * 256, V, vec, dv[h]);
+            for (int h = 0; h < 2; ++h) {
+                load8(c.t, e0 + h * 256, V, vec, tv[h]);
+                if (c.d) load8(c.d, e0 + h * 256, V, vec, dv[h]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) sr += residual_of(c, e0 + h * 256 + j, tv[h][j], c.d ? dv[h][j] : 0.f);   // past V: et is 0
         }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sr += residual_of(c, e0 + h * 256 + j, tv[h][j], c.d ? dv[h][j] : 0.f);   // past V: et is 0
         sr = warp_sum(sr);
         if (lane == 0) rrow[chunk] = sr;
     }
@@ -478,7 +487,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
     // ---- the entry: smallest index whose cumulative mass exceeds the target, else the last that carries mass
     int pick = -1, last = -1;
 #pragma unroll 1
-    for (int e = pick_chunk * RS_CHUNK; e < min(V, (pick_chunk + 1) * RS_CHUNK) && pick < 0; e += 256) {
+    for (int e = pick_chunk * SETS * RS_CHUNK; e < min(V, (pick_chunk + 1) * SETS * RS_CHUNK) && pick < 0; e += 256) {
         const int at = e + lane * 8;
         float tv[8], dv[8];
         load8(c.t, at, V, vec, tv);
@@ -937,13 +946,14 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
 
 struct AcceptLayout {
     size_t part_off, info_off, z_off, zsum_off, r_off, ticket_off, total;
-    int nchunk_a, nchunk_r;
+    int nchunk_a, nchunk_r, sets;
 };
 
-static AcceptLayout accept_layout(int rows, int k, int V) {
+static AcceptLayout accept_layout(int rows, int k, int V, int sets = 1) {
     AcceptLayout L;
     L.nchunk_a = (V + ST_CHUNK - 1) / ST_CHUNK;
-    L.nchunk_r = (V + RS_CHUNK - 1) / RS_CHUNK;
+    L.nchunk_r = (int)(((long long)V + sets * RS_CHUNK - 1) / (sets * RS_CHUNK));
+    L.sets = sets;
     size_t nvec = (size_t)rows * (2 * (size_t)k + 1);
     size_t off = 0;
     L.part_off = off;   off = align_up(off + nvec * L.nchunk_a * sizeof(StatPartial), 256);
@@ -954,6 +964,17 @@ static AcceptLayout accept_layout(int rows, int k, int V) {
     L.ticket_off = off; off = align_up(off + 2 * (size_t)rows * sizeof(unsigned), 256);   // normaliser pass, mass pass
     L.total = off;
     return L;
+}
+
+// The layout for `room` bytes of scratch: the resample passes keep 24 bytes per row and chunk, of 512 logits where that fits, else of
+// 2048.  (V = 128256, 512 / 2048: 64 rows, k = 4 123 / 131 us a call, k = 16 246 / 257; 320 rows, k = 1 315 / 274.)
+static csd_status accept_layout_in(int rows, int k, int V, size_t room, AcceptLayout& L) {
+    const AcceptLayout least = accept_layout(rows, k, V, 4);
+    if (room < least.total) return CSD_ERR_CAPACITY;
+    if (least.nchunk_r > 65535) return CSD_ERR_UNSUPPORTED;
+    L = accept_layout(rows, k, V);
+    if (room < L.total || L.nchunk_r > 65535) L = least;
+    return CSD_OK;
 }
 
 static int accept_sm_count() {
@@ -1140,11 +1161,12 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     } else if (!greedy) {
         const dim3 g2((unsigned)(((long long)rows * L.nchunk_r + RS_THREADS / 32 - 1) / (RS_THREADS / 32)));
         PdlLaunch lz(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lz.cfg, resample_z_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, zpart, zsum,
-                                    tickets, L.nchunk_r));
+        CSD_CUDA(cudaLaunchKernelEx(&lz.cfg, L.sets == 1 ? resample_z_kernel<1> : resample_z_kernel<4>, tl, dl, rows, k, V, temperature,
+                                    (const RowInfo*)info, zpart, zsum, tickets, L.nchunk_r));
         PdlLaunch lp(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, resample_pick_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info,
-                                    (const double2*)zpart, (const double2*)zsum, rpart, tickets + rows, L.nchunk_r, (int*)out_tok));
+        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, L.sets == 1 ? resample_pick_kernel<1> : resample_pick_kernel<4>, tl, dl, rows, k, V,
+                                    temperature, (const RowInfo*)info, (const double2*)zpart, (const double2*)zsum, rpart,
+                                    tickets + rows, L.nchunk_r, (int*)out_tok));
         count_launch(2);
     }
     CSD_CUDA(cudaGetLastError());
@@ -1171,9 +1193,9 @@ csd_status accept_into(const float* target_logits_dev, const float* draft_logits
     if (!target_logits_dev || !n_accepted_dev || !out_token_dev || !workspace_dev) return CSD_ERR_INVALID_ARG;
     if (k > 0 && !draft_tokens_dev) return CSD_ERR_INVALID_ARG;
     if (((uintptr_t)workspace_dev & 255) != 0) return CSD_ERR_INVALID_ARG;
-    const AcceptLayout L = accept_layout(rows, k, V);
-    if (workspace_bytes < L.total) return CSD_ERR_CAPACITY;
-    if (L.nchunk_r > 65535) return CSD_ERR_UNSUPPORTED;
+    AcceptLayout L;
+    const csd_status fits = accept_layout_in(rows, k, V, workspace_bytes, L);
+    if (fits != CSD_OK) return fits;
     int* status = status_word_device();
     if (!status) return CSD_ERR_CUDA;
     return run_accept(target_logits_dev, draft_logits_dev, onehot_dev, draft_tokens_dev, rows, k, V, temperature, lenience,
@@ -1301,9 +1323,9 @@ extern "C" csd_status csd_spec_accept_static(const float* target_logits_dev, con
     if (rows == 0) return CSD_OK;
     if (!target_logits_dev || !n_accepted_dev || !out_token_dev) return CSD_ERR_INVALID_ARG;
     if (k > 0 && !draft_tokens_dev) return CSD_ERR_INVALID_ARG;
-    const AcceptLayout L = accept_layout(rows, k, V);
-    if (L.total > STATIC_SCRATCH_BYTES) return CSD_ERR_CAPACITY;   // the problem does not fit the fixed scratch
-    if (L.nchunk_r > 65535) return CSD_ERR_UNSUPPORTED;
+    AcceptLayout L;
+    const csd_status fits = accept_layout_in(rows, k, V, STATIC_SCRATCH_BYTES, L);
+    if (fits != CSD_OK) return fits;
     // Set-up, once per device: in host code the array's name is only a handle, so ask the runtime
     // for the address the kernels can use.  Nothing is allocated here.
     int dev = 0;

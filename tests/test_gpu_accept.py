@@ -117,3 +117,21 @@ def test_distribution_on_tiny_vocab(b, orc):
     assert stats.chisquare(np.bincount(y1, minlength=V), p[0] * N).pvalue > 0.01
     y3 = o[n == 2]
     assert stats.chisquare(np.bincount(y3, minlength=V), p[2] * len(y3)).pvalue > 0.01
+
+
+@pytest.mark.parametrize("rows,k,V,sigma", [(3, 2, 131076, 0.5), (64, 4, 128256, 0.1), (64, 1, 200003, 2.0), (5, 0, 150000, 0.5)])
+def test_scratch_for_longer_chunks_only(b, orc, rows, k, V, sigma):
+    """A workspace that holds a quarter of the resample passes' chunk sums: chunks of 2048 logits instead of 512, the same law."""
+    t, d, tok = workloads.accept_case(rows, k, V, sigma, seed=rows + k, device="cuda")
+    full = b.lib.csd_spec_accept_workspace_bytes(rows, k, V)
+    short = full - 24 * rows * (-(-V // 512) - -(-V // 2048)) + 1024        # (1024: the parts start on 256-byte boundaries)
+    assert short < full
+    want = orc.spec_accept(t.cpu().numpy(), d.cpu().numpy() if k else None, tok.cpu().numpy(), 1.0, 1.0, 9, 4)
+    for nbytes in (full, short):
+        room = torch.zeros(nbytes + 4096, dtype=torch.uint8, device="cuda")
+        n, o = b.csd_spec_accept(t, d if k else None, tok, 1.0, seed=9, step=4, workspace=room[:nbytes])
+        assert b.csd_device_status() == 0 and (room[nbytes:] == 0).all()
+        ok = want[2] == 0
+        assert (n.cpu().numpy()[ok] == want[0][ok]).all() and (o.cpu().numpy()[ok] == want[1][ok]).all()
+    with pytest.raises(b.CsdError):
+        b.csd_spec_accept(t, d if k else None, tok, 1.0, workspace=room[:short - 2048 - 24 * rows])

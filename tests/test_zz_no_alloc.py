@@ -83,3 +83,14 @@ def test_refuses_what_does_not_fit_and_bad_arguments(b):
     code = b.lib.csd_spec_accept_static(t.data_ptr(), None, None, t.data_ptr(), 1, 1, 8, 1.0, 0.5, 0, 0,
                                         out[0].data_ptr(), out[1].data_ptr(), None)
     assert code == 1                        # lenience below 1
+
+
+def test_takes_what_fits_in_longer_chunks(b):
+    """Rows whose sums per 512 logits exceed the scratch, but not their sums per 2048."""
+    rows, k, V = 320, 1, 128256
+    assert b.lib.csd_spec_accept_workspace_bytes(rows, k, V) > b.lib.csd_spec_accept_static_capacity()
+    t, d, tok = workloads.accept_case(rows, k, V, 0.5, seed=12, device="cuda")
+    want = b.csd_spec_accept(t, d, tok, 1.0, seed=2)
+    got = b.csd_spec_accept_static(t, d, tok, 1.0, seed=2, out=outputs(rows))
+    assert torch.equal(got[0], want[0])
+    assert (got[1] != want[1]).sum() <= 1        # (fp64 sums in another order: a target within 1e-11 of an entry's edge)
