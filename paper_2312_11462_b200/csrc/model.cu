@@ -17,13 +17,13 @@ embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict
                              float* __restrict__ x, int* status) {
     pdl_wait();
     pdl_trigger();
-    const int r = blockIdx.y;
+    const int r = blockIdx.x;                  // (a source may have more tokens than a grid has room for in y)
     int t = tokens[r];
     if (t < 0 || t >= V) {
-        if (threadIdx.x == 0 && blockIdx.x == 0) set_status(status, CSD_ERR_BAD_TOKEN);
+        if (threadIdx.x == 0 && blockIdx.y == 0) set_status(status, CSD_ERR_BAD_TOKEN);
         t = 0;
     }
-    const int k = (blockIdx.x * 128 + threadIdx.x) * 8;
+    const int k = (blockIdx.y * 128 + threadIdx.x) * 8;
     if (k >= d) return;
     const uint4 e = *reinterpret_cast<const uint4*>(E + (size_t)t * d + k);
     float* dst = x + (size_t)r * d + k;
@@ -33,7 +33,7 @@ embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict
 
 static csd_status launch_embed(const int32_t* tokens, const __nv_bfloat16* E, int V, int d, int m, float* x, int* status,
                                cudaStream_t st) {
-    PdlLaunch L(dim3((unsigned)((d + 1023) / 1024), (unsigned)m), dim3(128), 0, st);
+    PdlLaunch L(dim3((unsigned)m, (unsigned)((d + 1023) / 1024)), dim3(128), 0, st);
     CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_kernel, tokens, E, V, d, x, status));
     count_launch();
     return CSD_OK;

@@ -79,3 +79,20 @@ def test_models_outside_keep_exact_rows(b, shape):
     rows = toks[120:125].contiguous()
     assert torch.equal(whole.csd_review_forward(rows, 120), blocks.csd_review_forward(rows, 120))
     assert b.csd_device_status() == 0
+
+
+def test_source_longer_than_a_grid_dimension(b):
+    """A source of more than 65535 tokens, all equal and without position biases: every position attends to the same value
+    whatever the length, so the decoder must see what a short source gives it."""
+    shape = t5_shape(1, 1, 64, 2, 32, 128, 64, 8, 65600)
+    blob = workloads.make_weights(shape, seed=45, device="cuda", gain_std=0.2)
+    at = {name: (off, int(np.prod(shp))) for name, off, shp in workloads.blob_layout(shape)[0]}
+    off, count = at["enc.rel_bias"]
+    blob[off:off + count] = 0
+    m = b.Model(shape, blob)
+    out = []
+    for n in (24, 65600):
+        m.csd_encoder_forward(torch.full((n,), 7, dtype=torch.int32, device="cuda"))
+        out.append(m.csd_review_forward(to_dev_i32([1, 2, 3]), 0))
+    assert b.csd_device_status() == 0 and torch.isfinite(out[0]).all()
+    assert rel_l2(out[1].cpu(), out[0].cpu()) <= 1e-4           # (sums of 65600 fp32 weights: sqrt(65600) 2^-24 each, and K and V entries that round to the neighbour)
