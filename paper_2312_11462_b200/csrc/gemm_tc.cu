@@ -657,6 +657,9 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
     if (*abort_flag) {              // (looked at behind the barrier: any warp may have given up last)
         if (tid == 0) set_status(p.status, CSD_ERR_TIMEOUT);
         __nanosleep(2000000);          // let copies already in flight land before the CTA's memory is released
+        // cluster split: the others may still write into this CTA's memory or signal its barriers.  All their waits end, and who
+        // has left the kernel is not waited for.
+        if (p.csplit > 1) cluster_barrier();
     }
     if (warp == 1) {
         tc_fence_after();

@@ -338,6 +338,8 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0u);
         unsigned g = 0;
+        bool ok = true;               // false: this warp waited in vain.  It goes on through every barrier (and stores what it has, under
+                                      // CSD_ERR_TIMEOUT): another warp's wait may still have ended well, and would wait for it there.
 #pragma unroll 1
         for (int i = 0; i < items;) {
             const int tile = (int)((u0 + i) / p.nkb), kb_begin = (int)((u0 + i) % p.nkb);
@@ -355,12 +357,11 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             float acc[NT * CH * 16];
 #pragma unroll
             for (int e = 0; e < NT * CH * 16; ++e) acc[e] = 0.f;
-            bool ok = true;
 #pragma unroll 1
-            for (int left = seg; left > 0; left -= WG_DRAIN, ++g) {
+            for (int left = seg; left > 0 && ok; left -= WG_DRAIN, ++g) {
                 const int b = g & 1;
                 ok = mbar_wait(&ctl->acc_full[b], (g >> 1) & 1);
-                if (!ok) break;
+                if (!ok) { *abort_flag = 1; break; }
                 tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * WG_SET + half * htok);
 #pragma unroll
@@ -380,7 +381,6 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     else remote_arrive(empty_bar + (uint32_t)(b * sizeof(uint64_t)));
                 }
             }
-            if (!ok) { *abort_flag = 1; break; }              // (the same outcome in all eight warps)
             if (p.pk == 1 && seg < p.nkb) {
                 // part of a tile: later contributors park and go on, the first one adds the parts in pair order.
                 // Parked layout [warp][chunk][quarter of 16][lane][4]: 512 contiguous bytes per warp access.
@@ -413,7 +413,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     int spins = 0;
 #pragma unroll 1
                     while (ld_acquire_gpu(&p.tickets[2 * tile + rank]) < want)
-                        if (++spins > SPIN_LIMIT) { *abort_flag = 1; break; }
+                        if (++spins > SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
                     p.tickets[2 * tile + rank] = 0u;          // everyone has arrived: ready for the next launch
                     __threadfence();
                     asm volatile("fence.proxy.async;" ::: "memory");
