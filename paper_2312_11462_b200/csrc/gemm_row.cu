@@ -66,6 +66,9 @@ template <int M, int R, int S, bool DUAL, bool GATHER>
 __global__ void __launch_bounds__(RW_THREADS, 2)
 row_gemm_kernel(const RowParams p) {
     constexpr int NT = DUAL ? 2 : 1, V = R * M, Q = (V + 31) / 32;     // sums, in groups of 32
+    // A lane's 8 S products of a sum run as one chain of adds for short K and as two beyond, or their rounding shows (768 x 3072
+    // against fp64: 1.9e-7 with one chain, 1.4e-7 with two, as the tensor-core kernel).
+    constexpr int CHAINS = S > 3 ? 2 : 1;
     extern __shared__ __align__(16) float rw_smem[];
     const int steps = p.steps, KP = steps * RW_STEP;
     float* xs = rw_smem;                             // [M][KP], each step stored as [half][lane][4]
@@ -166,11 +169,11 @@ row_gemm_kernel(const RowParams p) {
 
 #pragma unroll 1
     while (g < groups) {
-        float acc[NT][V];
+        float acc[NT][V], acc2[NT][V];
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
-            for (int v = 0; v < V; ++v) acc[t][v] = 0.f;
+            for (int v = 0; v < V; ++v) acc[t][v] = acc2[t][v] = 0.f;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             if (s >= steps) break;
@@ -187,11 +190,19 @@ row_gemm_kernel(const RowParams p) {
                         float d = acc[t][rr * M + r];
                         d = fmaf(bf16lo(u.x), xa.x, d); d = fmaf(bf16hi(u.x), xa.y, d);
                         d = fmaf(bf16lo(u.y), xa.z, d); d = fmaf(bf16hi(u.y), xa.w, d);
-                        d = fmaf(bf16lo(u.z), xb.x, d); d = fmaf(bf16hi(u.z), xb.y, d);
-                        d = fmaf(bf16lo(u.w), xb.z, d); d = fmaf(bf16hi(u.w), xb.w, d);
-                        acc[t][rr * M + r] = d;
+                        float e = CHAINS > 1 ? acc2[t][rr * M + r] : d;
+                        e = fmaf(bf16lo(u.z), xb.x, e); e = fmaf(bf16hi(u.z), xb.y, e);
+                        e = fmaf(bf16lo(u.w), xb.z, e); e = fmaf(bf16hi(u.w), xb.w, e);
+                        acc[t][rr * M + r] = CHAINS > 1 ? d : e;
+                        if (CHAINS > 1) acc2[t][rr * M + r] = e;
                     }
             }
+        }
+        if (CHAINS > 1) {
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[t][v] += acc2[t][v];
         }
         const int cur = g;
         g += stride;

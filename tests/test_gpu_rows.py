@@ -34,6 +34,20 @@ def test_shapes(b, m):
     assert b.csd_device_status() == 0
 
 
+@pytest.mark.parametrize("m", [1, 5, 6, 8])
+def test_rounding_of_long_sums(b, m):
+    """K = 3072: 96 products a lane.  In two chains of 48 adds, partial sums of sqrt(j) terms round to 2^-25 of themselves, rms
+    sqrt(2 / 3): sqrt(48 / 2) 2^-25 sqrt(2 / 3) = 1.2e-7 of the result, the tree over lanes and columns under 0.5e-7 more; in one chain
+    1.7e-7 and more."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m)
+    W = (0.05 * torch.randn(768, 3072, generator=g, device="cuda")).to(torch.bfloat16)
+    X = torch.randn(m, 3072, generator=g, device="cuda")
+    want = X.double() @ W.double().T
+    assert float((b.csd_linear(W, X).double() - want).norm() / want.norm()) < 1.65e-7
+    assert b.csd_device_status() == 0
+
+
 @pytest.mark.parametrize("shape", [llama_shape(2, 768, 12, 3072, 3001, 96), llama_shape(1, 512, 8, 776, 777, 96), t5_shape(1, 2, 512, 8, 64, 1000, 700, 96, 40)],
                          ids=["d768", "d512", "t5-d512"])
 def test_forwards(b, orc, shape):
