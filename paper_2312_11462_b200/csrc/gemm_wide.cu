@@ -17,8 +17,10 @@
 // fp32 accumulation.  The tensor core loses a little with every add of a long chain, so after WG_DRAIN
 // K blocks (64 adds) the accumulator set is added into fp32 registers of the epilogue warps while
 // the MMAs continue on the other set: shorter chains than in the earlier kernel (256 to 700
-// adds), and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to 11008:
-// 2.7e-6 (earlier 5.0e-6), which is what the two-term form itself leaves.
+// adds), and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to 11008: 2.7e-6 (earlier
+// 2.5e-6 to 5.0e-6, growing with the block), of which the two-term form itself leaves 2.45e-6.  Tiles of up to 32 tokens, where the
+// earlier kernel left 2.45e-6 to 2.65e-6, sum the low terms' products in columns of their own: 2.5e-6.  (8 layers of the 7B shape, 20
+// tokens: 1001 us, 965 so, the kernel of such tiles being short as well; sets of 4 K blocks, which leave the same, cost 2 to 7 % a GEMM.)
 //
 // Roles inside a CTA (384 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 of the pair's first CTA
 // issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
@@ -186,7 +188,8 @@ __device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigne
 // its 128 weight rows from shared memory for half the work, and those reads, not the tensor pipe, set the pace: gate and up of
 // the 7B shape at 1000 tokens 323 us in mode 1, 277 in mode 2; of the T5-xxl shape at 256 tokens 92 and 82.
 // Up to 128 tokens mode 1 moves fewer bytes: its tile is 256 outputs wide.)
-template <int MODE>
+// LOW: tiles of up to 32 tokens, the low terms' products in columns of their own (modes 0 and 1)
+template <int MODE, bool LOW>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmX, const WgParams p) {
@@ -194,8 +197,9 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     constexpr int NT = DUAL ? 2 : 1;
     constexpr int OUT_ROWS = MIXED ? WG_ROWS / 2 : WG_ROWS;   // outputs of a tile
     constexpr uint32_t WB = NT * STAGE_BYTES;                 // weight bytes per stage and CTA
-    constexpr int CH = DUAL ? 4 : 8;                          // 16-token chunks an epilogue warp holds at most
-    const int nt = p.nt, htok = nt >> 1;
+    constexpr int CH = LOW ? 1 : (DUAL ? 4 : 8);              // 16-token chunks an epilogue warp holds at most
+    const int nt = LOW ? 32 : p.nt, htok = nt >> 1;
+    constexpr uint32_t LOW_COLS = LOW ? 32 * NT : 0;          // columns between the high and the low terms' sums
     const uint32_t xterm = (uint32_t)htok * 128u;             // one term of this CTA's half of the tokens
     const uint32_t stage_bytes = WB + 2u * xterm;
     const uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) |
@@ -312,10 +316,10 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         for (int k = 0; k < KB / 16; ++k) {
                             const uint32_t acc = (j | k) != 0;
                             tc_mma_pair(d0, ad + 2 * k, bh + 2 * k, IDESC, acc);
-                            tc_mma_pair(d0, ad + 2 * k, bl + 2 * k, IDESC, 1u);
+                            tc_mma_pair(d0 + LOW_COLS, ad + 2 * k, bl + 2 * k, IDESC, LOW ? acc : 1u);
                             if (DUAL) {
                                 tc_mma_pair(d0 + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bh + 2 * k, IDESC, acc);
-                                tc_mma_pair(d0 + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bl + 2 * k, IDESC, 1u);
+                                tc_mma_pair(d0 + LOW_COLS + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bl + 2 * k, IDESC, LOW ? acc : 1u);
                             }
                         }
                         tc_commit_pair(&ctl->empty[s]);
@@ -337,9 +341,9 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const uint32_t part_bytes = (uint32_t)(TILE_N * NT * sizeof(float)) * (uint32_t)nt;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0u);
-        unsigned g = 0;
-        bool ok = true;               // false: this warp waited in vain.  It goes on through every barrier (and stores what it has, under
-                                      // CSD_ERR_TIMEOUT): another warp's wait may still have ended well, and would wait for it there.
+        // Accumulator sets read so far; negative once this warp has waited in vain.  It then goes on through every barrier (and stores
+        // what it has, under CSD_ERR_TIMEOUT): another warp's wait may still have ended well, and would wait for it there.
+        int g = 0;
 #pragma unroll 1
         for (int i = 0; i < items;) {
             const int tile = (int)((u0 + i) / p.nkb), kb_begin = (int)((u0 + i) % p.nkb);
@@ -358,10 +362,9 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll
             for (int e = 0; e < NT * CH * 16; ++e) acc[e] = 0.f;
 #pragma unroll 1
-            for (int left = seg; left > 0 && ok; left -= WG_DRAIN, ++g) {
+            for (int left = seg; left > 0 && g >= 0; left -= WG_DRAIN, ++g) {
                 const int b = g & 1;
-                ok = mbar_wait(&ctl->acc_full[b], (g >> 1) & 1);
-                if (!ok) { *abort_flag = 1; break; }
+                if (!mbar_wait(&ctl->acc_full[b], (uint32_t)(g >> 1) & 1u)) { *abort_flag = 1; g = -1; break; }
                 tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * WG_SET + half * htok);
 #pragma unroll
@@ -373,6 +376,11 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                             tc_ld16(taddr + (uint32_t)(u * nt + ch * 16), v);
 #pragma unroll
                             for (int e = 0; e < 16; ++e) acc[(u * CH + ch) * 16 + e] += v[e];
+                            if (LOW) {
+                                tc_ld16(taddr + LOW_COLS + (uint32_t)(u * nt), v);
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) acc[(u * CH + ch) * 16 + e] += v[e];
+                            }
                         }
                 tc_fence_before();
                 __syncwarp();
@@ -702,10 +710,12 @@ csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_b
     return CSD_OK;
 }
 
-template <int MODE>
+template <int MODE, bool LOW = false>
 static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const WgParams& wp,
                             const WgPlan& pl, cudaStream_t st) {
-    auto kern = wide_gemm_kernel<MODE>;
+    if constexpr (MODE < 2 && !LOW)
+        if (pl.nt == 32) return launch_wg<MODE, true>(tw, tw2, tx, wp, pl, st);
+    auto kern = wide_gemm_kernel<MODE, LOW>;
     static PerDevice ready;
     const csd_status ok = allow_smem(ready, kern, WG_SMEM_MAX);
     if (ok != CSD_OK) return ok;

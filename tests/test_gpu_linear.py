@@ -128,3 +128,24 @@ def test_wide_blocks_into_any_address(m, N, K):
         assert float((Y.double() - full).norm() / full.norm()) < 3e-5, off
         assert (room[:off] == 7.0).all() and (room[off + m * N:] == 7.0).all()
     assert b.csd_device_status() == 0
+
+
+@pytest.mark.parametrize("m", [18, 31, 32])
+@pytest.mark.parametrize("N,K", [(4096, 4096), (12288, 4096), (2304, 768)])
+def test_smallest_wide_blocks_sum_like_fp32(m, N, K):
+    """Blocks of up to 32 rows against the fp64 product of the two-term rows themselves: what is left is the fp32 accumulation,
+    in chains of 32 tensor-core adds, each truncating up to 2^-23 of the partial sum.  A chain is 512 of the K products, so its
+    sum is sqrt(512 / K) of the result and its partial sums 2/3 of that; the losses of a chain point one way and K / 512 chains add
+    up like their signs: 32 * 2/3 * 2^-24 * sqrt(512 / K) * sqrt(K / 512) / 2 = 6e-7, half of it on average over a mantissa's range.
+    Measured 4.7e-7; with both terms in one chain of 64 adds 1.1e-6."""
+    require_gpu()
+    from paper_2312_11462_b200 import binding as b
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + N)
+    W = (0.05 * torch.randn(N, K, generator=g, device="cuda")).to(torch.bfloat16)
+    X = torch.randn(m, K, generator=g, device="cuda")
+    hi = X.to(torch.bfloat16)
+    lo = (X - hi.float()).to(torch.bfloat16)
+    full = (hi.double() + lo.double()) @ W.double().T
+    assert float((b.csd_linear(W, X).double() - full).norm() / full.norm()) < 7e-7
+    assert b.csd_device_status() == 0
