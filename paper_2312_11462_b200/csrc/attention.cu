@@ -834,17 +834,12 @@ csd_status launch_attention(const AttnArgs& a, cudaStream_t st) {
     return CSD_OK;
 }
 
-csd_status launch_attention_batch(const AttnArgs* a, int n, cudaStream_t st) {
-    const bool together = n > 0 && (a[0].Dh == 64 || a[0].Dh == 128) && !g_attn_cuda_cores;
-    for (int i = 0; i < n;) {
-        int cnt = together ? (n - i < MAX_SEGS ? n - i : MAX_SEGS) : 1;
-        for (int j = i; j < i + cnt; ++j)
-            if (a[j].tree_mask || a[j].m > 16) cnt = 1;
-        const csd_status rc = launch_attention_block(a + i, cnt, st);
-        if (rc != CSD_OK) return rc;
-        i += cnt;
-    }
-    return CSD_OK;
+csd_status launch_attention_batch(const AttnArgs* a, int n, int* taken, cudaStream_t st) {
+    int cnt = n > 1 && (a[0].Dh == 64 || a[0].Dh == 128) && !g_attn_cuda_cores ? (n < MAX_SEGS ? n : MAX_SEGS) : 1;
+    for (int j = 0; j < cnt; ++j)
+        if (a[j].tree_mask || a[j].m > 16) cnt = 1;
+    *taken = cnt;
+    return cnt == 1 ? launch_attention(a[0], st) : launch_attention_block(a, cnt, st);
 }
 
 // The blocks of n sequences of one model (n <= MAX_SEGS; more than one on the tensor-core kernel only, without a tree).

@@ -50,8 +50,9 @@ struct AttnArgs {
 int attn_splits(int total_keys, int H, int Dh, int gemm_rows);   // gemm_rows: rows of the projection that follows
 void set_attention_cuda_cores(bool on);   // true: always the CUDA-core kernel (for comparison runs)
 csd_status launch_attention(const AttnArgs& a, cudaStream_t st);
-// The blocks of n sequences that share a model and an output buffer (batched review): one launch per four where it can.
-csd_status launch_attention_batch(const AttnArgs* a, int n, cudaStream_t st);
+// The first of the blocks of n sequences that share a model and an output buffer (batched review), in one launch: up to four
+// where it can; *taken says how many.
+csd_status launch_attention_batch(const AttnArgs* a, int n, int* taken, cudaStream_t st);
 // Whether the rows of a wide pass take launch_row_attention: head dimension 64 or 128, comparison switch off.
 bool row_attention_supported(int Dh);
 csd_status launch_row_attention(const AttnArgs& a, cudaStream_t st);

@@ -375,8 +375,11 @@ static csd_status attention(csd_model* M, const AttnArgs& a, cudaStream_t st) {
     return launch_attention(a, st);
 }
 static csd_status attention(csd_model* M, const AttnArgs* blocks, int n, cudaStream_t st) {
-    ProfScope ps(M, 1, st);
-    return n == 1 ? launch_attention(blocks[0], st) : launch_attention_batch(blocks, n, st);
+    for (int i = 0, taken = 0; i < n; i += taken) {
+        ProfScope ps(M, 1, st);
+        CSD_TRY(launch_attention_batch(blocks + i, n - i, &taken, st));
+    }
+    return CSD_OK;
 }
 
 // q|k|v projections of `m` rows with the norm fused; one GEMM when the three matrices are
@@ -851,13 +854,12 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
     // next) in three-term form, written by the epilogue of the GEMM that produced the rows (for the
     // embedded rows: by the gather itself, when the first projection takes that form)
     bool x_ready = false, gather = false;      // gather: the first projection fetches the embedded rows itself
-    {
+    const LayerW& y0 = M->dec[0];
+    const bool fused_qkv = y0.wk == y0.wq + (size_t)di * d && y0.wv == y0.wk + (size_t)di * d;
+    gather = fused_qkv && linear_gathers(m, 3 * di, d) && !linear_uses_tensor_cores(m, 3 * di, d, false);
+    if (!gather) {
         ProfScope ps(M, 2, st);
-        const LayerW& y0 = M->dec[0];
-        const bool fused_qkv = y0.wk == y0.wq + (size_t)di * d && y0.wv == y0.wk + (size_t)di * d;
-        gather = fused_qkv && linear_gathers(m, 3 * di, d) && !linear_uses_tensor_cores(m, 3 * di, d, false);
-        if (gather) {
-        } else if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
+        if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
             PdlLaunch L(dim3((unsigned)split_ssq_entries(d), (unsigned)m), dim3(128), 0, st);
             CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_split_kernel, block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x,
                                         M->ssq_x, M->status));
@@ -931,8 +933,8 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
         const bool last = l + 1 == c.n_layers;
         const __nv_bfloat16* next_gain = last ? M->final_norm : M->dec[l + 1].norm1;
         const LayerW* nx = last ? nullptr : &M->dec[l + 1];
-        const bool fused_qkv = nx && nx->wk == nx->wq + (size_t)di * d && nx->wv == nx->wk + (size_t)di * d;
-        const int next_N = last ? V : (fused_qkv ? 3 * di : di);
+        const bool next_fused = nx && nx->wk == nx->wq + (size_t)di * d && nx->wv == nx->wk + (size_t)di * d;
+        const int next_N = last ? V : (next_fused ? 3 * di : di);
         CSD_TRY(feed_forward(M, y, M->x, m, st, x_ready, next_gain, next_N, false, &x_ready));
     }
     if (!logits_out_dev) {                    // cache append only: nobody reads this block's laws

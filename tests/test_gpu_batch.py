@@ -104,3 +104,20 @@ def test_more_sequences_than_one_launch_takes(b, orc, rows):
     assert b.csd_device_status() == 0
     for i, (o, s, n, r) in enumerate(zip(oms, seqs, kv, rows)):
         assert rel_l2(got[i].cpu().numpy(), o.review_forward(s[n:n + r], n)) <= LOGIT_REL_L2, i
+
+
+def test_profile_counts_launches(b, request):
+    """csd_model_profile brackets launches: of five sequences' attention two a layer, or one per sequence on the CUDA cores; none for
+    the embedded rows where the first projection gathers them (rows of a small model, automatic choice)."""
+    shape = llama_shape(2, 768, 12, 3072, 3001, 96)
+    blob = workloads.make_weights(shape, seed=5, device="cuda")
+    ms = [b.Model(shape, blob) for _ in range(5)]
+    blocks = [to_dev_i32([3 + i]) for i in range(5)]
+    ms[0].csd_model_profile(True)
+    b.csd_review_forward_batch(ms, blocks, [0] * 5)
+    p = ms[0].csd_model_profile_read()
+    path = request.node.callspec.id
+    assert p["attn_launches"] == 2 * (5 if path == "cuda-core" else 2)
+    assert p["other_launches"] == (0 if path == "automatic" else 1)
+    assert p["gemm_launches"] == 2 * 4 + 1
+    assert b.csd_device_status() == 0
