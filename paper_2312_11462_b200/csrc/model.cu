@@ -288,8 +288,14 @@ static WsLayout ws_layout(const csd_model_config& c) {
     L.ssq_x = put((size_t)linear_ssq_capacity((int)d) * R * 4);
     if (L.wide) {
         const size_t WR = (size_t)L.wide_rows;
-        L.wx = put(WR * d * 4); L.wqkv = put(WR * 3 * di * 4); L.wattn = put(WR * di * 4);
-        L.wxs_x = put(2 * WR * d * 2); L.wxs_attn = put(2 * WR * di * 2); L.wxs_act = put(2 * WR * ff * 2);
+        // Two pairs of buffers are never live together and share their memory: the q|k|v rows (from their projection to the attention)
+        // and the activations (from gate and up to the down projection); the projections' two-term input rows and, where the
+        // attention has no two-term output, its fp32 rows.  (7B shape, 1024 rows: 120 MB of wide buffers instead of 182.)
+        const size_t qkv = WR * 3 * di * 4, act = 2 * WR * ff * 2, rows = 2 * WR * d * 2, attn = WR * di * 4;
+        L.wx = put(WR * d * 4);
+        L.wqkv = L.wxs_act = put(qkv > act ? qkv : act);
+        L.wxs_x = L.wattn = put(rows > attn ? rows : attn);
+        L.wxs_attn = put(2 * WR * di * 2);
         const size_t kmax_w = d > di ? (d > ff ? d : ff) : (di > ff ? di : ff);
         size_t pieces = (size_t)wide_ssq_capacity((int)d);
         if ((size_t)wide_split_pieces((int)kmax_w) > pieces) pieces = (size_t)wide_split_pieces((int)kmax_w);

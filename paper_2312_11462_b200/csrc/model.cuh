@@ -40,6 +40,7 @@ struct csd_model {
     int wide_rows = 0;
     float *wx = nullptr, *wqkv = nullptr, *wattn = nullptr;                             // [wide_rows][d], [wide_rows][3 d_inner], ...
     __nv_bfloat16 *wxs_x = nullptr, *wxs_attn = nullptr, *wxs_act = nullptr;            // two-term rows [2][wide_rows][K]
+    //   (wxs_act lies where wqkv does, wattn where wxs_x does: see ws_layout)
     float* wssq = nullptr;              // pieces of the rows' sums of squares
     float* wpart = nullptr;             // partial sums of wide GEMMs
     // optional per-kernel-class timing (csd_model_profile): event pairs around every launch

@@ -46,6 +46,16 @@ def test_weight_bytes_match_blob_layout(b):
         assert b.lib.csd_model_workspace_bytes(C.byref(cfg)) > 0
 
 
+def test_wide_buffers_share_what_is_never_live_together(b):
+    """Every sequence of a batch has a workspace of its own: beside the caches, 1024 wide rows of the 7B shape take the residual
+    rows, the larger of q|k|v rows and activations, two sets of two-term rows, and the partial sums, 120 MB; 15 MB are the rest."""
+    s = workloads.with_max_seq(workloads.SHAPES["llama7b"], 1024)
+    rows = 1024 * s.d_model * 4
+    caches = 2 * s.n_layers * s.d_inner * s.max_seq * 2
+    total = b.lib.csd_model_workspace_bytes(C.byref(b.config_from_shape(s)))
+    assert total - caches < rows + 3 * rows + 2 * rows + 74 * 256 * 256 * 4 + 16e6
+
+
 def test_config_validation(b):
     s = workloads.SHAPES["tiny_target"]
     cfg = b.config_from_shape(s)

@@ -53,6 +53,45 @@ def test_prompt_lengths(b, llama_refs, n):
     assert np.abs(g - refs[n]).max() <= LOGIT_MAX_ABS
 
 
+@pytest.mark.parametrize("n", [33, 300, 1190])
+def test_prompts_whose_attention_leaves_fp32_rows(b, llama_refs, n):
+    """The CUDA-core attention (the comparison switch; head dimension 32): rotation in the append, its fp32 rows split afterwards."""
+    blob, toks, refs = llama_refs
+    m = b.Model(LLAMA, blob.cuda())
+    try:
+        b.csd_set_attention_path(1)
+        m.csd_prefill(to_dev_i32(toks[:n]), 0)
+        g = m.csd_review_forward(to_dev_i32(toks[n:n + 3]), n).cpu().numpy()
+    finally:
+        b.csd_set_attention_path(0)
+    assert b.csd_device_status() == 0
+    assert rel_l2(g, refs[n]) <= LOGIT_REL_L2, rel_l2(g, refs[n])
+    assert np.abs(g - refs[n]).max() <= LOGIT_MAX_ABS
+
+
+@pytest.mark.parametrize("shape,n", [(llama_shape(2, 1088, 34, 1416, 500, 200), 190), (t5_shape(2, 2, 1088, 34, 32, 1416, 500, 32, 150), 150)], ids=["llama", "t5"])
+def test_head_dimension_32(b, orc, shape, n):
+    blob = workloads.make_weights(shape, seed=44, device="cpu", std=0.01 if shape.arch == 1 else 0.02, gain_std=0.2)
+    om, gm = orc.Model(shape, orc.blob_to_u16(blob)), b.Model(shape, blob.cuda())
+    toks = workloads.make_prompt(shape.vocab, n + 3, seed=n)
+    pos = 0
+    if shape.arch == 1:
+        om.encoder_forward(toks[:n])
+        gm.csd_encoder_forward(to_dev_i32(toks[:n]))
+        om.review_forward(toks[:20], 0)                    # (and a prompt of the decoder, through cross-attention)
+        gm.csd_prefill(to_dev_i32(toks[:20]), 0)
+        pos = 20
+    else:
+        om.review_forward(toks[:n], 0)
+        gm.csd_prefill(to_dev_i32(toks[:n]), 0)
+        pos = n
+    blk = toks[n:n + 3]
+    g, r = gm.csd_review_forward(to_dev_i32(blk), pos).cpu().numpy(), om.review_forward(blk, pos)
+    assert b.csd_device_status() == 0
+    assert rel_l2(g, r) <= LOGIT_REL_L2, rel_l2(g, r)
+    assert np.abs(g - r).max() <= LOGIT_MAX_ABS
+
+
 @pytest.mark.parametrize("n", [18, 33, 129, 256, 300])
 def test_source_lengths(b, orc, n):
     blob = workloads.make_weights(T5, seed=42, device="cpu", std=0.01, gain_std=0.2)
