@@ -755,18 +755,18 @@ bool row_attention_supported(int Dh) { return (Dh == 64 || Dh == 128) && !g_attn
 
 // Splits per head: one 64-key tile per CTA while that keeps the splits of a head inside one portable cluster (8) and the
 // grid near two CTAs per SM (short caches are latency-bound, and more splits mean more tiles in flight at once); long
-// caches walk several tiles per CTA, two requests ahead.  At head dimension 128 one CTA fits beside a GEMM's on an SM, and
-// how many more than the SMs there are pays depends on the output projection behind it (8 layers of the 7B shape):
-//   up to 5 rows it leaves SMs free.  Caches of 5 to 8 tiles do with a CTA per SM, each walking two (5 rows, 300 keys: 774 us
-//   with 5 splits, 761 with 3); longer ones gain from all 8 (1000 keys: 800 us, 806 with 7).
-//   larger blocks fill every SM with it, and the last CTAs of clusters of 8 start only when it is through (9 rows, 1000 keys:
-//   882 us with 8, 845 with 7; 17 rows, 1500 keys: 1105, 1031), so 7 at most.
+// caches walk several tiles per CTA, two requests ahead.  At head dimension 128 (8 layers of the 7B shape, 32 heads, us):
+//   up to 5 rows, caches of 5 to 8 tiles do with about a CTA per SM, each walking two (300 keys: 704 with 3 splits, 709 with 5;
+//     400: 709 with 4, 714 with 7); on longer ones 7 and 8 splits are level (1000 keys 742 both, 1500 757 and 763).  At 6 to 8 rows
+//     the half is level too, larger blocks want the splits (9 rows, 300 keys: 772 with 3, 757 with 5).
+//   from 6 rows on, at most 7: 6 rows 1000 keys 752 with 7, 782 with 8; 8 rows 769 and 800, 1500 keys 785 and 824; 17 rows 1000 keys
+//     918 and 974, 1500 keys 949 and 1022.  (At 2048 keys 8 splits of whole tiles are 7 anyway.)
 int attn_splits(int total_keys, int H, int Dh, int gemm_rows) {
-    const int by_sm = (2 * 148 + H - 1) / H, tiles = (total_keys + TILE - 1) / TILE;
+    const int sms = tc_sm_count(), by_sm = (2 * sms + H - 1) / H, tiles = (total_keys + TILE - 1) / TILE;
     int n = by_sm < tiles ? by_sm : tiles;
     if (n > MAX_SPLITS) n = MAX_SPLITS;
     if (Dh == 128 && gemm_rows > 5 && n == MAX_SPLITS) n = MAX_SPLITS - 1;
-    if (Dh == 128 && gemm_rows <= 5 && n == tiles && tiles > 4 && H * tiles > 148) n = (tiles + 1) / 2;
+    if (Dh == 128 && gemm_rows <= 5 && n == tiles && tiles > 4 && H * tiles > sms) n = (tiles + 1) / 2;
     return n < 1 ? 1 : n;
 }
 
