@@ -524,8 +524,8 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 // u2 * S.  That CTA scans its threads' sums in thread order and picks the entry.  All sums have a
 // fixed order (lanes by xor-shuffle or prefix scan, warps and CTAs in index order).
 // ---------------------------------------------------------------------------------------------
-constexpr int RF_THREADS = 512, RF_PER = 16, RF_SLICE = RF_THREADS * RF_PER, RF_MAXC = 16;
-constexpr int RF_USE_MAXC = 8;   // larger clusters run (one per GPC at a time) but lose to the two-pass kernels: 199 us against 145 at V = 128256
+constexpr int RF_THREADS = 512, RF_PER = 16, RF_SLICE = RF_THREADS * RF_PER;
+constexpr int RF_MAXC = 8;   // larger clusters run (one per GPC at a time) but lose to the two-pass kernels: 199 us against 145 at V = 128256
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -1007,8 +1007,8 @@ static csd_status exp_table_ready() {
 
 // Whether clusters of `csize` CTAs of the fused resample kernel can run on the current device.
 static bool fused_resample_ok(int csize) {
-    static PerDevice known[RF_USE_MAXC + 1];
-    if (csize < 1 || csize > RF_USE_MAXC) return false;
+    static PerDevice known[RF_MAXC + 1];
+    if (csize < 1 || csize > RF_MAXC) return false;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return false; }
     return known[csize].get(dev, [csize] {

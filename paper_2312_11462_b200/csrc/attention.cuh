@@ -22,8 +22,8 @@ struct AttnArgs {
     int out_xs_ld = 0;
     int out_xs_rows = 0;                  // rows per term of the out_xs buffer (0: m) and this block's first row in it
     int out_xs_row0 = 0;
-    // Many rows (launch_row_attention): rotation of q by these tables at positions q_pos0 + r, and the output as two bf16
-    // terms, row = term * out_xs_rows + r, instead of fp32 rows
+    // Many rows (launch_row_attention): rotation of q by these tables at positions q_pos0 + r; the output goes here as two bf16
+    // terms, row = term * out_xs_rows + r (out is not written)
     const float* q_rope_cos = nullptr;
     const float* q_rope_sin = nullptr;
     __nv_bfloat16* out_xs2 = nullptr;

@@ -5,7 +5,7 @@
 // nothing in the walk is block-wide: a warp keeps its rows' q fragments, online softmax and output in registers,
 // and the accumulator fragments of q.K^T are the operand fragments of P.V.  q (rotated here, from its fp32
 // projection) and the softmax weights are bf16 pairs, two MMAs each.  The output leaves through shared
-// memory in whole 16-byte pieces, as fp32 rows or directly as the two-term rows of the projection that follows.
+// memory in whole 16-byte pieces, as the two-term rows of the projection that follows.
 //
 // What bounds it: the MMAs (256 per warp and tile) and the softmax's instructions between them, two CTAs an SM
 // taking turns.  1000 rows on an empty cache, 32 heads of 128: 72 us (230 TFLOP/s of two-term products), against 228 us
@@ -21,15 +21,15 @@ constexpr int RSTAGES = 3;
 
 struct RowsParams {
     const float* q; const float* rope_cos; const float* rope_sin; const float* bias;
-    float* out; __nv_bfloat16* xs; int* status;
-    int ldq, m, cap, n_keys, causal, bias_len, bias_zero, q_pos0, ldo, xs_ld, xs_rows;
+    __nv_bfloat16* xs; int* status;
+    int ldq, m, cap, n_keys, causal, bias_len, bias_zero, q_pos0, xs_ld, xs_rows;
     float scale;
 };
 
 template <int DH> struct RowsCfg {
     static constexpr size_t TILE_BYTES = (size_t)TILE * DH * 2;
     static constexpr size_t SMEM = 1024 + 2 * RSTAGES * TILE_BYTES + 2 * RSTAGES * 8;
-    static constexpr int OP = DH * 4 + 16;                 // bytes of an output row: fp32, or two terms; one 16-byte skew
+    static constexpr int OP = DH * 4 + 16;                 // bytes of an output row: two terms, one 16-byte skew
     static_assert(RROWS * OP <= 2 * RSTAGES * (int)TILE_BYTES, "the output rows fit the stages");
 };
 
@@ -229,14 +229,10 @@ row_attention_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 #pragma unroll
         for (int t = 0; t < 2 * KS; ++t) {
             const float x = o[t][2 * hr] * inv, y = o[t][2 * hr + 1] * inv;
-            if (p.xs) {
-                uint32_t w1, w2;
-                pack_pair(x, y, w1, w2);
-                *reinterpret_cast<uint32_t*>(dst + (8 * t + c0) * 2) = w1;
-                *reinterpret_cast<uint32_t*>(dst + DH * 2 + (8 * t + c0) * 2) = w2;
-            } else {
-                *reinterpret_cast<float2*>(dst + (8 * t + c0) * 4) = make_float2(x, y);
-            }
+            uint32_t w1, w2;
+            pack_pair(x, y, w1, w2);
+            *reinterpret_cast<uint32_t*>(dst + (8 * t + c0) * 2) = w1;
+            *reinterpret_cast<uint32_t*>(dst + DH * 2 + (8 * t + c0) * 2) = w2;
         }
     }
     __syncwarp();                          // a warp stores its own rows
@@ -245,12 +241,8 @@ row_attention_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         const int r = warp * 16 + i / PER, c = i % PER;
         if (r >= rows) break;
         const uint4 v = *reinterpret_cast<const uint4*>(orow + (size_t)r * C::OP + c * 16);
-        if (p.xs) {
-            const int term = c / (PER / 2), cc = c % (PER / 2);
-            *reinterpret_cast<uint4*>(p.xs + ((size_t)term * p.xs_rows + r0 + r) * p.xs_ld + h * DH + cc * 8) = v;
-        } else {
-            *reinterpret_cast<uint4*>(p.out + (size_t)(r0 + r) * p.ldo + h * DH + c * 4) = v;
-        }
+        const int term = c / (PER / 2), cc = c % (PER / 2);
+        *reinterpret_cast<uint4*>(p.xs + ((size_t)term * p.xs_rows + r0 + r) * p.xs_ld + h * DH + cc * 8) = v;
     }
 }
 
@@ -267,18 +259,18 @@ static csd_status launch_rows(const CUtensorMap& tk, const CUtensorMap& tv, cons
 }
 
 csd_status launch_row_attention(const AttnArgs& a, cudaStream_t st) {
-    if (!a.q || !a.Kc || !a.Vc || (!a.out && !a.out_xs2) || a.m < 1 || a.m > CSD_WIDE_ROWS || a.H < 1 || a.n_keys < 1 || (a.Dh != 64 && a.Dh != 128))
+    if (!a.q || !a.Kc || !a.Vc || !a.out_xs2 || a.m < 1 || a.m > CSD_WIDE_ROWS || a.H < 1 || a.n_keys < 1 || (a.Dh != 64 && a.Dh != 128))
         return CSD_ERR_INVALID_ARG;
     if ((a.ldq & 1) || (((uintptr_t)a.q) & 7) || (((uintptr_t)a.Kc) & 15) || (((uintptr_t)a.Vc) & 15)) return CSD_ERR_INVALID_ARG;
-    if (a.out_xs2 ? ((a.out_xs_ld & 7) || (((uintptr_t)a.out_xs2) & 15)) : ((a.ldo & 3) || (((uintptr_t)a.out) & 15))) return CSD_ERR_INVALID_ARG;
+    if ((a.out_xs_ld & 7) || (((uintptr_t)a.out_xs2) & 15)) return CSD_ERR_INVALID_ARG;
     if ((a.causal ? a.n_keys + a.m - 1 : a.n_keys) > a.cap) return CSD_ERR_CAPACITY;
     CUtensorMap tk, tv;
     if (!tensor_map_2d(a.Kc, a.H * a.cap, a.Dh, TILE, &tk) || !tensor_map_2d(a.Vc, a.H * a.cap, a.Dh, TILE, &tv)) return CSD_ERR_UNSUPPORTED;
     RowsParams rp;
-    rp.q = a.q; rp.rope_cos = a.q_rope_cos; rp.rope_sin = a.q_rope_sin; rp.bias = a.bias; rp.out = a.out; rp.xs = a.out_xs2;
+    rp.q = a.q; rp.rope_cos = a.q_rope_cos; rp.rope_sin = a.q_rope_sin; rp.bias = a.bias; rp.xs = a.out_xs2;
     rp.status = status_word_device();
     rp.ldq = a.ldq; rp.m = a.m; rp.cap = a.cap; rp.n_keys = a.n_keys; rp.causal = a.causal; rp.bias_len = a.bias_len;
-    rp.bias_zero = a.bias_zero; rp.q_pos0 = a.q_pos0; rp.ldo = a.ldo; rp.xs_ld = a.out_xs_ld; rp.xs_rows = a.out_xs_rows;
+    rp.bias_zero = a.bias_zero; rp.q_pos0 = a.q_pos0; rp.xs_ld = a.out_xs_ld; rp.xs_rows = a.out_xs_rows;
     rp.scale = a.scale;
     return a.Dh == 64 ? launch_rows<64>(tk, tv, rp, a.H, st) : launch_rows<128>(tk, tv, rp, a.H, st);
 }

@@ -79,6 +79,12 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// activations of the gated feed-forwards
+__device__ __forceinline__ float gelu_tanh(float x) {
+    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
+}
+__device__ __forceinline__ float silu(float x) { return x / (1.f + expf(-x)); }
+
 // two bf16 packed in a 32-bit word -> two fp32 (bf16 is the top half of an fp32)
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }

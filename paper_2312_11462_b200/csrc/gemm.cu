@@ -90,11 +90,6 @@ struct GemmParams {
     float eps;
 };
 
-__device__ __forceinline__ float gelu_tanh_f(float x) {
-    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
-}
-__device__ __forceinline__ float silu_f(float x) { return x / (1.f + expf(-x)); }
-
 __device__ __forceinline__ float dot8(const uint4& w, const float4& a, const float4& b, float acc) {
     acc = fmaf(bf16lo(w.x), a.x, acc);
     acc = fmaf(bf16hi(w.x), a.y, acc);
@@ -283,7 +278,7 @@ skinny_gemm_kernel(const GemmParams p) {
             float val = red[v * 33 + 32] * scale;
             if (DUAL) {
                 const float up = red[(R * M + v) * 33 + 32] * scale;
-                val = (p.epilogue == EPI_GEGLU ? gelu_tanh_f(val) : silu_f(val)) * up;
+                val = (p.epilogue == EPI_GEGLU ? gelu_tanh(val) : silu(val)) * up;
             }
             float* y = p.Y + (size_t)r * p.ldy + n;
             if (p.epilogue == EPI_ADD) *y += val; else *y = val;

@@ -35,11 +35,6 @@ bool row_supported(int m, int N, int K, bool dual) {
     return steps <= (dual ? 3 : RW_MAX_STEPS) && row_smem(row_m(m), steps) <= RW_SMEM_MAX;
 }
 
-__device__ __forceinline__ float rw_gelu(float x) {
-    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
-}
-__device__ __forceinline__ float rw_silu(float x) { return x / (1.f + expf(-x)); }
-
 // sums over the lanes of V <= 32 values each; lane v returns the sum of value v (garbage beyond V)
 template <int V>
 __device__ __forceinline__ float lane_sums(float (&v)[V], int lane) {
@@ -227,7 +222,7 @@ row_gemm_kernel(const RowParams p) {
                     scale = 1.f / sqrtf(sq / (float)p.K + p.eps);
                 }
                 float val = sum[0] * scale;
-                if (DUAL) val = (p.epilogue == EPI_GEGLU ? rw_gelu(val) : rw_silu(val)) * (sum[NT - 1] * scale);
+                if (DUAL) val = (p.epilogue == EPI_GEGLU ? gelu_tanh(val) : silu(val)) * (sum[NT - 1] * scale);
                 p.Y[(size_t)r * p.ldy + n] = val + old[c];
             }
         }

@@ -108,11 +108,6 @@ struct RsParams {
     float eps;
 };
 
-__device__ __forceinline__ float rs_gelu(float x) {
-    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
-}
-__device__ __forceinline__ float rs_silu(float x) { return x / (1.f + expf(-x)); }
-
 template <int M, bool DUAL>
 __global__ void __launch_bounds__(TC_THREADS, 2)
 skinny_gemm_rs_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
@@ -306,7 +301,7 @@ skinny_gemm_rs_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 float val = sums[0][r] * scale;
                 if (DUAL) {
                     const float up = sums[NT - 1][r] * scale;
-                    val = (p.epilogue == EPI_GEGLU ? rs_gelu(val) : rs_silu(val)) * up;
+                    val = (p.epilogue == EPI_GEGLU ? gelu_tanh(val) : silu(val)) * up;
                 }
                 if (mine) {
                     if (p.epilogue == EPI_ADD) val += yold[r];

@@ -196,11 +196,6 @@ struct __align__(8) TcCtrl {
     float scale[32];
 };
 
-__device__ __forceinline__ float tc_gelu(float x) {
-    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
-}
-__device__ __forceinline__ float tc_silu(float x) { return x / (1.f + expf(-x)); }
-
 // ---- distributed shared memory (cluster split) ---------------------------------------------------
 __device__ __forceinline__ void remote_store(uint32_t cluster_addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
@@ -478,7 +473,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                 const int mid = tile / 2 * 3 + 1;
                 slot = tile & 1;
                 c_lo = mid - 1; c_hi = mid;
-                if (slot) { c_lo = cta == mid + 1 ? cta : mid + 1; c_hi = mid; }
+                if (slot) { c_lo = mid + 1; c_hi = mid; }
             } else if (part_of_tile) {
                 c_lo = cta_of_unit((unsigned)tile * p.nkb, units, ctas);
                 c_hi = cta_of_unit((unsigned)(tile + 1) * p.nkb - 1, units, ctas);
@@ -621,7 +616,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                     float val = sums[0][r] * scale;
                     if (DUAL) {
                         const float up = sums[NT - 1][r] * scale;
-                        val = (p.epilogue == EPI_GEGLU ? tc_gelu(val) : tc_silu(val)) * up;
+                        val = (p.epilogue == EPI_GEGLU ? gelu_tanh(val) : silu(val)) * up;
                     }
                     if (n < p.N) {
                         if (p.epilogue == EPI_ADD) val += yold[r];

@@ -146,11 +146,6 @@ struct WgParams {
     float eps;
 };
 
-__device__ __forceinline__ float wg_gelu(float x) {
-    return 0.5f * x * (1.f + tanhf(0.7978845608028654f * (x + 0.044715f * x * x * x)));
-}
-__device__ __forceinline__ float wg_silu(float x) { return x / (1.f + expf(-x)); }
-
 // x = hi + lo with bf16 terms (16 mantissa bits)
 __device__ __forceinline__ void split2f(float x, uint16_t& hi, uint16_t& lo) {
     hi = float_to_bf16_bits(x);
@@ -529,7 +524,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         const float u[4] = {u4.x, u4.y, u4.z, u4.w};
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            x[k][j] = (p.epilogue == EPI_GEGLU ? wg_gelu(x[k][j]) : wg_silu(x[k][j])) * (u[j] * sc);
+                            x[k][j] = (p.epilogue == EPI_GEGLU ? gelu_tanh(x[k][j]) : silu(x[k][j])) * (u[j] * sc);
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
