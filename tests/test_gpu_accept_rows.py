@@ -23,17 +23,17 @@ def b():
 @pytest.mark.parametrize("rows,k", [(1, 0), (1, 1), (3, 4), (9, 2)])
 def test_slices(b, orc, V, rows, k):
     t, d, tok = workloads.accept_case(rows, k, V, 0.7, seed=V + rows, device="cuda")
-    compare(b, orc, t, d, tok, 1.0, max_flag_frac=0.34)         # (a single near tie among few rows)
-    compare(b, orc, t, None, tok, 0.8, max_flag_frac=0.34)
+    compare(b, orc, t, d, tok, 1.0, max_flag_frac=0.0)
+    compare(b, orc, t, None, tok, 0.8, max_flag_frac=0.0)
     compare(b, orc, t, d, tok, 0.0)
 
 
 def test_most_drafts_and_one_wave(b, orc):
     t, d, tok = workloads.accept_case(2, 64, 5000, 0.2, seed=4, device="cuda")
-    compare(b, orc, t, d, tok, 1.0, max_flag_frac=0.5)
+    compare(b, orc, t, d, tok, 1.0, max_flag_frac=0.0)
     for rows in (15, 16, 17, 18, 19, 37, 74):                   # up to and past what is resident at once
         t, d, tok = workloads.accept_case(rows, 3, 32000, 0.5, seed=rows, device="cuda")
-        compare(b, orc, t, d, tok, 1.0, max_flag_frac=0.1)
+        compare(b, orc, t, d, tok, 1.0, max_flag_frac=1.0 / rows)       # (16 rows: one within 1e-5 of its threshold)
 
 
 def test_empty_residual_and_masked_entries(b, orc):
@@ -47,4 +47,4 @@ def test_empty_residual_and_masked_entries(b, orc):
     # equal laws whose drafts come from elsewhere are accepted; a stretch of masked entries carries no mass
     t3 = t.clone()
     t3[:, :, 100:8990] = float("-inf")
-    compare(b, orc, t3, d, tok, 1.0, max_flag_frac=0.25)
+    compare(b, orc, t3, d, tok, 1.0, max_flag_frac=0.0)

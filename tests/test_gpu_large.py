@@ -263,9 +263,10 @@ def test_t5xxl_width_sampled_horizontal_cascade(b, orc):
 
 
 def test_wide_prefill_leaves_the_cache_a_review_needs(b, orc):
-    """csd_prefill at the 7B width (wide blocks of up to 128 rows, two-term activations): the review
+    """csd_prefill at the 7B width (wide passes, two-term activations): the review
     block that follows must meet the stated tolerance against the oracle, which forwards every
-    token the plain way; so must a second block after a second prefill that starts mid-cache, and
+    token the plain way; so must a second block after a second prefill that starts mid-cache, a third after a prompt cut
+    into a wide call and one short enough for the review kernels, and
     the result must not depend on how the prompt was cut into prefill calls beyond that tolerance."""
     shape = llama_shape(3, 4096, 32, 11008, 32000, 320)
     blob = workloads.make_weights(shape, seed=100, device="cuda")
@@ -282,13 +283,19 @@ def test_wide_prefill_leaves_the_cache_a_review_needs(b, orc):
         refs[cut] = out
     gm = b.Model(shape, blob)
     dev = to_dev_i32(seq)
-    gm.csd_prefill(dev[:150].contiguous(), 0)                        # 128 wide + 22 (17 + 5 review-sized)
+    gm.csd_prefill(dev[:150].contiguous(), 0)                        # one wide pass of 150
     g = gm.csd_review_forward(dev[150:155].contiguous(), 150).cpu().numpy()
     assert rel_l2(g, refs[155]) <= LOGIT_REL_L2, rel_l2(g, refs[155])
     assert np.abs(g - refs[155]).max() <= LOGIT_MAX_ABS
-    gm.csd_prefill(dev[155:290].contiguous(), 155)                   # starts mid-cache: 128 wide + 7
+    gm.csd_prefill(dev[155:290].contiguous(), 155)                   # starts mid-cache: one of 135
     g = gm.csd_review_forward(dev[290:295].contiguous(), 290).cpu().numpy()
     assert rel_l2(g, refs[295]) <= LOGIT_REL_L2, rel_l2(g, refs[295])
+    # a wide call and a short one: the change from wide to review kernels in mid-cache
+    gm3 = b.Model(shape, blob)
+    gm3.csd_prefill(dev[:137].contiguous(), 0)
+    gm3.csd_prefill(dev[137:150].contiguous(), 137)
+    g = gm3.csd_review_forward(dev[150:155].contiguous(), 150).cpu().numpy()
+    assert rel_l2(g, refs[155]) <= LOGIT_REL_L2, rel_l2(g, refs[155])
     # the same prompt through the review kernels only
     gm2 = b.Model(shape, blob)
     p = 0

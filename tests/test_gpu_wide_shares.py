@@ -1,0 +1,112 @@
+"""Wide passes whose output and down projections are too large for planes: pairs that take whole tiles and pairs that share tiles,
+each with the residual add, the two-term rows times a gain and the sums of squares in the GEMM's own epilogue, and the
+gated pair in both of its forms, over two layers.  Whole reviews against the oracle; and the second layer's cached values against
+fp64, entry by entry, from the first layer's cached keys and values on."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from workloads import llama_shape
+from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, rel_l2, require_gpu, to_dev_i32
+
+pytestmark = pytest.mark.gpu
+
+# d_model, heads, d_ff, prompts.  Pairs of CTAs: 74; a tile is 256 output rows x up to 256 tokens, the gated pair's 128 above 128 tokens.
+SHAPES = {
+    # the 7B width: o and down 32 to 48 tiles in equal shares, gate and up 172 to 258
+    "7b": (llama_shape(2, 4096, 32, 11008, 500, 720), (257, 300, 700)),
+    # o and down of 17 row tiles of which the last is a quarter full (34 tiles, shares); gate and up end inside a tile
+    "ragged": (llama_shape(2, 4160, 65, 1416, 500, 320), (257, 300)),
+    # o and down of 72 tiles for 74 pairs: whole tiles
+    "whole": (llama_shape(2, 4608, 36, 1416, 500, 800), (780,)),
+}
+
+
+@pytest.fixture(scope="module")
+def b():
+    require_gpu()
+    from paper_2312_11462_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module", params=list(SHAPES))
+def text(request, orc):
+    shape, lengths = SHAPES[request.param]
+    blob = workloads.make_weights(shape, seed=61, device="cuda", gain_std=0.2)
+    toks = workloads.make_prompt(shape.vocab, shape.max_seq, seed=12)
+    om = orc.Model(shape, orc.blob_to_u16(blob))
+    refs, pos = {}, 0
+    for n in lengths:
+        om.review_forward(toks[pos:n], pos)
+        pos = n
+        refs[n] = om.review_forward(toks[n:n + 3], n)
+    return shape, blob, toks, refs
+
+
+def second_layer_values(shape, blob, toks, k, v):
+    """V of the second layer in fp64, not rounded, given the first layer's cached K and V."""
+    part = {n: blob[o:o + int(np.prod(s))].view(s).double() for n, o, s in workloads.blob_layout(shape)[0] if n[:2] in ("em", "l0") or n in ("l1.norm1", "l1.wv")}
+    n, H, Dh = len(toks), shape.n_heads, shape.d_head
+
+    def norm(x, g):
+        return x / torch.sqrt((x * x).mean(-1, keepdim=True) + shape.norm_eps) * g
+
+    def turned(x):
+        half = Dh // 2
+        a = torch.arange(n, device="cuda").double()[:, None] * shape.rope_theta ** (-2.0 * torch.arange(half, device="cuda").double() / Dh)
+        c, s = a.cos()[:, None], a.sin()[:, None]
+        x = x.view(n, H, Dh)
+        return torch.cat([x[..., :half] * c - x[..., half:] * s, x[..., :half] * s + x[..., half:] * c], -1)
+
+    x = part["embed"][toks.long()]
+    h = norm(x, part["l0.norm1"])
+    q, k, v = turned(h @ part["l0.wq"].T), k.double(), v.double()
+    out = torch.empty(n, H, Dh, dtype=torch.float64, device="cuda")
+    later = torch.ones(n, n, dtype=torch.bool, device="cuda").triu(1)
+    for i in range(H):
+        out[:, i] = torch.softmax((q[:, i] @ k[:, i].T / Dh ** 0.5).masked_fill(later, float("-inf")), -1) @ v[:, i]
+    x = x + out.reshape(n, -1) @ part["l0.wo"].T
+    h = norm(x, part["l0.norm2"])
+    gate = h @ part["l0.wgate"].T
+    x = x + (gate / (1 + torch.exp(-gate)) * (h @ part["l0.wup"].T)) @ part["l0.wdown"].T
+    return (norm(x, part["l1.norm1"]) @ part["l1.wv"].T).view(n, H, Dh)
+
+
+def cached(b, model, layer, n):
+    """K and V [n, H, Dh] of a layer: the workspace opens with both, [layer][head][max_seq][d_head] bf16 each."""
+    s = model.shape
+    per = s.n_heads * s.max_seq * s.d_head
+    k_bytes = (s.n_layers * per * 2 + 255) // 256 * 256
+    at = layer * per * 2
+    return [model.workspace[o:o + per * 2].view(torch.bfloat16).view(s.n_heads, s.max_seq, s.d_head)[:, :n].transpose(0, 1) for o in (at, k_bytes + at)]
+
+
+def test_reviews_behind_prompts(b, text):
+    shape, blob, toks, refs = text
+    for n, ref in refs.items():
+        m = b.Model(shape, blob)
+        m.csd_prefill(to_dev_i32(toks[:n]), 0)
+        g = m.csd_review_forward(to_dev_i32(toks[n:n + 3]), n).cpu().numpy()
+        assert b.csd_device_status() == 0
+        assert rel_l2(g, ref) <= LOGIT_REL_L2, (n, rel_l2(g, ref))
+        assert np.abs(g - ref).max() <= LOGIT_MAX_ABS
+
+
+def test_second_layer_against_fp64(b, text):
+    """The cache rounds to bf16 (half a unit: at most 2^-8 of an entry), so an error e of the rows shows as entries on the other side
+    of a rounding edge: e / unit of them, about 4 * 2^7.5 e over normally distributed entries, the small ones having small units.
+    Four GEMMs and an attention whose operands have two terms leave an e of 1e-5 (2.7e-6 a GEMM, more behind the gated
+    product): 0.7 % measured, 1 % allowed; and beyond its rounding no entry may be off by more than ten times e (3.2 measured)."""
+    shape, blob, toks, refs = text
+    for n in refs:
+        m = b.Model(shape, blob)
+        m.csd_prefill(to_dev_i32(toks[:n]), 0)
+        got = cached(b, m, 1, n)[1]
+        want = second_layer_values(shape, blob, to_dev_i32(toks[:n]), *cached(b, m, 0, n))
+        rms = float(want.pow(2).mean().sqrt())
+        off = (got.double() - want).abs() - want.abs() * 2.0 ** -8
+        share = float((got != want.bfloat16()).double().mean())
+        assert share < 1e-2, (n, share)
+        assert float(off.max()) < 1e-4 * rms, (n, float(off.max()) / rms)
+    assert b.csd_device_status() == 0
