@@ -341,7 +341,7 @@ def run_review_only(args):
     tb = workloads.make_weights(ts, seed=100, device="cuda")
     prompt = torch.from_numpy(workloads.make_prompt(ts.vocab, S + MAX_BLOCK + 1, seed=1000)).cuda()
     target = b.Model(ts, tb)
-    target.csd_prefill(prompt[:S].contiguous(), 0)              # wide passes of 128 rows
+    target.csd_prefill(prompt[:S].contiguous(), 0)              # in wide passes
     blk = prompt[S:S + MAX_BLOCK + 1].contiguous()
     logits = torch.empty(MAX_BLOCK + 1, ts.vocab, device="cuda")
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)

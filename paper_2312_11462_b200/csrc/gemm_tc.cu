@@ -9,10 +9,13 @@
 // by the epilogue of the kernel that produced the rows, or by split_rows_kernel) and its 64-wide
 // K block rides in the same stage as the weight tile; the epilogue adds the three partial results.
 //
-// Work is cut into (tile, K block) units and every CTA (one per SM) owns an equal contiguous share
-// of them, so all SMs stream the same number of bytes; a tile that straddles CTAs is finished by
-// the first of them (for which it comes last), adding the parts the others parked in CTA order
-// (deterministic).  Roles inside a CTA (192 or 320 threads): warp 0 lane 0 issues TMA, warp 1
+// Work is cut into (tile, K block) units, tile-major, and dealt out in one of three ways (tc_plan):
+//   shares    every CTA (one per SM) owns an equal contiguous share, so all SMs stream the same number of bytes;
+//   groups    up to 10 rows, where three CTAs per two tiles come to 3/4 of the SMs or more: 144 CTAs for the 96 tiles of the 7B
+//             shape's q|k|v, 129 for the 86 of gate and up; the middle CTA of a group takes a little less than the others;
+//   clusters  a single matrix of few tiles, up to 8 rows: four CTAs share a tile's K range and add up on chip.
+// A tile that straddles CTAs is finished by the first of them (for which it comes last), adding the parts the others parked in
+// CTA order (deterministic).  Roles inside a CTA (192 or 320 threads): warp 0 lane 0 issues TMA, warp 1
 // lane 0 issues MMA, the others read the accumulators from tensor memory (a quadrant each) and run the
 // epilogue: rms-norm factor, residual add or gated activation, and optionally the three-term
 // split and sum-of-squares pieces of the result for the next GEMM.  The first ring-full of weight
@@ -68,7 +71,7 @@ int tc_sm_count() {
     return n;
 }
 
-// One CTA per SM; the (tile, K block) units are dealt out in equal contiguous shares.
+// How a launch is divided: clusters, groups of three CTAs, or equal shares (see the top of the file).
 static TcPlan tc_plan(int m, int N, int K, bool dual) {
     TcPlan p{};
     p.npad = npad_for(m);

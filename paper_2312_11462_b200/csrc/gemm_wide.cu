@@ -10,17 +10,17 @@
 //
 // What bounds it: the bytes an SM takes in (about 70 GB/s) and the tensor pipe, nearly level.  A full tile takes
 // 48 KB per 1024 tensor clocks and SM; at 1024 rows, N 12288, K 4096 the copies alone need 114 us, the MMAs alone
-// 89 us, the kernel 157 us (1.29 PFLOP/s of two-term products, 77 % of the measured one-term cuBLAS rate; the
-// earlier kernel, one CTA per 84 weight rows and 128 tokens, took in 32 KB of token terms for every 11 KB of
-// weights: 8 x 46 us).  At 128 rows both kernels need 40 us; below, the weight stream bounds.
+// 89 us, the kernel 157 us (1.29 PFLOP/s of two-term products, 77 % of the measured one-term cuBLAS rate).  One CTA per 84 weight
+// rows and 128 tokens instead of pairs takes in 32 KB of token terms for every 11 KB of weights: 8 x 46 us.  At 128 rows both
+// divisions need 40 us; below, the weight stream bounds.
 //
 // fp32 accumulation.  The tensor core loses a little with every add of a long chain, so after WG_DRAIN
 // K blocks (64 adds) the accumulator set is added into fp32 registers of the epilogue warps while
-// the MMAs continue on the other set: shorter chains than in the earlier kernel (256 to 700
-// adds), and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to 11008: 2.7e-6 (earlier
-// 2.5e-6 to 5.0e-6, growing with the block), of which the two-term form itself leaves 2.45e-6.  Tiles of up to 32 tokens, where the
-// earlier kernel left 2.45e-6 to 2.65e-6, sum the low terms' products in columns of their own: 2.5e-6.  (8 layers of the 7B shape, 20
-// tokens: 1001 us, 965 so, the kernel of such tiles being short as well; sets of 4 K blocks, which leave the same, cost 2 to 7 % a GEMM.)
+// the MMAs continue on the other set, and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to
+// 11008 (csd_linear, 18 to 128 rows): 2.7e-6, of which the two-term form itself leaves 2.45e-6.  (Chains of 256 to 700 adds left
+// 2.45e-6 at 18 rows to 5.0e-6 at 128.)  Tiles of up to 32 tokens sum the low terms' products in columns of their own: 2.5e-6, and
+// being short the kernel of such tiles is the faster one as well (8 layers of the 7B shape, 20 tokens: 1001 us together, 965 so).  Sets
+// of 4 K blocks, which leave 2.5e-6 at every size, cost 2 to 7 % a GEMM.
 //
 // Roles inside a CTA (384 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 of the pair's first CTA
 // issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
