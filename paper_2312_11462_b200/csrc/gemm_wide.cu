@@ -158,6 +158,10 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* t
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y) : "memory");
 }
+__device__ __forceinline__ void tma_load_2d_pair_once(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y, uint64_t pol) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+                 ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
+}
 __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
     asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }"
                  ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
@@ -242,47 +246,51 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(WG_REGS_CTL));
+        struct Cursor { int kb, row, tok; };                  // K block, row tile, token tile
+        auto step = [&](Cursor& c) {
+            if (++c.kb == p.nkb) { c.kb = 0; if (++c.tok == p.ntok) { c.tok = 0; ++c.row; } }
+        };
+        const int tile0 = (int)(u0 / p.nkb);
+        Cursor cur{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
         if (warp == 0 && lane == 0) {
-            // ---- TMA producer of this CTA; all copies of the pair complete on the first CTA's barriers
-            struct Cursor { int kb, row, tok; };              // K block, row tile, token tile
-            auto step = [&](Cursor& c) {
-                if (++c.kb == p.nkb) { c.kb = 0; if (++c.tok == p.ntok) { c.tok = 0; ++c.row; } }
-            };
-            const int tile0 = (int)(u0 / p.nkb);
-            Cursor cw{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
-            Cursor cx = cw;
-            auto load_w = [&](int s) {
-                unsigned char* dst = ring + (size_t)s * stage_bytes;
-                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
-                if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
-                const int row = cw.row * OUT_ROWS + rank * (OUT_ROWS / 2);
-                tma_load_2d_pair(dst, &tmW, bar, cw.kb * KB, row);
-                if (DUAL) tma_load_2d_pair(dst + STAGE_BYTES, &tmW2, bar, cw.kb * KB, row);
-                if (MIXED) tma_load_2d_pair(dst + STAGE_BYTES / 2, &tmW2, bar, cw.kb * KB, row);
-                step(cw);
-            };
-            auto load_x = [&](int s) {
-                unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
-                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
-                const int r = cx.tok * nt + rank * htok;
-                tma_load_2d_pair(dst, &tmX, bar, cx.kb * KB, r);
-                tma_load_2d_pair(dst + xterm, &tmX, bar, cx.kb * KB, p.mpad + r);
-                step(cx);
-            };
-            const int pre = items < p.stages ? items : p.stages;
-#pragma unroll 1
-            for (int i = 0; i < pre; ++i) load_w(i);
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-#pragma unroll 1
-            for (int i = 0; i < pre; ++i) load_x(i);
+            // ---- TMA producer of this CTA's weights; all copies of the pair complete on the first CTA's barriers
+            const uint64_t once = policy_evict_first();
+            const bool reread = p.ntok > 1;                   // other token tiles take the same weights from L2
             int s = 0;
             uint32_t ph = 0;
 #pragma unroll 1
-            for (int i = pre; i < items && !*abort_flag; ++i) {
-                if (!mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
-                load_w(s);
-                load_x(s);
-                if (++s == p.stages) { s = 0; ph ^= 1u; }
+            for (int i = 0; i < items && !*abort_flag; ++i) {
+                if (i >= p.stages && !mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
+                unsigned char* dst = ring + (size_t)s * stage_bytes;
+                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+                if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
+                const int row = cur.row * OUT_ROWS + rank * (OUT_ROWS / 2);
+                auto load = [&](void* to, const CUtensorMap* tm) {
+                    if (reread) tma_load_2d_pair(to, tm, bar, cur.kb * KB, row);
+                    else tma_load_2d_pair_once(to, tm, bar, cur.kb * KB, row, once);
+                };
+                load(dst, &tmW);
+                if (DUAL) load(dst + STAGE_BYTES, &tmW2);
+                if (MIXED) load(dst + STAGE_BYTES / 2, &tmW2);
+                step(cur);
+                if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
+            }
+        } else if (warp == 2 && lane == 0) {
+            // ---- TMA producer of this CTA's half of the row terms, a warp of its own: three copies a stage from one thread
+            //      (about 100 ns each, with the wait before them) set the pace of tiles of up to 128 tokens
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            int s = 0;
+            uint32_t ph = 0;
+#pragma unroll 1
+            for (int i = 0; i < items && !*abort_flag; ++i) {
+                if (i >= p.stages && !mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
+                unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
+                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+                const int r = cur.tok * nt + rank * htok;
+                tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, r);
+                tma_load_2d_pair(dst + xterm, &tmX, bar, cur.kb * KB, p.mpad + r);
+                step(cur);
+                if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
             }
         } else if (warp == 1 && rank == 0 && lane == 0) {
             // ---- MMA issuer of the pair
