@@ -4,9 +4,9 @@
 //
 // Each fp32 value of X enters as TWO bf16 terms x = hi + lo (16 mantissa bits, relative error
 // 2^-17), laid out as [2][mpad][K].  A tile is 256 weight rows x nt <= 256 tokens (the gated pair:
-// 128 rows of each matrix, or up to 128 tokens 256 rows of each) and belongs to a PAIR of CTAs on
-// neighbouring SMs: tcgen05.mma with cta_group::2, 128 weight rows and half of the tokens staged by
-// each CTA, both terms accumulated into the same fp32 columns.
+// 128 rows of each matrix, or up to 64 tokens 256 rows of each) and belongs to a PAIR of CTAs on
+// neighbouring SMs: tcgen05.mma with cta_group::2, 128 weight rows and half of the tokens' terms staged by
+// each CTA; both terms are accumulated into the same fp32 columns, up to 128 tokens side by side.
 //
 // What bounds it: the bytes an SM takes in (about 70 GB/s) and the tensor pipe, nearly level.  A full tile takes
 // 48 KB per 1024 tensor clocks and SM; at 1024 rows, N 12288, K 4096 the copies alone need 114 us, the MMAs alone
@@ -35,9 +35,9 @@ namespace csd {
 constexpr size_t WG_SMEM_MAX = 227 * 1024;
 constexpr int WG_MAX_STAGES = 10;
 constexpr int WG_THREADS = 384;              // one control warpgroup, two epilogue warpgroups
-// Registers a thread: 168 at launch (65536 / 384); 128 x 56 + 256 x 224 = 384 x 168.  Without the split the
+// Registers a thread: 168 at launch (65536 / 384); 128 x 72 + 256 x 216 = 384 x 168.  Without the split the
 // accumulators spill.
-constexpr int WG_REGS_CTL = 56, WG_REGS_EPI = 224;
+constexpr int WG_REGS_CTL = 72, WG_REGS_EPI = 216;
 constexpr int WG_ROWS = 256;                 // weight rows of a pair's tile
 constexpr int WG_DRAIN = 8;                  // K blocks per accumulator set before it is added into registers
 constexpr int WG_SET = 256;                  // tensor-memory columns of a set
@@ -68,6 +68,7 @@ static_assert(8 * 16 * 32 + 4 * WG_SET <= 2 * 8 * 16 * 32, "sums of squares fit 
 // of a full tile (0.55 us each).
 struct WgPlan {
     int mpad, nt, ntok, tiles, nkb, pairs, pk, gran, stages;
+    bool merged;                             // both terms of a tile's tokens in one MMA (up to 128 tokens)
     bool mixed;                              // gated pair: a tile's weight rows are half gate, half up
     size_t stage, smem;
 };
@@ -77,12 +78,13 @@ int wide_split_pieces(int K) { return (K + 1023) / 1024; }
 // planes: whether the result may go through planes (their reduction stores 16 bytes at a time)
 static WgPlan wg_plan(int m, int N, int K, bool dual, bool planes = true) {
     WgPlan p{};
-    const int P = tc_sm_count() / 2, most = dual && m <= 128 ? 128 : 256;
-    p.mixed = dual && m > 128;
+    const int P = tc_sm_count() / 2, most = 256;
+    p.mixed = dual && m > 64;
     const int rows = p.mixed ? WG_ROWS / 2 : WG_ROWS;
     p.mpad = (m + 15) & ~15;
     p.ntok = (m + most - 1) / most;
     p.nt = ((m + p.ntok - 1) / p.ntok + 31) & ~31;
+    p.merged = p.nt <= 128;
     p.tiles = ((N + rows - 1) / rows) * p.ntok;
     p.nkb = (K + KB - 1) / KB;
     p.stage = (size_t)STAGE_BYTES * (dual && !p.mixed ? 2 : 1) + (size_t)p.nt * 128;
@@ -158,7 +160,7 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* t
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y) : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_pair_once(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y, uint64_t pol) {
+__device__ __forceinline__ void tma_load_2d_pair_keep(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y, uint64_t pol) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
 }
@@ -182,13 +184,18 @@ __device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigne
     return unit_begin(c, units / gran, pairs) * gran;
 }
 
-// MODE 0: one matrix; 1: a gated pair, both matrices' 256 rows in a stage (up to 128 tokens); 2: a gated pair, the CTA's
-// 128 rows are 64 of the gate and the same 64 of the up matrix, so that the MMAs are 256 tokens wide.  (At N = 128 an MMA reads
-// its 128 weight rows from shared memory for half the work, and those reads, not the tensor pipe, set the pace: gate and up of
-// the 7B shape at 1000 tokens 323 us in mode 1, 277 in mode 2; of the T5-xxl shape at 256 tokens 92 and 82.
-// Up to 128 tokens mode 1 moves fewer bytes: its tile is 256 outputs wide.)
-// LOW: tiles of up to 32 tokens, the low terms' products in columns of their own (modes 0 and 1)
-template <int MODE, bool LOW>
+// MODE 0: one matrix; 1: a gated pair, both matrices' 256 rows in a stage (up to 64 tokens); 2: a gated pair, the CTA's
+// 128 rows are 64 of the gate and the same 64 of the up matrix, so that the MMAs are up to 256 columns wide.  (An MMA reads
+// its 128 weight rows from shared memory whatever its width, and those reads, not the tensor pipe, set the pace of narrow ones:
+// gate and up of the 7B shape at 1000 tokens 323 us in mode 1, 277 in mode 2.)
+// MERGED (tiles of up to 128 tokens): one MMA multiplies both terms of the tile's tokens, 2 nt columns wide, the high terms'
+// sums in the first nt columns and the low terms' in the others; one CTA of the pair stages the high terms of all tokens, the
+// other the low ones.  An MMA of 256 x 64 takes little less time than one of 256 x 128, so two of them per term and K step set
+// the pace of small tiles (0.46 to 0.49 us a K block of a single matrix, whatever the tokens; weights alone need 0.37).  A layer
+// of the 7B shape at 20 / 64 / 128 tokens 134 -> 120, 151 -> 133, 173 -> 160 us; eight layers of the T5-xxl-shaped encoder at 64 /
+// 128 tokens 1373 -> 1217, 1568 -> 1385 us.  The gated pair at 100 / 128 tokens of that in mode 1, terms apart: 155 (7B), 1427 (T5);
+// in mode 2, merged: 150, 1385.
+template <int MODE, bool MERGED>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmX, const WgParams p) {
@@ -196,12 +203,13 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     constexpr int NT = DUAL ? 2 : 1;
     constexpr int OUT_ROWS = MIXED ? WG_ROWS / 2 : WG_ROWS;   // outputs of a tile
     constexpr uint32_t WB = NT * STAGE_BYTES;                 // weight bytes per stage and CTA
-    constexpr int CH = LOW ? 1 : (DUAL ? 4 : 8);              // 16-token chunks an epilogue warp holds at most
-    const int nt = LOW ? 32 : p.nt, htok = nt >> 1;
-    constexpr uint32_t LOW_COLS = LOW ? 32 * NT : 0;          // columns between the high and the low terms' sums
+    static_assert(MODE != 1 || MERGED, "both matrices' sums of both terms fit a set up to 64 tokens");
+    constexpr int CH = MERGED ? (DUAL ? 2 : 4) : 8;           // 16-token chunks an epilogue warp holds at most
+    const int nt = p.nt, htok = nt >> 1;
+    const uint32_t mma_cols = MERGED ? 2 * nt : nt;           // columns of an MMA
     const uint32_t xterm = (uint32_t)htok * 128u;             // one term of this CTA's half of the tokens
     const uint32_t stage_bytes = WB + 2u * xterm;
-    const uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) |
+    const uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((mma_cols >> 3) << 17) |
                            ((uint32_t)(WG_ROWS >> 4) << 24);  // f32 accumulate, bf16 x bf16, K-major both
 
     extern __shared__ unsigned char smem_raw[];
@@ -250,12 +258,16 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         auto step = [&](Cursor& c) {
             if (++c.kb == p.nkb) { c.kb = 0; if (++c.tok == p.ntok) { c.tok = 0; ++c.row; } }
         };
-        const int tile0 = (int)(u0 / p.nkb);
-        Cursor cur{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
+        auto first = [&] {
+            const int tile0 = (int)(u0 / p.nkb);
+            return Cursor{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
+        };
         if (warp == 0 && lane == 0) {
             // ---- TMA producer of this CTA's weights; all copies of the pair complete on the first CTA's barriers
-            const uint64_t once = policy_evict_first();
-            const bool reread = p.ntok > 1;                   // other token tiles take the same weights from L2
+            uint64_t keep;                                    // (other token tiles take the same weights from L2)
+            if (p.ntok > 1) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep));
+            else keep = policy_evict_first();
+            Cursor cur = first();
             int s = 0;
             uint32_t ph = 0;
 #pragma unroll 1
@@ -265,13 +277,9 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
                 if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
                 const int row = cur.row * OUT_ROWS + rank * (OUT_ROWS / 2);
-                auto load = [&](void* to, const CUtensorMap* tm) {
-                    if (reread) tma_load_2d_pair(to, tm, bar, cur.kb * KB, row);
-                    else tma_load_2d_pair_once(to, tm, bar, cur.kb * KB, row, once);
-                };
-                load(dst, &tmW);
-                if (DUAL) load(dst + STAGE_BYTES, &tmW2);
-                if (MIXED) load(dst + STAGE_BYTES / 2, &tmW2);
+                tma_load_2d_pair_keep(dst, &tmW, bar, cur.kb * KB, row, keep);
+                if (DUAL) tma_load_2d_pair_keep(dst + STAGE_BYTES, &tmW2, bar, cur.kb * KB, row, keep);
+                if (MIXED) tma_load_2d_pair_keep(dst + STAGE_BYTES / 2, &tmW2, bar, cur.kb * KB, row, keep);
                 step(cur);
                 if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
             }
@@ -279,6 +287,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             // ---- TMA producer of this CTA's half of the row terms, a warp of its own: three copies a stage from one thread
             //      (about 100 ns each, with the wait before them) set the pace of tiles of up to 128 tokens
             asm volatile("griddepcontrol.wait;" ::: "memory");
+            Cursor cur = first();
             int s = 0;
             uint32_t ph = 0;
 #pragma unroll 1
@@ -286,9 +295,13 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 if (i >= p.stages && !mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
                 unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
                 const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
-                const int r = cur.tok * nt + rank * htok;
-                tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, r);
-                tma_load_2d_pair(dst + xterm, &tmX, bar, cur.kb * KB, p.mpad + r);
+                if (MERGED) {
+                    tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, rank * p.mpad + cur.tok * nt);
+                } else {
+                    const int r = cur.tok * nt + rank * htok;
+                    tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, r);
+                    tma_load_2d_pair(dst + xterm, &tmX, bar, cur.kb * KB, p.mpad + r);
+                }
                 step(cur);
                 if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
             }
@@ -319,10 +332,10 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         for (int k = 0; k < KB / 16; ++k) {
                             const uint32_t acc = (j | k) != 0;
                             tc_mma_pair(d0, ad + 2 * k, bh + 2 * k, IDESC, acc);
-                            tc_mma_pair(d0 + LOW_COLS, ad + 2 * k, bl + 2 * k, IDESC, LOW ? acc : 1u);
+                            if (!MERGED) tc_mma_pair(d0, ad + 2 * k, bl + 2 * k, IDESC, 1u);
                             if (DUAL) {
-                                tc_mma_pair(d0 + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bh + 2 * k, IDESC, acc);
-                                tc_mma_pair(d0 + LOW_COLS + nt, ad + (STAGE_BYTES >> 4) + 2 * k, bl + 2 * k, IDESC, LOW ? acc : 1u);
+                                tc_mma_pair(d0 + mma_cols, ad + (STAGE_BYTES >> 4) + 2 * k, bh + 2 * k, IDESC, acc);
+                                if (!MERGED) tc_mma_pair(d0 + mma_cols, ad + (STAGE_BYTES >> 4) + 2 * k, bl + 2 * k, IDESC, 1u);
                             }
                         }
                         tc_commit_pair(&ctl->empty[s]);
@@ -376,11 +389,11 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     for (int ch = 0; ch < CH; ++ch)
                         if (ch < nch) {
                             float v[16];
-                            tc_ld16(taddr + (uint32_t)(u * nt + ch * 16), v);
+                            tc_ld16(taddr + u * mma_cols + (uint32_t)(ch * 16), v);
 #pragma unroll
                             for (int e = 0; e < 16; ++e) acc[(u * CH + ch) * 16 + e] += v[e];
-                            if (LOW) {
-                                tc_ld16(taddr + LOW_COLS + (uint32_t)(u * nt), v);
+                            if (MERGED) {
+                                tc_ld16(taddr + u * mma_cols + (uint32_t)(nt + ch * 16), v);
 #pragma unroll
                                 for (int e = 0; e < 16; ++e) acc[(u * CH + ch) * 16 + e] += v[e];
                             }
@@ -713,12 +726,10 @@ csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_b
     return CSD_OK;
 }
 
-template <int MODE, bool LOW = false>
+template <int MODE, bool MERGED>
 static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const WgParams& wp,
                             const WgPlan& pl, cudaStream_t st) {
-    if constexpr (MODE < 2 && !LOW)
-        if (pl.nt == 32) return launch_wg<MODE, true>(tw, tw2, tx, wp, pl, st);
-    auto kern = wide_gemm_kernel<MODE, LOW>;
+    auto kern = wide_gemm_kernel<MODE, MERGED>;
     static PerDevice ready;
     const csd_status ok = allow_smem(ready, kern, WG_SMEM_MAX);
     if (ok != CSD_OK) return ok;
@@ -751,7 +762,7 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     if (!tensor_map_2d(a.W, a.N, a.K, box, &tw)) return CSD_ERR_UNSUPPORTED;
     tw2 = tw;
     if (dual && !tensor_map_2d(a.W2, a.N, a.K, box, &tw2)) return CSD_ERR_UNSUPPORTED;
-    if (!tensor_map_2d(a.xs, 2 * pl.mpad, a.K, pl.nt / 2, &tx)) return CSD_ERR_UNSUPPORTED;
+    if (!tensor_map_2d(a.xs, 2 * pl.mpad, a.K, pl.merged ? pl.nt : pl.nt / 2, &tx)) return CSD_ERR_UNSUPPORTED;
     WgParams wp;
     wp.Y = a.Y; wp.partial = a.partial; wp.tickets = a.tickets; wp.status = status_word_device();
     wp.ssq_in = a.ssq; wp.ssq_cnt = a.ssq_cnt;
@@ -763,7 +774,7 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     if (pl.pk > 1) {                     // partial planes now, sums and epilogue in the small kernel after
         wp.Y = a.partial; wp.ldy = a.N; wp.plane = (size_t)a.m * a.N; wp.epilogue = EPI_STORE;
         wp.out_xs = nullptr; wp.out_ssq = nullptr; wp.out_gain = nullptr; wp.vec_y = 1;
-        const csd_status s = launch_wg<0>(tw, tw2, tx, wp, pl, st);
+        const csd_status s = pl.merged ? launch_wg<0, true>(tw, tw2, tx, wp, pl, st) : launch_wg<0, false>(tw, tw2, tx, wp, pl, st);
         if (s != CSD_OK) return s;
         PdlLaunch L(dim3((unsigned)wide_split_pieces(a.N), (unsigned)a.m), dim3(128), 0, st);
         CSD_CUDA(cudaLaunchKernelEx(&L.cfg, wide_reduce_kernel, (const float*)a.partial, pl.pk, wp.plane, a.N, a.m, pl.mpad, a.ssq,
@@ -772,8 +783,9 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
         count_launch();
         return CSD_OK;
     }
-    if (pl.mixed) return launch_wg<2>(tw, tw2, tx, wp, pl, st);
-    return dual ? launch_wg<1>(tw, tw2, tx, wp, pl, st) : launch_wg<0>(tw, tw2, tx, wp, pl, st);
+    if (dual && !pl.mixed) return launch_wg<1, true>(tw, tw2, tx, wp, pl, st);
+    if (dual) return pl.merged ? launch_wg<2, true>(tw, tw2, tx, wp, pl, st) : launch_wg<2, false>(tw, tw2, tx, wp, pl, st);
+    return pl.merged ? launch_wg<0, true>(tw, tw2, tx, wp, pl, st) : launch_wg<0, false>(tw, tw2, tx, wp, pl, st);
 }
 
 }  // namespace csd
