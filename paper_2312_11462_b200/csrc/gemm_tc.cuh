@@ -36,13 +36,12 @@ struct WideArgs {
     __nv_bfloat16* out_xs = nullptr;     // optional: (Y * out_gain) in two-term form [2][mpad][out_ld] for the next wide GEMM
     int out_ld = 0;
     const __nv_bfloat16* out_gain = nullptr;
-    float* out_ssq = nullptr;            // optional: [wide_ssq_pieces(...)][m] pieces of the sums of squares of the rows of Y
+    float* out_ssq = nullptr;            // optional: [wide_ssq_pieces(N)][m] pieces of the sums of squares of the rows of Y
     float* partial = nullptr;            // scratch of wide_partial_bytes(m) for partial sums
     unsigned* tickets = nullptr;         // zero-initialised, wide_ticket_count(m, N) entries
 };
 bool wide_supported(int m, int N, int K, bool dual);
-int wide_ssq_pieces(int m, int N, int K, bool dual);
-int wide_ssq_capacity(int N);
+int wide_ssq_pieces(int N);
 size_t wide_partial_bytes(int m);
 int wide_ticket_count(int m, int N);
 int wide_split_pieces(int K);

@@ -57,8 +57,12 @@ static_assert(8 * 16 * 32 + 4 * WG_SET <= 2 * 8 * 16 * 32, "sums of squares fit 
 
 // How a launch is divided.  tiles = row tiles x token tiles, tokens fastest, so that pairs running at the
 // same time share weight rows in L2.  Three ways:
-//   planes   few tiles (pairs / tiles >= 3): every tile goes to pk pairs that share its K range, each writes
-//            an fp32 plane and wide_reduce_kernel adds the planes and runs the epilogue;
+//   parts    few tiles of a single matrix (at most half as many as pairs): every tile goes to pk pairs that share its K range.
+//            Each of them finishes a pk-th of the tile's tokens and parks its sums of the others' (they stay in L2).  With fp32
+//            planes and a kernel behind that added them and ran the epilogue, the GEMM after o and down of a 7B-shaped
+//            layer of 64 tokens met its rows 9.7 us after their end.  A layer of 64 / 128 / 256 tokens 133 -> 129, 160 -> 145,
+//            245 -> 235 us; two parts instead of shares: 512 tokens 454 -> 440, eight T5-xxl-shaped encoder layers of 128 1326 -> 1291.
+//            (Clusters of four pairs that add up through distributed shared memory: 15 of them are resident, for 16 tiles.)
 //   whole    pair c takes whole tiles (no partial sums) where that leaves little of the last round empty;
 //   shares   otherwise the (tile, K block) units are dealt out in equal contiguous shares; a tile cut by a
 //            share boundary is finished by its first contributor from the partial sums the later
@@ -75,8 +79,7 @@ struct WgPlan {
 
 int wide_split_pieces(int K) { return (K + 1023) / 1024; }
 
-// planes: whether the result may go through planes (their reduction stores 16 bytes at a time)
-static WgPlan wg_plan(int m, int N, int K, bool dual, bool planes = true) {
+static WgPlan wg_plan(int m, int N, int K, bool dual) {
     WgPlan p{};
     const int P = tc_sm_count() / 2, most = 256;
     p.mixed = dual && m > 64;
@@ -93,7 +96,7 @@ static WgPlan wg_plan(int m, int N, int K, bool dual, bool planes = true) {
     p.smem = (size_t)p.stages * p.stage + 1024 + WG_STAGING + sizeof(WgCtrl);
     p.pk = 1; p.gran = 1;
     const int ratio = P / p.tiles;
-    if (planes && !dual && (N & 7) == 0 && ratio >= 3 && p.nkb >= 16) {
+    if (!dual && ratio >= 2 && p.nkb >= 16) {
         p.pk = ratio < 8 ? ratio : 8;
         if (p.pk > p.nkb / 8) p.pk = p.nkb / 8;
         p.pairs = p.tiles * p.pk;
@@ -119,15 +122,8 @@ bool wide_supported(int m, int N, int K, bool dual) {
     return tiles * ((K + KB - 1) / KB) * (tc_sm_count() + 1) < (1LL << 31);
 }
 
-int wide_ssq_pieces(int m, int N, int K, bool dual) {
-    const WgPlan p = wg_plan(m, N, K, dual);
-    return p.pk > 1 ? wide_split_pieces(N) : 2 * ((N + WG_ROWS - 1) / WG_ROWS);
-}
-int wide_ssq_capacity(int N) {
-    const int a = 2 * ((N + WG_ROWS - 1) / WG_ROWS), b = wide_split_pieces(N);
-    return a > b ? a : b;
-}
-// planes of at most one tile per pair, or one parked tile (of both matrices of a gated pair) per pair
+int wide_ssq_pieces(int N) { return 2 * ((N + WG_ROWS - 1) / WG_ROWS); }
+// one parked tile (of both matrices of a gated pair) per pair
 size_t wide_partial_bytes(int m) {
     const int cols = m < 128 ? 2 * ((m + 31) & ~31) : 256;
     return (size_t)(tc_sm_count() / 2) * WG_ROWS * cols * sizeof(float);
@@ -135,7 +131,8 @@ size_t wide_partial_bytes(int m) {
 int wide_ticket_count(int m, int N) {
     const int half = WG_ROWS / 2;
     const int a = ((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128), b = ((N + half - 1) / half) * ((m + 255) / 256);
-    return 2 * (a > b ? a : b);
+    const int tiles = a > b ? a : b, pairs = tc_sm_count() / 2;     // two words a tile, or a pair where tiles go by parts
+    return 2 * (tiles > pairs ? tiles : pairs);
 }
 
 struct WgParams {
@@ -144,7 +141,6 @@ struct WgParams {
     __nv_bfloat16* out_xs; const __nv_bfloat16* out_gain; float* out_ssq; int out_ld;
     int m, mpad, nt, ntok, tiles, nkb, pk, gran, N, K, ldy, stages, epilogue;
     int vec_y;                          // Y takes 16-byte accesses
-    size_t plane;                       // floats between the partial planes (pk > 1)
     float eps;
 };
 
@@ -195,7 +191,7 @@ __device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigne
 // of the 7B shape at 20 / 64 / 128 tokens 134 -> 120, 151 -> 133, 173 -> 160 us; eight layers of the T5-xxl-shaped encoder at 64 /
 // 128 tokens 1373 -> 1217, 1568 -> 1385 us.  The gated pair at 100 / 128 tokens of that in mode 1, terms apart: 155 (7B), 1427 (T5);
 // in mode 2, merged: 150, 1385.
-template <int MODE, bool MERGED>
+template <int MODE, bool MERGED, bool PARTS>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
                  const __grid_constant__ CUtensorMap tmX, const WgParams p) {
@@ -221,7 +217,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
     const unsigned units = (unsigned)p.tiles * (unsigned)p.nkb;
     unsigned u0, u1;
-    if (p.pk > 1) {
+    if (PARTS) {
         const unsigned t = (unsigned)(pair / p.pk) * (unsigned)p.nkb, part = (unsigned)(pair % p.pk);
         u0 = t + part * (unsigned)p.nkb / (unsigned)p.pk;
         u1 = t + (part + 1) * (unsigned)p.nkb / (unsigned)p.pk;
@@ -366,8 +362,12 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             const int seg = min(p.nkb - kb_begin, items - i);
             i += seg;
             const int row_tile = tile / p.ntok, tok0 = (tile % p.ntok) * nt;
+            // a tile in parts of K: this part finishes the 16-token chunks own0 .. own1 - 1
+            constexpr bool cut = PARTS;
+            const int chunks = nt >> 4, kpart = cut ? pair % p.pk : 0;
+            const int own0 = cut ? kpart * chunks / p.pk : 0, own1 = cut ? (kpart + 1) * chunks / p.pk : 0;
             asm volatile("bar.sync 1, 256;" ::: "memory");    // everyone is past the previous tile's scale factors
-            if (p.ssq_in && p.pk == 1 && et < nt && tok0 + et < m) {
+            if (p.ssq_in && et < nt && tok0 + et < m) {
                 float sq = 0.f;
                 const float* src = p.ssq_in + tok0 + et;
 #pragma unroll 8
@@ -405,7 +405,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     else remote_arrive(empty_bar + (uint32_t)(b * sizeof(uint64_t)));
                 }
             }
-            if (p.pk == 1 && seg < p.nkb) {
+            if (!PARTS && seg < p.nkb) {
                 // part of a tile: later contributors park and go on, the first one adds the parts in pair order.
                 // Parked layout [warp][chunk][quarter of 16][lane][4]: 512 contiguous bytes per warp access.
                 const int c_lo = cta_of_unit((unsigned)tile * p.nkb, units, pairs);
@@ -444,12 +444,12 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 }
                 const float* mine = reinterpret_cast<const float*>(ring) + at;
 #pragma unroll 1
-                for (int c = c_lo + 1; c <= c_hi; ++c) {
+                for (int from = c_lo + 1; from <= c_hi; ++from) {
                     if (et == 0) {
                         mbar_expect_tx(&ctl->part_full, part_bytes);
-                        bulk_to_smem(ring, p.partial + (size_t)(2 * c + rank) * TILE_N * nt * NT, part_bytes, &ctl->part_full);
+                        bulk_to_smem(ring, p.partial + (size_t)(2 * from + rank) * TILE_N * nt * NT, part_bytes, &ctl->part_full);
                     }
-                    if (!mbar_wait(&ctl->part_full, (uint32_t)(c - c_lo - 1) & 1u)) *abort_flag = 1;
+                    if (!mbar_wait(&ctl->part_full, (uint32_t)(from - c_lo - 1) & 1u)) *abort_flag = 1;
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
 #pragma unroll
@@ -464,6 +464,35 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                             }
                     asm volatile("bar.sync 1, 256;" ::: "memory");    // the ring may be overwritten
                 }
+            } else if (PARTS) {
+                // a part of K: the 16-token chunks are dealt out to the tile's parts; this one's own go into the ring, which is
+                // free (all MMAs are done), the others' are parked, [chunk][token][128 rows]
+#pragma unroll
+                for (int ch = 0; ch < CH; ++ch)
+                    if (ch < nch) {
+                        const int cc = half * nch + ch;
+                        if (cc >= own0 && cc < own1) {
+                            float* to = reinterpret_cast<float*>(ring) + (cc - own0) * (16 * TILE_N) + q * 32 + lane;
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) to[e * TILE_N] = acc[ch * 16 + e];
+                        } else {
+                            float* to = p.partial + ((size_t)blockIdx.x * chunks + cc) * (16 * TILE_N) + q * 32 + lane;
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) __stcg(to + e * TILE_N, acc[ch * 16 + e]);
+                        }
+                    }
+                __syncwarp();
+                if (lane < p.pk && lane != kpart) red_release_gpu(&p.tickets[2 * (pair - kpart + lane) + rank], 1u);
+                if (et == 0) {
+                    const unsigned want = 8u * (unsigned)(p.pk - 1);
+                    int spins = 0;
+#pragma unroll 1
+                    while (ld_acquire_gpu(&p.tickets[2 * pair + rank]) < want)
+                        if (++spins > SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
+                    p.tickets[2 * pair + rank] = 0u;          // everyone has arrived: ready for the next launch
+                    __threadfence();
+                }
+                asm volatile("bar.sync 1, 256;" ::: "memory");    // (the tile's scale factors are written as well)
             } else {
                 asm volatile("bar.sync 1, 256;" ::: "memory");    // the tile's scale factors are written
             }
@@ -471,7 +500,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             //      staging so that a lane then holds 4 neighbouring rows of a token, 8 lanes a token's whole 128 bytes.
             //      (Staged by four warps for 128 rows, a chunk waited at two barriers: T5-xxl-shaped source of
             //      256 tokens 7.5 ms, 6.8 so.)
-            const bool scaled = p.ssq_in && p.pk == 1;
+            const bool scaled = p.ssq_in != nullptr;
             const int c = (lane & 7) * 4, e0 = lane >> 3;     // this lane's rows of the warp's 32, first of its tokens (every 4th)
             const int n = row_tile * OUT_ROWS + rank * (OUT_ROWS / 2) + (MIXED ? q & 1 : q) * 32 + c;
             const int have = min(4, p.N - n);                 // weight rows of this lane inside the matrix
@@ -482,14 +511,17 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 for (int j = 0; j < 4; ++j)
                     if (j < have) gain[j] = __bfloat162float(p.out_gain[n + j]);
             }
-            float* Y = p.Y ? p.Y + (p.pk > 1 ? (size_t)(pair % p.pk) * p.plane : 0) + n : nullptr;
+            float* Y = p.Y ? p.Y + n : nullptr;
+            // chunks this warp finishes: its half's, or every other one of its part's
+            const int ch_end = cut ? own1 - own0 : nch, ch_step = cut ? 2 : 1, ch0 = cut ? half : 0;
+            auto column = [&](int ch) { return cut ? (own0 + ch) * 16 : half * htok + ch * 16; };   // in the tile
             float old[4][4];                                  // residual values of a chunk, requested a chunk ahead
             auto load_old = [&](int ch) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int r = tok0 + half * htok + ch * 16 + 4 * k + e0;
+                    const int r = tok0 + column(ch) + 4 * k + e0;
                     old[k][0] = old[k][1] = old[k][2] = old[k][3] = 0.f;
-                    if (add && ch < nch && r < m) {
+                    if (add && ch < ch_end && r < m) {
                         const float* y = Y + (size_t)r * p.ldy;
                         if (vec) {
                             const float4 v = __ldcg(reinterpret_cast<const float4*>(y));
@@ -502,7 +534,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     }
                 }
             };
-            load_old(0);
+            load_old(ch0);
             // (mixed: warps q and q + 2 hold gate and up of the same outputs; each finishes half of the chunk's tokens from
             //  both stagings, of which there are two in turn, so that one barrier of the two warps per chunk will do)
             float* buf = staging + ew * ((MIXED ? 2 : NT) * 16 * 32);
@@ -511,8 +543,8 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             const int k0 = MIXED ? (q >> 1) * 2 : 0;
             float* sums = staging + 8 * 16 * 32;              // [quadrant][token]: sums of squares over a warp's 32 rows
 #pragma unroll 1
-            for (int ch = 0; ch < nch; ++ch) {
-                const int c0 = half * htok + ch * 16, r0 = tok0 + c0;     // column in the tile, token
+            for (int ch = ch0; ch < ch_end; ch += ch_step) {
+                const int c0 = column(ch), r0 = tok0 + c0;    // column in the tile, token
                 if (r0 >= m) break;                           // (the same for the four warps of a half)
                 float* put = buf + lane + (MIXED ? (ch & 1) * (16 * 32) : 0);
                 // Registers have no index: one short copy per chunk, everything else is a loop over the chunks.  Unrolled
@@ -528,16 +560,32 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             }                                                                                                           \
         }                                                                                                               \
         break;
-                switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
+                if (!cut) switch (ch) { WG_PUT(0) WG_PUT(1) WG_PUT(2) WG_PUT(3) WG_PUT(4) WG_PUT(5) WG_PUT(6) WG_PUT(7) }
 #undef WG_PUT
                 if (MIXED) asm volatile("bar.sync %0, 64;" ::"r"(4 + half * 2 + (q & 1)) : "memory");
                 else __syncwarp();
                 float x[4][4];
+                if (cut) {                                    // the parts in order, this one's from the ring
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) x[k][0] = x[k][1] = x[k][2] = x[k][3] = 0.f;
+#pragma unroll 2
+                    for (int j = 0; j < p.pk; ++j) {
+                        const int at = e0 * TILE_N + q * 32 + c;
+                        const float* own = reinterpret_cast<const float*>(ring) + ch * (16 * TILE_N) + at;
+                        const float* part = p.partial + ((size_t)(2 * (pair - kpart + j) + rank) * chunks + own0 + ch) * (16 * TILE_N) + at;
+                        float4 v[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            v[k] = j == kpart ? *reinterpret_cast<const float4*>(own + 4 * k * TILE_N) : __ldcg(reinterpret_cast<const float4*>(part + 4 * k * TILE_N));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) { x[k][0] += v[k].x; x[k][1] += v[k].y; x[k][2] += v[k].z; x[k][3] += v[k].w; }
+                    }
+                }
 #pragma unroll
                 for (int k = 0; k < KC; ++k) {
                     const int e = 4 * (k0 + k) + e0;
                     const float* from = MIXED ? gate + (ch & 1) * (16 * 32) : buf;
-                    const float4 v = *reinterpret_cast<const float4*>(from + e * 32 + c);
+                    const float4 v = cut ? make_float4(x[k][0], x[k][1], x[k][2], x[k][3]) : *reinterpret_cast<const float4*>(from + e * 32 + c);
                     const float sc = scaled ? ctl->scale[c0 + e] : 1.f;
                     x[k][0] = v.x * sc; x[k][1] = v.y * sc; x[k][2] = v.z * sc; x[k][3] = v.w * sc;
                     if (DUAL || MIXED) {
@@ -551,7 +599,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     for (int j = 0; j < 4; ++j)
                         if (MODE == 0) x[k][j] += old[k][j];
                 }
-                if (add) load_old(ch + 1);
+                if (add) load_old(ch + ch_step);
                 if (MODE == 0 && p.out_ssq) {                     // (rows past the matrix came out as zeros)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -593,8 +641,8 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             }
             if (MODE == 0 && p.out_ssq) {                         // one piece per token and CTA: its 128 rows
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");
-                const int col = half * htok + (et & 127);
-                if ((et & 127) < htok && tok0 + col < m)
+                const int i0 = et & 127, col = (cut ? own0 * 16 : half * htok) + i0;
+                if ((cut ? i0 < (own1 - own0) * 16 && ((i0 >> 4) & 1) == half : i0 < htok) && tok0 + col < m)
                     p.out_ssq[(size_t)(row_tile * 2 + rank) * m + tok0 + col] =
                         (sums[col] + sums[WG_SET + col]) + (sums[2 * WG_SET + col] + sums[3 * WG_SET + col]);
             }
@@ -656,66 +704,6 @@ split2_rows_kernel(const float* __restrict__ X, int ldx, int K, int m, int mpad,
     if (threadIdx.x == 0 && ssq && r < m) ssq[(size_t)blockIdx.x * m + r] = (part[0] + part[1]) + (part[2] + part[3]);
 }
 
-// Adds the partial planes of a K-partitioned launch in plane order, then the epilogue: optional rms-norm
-// factor, residual add into Y, two-term split (times a gain) and sum-of-squares pieces.
-// grid = (N / 1024 rounded up, m); N a multiple of 8.
-__global__ void __launch_bounds__(128)
-wide_reduce_kernel(const float* __restrict__ P, int pk, size_t plane, int N, int m, int mpad, const float* __restrict__ ssq_in,
-                   int ssq_cnt, int K, float eps, float* __restrict__ Y, int ldy, int add, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ xs, int out_ld,
-                   float* __restrict__ ssq) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int r = blockIdx.y, k = (blockIdx.x * 128 + threadIdx.x) * 8;
-    float sq = 0.f, scale = 1.f;
-    if (ssq_in) {
-        float s = 0.f;
-        for (int c = (int)(threadIdx.x & 31); c < ssq_cnt; c += 32) s += __ldcg(ssq_in + (size_t)c * m + r);
-        scale = 1.f / sqrtf(warp_sum(s) / (float)K + eps);
-    }
-    if (k < N) {
-        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int j = 0; j < pk; ++j) {
-            const float* src = P + (size_t)j * plane + (size_t)r * N + k;
-            const float4 a = __ldcg(reinterpret_cast<const float4*>(src)), b = __ldcg(reinterpret_cast<const float4*>(src + 4));
-            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] *= scale;
-        float* y = Y + (size_t)r * ldy + k;
-        if (add) {
-            const float4 a = *reinterpret_cast<const float4*>(y), b = *reinterpret_cast<const float4*>(y + 4);
-            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
-        }
-        *reinterpret_cast<float4*>(y) = make_float4(v[0], v[1], v[2], v[3]);
-        *reinterpret_cast<float4*>(y + 4) = make_float4(v[4], v[5], v[6], v[7]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sq = fmaf(v[e], v[e], sq);
-        if (xs) {
-            if (gain) {
-                const uint4 g = *reinterpret_cast<const uint4*>(gain + k);
-                v[0] *= bf16lo(g.x); v[1] *= bf16hi(g.x); v[2] *= bf16lo(g.y); v[3] *= bf16hi(g.y);
-                v[4] *= bf16lo(g.z); v[5] *= bf16hi(g.z); v[6] *= bf16lo(g.w); v[7] *= bf16hi(g.w);
-            }
-            uint32_t t[2][4];
-#pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-                uint16_t a1, a2, c1, c2;
-                split2f(v[e], a1, a2);
-                split2f(v[e + 1], c1, c2);
-                t[0][e / 2] = a1 | ((uint32_t)c1 << 16); t[1][e / 2] = a2 | ((uint32_t)c2 << 16);
-            }
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-                *reinterpret_cast<uint4*>(xs + (size_t)(s * mpad + r) * out_ld + k) = make_uint4(t[s][0], t[s][1], t[s][2], t[s][3]);
-        }
-    }
-    __shared__ float part[4];
-    sq = warp_sum(sq);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sq;
-    __syncthreads();
-    if (threadIdx.x == 0 && ssq) ssq[(size_t)blockIdx.x * m + r] = (part[0] + part[1]) + (part[2] + part[3]);
-}
-
 csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_bfloat16* gain, __nv_bfloat16* xs,
                              float* ssq, cudaStream_t st, unsigned* clear, int clear_count) {
     if (!X || !xs || (((uintptr_t)X) & 15) || (ldx & 3) || (K & 7) || m < 1 || m > CSD_WIDE_ROWS) return CSD_ERR_INVALID_ARG;
@@ -726,10 +714,10 @@ csd_status launch_wide_split(const float* X, int ldx, int K, int m, const __nv_b
     return CSD_OK;
 }
 
-template <int MODE, bool MERGED>
+template <int MODE, bool MERGED, bool PARTS = false>
 static csd_status launch_wg(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& tx, const WgParams& wp,
                             const WgPlan& pl, cudaStream_t st) {
-    auto kern = wide_gemm_kernel<MODE, MERGED>;
+    auto kern = wide_gemm_kernel<MODE, MERGED, PARTS>;
     static PerDevice ready;
     const csd_status ok = allow_smem(ready, kern, WG_SMEM_MAX);
     if (ok != CSD_OK) return ok;
@@ -752,11 +740,7 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     if (!a.Y && (!dual || !a.out_xs)) return CSD_ERR_INVALID_ARG;
     if (dual != (a.epilogue == EPI_SWIGLU || a.epilogue == EPI_GEGLU) || (dual && a.out_ssq)) return CSD_ERR_INVALID_ARG;
     if (!wide_supported(a.m, a.N, a.K, dual)) return CSD_ERR_UNSUPPORTED;
-    WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
-    if (pl.pk > 1 && ((a.ldy & 3) || (((uintptr_t)a.Y) & 15) || (a.out_xs && (a.out_ld & 7)))) {
-        if (a.out_ssq) return CSD_ERR_INVALID_ARG;       // (its pieces are counted by the plan with planes)
-        pl = wg_plan(a.m, a.N, a.K, dual, false);
-    }
+    const WgPlan pl = wg_plan(a.m, a.N, a.K, dual);
     CUtensorMap tw, tw2, tx;
     const int box = pl.mixed ? TILE_N / 2 : TILE_N;
     if (!tensor_map_2d(a.W, a.N, a.K, box, &tw)) return CSD_ERR_UNSUPPORTED;
@@ -769,22 +753,10 @@ csd_status launch_linear_wide(const WideArgs& a, cudaStream_t st) {
     wp.out_xs = a.out_xs; wp.out_gain = a.out_gain; wp.out_ssq = a.out_ssq; wp.out_ld = a.out_ld;
     wp.m = a.m; wp.mpad = pl.mpad; wp.nt = pl.nt; wp.ntok = pl.ntok; wp.tiles = pl.tiles; wp.nkb = pl.nkb; wp.pk = pl.pk;
     wp.gran = pl.gran; wp.N = a.N; wp.K = a.K; wp.ldy = a.ldy; wp.stages = pl.stages; wp.epilogue = a.epilogue; wp.eps = a.eps;
-    wp.plane = 0;
     wp.vec_y = (a.ldy & 3) == 0 && (((uintptr_t)a.Y) & 15) == 0;
-    if (pl.pk > 1) {                     // partial planes now, sums and epilogue in the small kernel after
-        wp.Y = a.partial; wp.ldy = a.N; wp.plane = (size_t)a.m * a.N; wp.epilogue = EPI_STORE;
-        wp.out_xs = nullptr; wp.out_ssq = nullptr; wp.out_gain = nullptr; wp.vec_y = 1;
-        const csd_status s = pl.merged ? launch_wg<0, true>(tw, tw2, tx, wp, pl, st) : launch_wg<0, false>(tw, tw2, tx, wp, pl, st);
-        if (s != CSD_OK) return s;
-        PdlLaunch L(dim3((unsigned)wide_split_pieces(a.N), (unsigned)a.m), dim3(128), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&L.cfg, wide_reduce_kernel, (const float*)a.partial, pl.pk, wp.plane, a.N, a.m, pl.mpad, a.ssq,
-                                    a.ssq_cnt, a.K, a.eps, a.Y, a.ldy, a.epilogue == EPI_ADD ? 1 : 0, a.out_gain, a.out_xs,
-                                    a.out_ld, a.out_ssq));
-        count_launch();
-        return CSD_OK;
-    }
     if (dual && !pl.mixed) return launch_wg<1, true>(tw, tw2, tx, wp, pl, st);
     if (dual) return pl.merged ? launch_wg<2, true>(tw, tw2, tx, wp, pl, st) : launch_wg<2, false>(tw, tw2, tx, wp, pl, st);
+    if (pl.pk > 1) return pl.merged ? launch_wg<0, true, true>(tw, tw2, tx, wp, pl, st) : launch_wg<0, false, true>(tw, tw2, tx, wp, pl, st);
     return pl.merged ? launch_wg<0, true>(tw, tw2, tx, wp, pl, st) : launch_wg<0, false>(tw, tw2, tx, wp, pl, st);
 }
 

@@ -297,7 +297,7 @@ static WsLayout ws_layout(const csd_model_config& c) {
         L.wxs_x = L.wattn = put(rows > attn ? rows : attn);
         L.wxs_attn = put(2 * WR * di * 2);
         const size_t kmax_w = d > di ? (d > ff ? d : ff) : (di > ff ? di : ff);
-        size_t pieces = (size_t)wide_ssq_capacity((int)d);
+        size_t pieces = (size_t)wide_ssq_pieces((int)d);
         if ((size_t)wide_split_pieces((int)kmax_w) > pieces) pieces = (size_t)wide_split_pieces((int)kmax_w);
         L.wssq = put(pieces * WR * 4);
         L.wpart = put(wide_partial_bytes((int)WR));
@@ -501,7 +501,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
         const __nv_bfloat16* after_o = c.arch == 1 ? y.norm_x : y.norm2;
         CSD_TRY(wide_linear(M, y.wo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d, after_o,
                             M->wssq, st));
-        cnt = wide_ssq_pieces(m, d, di, false);
+        cnt = wide_ssq_pieces(d);
         if (c.arch == 1) {
             CSD_TRY(wide_linear(M, y.xq, nullptr, di, d, m, M->wxs_x, M->wssq, cnt, M->wqkv, 3 * di, EPI_STORE, nullptr, 0,
                                 nullptr, nullptr, st));
@@ -509,13 +509,13 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
                                    c.max_enc_len, M->enc_len, false, false, nullptr, 0, 0, 0, st));
             CSD_TRY(wide_linear(M, y.xo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d, y.norm2,
                                 M->wssq, st));
-            cnt = wide_ssq_pieces(m, d, di, false);
+            cnt = wide_ssq_pieces(d);
         }
         CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, cnt, nullptr, ff,
                             c.arch == 0 ? EPI_SWIGLU : EPI_GEGLU, M->wxs_act, ff, nullptr, nullptr, st));
         CSD_TRY(wide_linear(M, y.wdown, nullptr, d, ff, m, M->wxs_act, nullptr, 0, M->wx, d, EPI_ADD, M->wxs_x, d,
                             M->dec[l + 1].norm1, M->wssq, st));
-        cnt = wide_ssq_pieces(m, d, ff, false);
+        cnt = wide_ssq_pieces(d);
     }
     CSD_CUDA(cudaGetLastError());
     return CSD_OK;
@@ -532,8 +532,11 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
         const bool fused = y.wk == y.wq + (size_t)di * d && y.wv == y.wk + (size_t)di * d;
         for (int r0 = 0; r0 < n; r0 += WR) {
             const int m = n - r0 < WR ? n - r0 : WR;
-            CSD_TRY(launch_wide_split(M->xenc + (size_t)r0 * d, d, d, m, y.norm1, M->wxs_x, M->wssq, st));
-            const int cnt = wide_split_pieces(d);
+            int cnt = wide_ssq_pieces(d);                     // (of the layer before, where it has handed its rows on)
+            if (l == 0 || n > WR) {
+                CSD_TRY(launch_wide_split(M->xenc + (size_t)r0 * d, d, d, m, y.norm1, M->wxs_x, M->wssq, st));
+                cnt = wide_split_pieces(d);
+            }
             float* out = M->qkv_enc + (size_t)r0 * 3 * di;
             if (fused) {
                 CSD_TRY(wide_linear(M, y.wq, nullptr, 3 * di, d, m, M->wxs_x, M->wssq, cnt, out, 3 * di, EPI_STORE, nullptr, 0,
@@ -553,18 +556,24 @@ static csd_status wide_encoder(csd_model* M, int n, cudaStream_t st) {
                                    2 * E - 1, E - 1, r0, st));
             CSD_TRY(wide_linear(M, y.wo, nullptr, d, di, m, M->wxs_attn, nullptr, 0, xr, d, EPI_ADD, M->wxs_x, d, y.norm2,
                                 M->wssq, st));
-            CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, wide_ssq_pieces(m, d, di, false), nullptr, ff,
+            CSD_TRY(wide_linear(M, y.wgate, y.wup, ff, d, m, M->wxs_x, M->wssq, wide_ssq_pieces(d), nullptr, ff,
                                 EPI_GEGLU, M->wxs_act, ff, nullptr, nullptr, st));
-            CSD_TRY(wide_linear(M, y.wdown, nullptr, d, ff, m, M->wxs_act, nullptr, 0, xr, d, EPI_ADD, nullptr, 0, nullptr,
-                                nullptr, st));
+            // one block of rows: handed on to the next layer's first norm (the last layer's: to the cross-attention's projections)
+            const bool on = n <= WR;
+            const __nv_bfloat16* next = l + 1 < c.n_enc_layers ? M->enc[l + 1].norm1 : M->enc_final_norm;
+            CSD_TRY(wide_linear(M, y.wdown, nullptr, d, ff, m, M->wxs_act, nullptr, 0, xr, d, EPI_ADD, on ? M->wxs_x : nullptr, d,
+                                on ? next : nullptr, on ? M->wssq : nullptr, st));
         }
     }
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& y = M->dec[l];
         for (int r0 = 0; r0 < n; r0 += WR) {
-            const int m = n - r0 < WR ? n - r0 : WR, cnt = wide_split_pieces(d);
-            if (l == 0 || n > WR)            // (one block of rows: their terms serve all layers)
+            const int m = n - r0 < WR ? n - r0 : WR;
+            int cnt = wide_ssq_pieces(d);    // (one block of rows: their terms, left by the last encoder layer, serve all layers)
+            if (n > WR) {
                 CSD_TRY(launch_wide_split(M->xenc + (size_t)r0 * d, d, d, m, M->enc_final_norm, M->wxs_x, M->wssq, st));
+                cnt = wide_split_pieces(d);
+            }
             float* out = M->qkv_enc + (size_t)r0 * 3 * di;
             const bool fused = y.xv == y.xk + (size_t)di * d;
             CSD_TRY(wide_linear(M, y.xk, nullptr, fused ? 2 * di : di, d, m, M->wxs_x, M->wssq, cnt, out + di, 3 * di, EPI_STORE,
