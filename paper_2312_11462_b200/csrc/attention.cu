@@ -29,7 +29,7 @@ template <int DH> struct AttnCfg {
     static constexpr int RG = (MAXM + G - 1) / G;            // rows per group
     static constexpr int NC = DH / 32;                       // 8-element chunks per score thread
     static constexpr int QROW = NC * 36;                     // q row: 32-float groups, 4 floats of skew each
-    static constexpr int REC = DH + 2;                       // merge record: output row, max, sum
+    static constexpr int REC = DH + 4;                       // merge record: output row, max, sum (and 16-byte rows)
     static constexpr size_t TILE_BYTES = (size_t)TILE * DH * 2;
     static constexpr size_t QS_FLOATS = (size_t)MAXM * (QROW > REC ? QROW : REC);
     static constexpr size_t SMEM = 2 * STAGES * TILE_BYTES + QS_FLOATS * 4 + (size_t)MAXM * TILE * 4 +
@@ -76,46 +76,85 @@ __device__ __forceinline__ void store_split(__nv_bfloat16* xs, int ld, int m, in
     base[((size_t)(2 * m + r) * ld) >> 1] = a3 | ((uint32_t)c3 << 16);
 }
 
+// W neighbouring values
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[1]) { v[0] = *p; }
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[2]) {
+    const float2 f = *reinterpret_cast<const float2*>(p);
+    v[0] = f.x; v[1] = f.y;
+}
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[4]) {
+    const float4 f = *reinterpret_cast<const float4*>(p);
+    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+}
+__device__ __forceinline__ void store_words(void* p, const uint32_t (&w)[1]) { *reinterpret_cast<uint32_t*>(p) = w[0]; }
+__device__ __forceinline__ void store_words(void* p, const uint32_t (&w)[2]) { *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]); }
 
 // Merge of the splits' records (unnormalised output row, running max, running sum) through
-// distributed shared memory: the CTAs of a head share out the m*DH output elements; each thread
+// distributed shared memory: the CTAs of a head share out the m*DH output elements, W neighbours a thread; each thread
 // first fetches everything it needs from all splits in one batch of independent remote loads.
-template <int DH, int REC>
-__device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* rec, const AttnParams& p, float* out, int xs_r0,
+template <int DH, int REC, int W>
+__device__ __forceinline__ void merge_rows(cg::cluster_group& cluster, float* rec, const AttnParams& p, float* out, int xs_r0,
                                              int h, int split, int m) {
-    for (int i = split * AT + threadIdx.x; i < m * DH; i += p.nsplit * AT) {
-        const int r = i / DH, d = i % DH;
-        float ms[MAX_SPLITS], ls[MAX_SPLITS], vs[MAX_SPLITS];
+    for (int i = split * AT + threadIdx.x; i < m * (DH / W); i += p.nsplit * AT) {
+        const int r = i / (DH / W), d = i % (DH / W) * W;
+        float ms[MAX_SPLITS], ls[MAX_SPLITS], vs[MAX_SPLITS][W];
 #pragma unroll
         for (int s = 0; s < MAX_SPLITS; ++s) {
-            ms[s] = -INFINITY; ls[s] = 0.f; vs[s] = 0.f;
+            ms[s] = -INFINITY; ls[s] = 0.f;
+#pragma unroll
+            for (int w = 0; w < W; ++w) vs[s][w] = 0.f;
             if (s < p.nsplit) {
                 const float* rs = cluster.map_shared_rank(rec, s) + r * REC;
-                ms[s] = rs[DH]; ls[s] = rs[DH + 1]; vs[s] = rs[d];
+                ms[s] = rs[DH]; ls[s] = rs[DH + 1];
+                load_vec(rs + d, vs[s]);
             }
         }
         float M = -INFINITY;
 #pragma unroll
         for (int s = 0; s < MAX_SPLITS; ++s) M = fmaxf(M, ms[s]);
-        float num = 0.f, den = 0.f;
+        float num[W], den = 0.f;
+#pragma unroll
+        for (int w = 0; w < W; ++w) num[w] = 0.f;
 #pragma unroll
         for (int s = 0; s < MAX_SPLITS; ++s)
             if (ms[s] > -INFINITY) {
-                const float w = expf(ms[s] - M);
-                num = fmaf(vs[s], w, num);
-                den = fmaf(ls[s], w, den);
+                const float f = expf(ms[s] - M);
+#pragma unroll
+                for (int w = 0; w < W; ++w) num[w] = fmaf(vs[s][w], f, num[w]);
+                den = fmaf(ls[s], f, den);
             }
-        const float ov = den > 0.f ? num / den : 0.f;
-        out[(size_t)r * p.ldo + h * DH + d] = ov;
+        float ov[W];
+        uint16_t b[3][W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            ov[w] = den > 0.f ? num[w] / den : 0.f;
+            split3(ov[w], b[0][w], b[1][w], b[2][w]);
+        }
         if (p.out_xs) {
-            uint16_t b1, b2, b3;
-            split3(ov, b1, b2, b3);
-            uint16_t* xs = reinterpret_cast<uint16_t*>(p.out_xs) + h * DH + d;
-            xs[(size_t)(xs_r0 + r) * p.out_xs_ld] = b1;
-            xs[(size_t)(p.xs_m + xs_r0 + r) * p.out_xs_ld] = b2;
-            xs[(size_t)(2 * p.xs_m + xs_r0 + r) * p.out_xs_ld] = b3;
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                __nv_bfloat16* dst = p.out_xs + (size_t)(t * p.xs_m + xs_r0 + r) * p.out_xs_ld + h * DH + d;
+                if constexpr (W == 1) {
+                    *reinterpret_cast<uint16_t*>(dst) = b[t][0];
+                } else {
+                    uint32_t w2[W / 2];
+#pragma unroll
+                    for (int w = 0; w < W; w += 2) w2[w / 2] = b[t][w] | ((uint32_t)b[t][w + 1] << 16);
+                    store_words(dst, w2);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int w = 0; w < W; ++w) out[(size_t)r * p.ldo + h * DH + d + w] = ov[w];
         }
     }
+}
+// one element a thread while there are threads for all, four otherwise
+template <int DH, int REC>
+__device__ __forceinline__ void merge_splits(cg::cluster_group& cluster, float* rec, const AttnParams& p, float* out, int xs_r0,
+                                             int h, int split, int m) {
+    if (m * DH <= p.nsplit * AT) merge_rows<DH, REC, 1>(cluster, rec, p, out, xs_r0, h, split, m);
+    else merge_rows<DH, REC, 4>(cluster, rec, p, out, xs_r0, h, split, m);
 }
 
 template <int DH>
@@ -338,9 +377,9 @@ block_attention_kernel(const AttnParams p) {
             const int r = g + rr * C::G;
             if (r < m) {
                 const float inv = row_l[r] > 0.f ? 1.f / row_l[r] : 0.f;
-                float* o = p.out + (size_t)r * p.ldo + h * DH + 2 * dp;
-                o[0] = acc[rr][0] * inv; o[1] = acc[rr][1] * inv;
-                if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, p.xs_r0 + r, h * DH + 2 * dp, o[0], o[1]);
+                const float a = acc[rr][0] * inv, b = acc[rr][1] * inv;
+                if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, p.xs_r0 + r, h * DH + 2 * dp, a, b);
+                else *reinterpret_cast<float2*>(p.out + (size_t)r * p.ldo + h * DH + 2 * dp) = make_float2(a, b);
             }
         }
         return;
@@ -375,7 +414,7 @@ template <int DH> struct MmaCfg {
     static constexpr int QP = DH * 2 + 16;                   // bytes per q row: bf16 plus one 16-byte skew
     static constexpr int PP = TILE * 2 + 16;                 // bytes per row of softmax weights
     static constexpr int SP = TILE + 4;                      // floats per score row
-    static constexpr int REC = DH + 2;
+    static constexpr int REC = DH + 4;
     static constexpr int NBOX = DH / 64;                     // 64-dimension (128-byte) boxes per row
     static constexpr size_t TILE_BYTES = (size_t)TILE * DH * 2;
     static constexpr size_t smem(int rows) {                 // rows = 16 or 32 operand rows
@@ -440,16 +479,19 @@ block_attention_mma_kernel(const __grid_constant__ AttnSegs segs, const AttnPara
     // (see the CUDA-core kernel above for why the requests may precede the dependency wait)
     if (tid == 0 && p.early_loads)
         for (int it = 0; it < n_tiles && it < STAGES; ++it) request(it);
-    // this thread's (row, dimension pair) items of the block; their rotation factors are constants
-    constexpr int ITEMS = ((R < MAXM ? R : (MT == 2 ? R : MAXM)) * (DH / 2) + AT - 1) / AT;
-    float rc[ITEMS], rs[ITEMS];
+    // this thread's items of the block: W neighbouring rotation pairs of a row each; their factors are constants.  (One element an
+    // item cost 17 rows of the 7B shape 3 us a layer more and 12 rows 1.5; four of a one-tile block leave too few threads at work.)
+    constexpr int W = MT == 1 ? 2 : 4, PER_ROW = DH / 2 / W, ITEMS = (R * PER_ROW + AT - 1) / AT;
+    float rc[ITEMS][W], rs[ITEMS][W];
 #pragma unroll
     for (int e = 0; e < ITEMS; ++e) {
-        const int i = tid + e * AT;
-        rc[e] = 1.f; rs[e] = 0.f;
-        if (i < m * half && p.rope_cos) {
-            const size_t at = (size_t)(n_old + (p.tree ? (int)p.tdepth[i / half] : i / half)) * half + i % half;
-            rc[e] = p.rope_cos[at]; rs[e] = p.rope_sin[at];
+        const int i = tid + e * AT, r = i / PER_ROW;
+#pragma unroll
+        for (int w = 0; w < W; ++w) { rc[e][w] = 1.f; rs[e][w] = 0.f; }
+        if (r < m && p.rope_cos) {
+            const size_t at = (size_t)(n_old + (p.tree ? (int)p.tdepth[r] : r)) * half + i % PER_ROW * W;
+            load_vec(p.rope_cos + at, rc[e]);
+            load_vec(p.rope_sin + at, rs[e]);
         }
     }
     pdl_wait();
@@ -457,48 +499,67 @@ block_attention_mma_kernel(const __grid_constant__ AttnSegs segs, const AttnPara
     if (tid == 0 && !p.early_loads)
         for (int it = 0; it < n_tiles && it < STAGES; ++it) request(it);
 
-    // ---- the block's rows: q rotated and split into its bf16 pair; k rotated, v, both rounded to bf16.
-    //      All loads first (one round trip), then the arithmetic and the stores.
+    // ---- the block's rows: q rotated and split into its bf16 pair; k rotated, v, both rounded to bf16 (by the splits whose
+    //      range holds some of them).  All loads first (one round trip), then the arithmetic and the stores.
     {
-        float qv[ITEMS][2], kv[ITEMS][2], vv[ITEMS][2];
+        const bool fresh = sg.k_new && s_end > n_old;
+        float q0[ITEMS][W], q1[ITEMS][W], k0[ITEMS][W], k1[ITEMS][W], v0[ITEMS][W], v1[ITEMS][W];
 #pragma unroll
         for (int e = 0; e < ITEMS; ++e) {
-            const int i = tid + e * AT;
-            if (i < m * half) {
-                const int r = i / half, d = i % half;
-                const float* qr = sg.q + (size_t)r * p.ldq + h * DH;
-                qv[e][0] = qr[d]; qv[e][1] = qr[d + half];
-                if (sg.k_new) {
-                    const float* kr = sg.k_new + (size_t)r * p.ld_new + h * DH;
-                    const float* vr = sg.v_new + (size_t)r * p.ld_new + h * DH;
-                    kv[e][0] = kr[d]; kv[e][1] = kr[d + half];
-                    vv[e][0] = vr[d]; vv[e][1] = vr[d + half];
+            const int i = tid + e * AT, r = i / PER_ROW, d = i % PER_ROW * W;
+            if (r < m) {
+                const float* qr = sg.q + (size_t)r * p.ldq + h * DH + d;
+                load_vec(qr, q0[e]);
+                load_vec(qr + half, q1[e]);
+                if (fresh) {
+                    const float* kr = sg.k_new + (size_t)r * p.ld_new + h * DH + d;
+                    const float* vr = sg.v_new + (size_t)r * p.ld_new + h * DH + d;
+                    load_vec(kr, k0[e]);
+                    load_vec(kr + half, k1[e]);
+                    load_vec(vr, v0[e]);
+                    load_vec(vr + half, v1[e]);
                 }
             }
         }
 #pragma unroll
         for (int e = 0; e < ITEMS; ++e) {
-            const int i = tid + e * AT;
-            if (i < m * half) {
-                const int r = i / half, d = i % half, pos = n_old + r;
-                const float c = rc[e], s = rs[e];
-                __nv_bfloat16 h0, l0, h1, l1;
-                split2(qv[e][0] * c - qv[e][1] * s, h0, l0);
-                split2(qv[e][0] * s + qv[e][1] * c, h1, l1);
-                __nv_bfloat16* qhr = reinterpret_cast<__nv_bfloat16*>(qh + r * C::QP);
-                __nv_bfloat16* qlr = reinterpret_cast<__nv_bfloat16*>(ql + r * C::QP);
-                qhr[d] = h0; qhr[d + half] = h1; qlr[d] = l0; qlr[d + half] = l1;
-                if (sg.k_new) {
-                    const __nv_bfloat16 ka = __float2bfloat16_rn(kv[e][0] * c - kv[e][1] * s);
-                    const __nv_bfloat16 kb = __float2bfloat16_rn(kv[e][0] * s + kv[e][1] * c);
-                    const __nv_bfloat16 va = __float2bfloat16_rn(vv[e][0]), vb = __float2bfloat16_rn(vv[e][1]);
-                    newK[r * DH + d] = ka; newK[r * DH + d + half] = kb;
-                    newV[r * DH + d] = va; newV[r * DH + d + half] = vb;
-                    if (pos >= s_begin && pos < s_end) {
-                        Kh[(size_t)pos * DH + d] = ka; Kh[(size_t)pos * DH + d + half] = kb;
-                        Vh[(size_t)pos * DH + d] = va; Vh[(size_t)pos * DH + d + half] = vb;
-                    }
+            const int i = tid + e * AT, r = i / PER_ROW, d = i % PER_ROW * W, pos = n_old + r;
+            if (r >= m) continue;
+            auto turn = [&](float (&a)[W], float (&b)[W]) {
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const float x = a[w], y = b[w];
+                    a[w] = x * rc[e][w] - y * rs[e][w];
+                    b[w] = x * rs[e][w] + y * rc[e][w];
                 }
+            };
+            uint32_t hi[W / 2], lo[W / 2];
+            auto put_pair = [&](const float (&v)[W], int col) {
+#pragma unroll
+                for (int w = 0; w < W; w += 2) pack_pair(v[w], v[w + 1], hi[w / 2], lo[w / 2]);
+                store_words(qh + r * C::QP + col * 2, hi);
+                store_words(ql + r * C::QP + col * 2, lo);
+            };
+            turn(q0[e], q1[e]);
+            put_pair(q0[e], d);
+            put_pair(q1[e], d + half);
+            if (fresh) {
+                turn(k0[e], k1[e]);
+                const bool mine = pos >= s_begin && pos < s_end;
+                auto put = [&](const float (&v)[W], __nv_bfloat16* smem, __nv_bfloat16* cache, int col) {
+                    uint32_t t[W / 2];
+#pragma unroll
+                    for (int w = 0; w < W; w += 2) {
+                        const __nv_bfloat162 x = __floats2bfloat162_rn(v[w], v[w + 1]);
+                        t[w / 2] = *reinterpret_cast<const uint32_t*>(&x);
+                    }
+                    store_words(smem + r * DH + col, t);
+                    if (mine) store_words(cache + (size_t)pos * DH + col, t);
+                };
+                put(k0[e], newK, Kh, d);
+                put(k1[e], newK, Kh, d + half);
+                put(v0[e], newV, Vh, d);
+                put(v1[e], newV, Vh, d + half);
             }
         }
     }
@@ -720,9 +781,9 @@ block_attention_mma_kernel(const __grid_constant__ AttnSegs segs, const AttnPara
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
                         const int d = 16 * warp + 8 * t + 2 * (lane & 3);
-                        float* dst = sg.out + (size_t)r * p.ldo + h * DH + d;
-                        dst[0] = o[mt][t][2 * hr] * inv; dst[1] = o[mt][t][2 * hr + 1] * inv;
-                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, sg.xs_r0 + r, h * DH + d, dst[0], dst[1]);
+                        const float a = o[mt][t][2 * hr] * inv, b = o[mt][t][2 * hr + 1] * inv;
+                        if (p.out_xs) store_split(p.out_xs, p.out_xs_ld, p.xs_m, sg.xs_r0 + r, h * DH + d, a, b);
+                        else *reinterpret_cast<float2*>(sg.out + (size_t)r * p.ldo + h * DH + d) = make_float2(a, b);
                     }
                 }
         }
@@ -739,8 +800,7 @@ block_attention_mma_kernel(const __grid_constant__ AttnSegs segs, const AttnPara
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     const int d = 16 * warp + 8 * t + 2 * (lane & 3);
-                    rec[r * C::REC + d] = o[mt][t][2 * hr];
-                    rec[r * C::REC + d + 1] = o[mt][t][2 * hr + 1];
+                    *reinterpret_cast<float2*>(rec + r * C::REC + d) = make_float2(o[mt][t][2 * hr], o[mt][t][2 * hr + 1]);
                 }
             }
     }
@@ -853,6 +913,10 @@ static csd_status launch_attention_block(const AttnArgs* args, int n, cudaStream
         if (append && (!b.v_new || !b.causal || b.n_keys < 1)) return CSD_ERR_INVALID_ARG;
         if ((b.rope_cos != nullptr) != (b.rope_sin != nullptr) || (b.rope_cos && !append)) return CSD_ERR_INVALID_ARG;
         if ((((uintptr_t)b.Kc) & 15) || (((uintptr_t)b.Vc) & 15)) return CSD_ERR_INVALID_ARG;
+        // (rows are read and written four values at a time)
+        if ((((uintptr_t)b.q) & 15) || (((uintptr_t)b.k_new) & 15) || (((uintptr_t)b.v_new) & 15) || (((uintptr_t)b.out) & 15) || (((uintptr_t)b.out_xs) & 15) ||
+            (b.ldq & 3) || (b.ld_new & 3) || (b.ldo & 3) || (b.out_xs_ld & 3))
+            return CSD_ERR_INVALID_ARG;
         totals[i] = b.causal ? b.n_keys + b.m - 1 : b.n_keys;
         if (totals[i] < 1 || totals[i] > b.cap) return CSD_ERR_CAPACITY;
         if (totals[i] > longest) longest = totals[i];
