@@ -519,12 +519,12 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 // ---------------------------------------------------------------------------------------------
 // resample, one kernel: a row is a thread-block cluster of up to RF_MAXC CTAs; a CTA keeps its
 // slice of the two logit vectors (position n only) in registers, so global memory is read once.
-// First exchange: per-CTA sums of the exponentials, exchanged through distributed shared memory -> the
+// First exchange: per-CTA sums of the exponentials, exchanged through distributed shared memory (a lane per CTA) -> the
 // normalisers.  Second exchange: per-CTA residual mass -> total mass S and the CTA whose slice holds
 // u2 * S.  That CTA scans its threads' sums in thread order and picks the entry.  All sums have a
 // fixed order (lanes by xor-shuffle or prefix scan, warps and CTAs in index order).
 // ---------------------------------------------------------------------------------------------
-constexpr int RF_THREADS = 512, RF_PER = 16, RF_SLICE = RF_THREADS * RF_PER;
+constexpr int RF_THREADS = 512, RF_WARPS = RF_THREADS / 32, RF_PER = 16, RF_SLICE = RF_THREADS * RF_PER;
 constexpr int RF_MAXC = 8;   // larger clusters run (one per GPC at a time) but lose to the two-pass kernels: 199 us against 145 at V = 128256
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -544,18 +544,6 @@ __device__ __forceinline__ double cluster_read_f64(const double* local, uint32_t
     return v;
 }
 
-// ordered sum over the CTA; the result is valid in every thread
-__device__ __forceinline__ double rf_block_sum(double v, double* s_warp) {
-    v = warp_sum(v);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) s_warp[warp] = v;
-    __syncthreads();
-    double tot = 0.0;
-    for (int w = 0; w < RF_THREADS / 32; ++w) tot += s_warp[w];
-    return tot;
-}
-
 __global__ void __launch_bounds__(RF_THREADS, 1)
 resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int k, int V, float temperature,
                       const RowInfo* __restrict__ info, int csize, int* __restrict__ out_tok) {
@@ -565,17 +553,16 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
     pdl_trigger();
     const RowInfo ri = info[row];
     if (ri.mode == MODE_DONE) return;                 // (the same decision in every CTA of the cluster)
-    __shared__ double s_warp[RF_THREADS / 32];
-    __shared__ double s_ex[2];                        // this CTA's contribution to the current exchange
-    __shared__ double s_scan[RF_THREADS / 32];
-    __shared__ int s_pick, s_last;
+    __shared__ double s_warp[2 * RF_WARPS], s_ex[4];  // s_ex: this CTA's contributions to the exchanges
     __shared__ double s_tab[64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     exp_table_to_shared(s_tab);
     const double invT = 1.0 / (double)temperature;
     const float* t = tl + ((long long)row * (k + 1) + ri.n) * V;
     const float* d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
     const int e0 = (int)rank * RF_SLICE + threadIdx.x * RF_PER;
-    // ---- this thread's entries, read once; their exponentials stay in registers for both rounds
+    // ---- this thread's entries, read once; their exponentials stay in registers for both rounds (formed anew in the second one they
+    //      let two CTAs share an SM, but the fp64 pipe is what a wave waits for: 64 rows, k 16, V 32000 78.8 -> 80.9 us, V 60000 24.8 -> 30.1)
     double et[RF_PER], ed[RF_PER];
     const bool vec = (V % 4 == 0) && ((((uintptr_t)t) & 15) == 0) && (!d || (((uintptr_t)d) & 15) == 0);
     double sp = 0.0, sq = 0.0;
@@ -605,74 +592,79 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
             sq += ed[j + i];
         }
     }
-    // ---- first exchange: normalisers
-    sp = rf_block_sum(sp, s_warp);
-    sq = rf_block_sum(sq, s_warp);
-    if (threadIdx.x == 0) { s_ex[0] = sp; s_ex[1] = sq; }
-    cluster_sync_all();
-    double Zp = 0.0, Zq = 0.0;
-    for (int c = 0; c < csize; ++c) { Zp += cluster_read_f64(&s_ex[0], (uint32_t)c); Zq += cluster_read_f64(&s_ex[1], (uint32_t)c); }
-    cluster_sync_all();                               // everyone has read before s_ex is reused
-    const int xn = ri.x;
-    auto resid = [&](int j, int mode) -> double {
-        return e0 + j < V ? residual_from(mode, et[j], ed[j], Zp, Zq, e0 + j == xn) : 0.0;
+    // ---- first exchange: normalisers (lanes 0-15 hold the warps', then the CTAs' Zp, lanes 16-31 their Zq)
+    auto half_sum = [](double a) {
+#pragma unroll
+        for (int o = RF_WARPS / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        return a;
     };
+    sp = warp_sum(sp); sq = warp_sum(sq);
+    if (lane == 0) { s_warp[warp] = sp; s_warp[RF_WARPS + warp] = sq; }
+    __syncthreads();
+    if (warp == 0) {
+        const double a = half_sum(s_warp[lane]);
+        if (lane % RF_WARPS == 0) s_ex[lane / RF_WARPS] = a;
+    }
+    cluster_sync_all();
+    double Zp, Zq;
+    {
+        const double a = half_sum(lane % RF_WARPS < csize ? cluster_read_f64(&s_ex[lane / RF_WARPS], (uint32_t)(lane % RF_WARPS)) : 0.0);
+        Zp = __shfl_sync(0xffffffffu, a, 0); Zq = __shfl_sync(0xffffffffu, a, RF_WARPS);
+    }
+    const int xn = ri.x;
     // ---- second exchange: masses (a second time with the target law itself if the residual is empty)
-    int mode = ri.mode;
-    double local = 0.0, S = 0.0, base = 0.0, my_mass = 0.0;
-    int pick_cta = -1, last_pos = 0;
+    int mode = ri.mode, owner = 0;
+    bool forced = false;
+    double local = 0.0, run = 0.0, head = 0.0, target = 0.0;   // this thread's mass, the warps' up to lane, the CTAs' before this one
+    auto resid = [&](int j) -> double { return e0 + j < V ? residual_from(mode, et[j], ed[j], Zp, Zq, e0 + j == xn) : 0.0; };
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
         local = 0.0;
 #pragma unroll
-        for (int j = 0; j < RF_PER; ++j) local += resid(j, mode);
-        my_mass = rf_block_sum(local, s_warp);
-        if (threadIdx.x == 0) s_ex[0] = my_mass;
+        for (int j = 0; j < RF_PER; ++j) local += resid(j);
+        const double mass_w = warp_sum(local);
+        __syncthreads();
+        if (lane == 0) s_warp[warp] = mass_w;
+        __syncthreads();
+        run = warp_scan(lane < RF_WARPS ? s_warp[lane] : 0.0, lane);
+        if (threadIdx.x == RF_WARPS - 1) s_ex[2 + pass] = run;
         cluster_sync_all();
-        S = 0.0;
-        double masses[RF_MAXC];
-        for (int c = 0; c < csize; ++c) { masses[c] = cluster_read_f64(&s_ex[0], (uint32_t)c); S += masses[c]; }
-        cluster_sync_all();
-        const bool empty = !(S > 0.0) || !isfinite(S);
-        if (empty && pass == 0 && mode != MODE_TARGET_ONLY) { mode = MODE_TARGET_ONLY; continue; }
-        const double target = ri.u2 * S;
-        double acc = 0.0;
-        for (int c = 0; c < csize; ++c) {
-            if (masses[c] > 0.0) last_pos = c;
-            if (pick_cta < 0 && acc + masses[c] > target) { pick_cta = c; base = acc; }
-            if (pick_cta < 0) acc += masses[c];
-        }
+        const double m = lane < csize ? cluster_read_f64(&s_ex[2 + pass], (uint32_t)lane) : 0.0;
+        const double incl = warp_scan(m, lane), total = __shfl_sync(0xffffffffu, incl, csize - 1);
+        if (pass == 0 && mode != MODE_TARGET_ONLY && (!(total > 0.0) || !isfinite(total))) { mode = MODE_TARGET_ONLY; continue; }
+        // the CTA whose masses reach past u2 * total; rounding may leave none, then the last one that carries mass
+        target = ri.u2 * total;
+        const unsigned past = __ballot_sync(0xffffffffu, lane < csize && incl > target);
+        const unsigned some = __ballot_sync(0xffffffffu, m > 0.0);
+        forced = past == 0;
+        owner = past ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
+        head = __shfl_sync(0xffffffffu, incl - m, (int)rank);
         break;
     }
-    const double target = ri.u2 * S;
-    int forced = 0;
-    if (pick_cta < 0) { pick_cta = last_pos; forced = 1; }
-    if ((int)rank != pick_cta) return;
-    // ---- the picking CTA: exclusive prefix of the threads' sums in thread order, then the entry
-    if (threadIdx.x == 0) { s_pick = 0x7fffffff; s_last = -1; }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double incl = local;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has read what it needs of the others
+    if ((int)rank == owner) {
+        // ---- in it the warp, then the entry: the smallest index whose cumulative mass exceeds the target; forced, or where
+        //      rounding leaves none: the last entry that carries mass
+        const unsigned past = __ballot_sync(0xffffffffu, lane < RF_WARPS && head + run > target);
+        const unsigned some = __ballot_sync(0xffffffffu, lane < RF_WARPS && s_warp[lane % RF_WARPS] > 0.0);
+        const int wpick = past && !forced ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
+        const double before = __shfl_sync(0xffffffffu, run, (wpick + 31) & 31);
+        if (warp == wpick) {
+                double cum = head + (wpick > 0 ? before : 0.0) + (warp_scan(local, lane) - local);
+            int found = 0x7fffffff, my_last = -1;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+            for (int j = 0; j < RF_PER; ++j) {
+                const double r = resid(j);
+                if (r > 0.0) my_last = e0 + j;
+                cum += r;
+                if (!forced && found == 0x7fffffff && r > 0.0 && cum > target) found = e0 + j;
+            }
+            found = __reduce_min_sync(0xffffffffu, found);
+            my_last = __reduce_max_sync(0xffffffffu, my_last);
+            if (lane == 0) out_tok[row] = found != 0x7fffffff ? found : max(my_last, 0);
+        }
     }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    double woff = 0.0;
-    for (int w = 0; w < warp; ++w) woff += s_scan[w];
-    double cum = base + woff + (incl - local);
-    int found = 0x7fffffff, my_last = -1;
-#pragma unroll
-    for (int j = 0; j < RF_PER; ++j) {
-        const double r = resid(j, mode);
-        if (r > 0.0) my_last = e0 + j;
-        cum += r;
-        if (!forced && found == 0x7fffffff && r > 0.0 && cum > target) found = e0 + j;
-    }
-    if (found != 0x7fffffff) atomicMin(&s_pick, found);
-    if (my_last >= 0) atomicMax(&s_last, my_last);
-    __syncthreads();
-    if (threadIdx.x == 0) out_tok[row] = s_pick != 0x7fffffff ? s_pick : (s_last >= 0 ? s_last : 0);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1104,7 +1096,8 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     if (nvec > 0x7fffffffLL) return CSD_ERR_UNSUPPORTED;
     const bool vec_ok = (V % 4 == 0) && (((uintptr_t)tl & 15) == 0) && (!use_d || ((uintptr_t)dl & 15) == 0);
     // One kernel while its clusters are all resident; smallest power of two that leaves a CTA at most
-    // 4096 entries (8192 beyond 32768), doubled while that leaves it 512 and the rows still fit.
+    // 4096 entries (8192 beyond 32768), doubled while that leaves it 512 and the rows still fit, halved while it takes that for all
+    // rows to be resident (k 4, V 32000: 16 rows 24.4 -> 23.1 us, 30 rows 29.5 -> 23.9; in two waves of clusters of 8 27.4 and 30.7).
     if (!greedy) {
         const csd_status ts = exp_table_ready();
         if (ts != CSD_OK) return ts;
@@ -1113,16 +1106,20 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
         int csize = 1;
         while (csize < 8 && (V + csize - 1) / csize > 4096) csize *= 2;
         if (V > 8 * 8192) csize = 16;
-        const bool wide = ((V + csize - 1) / csize + 3) / 4 * 4 > 4096;
         while (csize < 8 && rows * csize * 2 <= accept_sm_count() && V / (csize * 2) >= 512) csize *= 2;
         bool done = false;
-        csd_status s;
-        if (vec_ok)
-            s = wide ? launch_accept_row<true, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
-                     : launch_accept_row<true, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
-        else
-            s = wide ? launch_accept_row<false, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
-                     : launch_accept_row<false, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
+        csd_status s = CSD_OK;
+        for (;; csize /= 2) {
+            const int S = ((V + csize - 1) / csize + 3) / 4 * 4;
+            if (S > 8192) break;
+            if (vec_ok)
+                s = S > 4096 ? launch_accept_row<true, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
+                             : launch_accept_row<true, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
+            else
+                s = S > 4096 ? launch_accept_row<false, 8>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done)
+                             : launch_accept_row<false, 4>(tl, dl, onehot, tokens, rows, k, V, temperature, lenience, seed, step, csize, n_acc, out_tok, seq, status, st, &done);
+            if (s != CSD_OK || done || csize == 1) break;
+        }
         if (seq_written) *seq_written = done && seq;
         if (s != CSD_OK || done) return s;
     }
