@@ -7,10 +7,10 @@
 //   decide   per row: merge the pieces, run the accept tests of all positions in parallel with
 //            the Philox uniforms, find the first rejection n.
 //   resample (temperature > 0 only) per row, at position n only, in fp64 so that the chosen token
-//            does not depend on summation order or on fp32 rounding: first the per-chunk sums
-//            of the exponentials (the normalisers), then per chunk the mass of the residual
-//            max(0, p - q) (or of p after k acceptances); the CTA that finishes a row last takes
-//            the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
+//            does not depend on summation order or on fp32 rounding: the sums of both laws'
+//            exponentials (the normalisers) and the mass of the residual max(0, p - q) (or of p after
+//            k acceptances), by a cluster of CTAs a row or, beyond V = 65536, by chunks in one pass, whose
+//            last one takes the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
 #include "model.cuh"
 #include "philox.cuh"
@@ -42,6 +42,7 @@ struct __align__(16) RowInfo {
     double max_t; // max target logit at position n
     double max_q; // max draft logit at position n
     double u2;    // resampling uniform
+    float z_t, z_q;   // sums of the exponentials at position n as the stats pass has them (fp32)
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -248,7 +249,7 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
     if (tid == 0 && tickets) { tickets[row] = 0u; tickets[rows + row] = 0u; }   // for the two resample passes
     __syncthreads();
     RowInfo ri;
-    ri.n = k; ri.mode = MODE_DONE; ri.x = 0; ri.pad = 0; ri.max_t = 0; ri.max_q = 0; ri.u2 = 0;
+    ri.n = k; ri.mode = MODE_DONE; ri.x = 0; ri.pad = 0; ri.max_t = 0; ri.max_q = 0; ri.u2 = 0; ri.z_t = ri.z_q = 1.f;
     if (tid < k) {                              // a drafted id outside the vocabulary is rejected and recorded
         if (bad) set_status(status, CSD_ERR_BAD_TOKEN);
         s_x[tid] = bad ? 0 : x; s_point[tid] = point ? 1 : 0;
@@ -276,6 +277,7 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         ri.max_t = (double)s_mx[n];
         ri.max_q = s_point[n] ? 0.0 : (double)s_mx[k + 1 + n];
         ri.u2 = s_u2[n];
+        ri.z_t = s_z[n]; ri.z_q = s_point[n] ? 1.f : s_z[k + 1 + n];
     } else {
         const Philox4 r = philox4x32_10((uint32_t)k, (uint32_t)row, c2, c3, k0, k1);
         ri.mode = MODE_TARGET_ONLY;
@@ -288,13 +290,27 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 }
 
 // ---------------------------------------------------------------------------------------------
-// resample passes (fp64).  A WARP owns a chunk of 512 logits of a row (8 neighbours a lane, twice, all
-// requested at once); no block-wide synchronisation.  The fp64 pipe (about 13
-// instructions an exponential) needs 12 us a pass at 64 rows and V = 128256, the table reads from shared memory as
-// much; measured 30 and 46 us (a block of 256 threads per chunk with barriers: 38 and 54 us; 2048 logits a warp: 43
-// and 58; persistent blocks with a conflict-free copy of the table per lane: 35 and 91, the picks wait).
+// resample pass (fp64) of long vocabularies.  A WARP owns a chunk of a row (two sets of 512 logits, or eight where the scratch is small;
+// 8 neighbours a lane and load); no block-wide synchronisation.  The residual max(0, p - q) needs both normalisers, which are known
+// when every entry has been seen; but which entries it keeps is known before that for all but a few, from the fp32 sums of
+// the stats pass and a bound on their error.  So one pass sums, per chunk, both laws' exponentials (the normalisers) and, apart, those
+// of the entries that stay: a chunk's residual mass is then A Zq - B Zp, plus the few undecided entries, which are listed
+// and taken up when the normalisers are known (a chunk with more of them than its list holds is formed anew).  The warp that
+// finishes a row last does that and picks.  With a pass for the
+// normalisers and one for the masses (31 and 47 us at 64 rows, V = 128256) a call of 64 rows took k = 16 246.0 us, 233.2 so, k = 4
+// 123.6 and 107.2; 16 rows, k = 8 61.3 and 58.0.  (For rows up to V = 65536 the fused kernel below stays the faster one but for many
+// of them: 10 rows, k 8, V 50000 29.2 us, 37.6 by this pass; 64 rows, k 16, V 32000 77.7 and 76.6.)
 // Every sum has one fixed order: a lane's entries, lanes by xor-shuffle or prefix scan, chunks in index order.
 // ---------------------------------------------------------------------------------------------
+constexpr int RS_SETS = 2;             // sets of 512 logits of a chunk (times 4 where the scratch is small)
+constexpr int RS_LIST = 6;             // undecided entries a chunk can list
+constexpr unsigned short RS_NONE = 0xffff, RS_FULL = 0xfffe;
+// Distance of the laws' logarithms within which an entry is undecided.  The fp32 sums are off by at most the terms' own errors (2 ulp
+// of __expf, 1.2 more for each unit of the exponent, whose mean under a law is below ln V) and 300 roundings: 2e-5 each; the
+// comparison itself by 2^-23 of the exponents.
+constexpr float RS_BAND = 5e-5f;
+struct ChunkSums { double p, q, a, b; };   // all entries' exponentials of both laws; those of the entries that stay; later b: the mass
+
 // eight consecutive logits of a vector (two 16-byte loads when the vector allows it); past V: -inf
 __device__ __forceinline__ void load8(const float* __restrict__ src, int e0, int V, bool vec, float (&v)[8]) {
     if (vec && e0 + 7 < V) {
@@ -349,13 +365,10 @@ __device__ __forceinline__ bool last_of_row(unsigned* ticket, int nchunk, int la
     return true;
 }
 
-// pass 1: per-chunk sums of exp((t - max_t)/T) and exp((d - max_q)/T), and their totals
-// SETS: a chunk is SETS times 512 logits (1; 4 where the scratch at hand does not hold the sums of the short ones)
-template <int SETS>
-__global__ void __launch_bounds__(RS_THREADS, 3)
-resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
-                  const RowInfo* __restrict__ info, double2* __restrict__ zpart, double2* __restrict__ zsum,
-                  unsigned* __restrict__ tickets, int nchunk) {
+__global__ void __launch_bounds__(RS_THREADS, 2)
+resample_once_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
+                     const RowInfo* __restrict__ info, ChunkSums* sums, unsigned short* lists, unsigned* __restrict__ tickets,
+                     int nchunk, int sets, int* __restrict__ out_tok) {
     __shared__ double s_tab[64];
     exp_table_to_shared(s_tab);
     pdl_wait();            // the row records come from the decide pass
@@ -365,107 +378,160 @@ resample_z_kernel(const float* __restrict__ tl, const float* __restrict__ dl, in
     const int row = (int)(item / nchunk), chunk = (int)(item % nchunk);
     if (row >= rows) return;
     const RowInfo ri = info[row];
-    const double invT = 1.0 / (double)temperature;
-    const float* t = tl + ((long long)row * (k + 1) + ri.n) * V;
-    const float* d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
-    const bool vec = (V % 4 == 0) && ((((uintptr_t)t) & 15) == 0) && (!d || (((uintptr_t)d) & 15) == 0);
-    double sp = 0.0, sq = 0.0;
-#pragma unroll 1
-    for (int set = 0; set < SETS; ++set) {
-        const int e0 = (chunk * SETS + set) * RS_CHUNK + lane * 8;
-        float tv[2][8], dv[2][8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            load8(t, e0 + h * 256, V, vec, tv[h]);
-            if (d) load8(d, e0 + h * 256, V, vec, dv[h]);
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sp += exp_neg(((double)tv[h][j] - ri.max_t) * invT, s_tab);      // -inf (past V) gives 0
-        if (d) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) sq += exp_neg(((double)dv[h][j] - ri.max_q) * invT, s_tab);
-        }
-    }
-    sp = warp_sum(sp);
-    sq = warp_sum(sq);
-    double2* zrow = zpart + (long long)row * nchunk;
-    if (lane == 0) zrow[chunk] = make_double2(sp, sq);
-    if (!last_of_row(&tickets[row], nchunk, lane)) return;
-    sp = sq = 0.0;
-    for (int c = lane; c < nchunk; c += 32) { sp += __ldcg(&zrow[c].x); sq += __ldcg(&zrow[c].y); }
-    sp = warp_sum(sp);
-    sq = warp_sum(sq);
-    if (lane == 0) zsum[row] = make_double2(sp, sq);
-}
-
-// pass 2: per-chunk mass of the residual; the warp that arrives last at the row's ticket picks the token
-template <int SETS>
-__global__ void __launch_bounds__(RS_THREADS, 3)
-resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
-                     const RowInfo* __restrict__ info, const double2* __restrict__ zpart,
-                     const double2* __restrict__ zsum, double* __restrict__ rpart, unsigned* __restrict__ tickets,
-                     int nchunk, int* __restrict__ out_tok) {
-    __shared__ double s_tab[64];
-    exp_table_to_shared(s_tab);
-    pdl_wait();            // the normalisers come from the pass before this one
-    pdl_trigger();
-    const int lane = threadIdx.x & 31;
-    const long long item = (long long)blockIdx.x * (RS_THREADS / 32) + (threadIdx.x >> 5);
-    const int row = (int)(item / nchunk), chunk = (int)(item % nchunk);
-    if (row >= rows) return;
-    const RowInfo ri = info[row];
-    const double2* zrow = zpart + (long long)row * nchunk;
-    double* rrow = rpart + (long long)row * nchunk;
     ResidualCtx c;
     c.t = tl + ((long long)row * (k + 1) + ri.n) * V;
     c.d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
-    c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature;
-    c.Zp = zsum[row].x; c.Zq = zsum[row].y;
+    c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature; c.Zp = c.Zq = 0.0;
     c.mode = ri.mode; c.x = ri.x; c.tab = s_tab;
     const bool vec = (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
+    ChunkSums* mine = sums + (long long)row * nchunk;
+    unsigned short* list = lists + ((long long)row * nchunk + chunk) * RS_LIST;
     {
-        double sr = 0.0;
+        const float fT = 1.f / temperature, edge = c.d ? logf(ri.z_t) - logf(ri.z_q) : 0.f;   // stays: x_t - x_d > edge
+        const float mt = (float)ri.max_t, mq = (float)ri.max_q;
+        ChunkSums acc{0.0, 0.0, 0.0, 0.0};
+        int listed = 0;
+        float nt[8], nd[8];
+        load8(c.t, chunk * sets * RS_CHUNK + lane * 8, V, vec, nt);
+        if (c.d) load8(c.d, chunk * sets * RS_CHUNK + lane * 8, V, vec, nd);
 #pragma unroll 1
-        for (int set = 0; set < SETS; ++set) {
-            const int e0 = (chunk * SETS + set) * RS_CHUNK + lane * 8;
-            float tv[2][8], dv[2][8];
+        for (int half = 0; half < 2 * sets; ++half) {
+            const int at = (chunk * sets * 2 + half) * 256 + lane * 8;
+            float tv[8], dv[8];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                load8(c.t, e0 + h * 256, V, vec, tv[h]);
-                if (c.d) load8(c.d, e0 + h * 256, V, vec, dv[h]);
+            for (int j = 0; j < 8; ++j) { tv[j] = nt[j]; dv[j] = nd[j]; }
+            if (half + 1 < 2 * sets) {                                       // in flight while this half is summed
+                load8(c.t, at + 256, V, vec, nt);
+                if (c.d) load8(c.d, at + 256, V, vec, nd);
             }
+            unsigned open = 0;
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) sr += residual_of(c, e0 + h * 256 + j, tv[h][j], c.d ? dv[h][j] : 0.f);   // past V: et is 0
+            for (int j = 0; j < 8; ++j) {
+                const double et = exp_neg(((double)tv[j] - c.max_t) * c.invT, s_tab);         // -inf (past V) gives 0
+                acc.p += et;
+                if (c.d) {
+                    const double ed = exp_neg(((double)dv[j] - c.max_q) * c.invT, s_tab);
+                    const float over = (tv[j] - mt) * fT - (dv[j] - mq) * fT - edge;
+                    const float band = RS_BAND + 3e-7f * (fabsf((tv[j] - mt) * fT) + fabsf((dv[j] - mq) * fT));
+                    const bool stays = over > band || dv[j] == -INFINITY;
+                    acc.q += ed;
+                    acc.a += stays ? et : 0.0;
+                    acc.b += stays ? ed : 0.0;
+                    // (also what does not compare: both laws without the entry, not-a-number)
+                    if (!stays && !(over < -band) && at + j < V && !(tv[j] == -INFINITY)) open |= 1u << j;
+                } else {
+                    acc.a += at + j != c.x || c.mode != MODE_RESID_POINT ? et : 0.0;
+                }
+            }
+            while (__any_sync(0xffffffffu, open != 0)) {                     // rare
+                const unsigned who = __ballot_sync(0xffffffffu, open != 0);
+                const int place = listed + __popc(who & ((1u << lane) - 1u));
+                if (open && place < RS_LIST) list[place] = (unsigned short)(at + __ffs(open) - 1 - chunk * sets * RS_CHUNK);
+                open &= open - 1;
+                listed += __popc(who);
+            }
         }
-        sr = warp_sum(sr);
-        if (lane == 0) rrow[chunk] = sr;
+        acc.p = warp_sum(acc.p);
+        if (c.d) { acc.q = warp_sum(acc.q); acc.b = warp_sum(acc.b); }
+        acc.a = warp_sum(acc.a);
+        if (lane == 0) {
+            mine[chunk] = acc;
+            if (listed > RS_LIST) list[0] = RS_FULL;
+            else if (listed < RS_LIST) list[listed] = RS_NONE;
+        }
+        __syncwarp();
     }
     if (!last_of_row(&tickets[row], nchunk, lane)) return;
+    // ---- the normalisers, then each chunk's mass into its b
+    {
+        double sp = 0.0, sq = 0.0;
+#pragma unroll 4
+        for (int ch = lane; ch < nchunk; ch += 32) { sp += __ldcg(&mine[ch].p); sq += __ldcg(&mine[ch].q); }
+        c.Zp = warp_sum(sp);
+        c.Zq = warp_sum(sq);
+    }
+    if (c.mode != MODE_TARGET_ONLY) {
+        // four chunks a lane at a time: their sums and lists are fetched together, then one listed entry of each
+#pragma unroll 1
+        for (int base = 0; base < nchunk; base += 128) {
+            double mass[4];
+            uint32_t words[4][RS_LIST / 2];
+            bool open[4], full[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int ch = min(base + 32 * u + lane, nchunk - 1);
+                const uint32_t* from = reinterpret_cast<const uint32_t*>(lists + ((long long)row * nchunk + ch) * RS_LIST);
+                const double a = __ldcg(&mine[ch].a), b = c.d ? __ldcg(&mine[ch].b) : 0.0;
+#pragma unroll
+                for (int w = 0; w < RS_LIST / 2; ++w) words[u][w] = c.d ? __ldcg(from + w) : 0xffffffffu;
+                mass[u] = c.d ? a * c.Zq - b * c.Zp : a;
+                full[u] = base + 32 * u + lane < nchunk && (words[u][0] & 0xffffu) == RS_FULL;
+                open[u] = base + 32 * u + lane < nchunk && !full[u];
+            }
+#pragma unroll
+            for (int i = 0; i < RS_LIST; ++i) {
+                float tv[4], dv[4];
+                int at[4];
+                bool any = false;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned e = (words[u][i / 2] >> (16 * (i & 1))) & 0xffffu;
+                    open[u] = open[u] && e != RS_NONE;
+                    at[u] = (base + 32 * u + lane) * sets * RS_CHUNK + (int)e;
+                    tv[u] = dv[u] = 0.f;
+                    if (open[u]) { tv[u] = c.t[at[u]]; dv[u] = c.d[at[u]]; any = true; }
+                }
+                if (!__any_sync(0xffffffffu, any)) break;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (open[u]) mass[u] += residual_of(c, at[u], tv[u], dv[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int ch = base + 32 * u + lane;
+                if (ch < nchunk && !full[u]) __stcg(&mine[ch].b, mass[u] > 0.0 ? mass[u] : 0.0);     // (rounding of the difference)
+                unsigned todo = __ballot_sync(0xffffffffu, full[u]);
+                while (todo) {                                               // a chunk of laws that nearly agree throughout
+                    const int ch2 = base + 32 * u + __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    double sr = 0.0;
+#pragma unroll 1
+                    for (int half = 0; half < 2 * sets; ++half) {
+                        const int at = (ch2 * sets * 2 + half) * 256 + lane * 8;
+                        float tv[8], dv[8];
+                        load8(c.t, at, V, vec, tv);
+                        load8(c.d, at, V, vec, dv);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) sr += residual_of(c, at + j, tv[j], dv[j]);
+                    }
+                    sr = warp_sum(sr);
+                    if (lane == 0) __stcg(&mine[ch2].b, sr);
+                }
+            }
+        }
+        __threadfence_block();
+        __syncwarp();
+    }
     // ---- which chunk holds u2 * S: a lane owns neighbouring chunks; a second time with the target law itself if the
     //      residual is empty.  Rounding may leave none, then the last chunk that carries mass.
     const int each = (nchunk + 31) / 32, c_lo = min(nchunk, lane * each), c_hi = min(nchunk, c_lo + each);
-    double mine = 0.0, incl = 0.0, S = 0.0;
-    auto mass_of = [&](int ch) -> double { return c.mode == MODE_TARGET_ONLY ? __ldcg(&zrow[ch].x) : __ldcg(rrow + ch); };
+    double own = 0.0, incl = 0.0, S = 0.0;
+    auto mass_of = [&](int ch) -> double { return c.mode == MODE_TARGET_ONLY ? __ldcg(&mine[ch].p) : __ldcg(&mine[ch].b); };
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-        mine = 0.0;
-        for (int ch = c_lo; ch < c_hi; ++ch) mine += mass_of(ch);
-        incl = warp_scan(mine, lane);
+        own = 0.0;
+#pragma unroll 4
+        for (int ch = c_lo; ch < c_hi; ++ch) own += mass_of(ch);
+        incl = warp_scan(own, lane);
         S = __shfl_sync(0xffffffffu, incl, 31);
         if (pass == 0 && c.mode != MODE_TARGET_ONLY && (!(S > 0.0) || !isfinite(S))) { c.mode = MODE_TARGET_ONLY; continue; }
         break;
     }
     const double target = ri.u2 * S;
-    const unsigned past = __ballot_sync(0xffffffffu, incl > target), some = __ballot_sync(0xffffffffu, mine > 0.0);
+    const unsigned past = __ballot_sync(0xffffffffu, incl > target), some = __ballot_sync(0xffffffffu, own > 0.0);
     const bool forced = past == 0;
     const int src = past ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
-    double cum = incl - mine;
+    double cum = incl - own;
     int pick_chunk = c_lo;
     if (lane == src) {
         int last_pos = c_lo, hit = -1;
@@ -477,7 +543,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         }
         if (hit < 0) {                                  // the last chunk with mass, from its own start
             hit = last_pos;
-            cum = incl - mine;
+            cum = incl - own;
             for (int ch = c_lo; ch < last_pos; ++ch) cum += mass_of(ch);
         }
         pick_chunk = hit;
@@ -487,7 +553,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
     // ---- the entry: smallest index whose cumulative mass exceeds the target, else the last that carries mass
     int pick = -1, last = -1;
 #pragma unroll 1
-    for (int e = pick_chunk * SETS * RS_CHUNK; e < min(V, (pick_chunk + 1) * SETS * RS_CHUNK) && pick < 0; e += 256) {
+    for (int e = pick_chunk * sets * RS_CHUNK; e < min(V, (pick_chunk + 1) * sets * RS_CHUNK) && pick < 0; e += 256) {
         const int at = e + lane * 8;
         float tv[8], dv[8];
         load8(c.t, at, V, vec, tv);
@@ -958,8 +1024,8 @@ static AcceptLayout accept_layout(int rows, int k, int V, int sets = 1) {
     return L;
 }
 
-// The layout for `room` bytes of scratch: the resample passes keep 24 bytes per row and chunk, of 512 logits where that fits, else of
-// 2048.  (V = 128256, 512 / 2048: 64 rows, k = 4 123 / 131 us a call, k = 16 246 / 257; 320 rows, k = 1 315 / 274.)
+// The layout for `room` bytes of scratch: 24 bytes per row and 512 logits for the resample's sums and lists (44 bytes a chunk of
+// 1024) where that fits, else per 2048.  (V = 128256, 512 / 2048: 64 rows, k = 4 123 / 131 us a call, k = 16 246 / 257; 320 rows, k = 1 315 / 274.)
 static csd_status accept_layout_in(int rows, int k, int V, size_t room, AcceptLayout& L) {
     const AcceptLayout least = accept_layout(rows, k, V, 4);
     if (room < least.total) return CSD_ERR_CAPACITY;
@@ -1083,9 +1149,6 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
                              cudaStream_t st, int32_t* seq = nullptr, bool* seq_written = nullptr) {
     StatPartial* part = (StatPartial*)(ws + L.part_off);
     RowInfo* info = (RowInfo*)(ws + L.info_off);
-    double2* zpart = (double2*)(ws + L.z_off);
-    double* rpart = (double*)(ws + L.r_off);
-    double2* zsum = (double2*)(ws + L.zsum_off);
     unsigned* tickets = (unsigned*)(ws + L.ticket_off);
     const bool greedy = temperature == 0.f;
     const float invT = greedy ? 1.f : 1.f / temperature;
@@ -1156,15 +1219,14 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
                                     (int*)out_tok));
         count_launch();
     } else if (!greedy) {
-        const dim3 g2((unsigned)(((long long)rows * L.nchunk_r + RS_THREADS / 32 - 1) / (RS_THREADS / 32)));
-        PdlLaunch lz(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lz.cfg, L.sets == 1 ? resample_z_kernel<1> : resample_z_kernel<4>, tl, dl, rows, k, V, temperature,
-                                    (const RowInfo*)info, zpart, zsum, tickets, L.nchunk_r));
-        PdlLaunch lp(g2, dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, L.sets == 1 ? resample_pick_kernel<1> : resample_pick_kernel<4>, tl, dl, rows, k, V,
-                                    temperature, (const RowInfo*)info, (const double2*)zpart, (const double2*)zsum, rpart,
-                                    tickets + rows, L.nchunk_r, (int*)out_tok));
-        count_launch(2);
+        const int nch = (L.nchunk_r + RS_SETS - 1) / RS_SETS;     // chunks of twice the layout's
+        ChunkSums* sums = (ChunkSums*)(ws + L.z_off);
+        unsigned short* lists = (unsigned short*)(sums + (size_t)rows * nch);
+        if ((size_t)rows * nch * (sizeof(ChunkSums) + RS_LIST * 2) > L.zsum_off - L.z_off) return CSD_ERR_UNSUPPORTED;   // (fewer than six chunks)
+        PdlLaunch lo(dim3((unsigned)(((long long)rows * nch + RS_THREADS / 32 - 1) / (RS_THREADS / 32))), dim3(RS_THREADS), 0, st);
+        CSD_CUDA(cudaLaunchKernelEx(&lo.cfg, resample_once_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, sums, lists,
+                                    tickets, nch, L.sets * RS_SETS, (int*)out_tok));
+        count_launch();
     }
     CSD_CUDA(cudaGetLastError());
     return CSD_OK;

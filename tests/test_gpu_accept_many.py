@@ -64,3 +64,24 @@ def test_scratch_that_holds_anything_and_calls_in_a_row(b):
     bad[7, 2] = 20000
     b.csd_spec_accept(t, d, bad, 1.0, seed=3)
     assert b.csd_device_status() == 6                           # a token outside the vocabulary is recorded
+
+
+@pytest.mark.parametrize("V", [65537, 70001, 131584])
+@pytest.mark.parametrize("sigma", [0.0, 1e-5, 1e-3, 0.03, 0.5])
+def test_laws_that_nearly_agree(b, orc, V, sigma):
+    """Long vocabularies: the entries the residual keeps are told before the normalisers are known but where the laws nearly agree
+    (within 5e-5 of their logarithms); those are listed, six a chunk of 1024, and chunks with more are summed anew.  Two entries
+    of each draft law are swapped, the drafted one gaining, so that it is refused while all others agree up to sigma."""
+    rows, k = 20, 2
+    t, _, _ = workloads.accept_case(rows, k, V, 0.5, seed=V, device="cuda")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(V)
+    d = t[:, :k].clone()
+    top = d.argmax(-1, keepdim=True)
+    low = torch.randint(0, V, (rows, k, 1), generator=g, device="cuda")
+    low = torch.where(low == top, (low + 1) % V, low)
+    hi_v, lo_v = d.gather(-1, top), d.gather(-1, low)
+    d.scatter_(-1, top, lo_v).scatter_(-1, low, hi_v)
+    d = (d + sigma * torch.randn(d.shape, generator=g, device="cuda")).contiguous()
+    compare(b, orc, t, d, low[..., 0].to(torch.int32).contiguous(), 1.0)
+    compare(b, orc, t, d, low[..., 0].to(torch.int32).contiguous(), 0.6)
