@@ -1025,7 +1025,7 @@ static AcceptLayout accept_layout(int rows, int k, int V, int sets = 1) {
 }
 
 // The layout for `room` bytes of scratch: 24 bytes per row and 512 logits for the resample's sums and lists (44 bytes a chunk of
-// 1024) where that fits, else per 2048.  (V = 128256, 512 / 2048: 64 rows, k = 4 123 / 131 us a call, k = 16 246 / 257; 320 rows, k = 1 315 / 274.)
+// 1024) where that fits, else per 2048.  (V = 128256: 64 rows, k = 4 107 / 125 us a call, k = 16 233 / 250; 320 rows, k = 1 244 / 241.)
 static csd_status accept_layout_in(int rows, int k, int V, size_t room, AcceptLayout& L) {
     const AcceptLayout least = accept_layout(rows, k, V, 4);
     if (room < least.total) return CSD_ERR_CAPACITY;
@@ -1118,8 +1118,16 @@ static csd_status launch_accept_row(const float* tl, const float* dl, const int*
     // (a CTA takes in about 40 GB/s here: beyond about 320 KB of slices the stats pass over all SMs is faster; one row,
     // V = 128256: k = 4, 289 KB, 29.6 us against 34.3; k = 8, 545 KB, 35.0 against 34.3)
     if ((long long)nvec * S * 4 > 320 * 1024 || row_clusters<VEC, PER>(csize) < rows) return CSD_OK;
-    int pieces = (AR_WARPS + nvec - 1) / nvec;           // enough pieces for every warp, of at least 1024 logits
+    // pieces of a vector's slice, of at least 1024 logits: enough for every warp, fewer where that saves batches of the busiest warp (2 rows,
+    // k 6, V 50000, 13 vectors: 39 tasks for 32 warps 19.7 us, 26 of them 17.8)
+    auto batches = [&](int n) {
+        const int plen = (S + n * 128 - 1) / (n * 128) * 128;
+        return (nvec * n + AR_WARPS - 1) / AR_WARPS * ((plen + ST_SUB - 1) / ST_SUB);
+    };
+    int pieces = (AR_WARPS + nvec - 1) / nvec;
     if (pieces > (S + ST_SUB - 1) / ST_SUB) pieces = (S + ST_SUB - 1) / ST_SUB;
+    for (int n = pieces - 1; n >= 1; --n)
+        if (batches(n) < batches(pieces)) pieces = n;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
     cudaLaunchAttribute attr[2];
     cfg.gridDim = dim3((unsigned)(rows * csize)); cfg.blockDim = dim3(AR_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
@@ -1159,7 +1167,7 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     if (nvec > 0x7fffffffLL) return CSD_ERR_UNSUPPORTED;
     const bool vec_ok = (V % 4 == 0) && (((uintptr_t)tl & 15) == 0) && (!use_d || ((uintptr_t)dl & 15) == 0);
     // One kernel while its clusters are all resident; smallest power of two that leaves a CTA at most
-    // 4096 entries (8192 beyond 32768), doubled while that leaves it 512 and the rows still fit, halved while it takes that for all
+    // 4096 entries and 320 KB, doubled while that leaves it 512 and the rows still fit, halved while it takes that for all
     // rows to be resident (k 4, V 32000: 16 rows 24.4 -> 23.1 us, 30 rows 29.5 -> 23.9; in two waves of clusters of 8 27.4 and 30.7).
     if (!greedy) {
         const csd_status ts = exp_table_ready();
@@ -1168,7 +1176,8 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     if (V <= AR_MAXC * 8192) {
         int csize = 1;
         while (csize < 8 && (V + csize - 1) / csize > 4096) csize *= 2;
-        if (V > 8 * 8192) csize = 16;
+        // (clusters of 16: 2 rows, k 6, V 50000 24.0 -> 17.8 us, 1 row, k 4, V 64000 22.0 -> 17.8, k 16, V 32000 23.3 -> 21.2; k 4, V 32000 13.6 -> 14.2)
+        if (V > 8 * 4096 || (csize == 8 && (long long)(use_d ? 2 * k + 1 : k + 1) * V / 8 * 4 > 320 * 1024)) csize = 16;
         while (csize < 8 && rows * csize * 2 <= accept_sm_count() && V / (csize * 2) >= 512) csize *= 2;
         bool done = false;
         csd_status s = CSD_OK;
