@@ -8,21 +8,19 @@
 // neighbouring SMs: tcgen05.mma with cta_group::2, 128 weight rows and half of the tokens' terms staged by
 // each CTA; both terms are accumulated into the same fp32 columns, up to 128 tokens side by side.
 //
-// What bounds it: the bytes an SM takes in (about 70 GB/s) and the tensor pipe, nearly level.  A full tile takes
-// 48 KB per 1024 tensor clocks and SM; at 1024 rows, N 12288, K 4096 the copies alone need 114 us, the MMAs alone
-// 89 us, the kernel 157 us (1.29 PFLOP/s of two-term products, 77 % of the measured one-term cuBLAS rate).  One CTA per 84 weight
-// rows and 128 tokens instead of pairs takes in 32 KB of token terms for every 11 KB of weights: 8 x 46 us.  At 128 rows both
-// divisions need 40 us; below, the weight stream bounds.
+// What bounds it: beyond 128 tokens the MMAs and what they read from shared memory (a full tile: 112 KB per 1024 tensor clocks and SM, of
+// 128 KB that it can give; copies into it 48 KB, where each of 148 SMs can draw 130 GB/s from L2), under the power limit;
+// 1024 rows, N 12288, K 4096: MMAs alone 89 us, the kernel 157 us (1.29 PFLOP/s of two-term products, 77 % of the measured one-term cuBLAS
+// rate).  Up to 128 tokens the weight stream and, since a CTA fills an SM, each launch's start from an empty ring and its finish:
+// q|k|v of the 7B shape at 64 tokens 28 us, of which 18 are the stream.
 //
 // fp32 accumulation.  The tensor core loses a little with every add of a long chain, so after WG_DRAIN
 // K blocks (64 adds) the accumulator set is added into fp32 registers of the epilogue warps while
 // the MMAs continue on the other set, and the epilogue of one tile overlaps the MMAs of the next.  Error against fp64 at K = 4096 to
-// 11008 (csd_linear, 18 to 128 rows): 2.7e-6, of which the two-term form itself leaves 2.45e-6.  (Chains of 256 to 700 adds left
-// 2.45e-6 at 18 rows to 5.0e-6 at 128.)  Tiles of up to 32 tokens sum the low terms' products in columns of their own: 2.5e-6, and
-// being short the kernel of such tiles is the faster one as well (8 layers of the 7B shape, 20 tokens: 1001 us together, 965 so).  Sets
-// of 4 K blocks, which leave 2.5e-6 at every size, cost 2 to 7 % a GEMM.
+// 12288 (csd_linear, 18 to 128 rows, where the low terms' products have columns of their own): 2.50e-6, of which the two-term form
+// itself leaves 2.45e-6; both terms in one chain 2.7e-6.  Sets of 4 K blocks, which leave 2.5e-6 either way, cost 2 to 7 % a GEMM.
 //
-// Roles inside a CTA (384 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 of the pair's first CTA
+// Roles inside a CTA (384 threads): lane 0 of warps 0 and 2 issues TMA (weights, row terms), warp 1 lane 0 of the pair's first CTA
 // issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
 // tokens) and finish tiles; they hold 128 accumulators each, hence the register split.  Every
 // mbarrier wait is bounded; on a time-out the CTA records CSD_ERR_TIMEOUT, stops, frees its tensor
