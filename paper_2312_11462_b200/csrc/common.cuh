@@ -102,6 +102,13 @@ __device__ __forceinline__ void split3(float x, uint16_t& b1, uint16_t& b2, uint
     b3 = float_to_bf16_bits(r1 - bf16_bits_to_float(b2));
 }
 
+// The kernels that open a forward, and the splits in front of csd_linear's GEMMs, zero the tickets of the GEMMs behind them: a launch
+// that has given up waiting (CSD_ERR_TIMEOUT) leaves any count there.  After pdl_wait; 2D grid of THREADS-thread blocks.
+template <int THREADS = 128>
+__device__ __forceinline__ void clear_words(unsigned* words, int count) {
+    for (int i = (int)((blockIdx.y * gridDim.x + blockIdx.x) * THREADS + threadIdx.x); i < count; i += (int)(gridDim.x * gridDim.y * THREADS)) words[i] = 0u;
+}
+
 // 128-bit streaming load that does not allocate in L1 (weights are read exactly once)
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     uint4 v;

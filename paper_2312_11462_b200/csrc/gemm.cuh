@@ -18,7 +18,7 @@ struct LinearArgs {
     int ldy = 0;
     int epilogue = EPI_STORE;
     float* partial = nullptr;            // split-K scratch (linear_scratch_bytes)
-    unsigned* tickets = nullptr;         // zero-initialised, linear_ticket_count entries
+    unsigned* tickets = nullptr;         // zeroed since a launch on them last gave up; linear_ticket_count entries
     // ---- tensor-core path only: the block's rows as three bf16 terms x = b1 + b2 + b3
     __nv_bfloat16* xs = nullptr;         // [3m][K] row-major, row = term * m + r
     bool xs_ready = false;               // false: launch_linear splits X (times gain) into xs first
@@ -36,6 +36,7 @@ struct LinearArgs {
     const __nv_bfloat16* embed = nullptr;
     int vocab = 0;
     float* x_out = nullptr;
+    int n_clear = 0;                     // the first n_clear tickets are zeroed on the way
 };
 
 int split_rows(int m);                   // 16, 32, 48 or 64 operand rows hold the 3m terms

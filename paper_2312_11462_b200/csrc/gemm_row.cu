@@ -20,8 +20,8 @@ constexpr size_t RW_SMEM_MAX = 110 * 1024; // two CTAs share an SM
 
 struct RowParams {
     const __nv_bfloat16* W; const __nv_bfloat16* W2; const float* X; const __nv_bfloat16* gain; float* Y;
-    const int32_t* tokens; const __nv_bfloat16* embed; float* x_out; int* status;
-    int N, K, ldx, ldy, m, steps, epilogue, vocab;
+    const int32_t* tokens; const __nv_bfloat16* embed; float* x_out; int* status; unsigned* tickets;
+    int N, K, ldx, ldy, m, steps, epilogue, vocab, n_clear;
     float eps;
 };
 
@@ -93,6 +93,7 @@ row_gemm_kernel(const RowParams p) {
         for (int i = tid * 4; i < M * KP; i += RW_THREADS * 4) *reinterpret_cast<float4*>(xs + i) = make_float4(0.f, 0.f, 0.f, 0.f);
     pdl_wait();
     pdl_trigger();
+    if (GATHER) clear_words<RW_THREADS>(p.tickets, p.n_clear);   // (the first launch of a forward)
     __syncthreads();
 
     // ---- the block's rows: task (row, step) to a warp, four tasks' loads in flight; then each lane scales what it
@@ -266,6 +267,7 @@ csd_status launch_linear_row(const LinearArgs& a, cudaStream_t st) {
     RowParams rp;
     rp.W = a.W; rp.W2 = a.W2; rp.X = a.X; rp.gain = a.gain; rp.Y = a.Y; rp.N = a.N; rp.K = a.K; rp.ldx = a.ldx; rp.ldy = a.ldy;
     rp.tokens = a.tokens; rp.embed = a.embed; rp.x_out = a.x_out; rp.vocab = a.vocab; rp.status = a.tokens ? status_word_device() : nullptr;
+    rp.tickets = a.tickets; rp.n_clear = a.n_clear;
     rp.m = a.m; rp.steps = (a.K + RW_STEP - 1) / RW_STEP; rp.epilogue = a.epilogue; rp.eps = a.eps;
 #define CSD_ROW_CASE(MM) case MM: return dual ? launch_row_m<MM, true>(rp, st) : launch_row_m<MM, false>(rp, st);
     switch (row_m(a.m)) {

@@ -510,7 +510,7 @@ skinny_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_cons
                     while (ld_acquire_gpu(ticket) < want) {
                         if (++spins > SPIN_LIMIT) { *abort_flag = 1; break; }
                     }
-                    *ticket = 0u;                       // everyone has arrived: ready for the next launch
+                    *ticket = 0u;                       // ready for the next launch, if everyone has arrived (clear_words)
                 }
                 __syncwarp();
                 // the other parts in CTA order (deterministic); as many contributors' loads in flight together as about
@@ -706,6 +706,7 @@ split_rows_kernel(const float* __restrict__ X, int ldx, int K, int m, const __nv
     if (threadIdx.x == 0 && ssq) ssq[(size_t)blockIdx.x * m + r] = (part[0] + part[1]) + (part[2] + part[3]);
 }
 
+int tc_ticket_count(int N) { return (N + TILE_N - 1) / TILE_N * 8; }
 int split_rows(int m) { return npad_for(m); }
 int split_ssq_entries(int K) { return (K + 1023) / 1024; }
 
@@ -727,7 +728,7 @@ csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st) {
     pdl_config(cfg, attr, dim3((unsigned)split_ssq_entries(a.K), (unsigned)a.m), dim3(128), 0, st);
     CSD_CUDA(cudaLaunchKernelEx(&cfg, split_rows_kernel, a.X, a.ldx, a.K, a.m, a.gain, a.xs,
                                 a.gain ? a.ssq : (float*)nullptr, a.clear_tickets ? a.tickets : (unsigned*)nullptr,
-                                a.clear_tickets ? (a.N + TILE_N - 1) / TILE_N * 8 : 0));
+                                a.clear_tickets ? tc_ticket_count(a.N) : 0));
     count_launch();
     return CSD_OK;
 }

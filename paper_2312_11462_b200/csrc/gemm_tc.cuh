@@ -7,6 +7,7 @@ namespace csd {
 int tc_sm_count();
 bool tc_supported(int m, int N, int K, bool dual);
 size_t tc_scratch_bytes(int m, int N, int K, bool dual);
+int tc_ticket_count(int N);
 csd_status launch_linear_tc(const LinearArgs& a, cudaStream_t st);
 csd_status launch_split_rows(const LinearArgs& a, cudaStream_t st);   // a.X (times a.gain) -> a.xs, a.ssq
 
@@ -38,7 +39,7 @@ struct WideArgs {
     const __nv_bfloat16* out_gain = nullptr;
     float* out_ssq = nullptr;            // optional: [wide_ssq_pieces(N)][m] pieces of the sums of squares of the rows of Y
     float* partial = nullptr;            // scratch of wide_partial_bytes(m) for partial sums
-    unsigned* tickets = nullptr;         // zero-initialised, wide_ticket_count(m, N) entries
+    unsigned* tickets = nullptr;         // zeroed since a launch on them last gave up; wide_ticket_count(m, N) entries
 };
 bool wide_supported(int m, int N, int K, bool dual);
 int wide_ssq_pieces(int N);

@@ -436,7 +436,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll 1
                     while (ld_acquire_gpu(&p.tickets[2 * tile + rank]) < want)
                         if (++spins > SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
-                    p.tickets[2 * tile + rank] = 0u;          // everyone has arrived: ready for the next launch
+                    p.tickets[2 * tile + rank] = 0u;          // ready for the next launch, if everyone has arrived (clear_words)
                     __threadfence();
                     asm volatile("fence.proxy.async;" ::: "memory");
                 }
@@ -487,7 +487,7 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll 1
                     while (ld_acquire_gpu(&p.tickets[2 * pair + rank]) < want)
                         if (++spins > SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
-                    p.tickets[2 * pair + rank] = 0u;          // everyone has arrived: ready for the next launch
+                    p.tickets[2 * pair + rank] = 0u;          // ready for the next launch, if everyone has arrived (clear_words)
                     __threadfence();
                 }
                 asm volatile("bar.sync 1, 256;" ::: "memory");    // (the tile's scale factors are written as well)

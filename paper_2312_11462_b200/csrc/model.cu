@@ -14,9 +14,10 @@ namespace csd {
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128)
 embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict__ E, int V, int d,
-                             float* __restrict__ x, int* status) {
+                             float* __restrict__ x, int* status, unsigned* __restrict__ tickets, int n_tickets) {
     pdl_wait();
     pdl_trigger();
+    clear_words(tickets, n_tickets);
     const int r = blockIdx.x;                  // (a source may have more tokens than a grid has room for in y)
     int t = tokens[r];
     if (t < 0 || t >= V) {
@@ -31,10 +32,10 @@ embed_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict
     *reinterpret_cast<float4*>(dst + 4) = make_float4(bf16lo(e.z), bf16hi(e.z), bf16lo(e.w), bf16hi(e.w));
 }
 
-static csd_status launch_embed(const int32_t* tokens, const __nv_bfloat16* E, int V, int d, int m, float* x, int* status,
-                               cudaStream_t st) {
+static csd_status launch_embed(csd_model* M, const int32_t* tokens, int m, float* x, cudaStream_t st) {
+    const int d = M->cfg.d_model;
     PdlLaunch L(dim3((unsigned)m, (unsigned)((d + 1023) / 1024)), dim3(128), 0, st);
-    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_kernel, tokens, E, V, d, x, status));
+    CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_kernel, tokens, M->embed, M->cfg.vocab, d, x, M->status, M->gemm_tickets, M->n_tickets));
     count_launch();
     return CSD_OK;
 }
@@ -45,9 +46,10 @@ static csd_status launch_embed(const int32_t* tokens, const __nv_bfloat16* E, in
 __global__ void __launch_bounds__(128)
 embed_split_kernel(const int32_t* __restrict__ tokens, const __nv_bfloat16* __restrict__ E, int V, int d, int m,
                    const __nv_bfloat16* __restrict__ gain, float* __restrict__ x, __nv_bfloat16* __restrict__ xs,
-                   float* __restrict__ ssq, int* status) {
+                   float* __restrict__ ssq, int* status, unsigned* __restrict__ tickets, int n_tickets) {
     pdl_wait();
     pdl_trigger();
+    clear_words(tickets, n_tickets);
     const int r = blockIdx.y, k = (blockIdx.x * 128 + threadIdx.x) * 8;
     int t = tokens[r];
     if (t < 0 || t >= V) {
@@ -222,7 +224,7 @@ struct WsLayout {
         buckets, gemm_partial, gemm_tickets, xs_tmp, ssq_tmp, xs_x, xs_attn, xs_act, ssq_x,
         wx, wqkv, wattn, wxs_x, wxs_attn, wxs_act, wssq, wpart, total;
     bool wide;
-    int wide_rows;
+    int wide_rows, n_tickets;
     size_t layer_kv, layer_x;
 };
 
@@ -279,6 +281,9 @@ static WsLayout ws_layout(const csd_model_config& c) {
     const size_t widest = 3 * di > ff ? (3 * di > d ? 3 * di : d) : (ff > d ? ff : d);        // widest matrix of a wide pass
     if (L.wide && (size_t)wide_ticket_count(L.wide_rows, (int)widest) > tickets) tickets = (size_t)wide_ticket_count(L.wide_rows, (int)widest);
     L.gemm_tickets = put(tickets * 4);
+    // words in which a launch that gives up may leave a count: those of the kernels that wait for one another's parts
+    L.n_tickets = tc_ticket_count((int)nmax);
+    if (L.wide && wide_ticket_count(L.wide_rows, (int)widest) > L.n_tickets) L.n_tickets = wide_ticket_count(L.wide_rows, (int)widest);
     const size_t kmax = d > di ? (d > ff ? d : ff) : (di > ff ? di : ff);
     L.xs_tmp = put(3 * R * kmax * 2);
     L.ssq_tmp = put((size_t)split_ssq_entries((int)kmax) * R * 4);
@@ -361,7 +366,7 @@ static csd_status linear(csd_model* M, const __nv_bfloat16* W, const __nv_bfloat
             a.xs = const_cast<__nv_bfloat16*>(o->xs_in); a.xs_ready = true;
             a.ssq = const_cast<float*>(o->ssq_in); a.ssq_cnt = o->ssq_cnt;
         }
-        if (o->tokens) { a.tokens = o->tokens; a.embed = M->embed; a.vocab = M->cfg.vocab; a.x_out = M->x; }
+        if (o->tokens) { a.tokens = o->tokens; a.embed = M->embed; a.vocab = M->cfg.vocab; a.x_out = M->x; a.n_clear = M->n_tickets; }
         a.out_xs = o->out_xs; a.out_ld = o->out_ld; a.out_gain = o->out_gain; a.out_ssq = o->out_ssq;
         if (o->out_ssq == M->ssq_x) M->ssq_x_cnt = linear_ssq_pieces(m, N, K, W2 != nullptr);
     }
@@ -470,7 +475,7 @@ static csd_status wide_decoder_pass(csd_model* M, const int32_t* tokens, int m, 
     const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, ff = c.d_ff;
     {
         ProfScope ps(M, 2, st);
-        CSD_TRY(launch_embed(tokens, M->embed, c.vocab, d, m, M->wx, M->status, st));
+        CSD_TRY(launch_embed(M, tokens, m, M->wx, st));
     }
     int cnt = 0;                       // pieces in wssq that describe the rows in wxs_x (0: wxs_x not current)
     for (int l = 0; l < c.n_layers; ++l) {
@@ -644,7 +649,7 @@ extern "C" csd_status csd_model_create(const csd_model_config* cfg, const void* 
     M->layer_kv = L.layer_kv; M->layer_x = L.layer_x;
     M->x = (float*)(ws + L.x); M->qkv = (float*)(ws + L.qkv); M->attn = (float*)(ws + L.attn);
     M->act = (float*)(ws + L.act);
-    M->gemm_partial = (float*)(ws + L.gemm_partial); M->gemm_tickets = (unsigned*)(ws + L.gemm_tickets);
+    M->gemm_partial = (float*)(ws + L.gemm_partial); M->gemm_tickets = (unsigned*)(ws + L.gemm_tickets); M->n_tickets = L.n_tickets;
     M->xs_tmp = (__nv_bfloat16*)(ws + L.xs_tmp); M->ssq_tmp = (float*)(ws + L.ssq_tmp);
     M->xs_x = (__nv_bfloat16*)(ws + L.xs_x); M->xs_attn = (__nv_bfloat16*)(ws + L.xs_attn);
     M->xs_act = (__nv_bfloat16*)(ws + L.xs_act); M->ssq_x = (float*)(ws + L.ssq_x);
@@ -734,7 +739,7 @@ extern "C" csd_status csd_encoder_forward(csd_model* M, const int32_t* enc_token
     cudaStream_t st = (cudaStream_t)stream;
     const int d = c.d_model, H = c.n_heads, Dh = c.d_head, di = M->di, E = c.max_enc_len;
     const int CH = 16;
-    CSD_TRY(launch_embed(enc_tokens_dev, M->embed, c.vocab, d, n, M->xenc, M->status, st));
+    CSD_TRY(launch_embed(M, enc_tokens_dev, n, M->xenc, st));
     if (M->wide && gemm_path() != 1 && n > CSD_MAX_ROWS) {      // large model: wide blocks
         CSD_TRY(wide_encoder(M, n, st));
         M->enc_len = n;
@@ -877,12 +882,12 @@ static csd_status review_forward_impl(csd_model* M, const int32_t* block_tokens_
         if ((d & 7) == 0 && linear_uses_tensor_cores(m, fused_qkv ? 3 * di : di, d, false)) {
             PdlLaunch L(dim3((unsigned)split_ssq_entries(d), (unsigned)m), dim3(128), 0, st);
             CSD_CUDA(cudaLaunchKernelEx(&L.cfg, embed_split_kernel, block_tokens_dev, M->embed, V, d, m, y0.norm1, M->x, M->xs_x,
-                                        M->ssq_x, M->status));
+                                        M->ssq_x, M->status, M->gemm_tickets, M->n_tickets));
             M->ssq_x_cnt = split_ssq_entries(d);
             x_ready = true;
             count_launch();
         } else {
-            CSD_TRY(launch_embed(block_tokens_dev, M->embed, V, d, m, M->x, M->status, st));
+            CSD_TRY(launch_embed(M, block_tokens_dev, m, M->x, st));
         }
     }
     const int ff = c.d_ff;

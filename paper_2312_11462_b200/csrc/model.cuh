@@ -28,6 +28,7 @@ struct csd_model {
     float *rope_c = nullptr, *rope_s = nullptr, *dec_bias = nullptr, *enc_bias = nullptr;
     float* gemm_partial = nullptr;
     unsigned* gemm_tickets = nullptr;
+    int n_tickets = 0;                  // of them, those that every forward zeroes before its first GEMM
     __nv_bfloat16* xs_tmp = nullptr;    // three-term bf16 split of a GEMM's input rows (tensor-core path)
     float* ssq_tmp = nullptr;           // pieces of the rows' sums of squares written with it
     // activations handed from kernel to kernel in three-term form (tensor-core path)

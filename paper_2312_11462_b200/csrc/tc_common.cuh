@@ -131,11 +131,6 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// the split kernels (2D grid of 128-thread blocks) zero the tickets of a caller's scratch before the GEMM behind them
-__device__ __forceinline__ void clear_words(unsigned* words, int count) {
-    for (int i = (int)((blockIdx.y * gridDim.x + blockIdx.x) * 128 + threadIdx.x); i < count; i += (int)(gridDim.x * gridDim.y * 128)) words[i] = 0u;
-}
-
 __device__ __forceinline__ void red_release_gpu(unsigned* p, unsigned v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
