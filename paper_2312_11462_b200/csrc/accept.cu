@@ -434,6 +434,7 @@ resample_once_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         acc.p = warp_sum(acc.p);
         if (c.d) { acc.q = warp_sum(acc.q); acc.b = warp_sum(acc.b); }
         acc.a = warp_sum(acc.a);
+        __syncwarp();                                                        // (a lane's entry in list[0] before the mark there)
         if (lane == 0) {
             mine[chunk] = acc;
             if (listed > RS_LIST) list[0] = RS_FULL;
