@@ -9,8 +9,8 @@
 //   resample (temperature > 0 only) per row, at position n only, in fp64 so that the chosen token
 //            does not depend on summation order or on fp32 rounding: the sums of both laws'
 //            exponentials (the normalisers) and the mass of the residual max(0, p - q) (or of p after
-//            k acceptances), by a cluster of CTAs a row or, beyond V = 65536, by chunks in one pass, whose
-//            last one takes the inverse-CDF pick.  exp() here is a short fp64 routine of this file (exp_neg), and no
+//            k acceptances), by a cluster of CTAs a row or, beyond V = 65536, by chunks in one pass and
+//            a kernel that takes the inverse-CDF pick from their sums.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
 #include "model.cuh"
 #include "philox.cuh"
@@ -246,7 +246,7 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
         merge_stat_lanes<DC_LANES>(a, invT);
         if (i < nvec_row && l == 0) { s_mx[i] = a.mx; s_z[i] = a.sum; s_arg[i] = a.arg; }
     }
-    if (tid == 0 && tickets) { tickets[row] = 0u; tickets[rows + row] = 0u; }   // for the two resample passes
+    if (tid == 0 && tickets) tickets[row] = 0u;        // for the resample's CTAs of a row
     __syncthreads();
     RowInfo ri;
     ri.n = k; ri.mode = MODE_DONE; ri.x = 0; ri.pad = 0; ri.max_t = 0; ri.max_q = 0; ri.u2 = 0; ri.z_t = ri.z_q = 1.f;
@@ -290,16 +290,18 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 }
 
 // ---------------------------------------------------------------------------------------------
-// resample pass (fp64) of long vocabularies.  A WARP owns a chunk of a row (two sets of 512 logits, or eight where the scratch is small;
-// 8 neighbours a lane and load); no block-wide synchronisation.  The residual max(0, p - q) needs both normalisers, which are known
-// when every entry has been seen; but which entries it keeps is known before that for all but a few, from the fp32 sums of
-// the stats pass and a bound on their error.  So one pass sums, per chunk, both laws' exponentials (the normalisers) and, apart, those
-// of the entries that stay: a chunk's residual mass is then A Zq - B Zp, plus the few undecided entries, which are listed
-// and taken up when the normalisers are known (a chunk with more of them than its list holds is formed anew).  The warp that
-// finishes a row last does that and picks.  With a pass for the
-// normalisers and one for the masses (31 and 47 us at 64 rows, V = 128256) a call of 64 rows took k = 16 246.0 us, 233.2 so, k = 4
-// 123.6 and 107.2; 16 rows, k = 8 61.3 and 58.0.  (For rows up to V = 65536 the fused kernel below stays the faster one but for many
-// of them: 10 rows, k 8, V 50000 29.2 us, 37.6 by this pass; 64 rows, k 16, V 32000 77.7 and 76.6.)
+// resample passes (fp64) of long vocabularies: sums, then the pick.  In the first a WARP owns a chunk of a row (two sets of 512 logits,
+// or eight where the scratch is small; 8 neighbours a lane and load); no block-wide synchronisation.  The residual max(0, p - q) needs
+// both normalisers, which are known when every entry has been seen; but which entries it keeps is known before that for all but a
+// few, from the fp32 sums of the stats pass and a bound on their error.  So one pass sums, per chunk, both laws' exponentials (the
+// normalisers) and, apart, those of the entries that stay: a chunk's residual mass is then A Zq - B Zp, plus the few undecided
+// entries, which are listed and taken up by the second kernel; it reads a row's sums, not its logits, but for the chunk it picks
+// from and for chunks with more undecided entries than a list holds, which it forms anew.
+// Bound by the fp64 pipe (about 13 instructions an exponential).  Against a pass for the normalisers and one for the masses of all
+// entries (31 and 47 us at 64 rows, V = 128256), us a call: 64 rows, k = 16 245 -> 217, k = 4 122 -> 92; 16 rows, k 8, V 98315
+// 63.5 -> 45.0; 2 rows, k 15 38.6 -> 29.0.  Laws that nearly agree have full lists throughout (logits apart by 0.005 and less, 64 rows
+// 109 -> 106 to 112, 20 rows 54 -> 49 to 53): formed by one warp a row they took 1090 and 940, by the warps that had
+// summed them, staying for the normalisers, 187 and 96.  Three blocks an SM: with two, 64 rows, k = 16 222.
 // Every sum has one fixed order: a lane's entries, lanes by xor-shuffle or prefix scan, chunks in index order.
 // ---------------------------------------------------------------------------------------------
 constexpr int RS_SETS = 2;             // sets of 512 logits of a chunk (times 4 where the scratch is small)
@@ -338,6 +340,19 @@ struct ResidualCtx {
     double max_t, max_q, invT, Zp, Zq;
     int mode, x;
 };
+__device__ __forceinline__ ResidualCtx residual_ctx(const RowInfo& ri, int row, const float* tl, const float* dl, int k, int V, float temperature,
+                                                    const double* tab) {
+    ResidualCtx c;
+    c.t = tl + ((long long)row * (k + 1) + ri.n) * V;
+    c.d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
+    c.tab = tab;
+    c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature; c.Zp = c.Zq = 0.0;
+    c.mode = ri.mode; c.x = ri.x;
+    return c;
+}
+__device__ __forceinline__ bool residual_vec(const ResidualCtx& c, int V) {      // 16-byte loads
+    return (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
+}
 __device__ __forceinline__ double residual_of(const ResidualCtx& c, int e, float tv, float dv) {
     const double et = exp_neg(((double)tv - c.max_t) * c.invT, c.tab);
     const double ed = c.mode == MODE_RESID_LOGITS ? exp_neg(((double)dv - c.max_q) * c.invT, c.tab) : 0.0;
@@ -352,189 +367,221 @@ __device__ __forceinline__ double warp_scan(double v, int lane) {      // inclus
     }
     return v;
 }
-// one warp of a row's chunks has finished: true in the whole warp for the last of them
-__device__ __forceinline__ bool last_of_row(unsigned* ticket, int nchunk, int lane) {
-    unsigned old = 0;
-    if (lane == 0) {
-        __threadfence();
-        old = atomicAdd(ticket, 1u);
-    }
-    old = __shfl_sync(0xffffffffu, old, 0);
-    if (old != (unsigned)nchunk - 1u) return false;
-    __threadfence();
-    return true;
-}
-
-__global__ void __launch_bounds__(RS_THREADS, 2)
-resample_once_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
-                     const RowInfo* __restrict__ info, ChunkSums* sums, unsigned short* lists, unsigned* __restrict__ tickets,
-                     int nchunk, int sets, int* __restrict__ out_tok) {
+__global__ void __launch_bounds__(RS_THREADS, 3)
+resample_sums_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int rows, int k, int V, float temperature,
+                     const RowInfo* __restrict__ info, ChunkSums* __restrict__ sums, unsigned short* __restrict__ lists, int nchunk, int sets) {
     __shared__ double s_tab[64];
     exp_table_to_shared(s_tab);
     pdl_wait();            // the row records come from the decide pass
     pdl_trigger();
     const int lane = threadIdx.x & 31;
-    const long long item = (long long)blockIdx.x * (RS_THREADS / 32) + (threadIdx.x >> 5);
+    const long long item = (long long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int row = (int)(item / nchunk), chunk = (int)(item % nchunk);
     if (row >= rows) return;
     const RowInfo ri = info[row];
-    ResidualCtx c;
-    c.t = tl + ((long long)row * (k + 1) + ri.n) * V;
-    c.d = ri.mode == MODE_RESID_LOGITS ? dl + ((long long)row * k + ri.n) * V : nullptr;
-    c.max_t = ri.max_t; c.max_q = ri.max_q; c.invT = 1.0 / (double)temperature; c.Zp = c.Zq = 0.0;
-    c.mode = ri.mode; c.x = ri.x; c.tab = s_tab;
-    const bool vec = (V % 4 == 0) && ((((uintptr_t)c.t) & 15) == 0) && (!c.d || (((uintptr_t)c.d) & 15) == 0);
+    const ResidualCtx c = residual_ctx(ri, row, tl, dl, k, V, temperature, s_tab);
+    const bool vec = residual_vec(c, V);
+    unsigned short* list = lists + item * RS_LIST;
+    const float fT = 1.f / temperature, edge = c.d ? logf(ri.z_t) - logf(ri.z_q) : 0.f;   // stays: x_t - x_d > edge
+    const float mt = (float)ri.max_t, mq = (float)ri.max_q;
+    ChunkSums acc{0.0, 0.0, 0.0, 0.0};
+    int listed = 0;
+    float nt[8], nd[8];
+    load8(c.t, chunk * sets * RS_CHUNK + lane * 8, V, vec, nt);
+    if (c.d) load8(c.d, chunk * sets * RS_CHUNK + lane * 8, V, vec, nd);
+#pragma unroll 1
+    for (int half = 0; half < 2 * sets; ++half) {
+        const int at = (chunk * sets * 2 + half) * 256 + lane * 8;
+        float tv[8], dv[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { tv[j] = nt[j]; dv[j] = nd[j]; }
+        if (half + 1 < 2 * sets) {                                       // in flight while this half is summed
+            load8(c.t, at + 256, V, vec, nt);
+            if (c.d) load8(c.d, at + 256, V, vec, nd);
+        }
+        unsigned open = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const double et = exp_neg(((double)tv[j] - c.max_t) * c.invT, s_tab);         // -inf (past V) gives 0
+            acc.p += et;
+            if (c.d) {
+                const double ed = exp_neg(((double)dv[j] - c.max_q) * c.invT, s_tab);
+                acc.q += ed;
+                if (listed > RS_LIST) continue;                              // a full list: formed anew in any case
+                const float over = (tv[j] - mt) * fT - (dv[j] - mq) * fT - edge;
+                const float band = RS_BAND + 3e-7f * (fabsf((tv[j] - mt) * fT) + fabsf((dv[j] - mq) * fT));
+                const bool stays = over > band || dv[j] == -INFINITY;
+                acc.a += stays ? et : 0.0;
+                acc.b += stays ? ed : 0.0;
+                // (also what does not compare: both laws without the entry, not-a-number)
+                if (!stays && !(over < -band) && at + j < V && !(tv[j] == -INFINITY)) open |= 1u << j;
+            } else {
+                acc.a += at + j != c.x || c.mode != MODE_RESID_POINT ? et : 0.0;
+            }
+        }
+        while (listed <= RS_LIST && __any_sync(0xffffffffu, open != 0)) {     // rare
+            const unsigned who = __ballot_sync(0xffffffffu, open != 0);
+            const int place = listed + __popc(who & ((1u << lane) - 1u));
+            if (open && place < RS_LIST) list[place] = (unsigned short)(at + __ffs(open) - 1 - chunk * sets * RS_CHUNK);
+            open &= open - 1;
+            listed += __popc(who);
+        }
+    }
+    acc.p = warp_sum(acc.p);
+    if (c.d) { acc.q = warp_sum(acc.q); acc.b = warp_sum(acc.b); }
+    acc.a = warp_sum(acc.a);
+    __syncwarp();                                                        // (a lane's entry in list[0] before the mark there)
+    if (lane == 0) {
+        sums[item] = acc;
+        if (listed > RS_LIST) list[0] = RS_FULL;
+        else if (listed < RS_LIST) list[listed] = RS_NONE;
+    }
+}
+
+// mass of the residual of two laws over one chunk, by a warp
+__device__ __forceinline__ double chunk_mass(const ResidualCtx& c, int at, int end, int V, bool vec, int lane) {
+    double sr = 0.0;
+    float nt[8], nd[8];
+    load8(c.t, at + lane * 8, V, vec, nt);
+    load8(c.d, at + lane * 8, V, vec, nd);
+#pragma unroll 1
+    for (; at < end; at += 256) {
+        float tv[8], dv[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { tv[j] = nt[j]; dv[j] = nd[j]; }
+        if (at + 256 < end) {                                                // in flight while these are summed
+            load8(c.t, at + 256 + lane * 8, V, vec, nt);
+            load8(c.d, at + 256 + lane * 8, V, vec, nd);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sr += residual_of(c, at + lane * 8 + j, tv[j], dv[j]);
+    }
+    return warp_sum(sr);
+}
+
+// The normalisers, every chunk's mass into its b, the pick.  A row's first CTA does it, unless some of its chunks have full lists:
+// then all `per_row` CTAs of the row form those anew, a warp a chunk, and the last of them to finish does the rest.
+__global__ void __launch_bounds__(RS_THREADS, 3)
+resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int k, int V, float temperature,
+                     const RowInfo* __restrict__ info, ChunkSums* sums, const unsigned short* __restrict__ lists,
+                     unsigned* __restrict__ tickets, int nchunk, int sets, int per_row, int* __restrict__ out_tok) {
+    constexpr int WARPS = RS_THREADS / 32;
+    __shared__ double s_tab[64], s_warp[2 * WARPS];
+    __shared__ int s_int[2 * WARPS], s_chunk;
+    __shared__ double s_cum;
+    exp_table_to_shared(s_tab);
+    pdl_wait();            // the chunks' sums come from the pass before this one
+    pdl_trigger();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row = blockIdx.x / per_row, share = blockIdx.x % per_row;
+    const RowInfo ri = info[row];
+    ResidualCtx c = residual_ctx(ri, row, tl, dl, k, V, temperature, s_tab);
+    const bool vec = residual_vec(c, V);
+    const int len = sets * RS_CHUNK;                     // logits of a chunk
     ChunkSums* mine = sums + (long long)row * nchunk;
-    unsigned short* list = lists + ((long long)row * nchunk + chunk) * RS_LIST;
-    {
-        const float fT = 1.f / temperature, edge = c.d ? logf(ri.z_t) - logf(ri.z_q) : 0.f;   // stays: x_t - x_d > edge
-        const float mt = (float)ri.max_t, mq = (float)ri.max_q;
-        ChunkSums acc{0.0, 0.0, 0.0, 0.0};
-        int listed = 0;
-        float nt[8], nd[8];
-        load8(c.t, chunk * sets * RS_CHUNK + lane * 8, V, vec, nt);
-        if (c.d) load8(c.d, chunk * sets * RS_CHUNK + lane * 8, V, vec, nd);
-#pragma unroll 1
-        for (int half = 0; half < 2 * sets; ++half) {
-            const int at = (chunk * sets * 2 + half) * 256 + lane * 8;
-            float tv[8], dv[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) { tv[j] = nt[j]; dv[j] = nd[j]; }
-            if (half + 1 < 2 * sets) {                                       // in flight while this half is summed
-                load8(c.t, at + 256, V, vec, nt);
-                if (c.d) load8(c.d, at + 256, V, vec, nd);
-            }
-            unsigned open = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const double et = exp_neg(((double)tv[j] - c.max_t) * c.invT, s_tab);         // -inf (past V) gives 0
-                acc.p += et;
-                if (c.d) {
-                    const double ed = exp_neg(((double)dv[j] - c.max_q) * c.invT, s_tab);
-                    const float over = (tv[j] - mt) * fT - (dv[j] - mq) * fT - edge;
-                    const float band = RS_BAND + 3e-7f * (fabsf((tv[j] - mt) * fT) + fabsf((dv[j] - mq) * fT));
-                    const bool stays = over > band || dv[j] == -INFINITY;
-                    acc.q += ed;
-                    acc.a += stays ? et : 0.0;
-                    acc.b += stays ? ed : 0.0;
-                    // (also what does not compare: both laws without the entry, not-a-number)
-                    if (!stays && !(over < -band) && at + j < V && !(tv[j] == -INFINITY)) open |= 1u << j;
-                } else {
-                    acc.a += at + j != c.x || c.mode != MODE_RESID_POINT ? et : 0.0;
-                }
-            }
-            while (__any_sync(0xffffffffu, open != 0)) {                     // rare
-                const unsigned who = __ballot_sync(0xffffffffu, open != 0);
-                const int place = listed + __popc(who & ((1u << lane) - 1u));
-                if (open && place < RS_LIST) list[place] = (unsigned short)(at + __ffs(open) - 1 - chunk * sets * RS_CHUNK);
-                open &= open - 1;
-                listed += __popc(who);
-            }
-        }
-        acc.p = warp_sum(acc.p);
-        if (c.d) { acc.q = warp_sum(acc.q); acc.b = warp_sum(acc.b); }
-        acc.a = warp_sum(acc.a);
-        __syncwarp();                                                        // (a lane's entry in list[0] before the mark there)
-        if (lane == 0) {
-            mine[chunk] = acc;
-            if (listed > RS_LIST) list[0] = RS_FULL;
-            else if (listed < RS_LIST) list[listed] = RS_NONE;
-        }
-        __syncwarp();
+    auto words = [&](int ch) { return reinterpret_cast<const uint32_t*>(lists + ((long long)row * nchunk + ch) * RS_LIST); };
+    auto is_full = [&](int ch) { return c.d && (words(ch)[0] & 0xffffu) == RS_FULL; };
+    bool full = false;
+    double sp = 0.0, sq = 0.0;
+    for (int ch = tid; ch < nchunk; ch += RS_THREADS) {
+        full = full || is_full(ch);
+        sp += mine[ch].p; sq += mine[ch].q;
     }
-    if (!last_of_row(&tickets[row], nchunk, lane)) return;
-    // ---- the normalisers, then each chunk's mass into its b
-    {
-        double sp = 0.0, sq = 0.0;
-#pragma unroll 4
-        for (int ch = lane; ch < nchunk; ch += 32) { sp += __ldcg(&mine[ch].p); sq += __ldcg(&mine[ch].q); }
-        c.Zp = warp_sum(sp);
-        c.Zq = warp_sum(sq);
-    }
-    if (c.mode != MODE_TARGET_ONLY) {
-        // four chunks a lane at a time: their sums and lists are fetched together, then one listed entry of each
+    full = __syncthreads_or(full);
+    if (share != 0 && !full) return;
+    // ---- the normalisers (every CTA of the row adds the same numbers in the same order)
+    sp = warp_sum(sp); sq = warp_sum(sq);
+    if (lane == 0) { s_warp[warp] = sp; s_warp[WARPS + warp] = sq; }
+    __syncthreads();
+    sp = sq = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) { sp += s_warp[w]; sq += s_warp[WARPS + w]; }
+    c.Zp = sp; c.Zq = sq;
+    if (full) {
 #pragma unroll 1
-        for (int base = 0; base < nchunk; base += 128) {
-            double mass[4];
-            uint32_t words[4][RS_LIST / 2];
-            bool open[4], full[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int ch = min(base + 32 * u + lane, nchunk - 1);
-                const uint32_t* from = reinterpret_cast<const uint32_t*>(lists + ((long long)row * nchunk + ch) * RS_LIST);
-                const double a = __ldcg(&mine[ch].a), b = c.d ? __ldcg(&mine[ch].b) : 0.0;
-#pragma unroll
-                for (int w = 0; w < RS_LIST / 2; ++w) words[u][w] = c.d ? __ldcg(from + w) : 0xffffffffu;
-                mass[u] = c.d ? a * c.Zq - b * c.Zp : a;
-                full[u] = base + 32 * u + lane < nchunk && (words[u][0] & 0xffffu) == RS_FULL;
-                open[u] = base + 32 * u + lane < nchunk && !full[u];
+        for (int ch = share * WARPS + warp; ch < nchunk; ch += per_row * WARPS)
+            if (is_full(ch)) {
+                const double m = chunk_mass(c, ch * len, (ch + 1) * len, V, vec, lane);
+                if (lane == 0) __stcg(&mine[ch].b, m);
             }
-#pragma unroll
-            for (int i = 0; i < RS_LIST; ++i) {
-                float tv[4], dv[4];
-                int at[4];
-                bool any = false;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const unsigned e = (words[u][i / 2] >> (16 * (i & 1))) & 0xffffu;
-                    open[u] = open[u] && e != RS_NONE;
-                    at[u] = (base + 32 * u + lane) * sets * RS_CHUNK + (int)e;
-                    tv[u] = dv[u] = 0.f;
-                    if (open[u]) { tv[u] = c.t[at[u]]; dv[u] = c.d[at[u]]; any = true; }
-                }
-                if (!__any_sync(0xffffffffu, any)) break;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (open[u]) mass[u] += residual_of(c, at[u], tv[u], dv[u]);
+        if (per_row > 1) {
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                s_chunk = (int)atomicAdd(&tickets[row], 1u);
+                __threadfence();
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int ch = base + 32 * u + lane;
-                if (ch < nchunk && !full[u]) __stcg(&mine[ch].b, mass[u] > 0.0 ? mass[u] : 0.0);     // (rounding of the difference)
-                unsigned todo = __ballot_sync(0xffffffffu, full[u]);
-                while (todo) {                                               // a chunk of laws that nearly agree throughout
-                    const int ch2 = base + 32 * u + __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    double sr = 0.0;
-#pragma unroll 1
-                    for (int half = 0; half < 2 * sets; ++half) {
-                        const int at = (ch2 * sets * 2 + half) * 256 + lane * 8;
-                        float tv[8], dv[8];
-                        load8(c.t, at, V, vec, tv);
-                        load8(c.d, at, V, vec, dv);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) sr += residual_of(c, at + j, tv[j], dv[j]);
-                    }
-                    sr = warp_sum(sr);
-                    if (lane == 0) __stcg(&mine[ch2].b, sr);
-                }
-            }
+            __syncthreads();
+            if (s_chunk != per_row - 1) return;
         }
-        __threadfence_block();
-        __syncwarp();
     }
-    // ---- which chunk holds u2 * S: a lane owns neighbouring chunks; a second time with the target law itself if the
+    // ---- the other chunks' masses: a thread a chunk
+    if (c.mode != MODE_TARGET_ONLY)
+        for (int ch = tid; ch < nchunk; ch += RS_THREADS) {
+            if (is_full(ch)) continue;
+            double mass = mine[ch].a;
+            if (c.d) {
+                mass = mass * c.Zq - mine[ch].b * c.Zp;
+                float tv[RS_LIST], dv[RS_LIST];
+                int at[RS_LIST], n = 0;
+#pragma unroll
+                for (int i = 0; i < RS_LIST; ++i) {
+                    const unsigned e = (words(ch)[i / 2] >> (16 * (i & 1))) & 0xffffu;
+                    if (n == i && e != RS_NONE) { at[i] = ch * len + (int)e; tv[i] = c.t[at[i]]; dv[i] = c.d[at[i]]; n = i + 1; }
+                }
+#pragma unroll
+                for (int i = 0; i < RS_LIST; ++i)
+                    if (i < n) mass += residual_of(c, at[i], tv[i], dv[i]);
+            }
+            __stcg(&mine[ch].b, mass > 0.0 ? mass : 0.0);                    // (rounding of the difference)
+        }
+    __syncthreads();
+    // inclusive prefix over the CTA's threads; `total` of all
+    auto block_scan = [&](double v, double& total) {
+        const double in = warp_scan(v, lane);
+        __syncthreads();
+        if (lane == 31) s_warp[warp] = in;
+        __syncthreads();
+        double before = 0.0;
+        total = 0.0;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+            if (w == warp) before = total;
+            total += s_warp[w];
+        }
+        return before + in;
+    };
+    // ---- which chunk holds u2 * S: a thread owns neighbouring chunks; a second time with the target law itself if the
     //      residual is empty.  Rounding may leave none, then the last chunk that carries mass.
-    const int each = (nchunk + 31) / 32, c_lo = min(nchunk, lane * each), c_hi = min(nchunk, c_lo + each);
+    const int each = (nchunk + RS_THREADS - 1) / RS_THREADS, c_lo = min(nchunk, tid * each), c_hi = min(nchunk, c_lo + each);
     double own = 0.0, incl = 0.0, S = 0.0;
-    auto mass_of = [&](int ch) -> double { return c.mode == MODE_TARGET_ONLY ? __ldcg(&mine[ch].p) : __ldcg(&mine[ch].b); };
+    auto mass_of = [&](int ch) -> double { return c.mode == MODE_TARGET_ONLY ? mine[ch].p : __ldcg(&mine[ch].b); };
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
         own = 0.0;
-#pragma unroll 4
         for (int ch = c_lo; ch < c_hi; ++ch) own += mass_of(ch);
-        incl = warp_scan(own, lane);
-        S = __shfl_sync(0xffffffffu, incl, 31);
+        incl = block_scan(own, S);
         if (pass == 0 && c.mode != MODE_TARGET_ONLY && (!(S > 0.0) || !isfinite(S))) { c.mode = MODE_TARGET_ONLY; continue; }
         break;
     }
     const double target = ri.u2 * S;
-    const unsigned past = __ballot_sync(0xffffffffu, incl > target), some = __ballot_sync(0xffffffffu, own > 0.0);
-    const bool forced = past == 0;
-    const int src = past ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
-    double cum = incl - own;
-    int pick_chunk = c_lo;
-    if (lane == src) {
+    // first thread whose prefix exceeds the target, last thread with mass
+    auto first_last = [&](bool past, bool some, int& first, int& last) {
+        const unsigned a = __ballot_sync(0xffffffffu, past), z = __ballot_sync(0xffffffffu, some);
+        if (lane == 0) { s_int[warp] = a ? warp * 32 + __ffs(a) - 1 : -1; s_int[WARPS + warp] = z ? warp * 32 + 31 - __clz(z) : -1; }
+        __syncthreads();
+        first = last = -1;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+            if (first < 0) first = s_int[w];
+            if (s_int[WARPS + w] >= 0) last = s_int[WARPS + w];
+        }
+        __syncthreads();
+    };
+    int first, last;
+    first_last(incl > target, own > 0.0, first, last);
+    const bool forced = first < 0;
+    if (tid == (forced ? max(last, 0) : first)) {
+        double cum = incl - own;
         int last_pos = c_lo, hit = -1;
         for (int ch = c_lo; ch < c_hi; ++ch) {
             const double m = mass_of(ch);
@@ -547,40 +594,42 @@ resample_once_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
             cum = incl - own;
             for (int ch = c_lo; ch < last_pos; ++ch) cum += mass_of(ch);
         }
-        pick_chunk = hit;
+        s_chunk = hit; s_cum = cum;
     }
-    pick_chunk = __shfl_sync(0xffffffffu, pick_chunk, src);
-    cum = __shfl_sync(0xffffffffu, cum, src);
+    __syncthreads();
+    double cum = s_cum;
+    const int begin = s_chunk * len, end = min(V, begin + len);
     // ---- the entry: smallest index whose cumulative mass exceeds the target, else the last that carries mass
-    int pick = -1, last = -1;
+    int pick = -1, carries = -1;
 #pragma unroll 1
-    for (int e = pick_chunk * sets * RS_CHUNK; e < min(V, (pick_chunk + 1) * sets * RS_CHUNK) && pick < 0; e += 256) {
-        const int at = e + lane * 8;
-        float tv[8], dv[8];
-        load8(c.t, at, V, vec, tv);
-        if (c.mode == MODE_RESID_LOGITS) load8(c.d, at, V, vec, dv);
-        double r[8], local = 0.0;
+    for (int e = begin; e < end && pick < 0; e += RS_THREADS * 4) {
+        const int at = e + tid * 4;
+        double r[4], local = 0.0, total;
         int my_last = -1;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            r[j] = residual_of(c, at + j, tv[j], c.mode == MODE_RESID_LOGITS ? dv[j] : 0.f);
-            if (r[j] > 0.0) my_last = at + j;
+        for (int j = 0; j < 4; ++j) {
+            const bool in = at + j < end;
+            r[j] = in ? residual_of(c, at + j, c.t[at + j], c.mode == MODE_RESID_LOGITS ? c.d[at + j] : 0.f) : 0.0;
+            if (r[j] > 0.0) my_last = j;
             local += r[j];
         }
-        const double in = warp_scan(local, lane);
-        double run = cum + (in - local);
-        int found = 0x7fffffff;
+        double run = cum + (block_scan(local, total) - local);
+        int found = -1;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
             run += r[j];
-            if (!forced && found == 0x7fffffff && r[j] > 0.0 && run > target) found = at + j;
+            if (!forced && found < 0 && r[j] > 0.0 && run > target) found = j;
         }
-        found = __reduce_min_sync(0xffffffffu, found);
-        if (found != 0x7fffffff) pick = found;
-        last = max(last, __reduce_max_sync(0xffffffffu, my_last));
-        cum += __shfl_sync(0xffffffffu, in, 31);
+        first_last(found >= 0, my_last >= 0, first, last);
+        if (tid == first || tid == last) s_int[tid == first ? 0 : 1] = at + (tid == first ? found : my_last);
+        if (tid == first && tid == last) s_int[1] = at + my_last;
+        __syncthreads();
+        if (first >= 0) pick = s_int[0];
+        if (last >= 0) carries = s_int[1];
+        __syncthreads();
+        cum += total;
     }
-    if (lane == 0) out_tok[row] = pick >= 0 ? pick : max(last, 0);
+    if (tid == 0) out_tok[row] = pick >= 0 ? pick : max(carries, 0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1233,10 +1282,20 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
         ChunkSums* sums = (ChunkSums*)(ws + L.z_off);
         unsigned short* lists = (unsigned short*)(sums + (size_t)rows * nch);
         if ((size_t)rows * nch * (sizeof(ChunkSums) + RS_LIST * 2) > L.zsum_off - L.z_off) return CSD_ERR_UNSUPPORTED;   // (fewer than six chunks)
-        PdlLaunch lo(dim3((unsigned)(((long long)rows * nch + RS_THREADS / 32 - 1) / (RS_THREADS / 32))), dim3(RS_THREADS), 0, st);
-        CSD_CUDA(cudaLaunchKernelEx(&lo.cfg, resample_once_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, sums, lists,
-                                    tickets, nch, L.sets * RS_SETS, (int*)out_tok));
-        count_launch();
+        // warps a block: fewer while that leaves SMs without one (2 rows, k 15, V 128256 31.8 -> 29.2 us, 4 rows, k 16 34.8 -> 34.1)
+        int warps = RS_THREADS / 32;
+        while (warps > 1 && (long long)rows * nch < (long long)warps * accept_sm_count()) warps /= 2;
+        PdlLaunch lo(dim3((unsigned)(((long long)rows * nch + warps - 1) / warps)), dim3((unsigned)warps * 32), 0, st);
+        CSD_CUDA(cudaLaunchKernelEx(&lo.cfg, resample_sums_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, sums, lists, nch,
+                                    L.sets * RS_SETS));
+        // CTAs a row, for chunks that are formed anew: as many as fit at once, at least a chunk a warp.  (A chunk a warp at any number
+        // of rows: 64 rows of laws that nearly agree 106 -> 102 us, others, whose further CTAs leave at once, 217 -> 220.)
+        int per_row = (nch + RS_THREADS / 32 - 1) / (RS_THREADS / 32);
+        if ((long long)per_row * rows > 3 * accept_sm_count()) per_row = max(1, 3 * accept_sm_count() / rows);
+        PdlLaunch lp(dim3((unsigned)(rows * per_row)), dim3(RS_THREADS), 0, st);
+        CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, resample_pick_kernel, tl, dl, k, V, temperature, (const RowInfo*)info, sums, (const unsigned short*)lists,
+                                    tickets, nch, L.sets * RS_SETS, per_row, (int*)out_tok));
+        count_launch(2);
     }
     CSD_CUDA(cudaGetLastError());
     return CSD_OK;

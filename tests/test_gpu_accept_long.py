@@ -53,9 +53,36 @@ def laws_that_agree_but_for_one_entry(rows, V, each, seed):
     return torch.stack([t, t], 1).contiguous(), d[:, None].contiguous(), x.to(torch.int32)
 
 
-@pytest.mark.parametrize("each", [lambda c: 4 + c % 5, lambda c: c % 3, lambda c: 1024, lambda c: (0, 3, 7)[c % 3]],
-                         ids=["around-a-full-list", "few", "all", "mixed"])
-def test_undecided_entries(b, orc, each):
-    t, d, tok = laws_that_agree_but_for_one_entry(40, 66560, each, seed=3)
+@pytest.mark.parametrize("rows,each", [(40, lambda c: 4 + c % 5), (40, lambda c: c % 3), (40, lambda c: 1024), (40, lambda c: (0, 3, 7)[c % 3]),
+                                       (300, lambda c: 1024)],
+                         ids=["around-a-full-list", "few", "all", "mixed", "all, many waves of blocks"])
+def test_undecided_entries(b, orc, rows, each):
+    t, d, tok = laws_that_agree_but_for_one_entry(rows, 66560, each, seed=3)
     n, o = compare(b, orc, t, d, tok)
     assert n.mean() < 0.2 and len(set(o // 1024)) > 15           # the residual is drawn from all over the vocabulary
+
+
+def test_full_lists_do_not_stand_in_line(b):
+    """Chunks with full lists are formed anew by as many CTAs as fit, so such a call takes at most one more pass over the laws it has been
+    through twice.  (By one warp a row it took twelve to twenty times as long.)"""
+    V, rows = 66560, 20
+    near = laws_that_agree_but_for_one_entry(rows, V, lambda c: 1024, seed=4)
+    far = (near[0], near[0][:, :1] + 0.5 * torch.randn(rows, 1, V, device="cuda"), near[2])
+    out = tuple(torch.empty(rows, dtype=torch.int32, device="cuda") for _ in range(2))
+    ws = b.csd_spec_accept_workspace(rows, 1, V, "cuda")
+
+    def us(t, d, tok):
+        best = []
+        for _ in range(7):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            for _ in range(20):
+                b.csd_spec_accept(t, d, tok, 1.0, seed=7, step=3, workspace=ws, out=out)
+            end.record()
+            end.synchronize()
+            best.append(start.elapsed_time(end) / 20 * 1e3)
+        return sorted(best)[3]
+
+    a, c = us(*near), us(*far)
+    print("us", a, c)
+    assert a < 3 * c, (a, c)
