@@ -12,6 +12,7 @@
 //            k acceptances), by a cluster of CTAs a row or, beyond V = 65536, by chunks in one pass and
 //            a kernel that takes the inverse-CDF pick from their sums.  exp() here is a short fp64 routine of this file (exp_neg), and no
 //            law is normalised: every comparison is made on products instead of quotients.
+#include "accept_layout.cuh"
 #include "model.cuh"
 #include "philox.cuh"
 #include <math.h>
@@ -20,30 +21,10 @@
 namespace csd {
 
 constexpr int ST_THREADS = 256;
-constexpr int ST_CHUNK = 8192;   // logits per warp item of the stats pass
 constexpr int ST_SUB = 1024;     // logits a warp has in registers at a time (8 x float4 per lane)
 constexpr int RS_THREADS = 256;
-constexpr int RS_CHUNK = 512;    // logits per warp of the resample passes: 8 neighbours a lane, twice
-
-struct __align__(16) StatPartial {
-    float mx;
-    float sum;   // sum exp((x - mx) * invT) over the piece
-    int arg;     // smallest index attaining mx
-    int pad;
-};
 
 enum : int { MODE_DONE = 0, MODE_RESID_LOGITS = 1, MODE_RESID_POINT = 2, MODE_TARGET_ONLY = 3 };
-
-struct __align__(16) RowInfo {
-    int n;        // first rejected position (k if none)
-    int mode;
-    int x;        // drafted token at position n (point-mass / validation)
-    int pad;
-    double max_t; // max target logit at position n
-    double max_q; // max draft logit at position n
-    double u2;    // resampling uniform
-    float z_t, z_q;   // sums of the exponentials at position n as the stats pass has them (fp32)
-};
 
 // ---------------------------------------------------------------------------------------------
 // stats pass: grid-stride loop of warps over (vector, piece) items
@@ -304,14 +285,11 @@ accept_decide_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 // summed them, staying for the normalisers, 187 and 96.  Three blocks an SM: with two, 64 rows, k = 16 222.
 // Every sum has one fixed order: a lane's entries, lanes by xor-shuffle or prefix scan, chunks in index order.
 // ---------------------------------------------------------------------------------------------
-constexpr int RS_SETS = 2;             // sets of 512 logits of a chunk (times 4 where the scratch is small)
-constexpr int RS_LIST = 6;             // undecided entries a chunk can list
 constexpr unsigned short RS_NONE = 0xffff, RS_FULL = 0xfffe;
 // Distance of the laws' logarithms within which an entry is undecided.  The fp32 sums are off by at most the terms' own errors (2 ulp
 // of __expf, 1.2 more for each unit of the exponent, whose mean under a law is below ln V) and 300 roundings: 2e-5 each; the
 // comparison itself by 2^-23 of the exponents.
 constexpr float RS_BAND = 5e-5f;
-struct ChunkSums { double p, q, a, b; };   // all entries' exponentials of both laws; those of the entries that stay; later b: the mass
 
 // eight consecutive logits of a vector (two 16-byte loads when the vector allows it); past V: -inf
 __device__ __forceinline__ void load8(const float* __restrict__ src, int e0, int V, bool vec, float (&v)[8]) {
@@ -1052,36 +1030,13 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
 }
 
-struct AcceptLayout {
-    size_t part_off, info_off, z_off, zsum_off, r_off, ticket_off, total;
-    int nchunk_a, nchunk_r, sets;
-};
-
-static AcceptLayout accept_layout(int rows, int k, int V, int sets = 1) {
-    AcceptLayout L;
-    L.nchunk_a = (V + ST_CHUNK - 1) / ST_CHUNK;
-    L.nchunk_r = (int)(((long long)V + sets * RS_CHUNK - 1) / (sets * RS_CHUNK));
-    L.sets = sets;
-    size_t nvec = (size_t)rows * (2 * (size_t)k + 1);
-    size_t off = 0;
-    L.part_off = off;   off = align_up(off + nvec * L.nchunk_a * sizeof(StatPartial), 256);
-    L.info_off = off;   off = align_up(off + (size_t)rows * sizeof(RowInfo), 256);
-    L.z_off = off;      off = align_up(off + (size_t)rows * L.nchunk_r * sizeof(double2), 256);
-    L.r_off = off;      off = align_up(off + (size_t)rows * L.nchunk_r * sizeof(double), 256);
-    L.zsum_off = off;   off = align_up(off + (size_t)rows * sizeof(double2), 256);
-    L.ticket_off = off; off = align_up(off + 2 * (size_t)rows * sizeof(unsigned), 256);   // normaliser pass, mass pass
-    L.total = off;
-    return L;
-}
-
-// The layout for `room` bytes of scratch: 24 bytes per row and 512 logits for the resample's sums and lists (44 bytes a chunk of
-// 1024) where that fits, else per 2048.  (V = 128256: 64 rows, k = 4 107 / 125 us a call, k = 16 233 / 250; 320 rows, k = 1 244 / 241.)
+// The layout for `room` bytes of scratch: chunks of 1024 logits for the resample where that holds them, else of 4096.  (V = 128256: 64 rows, k = 4 107 / 125 us a call, k = 16 233 / 250; 320 rows, k = 1 244 / 241.)
 static csd_status accept_layout_in(int rows, int k, int V, size_t room, AcceptLayout& L) {
     const AcceptLayout least = accept_layout(rows, k, V, 4);
     if (room < least.total) return CSD_ERR_CAPACITY;
-    if (least.nchunk_r > 65535) return CSD_ERR_UNSUPPORTED;
+    if (least.pieces > 65535) return CSD_ERR_UNSUPPORTED;
     L = accept_layout(rows, k, V);
-    if (room < L.total || L.nchunk_r > 65535) L = least;
+    if (room < L.total || L.pieces > 65535) L = least;
     return CSD_OK;
 }
 
@@ -1278,23 +1233,22 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
                                     (int*)out_tok));
         count_launch();
     } else if (!greedy) {
-        const int nch = (L.nchunk_r + RS_SETS - 1) / RS_SETS;     // chunks of twice the layout's
-        ChunkSums* sums = (ChunkSums*)(ws + L.z_off);
-        unsigned short* lists = (unsigned short*)(sums + (size_t)rows * nch);
-        if ((size_t)rows * nch * (sizeof(ChunkSums) + RS_LIST * 2) > L.zsum_off - L.z_off) return CSD_ERR_UNSUPPORTED;   // (fewer than six chunks)
+        const int nch = L.chunks;
+        ChunkSums* sums = (ChunkSums*)(ws + L.sums_off);
+        unsigned short* lists = (unsigned short*)(ws + L.lists_off);
         // warps a block: fewer while that leaves SMs without one (2 rows, k 15, V 128256 31.8 -> 29.2 us, 4 rows, k 16 34.8 -> 34.1)
         int warps = RS_THREADS / 32;
         while (warps > 1 && (long long)rows * nch < (long long)warps * accept_sm_count()) warps /= 2;
         PdlLaunch lo(dim3((unsigned)(((long long)rows * nch + warps - 1) / warps)), dim3((unsigned)warps * 32), 0, st);
         CSD_CUDA(cudaLaunchKernelEx(&lo.cfg, resample_sums_kernel, tl, dl, rows, k, V, temperature, (const RowInfo*)info, sums, lists, nch,
-                                    L.sets * RS_SETS));
+                                    L.sets));
         // CTAs a row, for chunks that are formed anew: as many as fit at once, at least a chunk a warp.  (A chunk a warp at any number
         // of rows: 64 rows of laws that nearly agree 106 -> 102 us, others, whose further CTAs leave at once, 217 -> 220.)
         int per_row = (nch + RS_THREADS / 32 - 1) / (RS_THREADS / 32);
         if ((long long)per_row * rows > 3 * accept_sm_count()) per_row = max(1, 3 * accept_sm_count() / rows);
         PdlLaunch lp(dim3((unsigned)(rows * per_row)), dim3(RS_THREADS), 0, st);
         CSD_CUDA(cudaLaunchKernelEx(&lp.cfg, resample_pick_kernel, tl, dl, k, V, temperature, (const RowInfo*)info, sums, (const unsigned short*)lists,
-                                    tickets, nch, L.sets * RS_SETS, per_row, (int*)out_tok));
+                                    tickets, nch, L.sets, per_row, (int*)out_tok));
         count_launch(2);
     }
     CSD_CUDA(cudaGetLastError());
