@@ -38,6 +38,7 @@ constexpr int WG_THREADS = 384;              // one control warpgroup, two epilo
 constexpr int WG_REGS_CTL = 72, WG_REGS_EPI = 216;
 constexpr int WG_ROWS = 256;                 // weight rows of a pair's tile
 constexpr int WG_DRAIN = 8;                  // K blocks per accumulator set before it is added into registers
+constexpr int WG_MAX_PARTS = 8;              // most parts of K a tile goes by
 constexpr int WG_SET = 256;                  // tensor-memory columns of a set
 
 struct __align__(8) WgCtrl {
@@ -95,7 +96,7 @@ static WgPlan wg_plan(int m, int N, int K, bool dual) {
     p.pk = 1; p.gran = 1;
     const int ratio = P / p.tiles;
     if (!dual && ratio >= 2 && p.nkb >= 16) {
-        p.pk = ratio < 8 ? ratio : 8;
+        p.pk = ratio < WG_MAX_PARTS ? ratio : WG_MAX_PARTS;
         if (p.pk > p.nkb / 8) p.pk = p.nkb / 8;
         p.pairs = p.tiles * p.pk;
         return p;
@@ -129,8 +130,9 @@ size_t wide_partial_bytes(int m) {
 int wide_ticket_count(int m, int N) {
     const int half = WG_ROWS / 2;
     const int a = ((N + WG_ROWS - 1) / WG_ROWS) * ((m + 127) / 128), b = ((N + half - 1) / half) * ((m + 255) / 256);
-    const int tiles = a > b ? a : b, pairs = tc_sm_count() / 2;     // two words a tile, or a pair where tiles go by parts
-    return 2 * (tiles > pairs ? tiles : pairs);
+    const int tiles = a > b ? a : b, pairs = tc_sm_count() / 2;
+    const int parts = WG_MAX_PARTS * tiles < pairs ? WG_MAX_PARTS * tiles : pairs;      // most pairs where tiles go by parts
+    return 2 * (tiles > parts ? tiles : parts);                                         // two words a tile, or a pair
 }
 
 struct WgParams {

@@ -56,6 +56,14 @@ def test_wide_buffers_share_what_is_never_live_together(b):
     assert total - caches < rows + 3 * rows + 2 * rows + 74 * 256 * 256 * 4 + 16e6
 
 
+@pytest.mark.parametrize("m,N,K,asked", [(18, 1, 512, 2970368), (18, 56, 4096, 5724416), (64, 57, 1024, 3363840), (128, 120, 4096, 5724672),
+                                         (100, 139, 11008, 27859200)])
+def test_linear_scratch_of_narrow_matrices(b, m, N, K, asked):
+    """Callers that keep their scratch keep its size: the tickets of a wide block, which lie in the room of those of a CUDA-core launch
+    (a word per output), must not ask for more than that."""
+    assert b.lib.csd_linear_workspace_bytes(m, N, K) == asked
+
+
 def test_config_validation(b):
     s = workloads.SHAPES["tiny_target"]
     cfg = b.config_from_shape(s)

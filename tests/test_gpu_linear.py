@@ -149,3 +149,20 @@ def test_smallest_wide_blocks_sum_like_fp32(m, N, K):
     full = (hi.double() + lo.double()) @ W.double().T
     assert float((b.csd_linear(W, X).double() - full).norm() / full.norm()) < 7e-7
     assert b.csd_device_status() == 0
+
+
+@pytest.mark.parametrize("m,N,K", [(18, 64, 16384), (128, 120, 11008), (33, 139, 8192), (100, 57, 20480)])
+def test_narrow_wide_blocks(m, N, K):
+    """One tile by up to eight parts of K, in scratch of the asked size and with nothing touched behind it."""
+    require_gpu()
+    from paper_2312_11462_b200 import binding as b
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    W = (0.05 * torch.randn(N, K, generator=g, device="cuda")).to(torch.bfloat16)
+    X = torch.randn(m, K, generator=g, device="cuda")
+    full = X.double() @ W.double().T
+    n = b.lib.csd_linear_workspace_bytes(m, N, K)
+    room = torch.full((n + 4096,), 0x5a, dtype=torch.uint8, device="cuda")
+    assert float((b.csd_linear(W, X, room[:n]).double() - full).norm() / full.norm()) < 3e-5
+    assert (room[n:] == 0x5a).all()
+    assert b.csd_device_status() == 0
