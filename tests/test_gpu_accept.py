@@ -121,7 +121,7 @@ def test_distribution_on_tiny_vocab(b, orc):
 
 @pytest.mark.parametrize("rows,k,V,sigma", [(3, 2, 131076, 0.5), (64, 4, 128256, 0.1), (64, 1, 200003, 2.0), (5, 0, 150000, 0.5)])
 def test_scratch_for_longer_chunks_only(b, orc, rows, k, V, sigma):
-    """A workspace that holds a quarter of the resample passes' chunk sums: chunks of 2048 logits instead of 512, the same law."""
+    """A workspace that holds a quarter of the resample passes' chunk sums: chunks of 4096 logits instead of 1024, the same law."""
     t, d, tok = workloads.accept_case(rows, k, V, sigma, seed=rows + k, device="cuda")
     full = b.lib.csd_spec_accept_workspace_bytes(rows, k, V)
     short = full - 24 * rows * (-(-V // 512) - -(-V // 2048)) + 1024        # (1024: the parts start on 256-byte boundaries)

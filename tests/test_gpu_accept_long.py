@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import workloads
 from gpu_util import require_gpu
 
 pytestmark = pytest.mark.gpu
@@ -86,3 +87,59 @@ def test_full_lists_do_not_stand_in_line(b):
     a, c = us(*near), us(*far)
     print("us", a, c)
     assert a < 3 * c, (a, c)
+
+
+@pytest.mark.parametrize("V", [65537, 66559, 66560, 66561, 69631, 69632, 69633])
+@pytest.mark.parametrize("rows,k", [(150, 1), (1, 16)])
+def test_chunk_edges(b, orc, V, rows, k):
+    """One more and one less logit than whole chunks of 1024 and 4096; many rows, and so few that blocks are smaller."""
+    t, d, tok = workloads.accept_case(rows, k, V, 0.5, seed=V + rows, device="cuda")
+    compare(b, orc, t, d, tok)
+
+
+def masked(law, rows, k, V):
+    """A block whose target law, draft law or both leave entries out."""
+    t, d, tok = workloads.accept_case(rows, k, V, 0.5, seed=V, device="cuda")
+    every = torch.arange(V, device="cuda")
+    x = torch.full_like(tok, V - 3)
+    if law == "target":
+        t[:, :, every % 3 != 0] = float("-inf")
+    elif law == "draft":
+        d[:, :, every % 3 != 0] = float("-inf")
+        tok = tok // 3 * 3
+    elif law == "both":
+        t[:, :, every % 2 == 0] = float("-inf")
+        d[:, :, every % 3 != 0] = float("-inf")
+        tok = tok // 3 * 3
+    elif law == "apart":                                     # no entry in common: all of the target's stay
+        t[:, :, every % 2 == 0] = float("-inf")
+        d[:, :, every % 2 == 1] = float("-inf")
+        tok = tok // 2 * 2
+    elif law == "one entry":                                 # the whole draft law on an entry that the target has, or has not
+        d.fill_(float("-inf"))
+        d.scatter_(2, x[..., None].long(), 0.0)
+        t[::2, :, V - 3] = float("-inf")
+        tok = x
+    elif law == "chunks":                                    # whole chunks without an entry, the ends among them
+        t[:, :, (every // 4096) % 3 == 0] = float("-inf")
+        t[:, :, 65000:] = float("-inf")
+    elif law == "near":                                      # laws that nearly agree on half of the vocabulary, which both leave otherwise out
+        d = t[:, :k] + 1e-6 * torch.randn(d.shape, device="cuda")
+        low = t[:, :k].argmin(-1, keepdim=True)
+        d.scatter_add_(2, low, torch.full_like(low, 4.0, dtype=torch.float32))
+        gone = (every % 2 == 0)[None, None].expand(rows, k, V) & (every[None, None] != low)
+        t[:, :k][gone], d[gone] = float("-inf"), float("-inf")
+        tok = low[..., 0].to(torch.int32)
+    return t.contiguous(), d.contiguous(), tok.contiguous()
+
+
+@pytest.mark.parametrize("V", [70001, 131584])
+@pytest.mark.parametrize("law", ["target", "draft", "both", "apart", "one entry", "chunks", "near"])
+def test_masked_laws(b, orc, law, V):
+    rows, k = 12, 2
+    t, d, tok = masked(law, rows, k, V)
+    compare(b, orc, t, d, tok)
+    compare(b, orc, t, d, tok, 0.7)
+    # some positions drafted by a statistical model: point masses beside laws
+    on = (torch.arange(rows * k, device="cuda").reshape(rows, k) % 3 == 0).to(torch.int32)
+    compare(b, orc, t, d, tok, onehot=on)

@@ -1,5 +1,5 @@
 """Accept calls that take the passes (more rows or longer vectors than the one-kernel form holds): sizes
-at the edges of their pieces (8192 logits) and resample chunks (512; 2048 where the scratch is small), the most drafts, scratch
+at the edges of their pieces (8192 logits) and, beyond 65536, of the resample chunks (1024), the most drafts, scratch
 that holds anything, masked and empty laws, and calls that follow one another on a stream, against the oracle."""
 import pytest
 import torch
@@ -70,7 +70,7 @@ def test_scratch_that_holds_anything_and_calls_in_a_row(b):
 @pytest.mark.parametrize("sigma", [0.0, 1e-5, 1e-3, 0.03, 0.5])
 def test_laws_that_nearly_agree(b, orc, V, sigma):
     """Long vocabularies: the entries the residual keeps are told before the normalisers are known but where the laws nearly agree
-    (within 5e-5 of their logarithms); those are listed, six a chunk of 1024, and chunks with more are summed anew.  Two entries
+    (within 5e-5 of their logarithms); those are listed, six a chunk of 1024, and chunks with more are formed anew.  Two entries
     of each draft law are swapped, the drafted one gaining, so that it is refused while all others agree up to sigma."""
     rows, k = 20, 2
     t, _, _ = workloads.accept_case(rows, k, V, 0.5, seed=V, device="cuda")

@@ -113,7 +113,7 @@ def test_workspaces_that_hold_anything(orc):
 
 @pytest.mark.parametrize("m,N,K", [(18, 1536, 1024), (128, 2304, 1536), (64, 4096, 4096), (33, 4099, 520)])
 def test_wide_blocks_into_any_address(m, N, K):
-    """A result that starts on a 4-byte boundary only (K parts then go through shares instead of planes)."""
+    """A result that starts on a 4-byte boundary only: parts of K as elsewhere, without 16-byte accesses to the result."""
     require_gpu()
     from paper_2312_11462_b200 import binding as b
     g = torch.Generator(device="cuda")

@@ -1,4 +1,4 @@
-"""Wide passes whose output and down projections are too large for planes: pairs that take whole tiles and pairs that share tiles,
+"""Wide passes of 257 tokens and more: output and down projections by parts of K, pairs that take whole tiles and pairs that share tiles,
 each with the residual add, the two-term rows times a gain and the sums of squares in the GEMM's own epilogue, and the
 gated pair in both of its forms, over two layers.  Whole reviews against the oracle; and the second layer's cached values against
 fp64, entry by entry, from the first layer's cached keys and values on."""
@@ -12,12 +12,14 @@ from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, rel_l2, require_gpu, to_dev_i3
 
 pytestmark = pytest.mark.gpu
 
-# d_model, heads, d_ff, prompts.  Pairs of CTAs: 74; a tile is 256 output rows x up to 256 tokens, the gated pair's 128 above 128 tokens.
+# d_model, heads, d_ff, prompts.  Pairs of CTAs: 74; a tile is 256 output rows x up to 256 tokens, the gated pair's 128 above 64 tokens.
 SHAPES = {
-    # the 7B width: o and down 32 to 48 tiles in equal shares, gate and up 172 to 258
+    # the 7B width: o and down 32 tiles by two parts of K each, at 700 tokens 48 in equal shares; gate and up 172 to 258
     "7b": (llama_shape(2, 4096, 32, 11008, 500, 720), (257, 300, 700)),
-    # o and down of 17 row tiles of which the last is a quarter full (34 tiles, shares); gate and up end inside a tile
+    # o and down of 17 row tiles of which the last is a quarter full (34 tiles, two parts of K each); gate and up end inside a tile
     "ragged": (llama_shape(2, 4160, 65, 1416, 500, 320), (257, 300)),
+    # the same 17 row tiles by three token tiles, the last of them not full: 51 tiles in equal shares
+    "ragged shares": (llama_shape(2, 4160, 65, 2824, 500, 620), (600,)),
     # o and down of 72 tiles for 74 pairs: whole tiles
     "whole": (llama_shape(2, 4608, 36, 1416, 500, 800), (780,)),
 }
