@@ -638,6 +638,9 @@ __device__ __forceinline__ double cluster_read_f64(const double* local, uint32_t
     return v;
 }
 
+// ALONE: a row of one CTA, which exchanges with nobody (barriers of a cluster of one and reads through its window: 200 rows, k 1,
+// V 512 24.8 us a call, 21.9 so; asked at run time, larger clusters lose 1 to 2 %)
+template <bool ALONE>
 __global__ void __launch_bounds__(RF_THREADS, 1)
 resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl, int k, int V, float temperature,
                       const RowInfo* __restrict__ info, int csize, int* __restrict__ out_tok) {
@@ -650,6 +653,8 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
     __shared__ double s_warp[2 * RF_WARPS], s_ex[4];  // s_ex: this CTA's contributions to the exchanges
     __shared__ double s_tab[64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto sync_row = [] { if (ALONE) __syncthreads(); else cluster_sync_all(); };
+    auto read_of = [](const double* p, uint32_t r) { return ALONE ? *p : cluster_read_f64(p, r); };
     exp_table_to_shared(s_tab);
     const double invT = 1.0 / (double)temperature;
     const float* t = tl + ((long long)row * (k + 1) + ri.n) * V;
@@ -699,10 +704,10 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
         const double a = half_sum(s_warp[lane]);
         if (lane % RF_WARPS == 0) s_ex[lane / RF_WARPS] = a;
     }
-    cluster_sync_all();
+    sync_row();
     double Zp, Zq;
     {
-        const double a = half_sum(lane % RF_WARPS < csize ? cluster_read_f64(&s_ex[lane / RF_WARPS], (uint32_t)(lane % RF_WARPS)) : 0.0);
+        const double a = half_sum(lane % RF_WARPS < csize ? read_of(&s_ex[lane / RF_WARPS], (uint32_t)(lane % RF_WARPS)) : 0.0);
         Zp = __shfl_sync(0xffffffffu, a, 0); Zq = __shfl_sync(0xffffffffu, a, RF_WARPS);
     }
     const int xn = ri.x;
@@ -722,8 +727,8 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
         __syncthreads();
         run = warp_scan(lane < RF_WARPS ? s_warp[lane] : 0.0, lane);
         if (threadIdx.x == RF_WARPS - 1) s_ex[2 + pass] = run;
-        cluster_sync_all();
-        const double m = lane < csize ? cluster_read_f64(&s_ex[2 + pass], (uint32_t)lane) : 0.0;
+        sync_row();
+        const double m = lane < csize ? read_of(&s_ex[2 + pass], (uint32_t)lane) : 0.0;
         const double incl = warp_scan(m, lane), total = __shfl_sync(0xffffffffu, incl, csize - 1);
         if (pass == 0 && mode != MODE_TARGET_ONLY && (!(total > 0.0) || !isfinite(total))) { mode = MODE_TARGET_ONLY; continue; }
         // the CTA whose masses reach past u2 * total; rounding may leave none, then the last one that carries mass
@@ -735,7 +740,7 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
         head = __shfl_sync(0xffffffffu, incl - m, (int)rank);
         break;
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has read what it needs of the others
+    if (!ALONE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has read what it needs of the others
     if ((int)rank == owner) {
         // ---- in it the warp, then the entry: the smallest index whose cumulative mass exceeds the target; forced, or where
         //      rounding leaves none: the last entry that carries mass
@@ -744,7 +749,7 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
         const int wpick = past && !forced ? __ffs(past) - 1 : (some ? 31 - __clz(some) : 0);
         const double before = __shfl_sync(0xffffffffu, run, (wpick + 31) & 31);
         if (warp == wpick) {
-                double cum = head + (wpick > 0 ? before : 0.0) + (warp_scan(local, lane) - local);
+            double cum = head + (wpick > 0 ? before : 0.0) + (warp_scan(local, lane) - local);
             int found = 0x7fffffff, my_last = -1;
 #pragma unroll
             for (int j = 0; j < RF_PER; ++j) {
@@ -758,7 +763,7 @@ resample_fused_kernel(const float* __restrict__ tl, const float* __restrict__ dl
             if (lane == 0) out_tok[row] = found != 0x7fffffff ? found : max(my_last, 0);
         }
     }
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
+    if (!ALONE) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1082,7 +1087,7 @@ static bool fused_resample_ok(int csize) {
         attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int n = 0;
-        const bool ok = cudaOccupancyMaxActiveClusters(&n, resample_fused_kernel, &cfg) == cudaSuccess && n >= 1;
+        const bool ok = cudaOccupancyMaxActiveClusters(&n, csize == 1 ? resample_fused_kernel<true> : resample_fused_kernel<false>, &cfg) == cudaSuccess && n >= 1;
         if (!ok) (void)cudaGetLastError();
         return ok ? 1 : 0;
     }) == 1;
@@ -1229,7 +1234,7 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 2;
-        CSD_CUDA(cudaLaunchKernelEx(&cfg, resample_fused_kernel, tl, dl, k, V, temperature, (const RowInfo*)info, csize,
+        CSD_CUDA(cudaLaunchKernelEx(&cfg, csize == 1 ? resample_fused_kernel<true> : resample_fused_kernel<false>, tl, dl, k, V, temperature, (const RowInfo*)info, csize,
                                     (int*)out_tok));
         count_launch();
     } else if (!greedy) {
