@@ -619,7 +619,7 @@ resample_pick_kernel(const float* __restrict__ tl, const float* __restrict__ dl,
 // fixed order (lanes by xor-shuffle or prefix scan, warps and CTAs in index order).
 // ---------------------------------------------------------------------------------------------
 constexpr int RF_THREADS = 512, RF_WARPS = RF_THREADS / 32, RF_PER = 16, RF_SLICE = RF_THREADS * RF_PER;
-constexpr int RF_MAXC = 8;   // larger clusters run (one per GPC at a time) but lose to the two-pass kernels: 199 us against 145 at V = 128256
+constexpr int RF_MAXC = 8;   // (clusters of 16 run one per GPC at a time: 64 rows, k 4, V 128256 199 us a call; the passes take 92)
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -1035,7 +1035,8 @@ accept_row_kernel(const float* __restrict__ tl, const float* __restrict__ dl, co
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // no CTA leaves while its results may still be read
 }
 
-// The layout for `room` bytes of scratch: chunks of 1024 logits for the resample where that holds them, else of 4096.  (V = 128256: 64 rows, k = 4 107 / 125 us a call, k = 16 233 / 250; 320 rows, k = 1 244 / 241.)
+// The layout for `room` bytes of scratch: chunks of 1024 logits for the resample where that holds them, else of 4096.  (V = 128256: 64
+// rows, k = 4 92 / 104 us a call, k = 16 214 / 223; 320 rows, k = 1 196 / 207.)
 static csd_status accept_layout_in(int rows, int k, int V, size_t room, AcceptLayout& L) {
     const AcceptLayout least = accept_layout(rows, k, V, 4);
     if (room < least.total) return CSD_ERR_CAPACITY;
@@ -1225,7 +1226,10 @@ static csd_status run_accept(const float* tl, const float* dl_in, const int32_t*
     }
     count_launch(2);
     const int csize = (V + RF_SLICE - 1) / RF_SLICE;
-    if (!greedy && fused_resample_ok(csize)) {  // a row fits one cluster: the fused resample kernel
+    // A row that fits one cluster goes to the fused kernel.  Measured, fused / passes: 10 rows, k 8, V 50000 29.7 / 31.4 us a call, 20 rows 44.9
+    // / 39.5; 64 rows, k 16, V 32000 77.9 / 71.7, k 4 43.0 / 37.4; 64 rows, k 4, V 60000 75.9 / 54.5: since the passes end in a kernel
+    // of their own, the line lies too high.
+    if (!greedy && fused_resample_ok(csize)) {
         cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
         cudaLaunchAttribute attr[2];
         cfg.gridDim = dim3((unsigned)(rows * csize)); cfg.blockDim = dim3(RF_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;

@@ -321,7 +321,7 @@ size_t linear_scratch_bytes(int m, int N, int K, bool dual) {
 }
 
 // One per row group of at least one row (CUDA-core kernel); eight per 128-row tile (tensor-core kernel) are fewer.  The wide kernel's
-// (at most four per 128 rows and 256 tokens: wide_ticket_count) are looked after where its tickets are handed out.
+// (wide_ticket_count) are looked after where its tickets are handed out.
 int linear_ticket_count(int N) { return N + 8; }
 
 // The row kernel (automatic choice only).  Measured back to back, us for row / tensor-core / split-K CUDA-core kernel:

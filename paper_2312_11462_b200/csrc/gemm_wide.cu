@@ -62,6 +62,8 @@ static_assert(8 * 16 * 32 + 4 * WG_SET <= 2 * 8 * 16 * 32, "sums of squares fit 
 //            layer of 64 tokens met its rows 9.7 us after their end.  A layer of 64 / 128 / 256 tokens 133 -> 129, 160 -> 145,
 //            245 -> 235 us; two parts instead of shares: 512 tokens 454 -> 440, eight T5-xxl-shaped encoder layers of 128 1326 -> 1291.
 //            (Clusters of four pairs that add up through distributed shared memory: 15 of them are resident, for 16 tiles.)
+//            A tile's pairs wait for one another, so all of them must come to be resident: they are neighbours in a grid that is dispatched
+//            in order, so of a launch that shares the GPU at most one tile waits for places, which the tiles before it give back;
 //   whole    pair c takes whole tiles (no partial sums) where that leaves little of the last round empty;
 //   shares   otherwise the (tile, K block) units are dealt out in equal contiguous shares; a tile cut by a
 //            share boundary is finished by its first contributor from the partial sums the later
@@ -182,8 +184,7 @@ __device__ __forceinline__ unsigned wg_begin(unsigned c, unsigned units, unsigne
 
 // MODE 0: one matrix; 1: a gated pair, both matrices' 256 rows in a stage (up to 64 tokens); 2: a gated pair, the CTA's
 // 128 rows are 64 of the gate and the same 64 of the up matrix, so that the MMAs are up to 256 columns wide.  (An MMA reads
-// its 128 weight rows from shared memory whatever its width, and those reads, not the tensor pipe, set the pace of narrow ones:
-// gate and up of the 7B shape at 1000 tokens 323 us in mode 1, 277 in mode 2.)
+// its 128 weight rows from shared memory whatever its width, and those reads, not the tensor pipe, set the pace of narrow ones.)
 // MERGED (tiles of up to 128 tokens): one MMA multiplies both terms of the tile's tokens, 2 nt columns wide, the high terms'
 // sums in the first nt columns and the low terms' in the others; one CTA of the pair stages the high terms of all tokens, the
 // other the low ones.  An MMA of 256 x 64 takes little less time than one of 256 x 128, so two of them per term and K step set
