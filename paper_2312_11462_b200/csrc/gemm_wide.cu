@@ -20,8 +20,8 @@
 // 12288 (csd_linear, 18 to 128 rows, where the low terms' products have columns of their own): 2.50e-6, of which the two-term form
 // itself leaves 2.45e-6; both terms in one chain 2.7e-6.  Sets of 4 K blocks, which leave 2.5e-6 either way, cost 2 to 7 % a GEMM.
 //
-// Roles inside a CTA (384 threads): lane 0 of warps 0 and 2 issues TMA (weights, row terms), warp 1 lane 0 of the pair's first CTA
-// issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
+// Roles inside a CTA (384 threads): lane 0 of warp 0 issues TMA (up to 128 tokens and for parts of K lane 0 of warp 2 that of the row
+// terms), warp 1 lane 0 of the pair's first CTA issues the MMAs for both, warps 4-11 read tensor memory (two warps per quadrant, each half of the
 // tokens) and finish tiles; they hold 128 accumulators each, hence the register split.  Every
 // mbarrier wait is bounded; on a time-out the CTA records CSD_ERR_TIMEOUT, stops, frees its tensor
 // memory, returns.
@@ -158,7 +158,7 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* t
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y) : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_pair_keep(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y, uint64_t pol) {
+__device__ __forceinline__ void tma_load_2d_pair_hint(void* dst, const CUtensorMap* tm, uint32_t bar, int x, int y, uint64_t pol) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)tm), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
 }
@@ -259,47 +259,71 @@ wide_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             const int tile0 = (int)(u0 / p.nkb);
             return Cursor{(int)(u0 % p.nkb), tile0 / p.ntok, tile0 % p.ntok};
         };
-        if (warp == 0 && lane == 0) {
-            // ---- TMA producer of this CTA's weights; all copies of the pair complete on the first CTA's barriers
-            uint64_t keep;                                    // (other token tiles take the same weights from L2)
-            if (p.ntok > 1) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep));
-            else keep = policy_evict_first();
-            Cursor cur = first();
-            int s = 0;
-            uint32_t ph = 0;
-#pragma unroll 1
-            for (int i = 0; i < items && !*abort_flag; ++i) {
-                if (i >= p.stages && !mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
-                unsigned char* dst = ring + (size_t)s * stage_bytes;
-                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
-                if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
-                const int row = cur.row * OUT_ROWS + rank * (OUT_ROWS / 2);
-                tma_load_2d_pair_keep(dst, &tmW, bar, cur.kb * KB, row, keep);
-                if (DUAL) tma_load_2d_pair_keep(dst + STAGE_BYTES, &tmW2, bar, cur.kb * KB, row, keep);
-                if (MIXED) tma_load_2d_pair_keep(dst + STAGE_BYTES / 2, &tmW2, bar, cur.kb * KB, row, keep);
-                step(cur);
-                if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
+        // All copies of the pair complete on the first CTA's barriers.
+        auto load_w = [&](int s, const Cursor& c, uint64_t once) {
+            unsigned char* dst = ring + (size_t)s * stage_bytes;
+            const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+            if (rank == 0) mbar_expect_tx(&ctl->full[s], 2u * stage_bytes);
+            const int row = c.row * OUT_ROWS + rank * (OUT_ROWS / 2);
+            if (p.ntok == 1) {                                // no other token tile takes these weights from L2
+                tma_load_2d_pair_hint(dst, &tmW, bar, c.kb * KB, row, once);
+                if (DUAL) tma_load_2d_pair_hint(dst + STAGE_BYTES, &tmW2, bar, c.kb * KB, row, once);
+                if (MIXED) tma_load_2d_pair_hint(dst + STAGE_BYTES / 2, &tmW2, bar, c.kb * KB, row, once);
+            } else {
+                tma_load_2d_pair(dst, &tmW, bar, c.kb * KB, row);
+                if (DUAL) tma_load_2d_pair(dst + STAGE_BYTES, &tmW2, bar, c.kb * KB, row);
+                if (MIXED) tma_load_2d_pair(dst + STAGE_BYTES / 2, &tmW2, bar, c.kb * KB, row);
             }
-        } else if (warp == 2 && lane == 0) {
-            // ---- TMA producer of this CTA's half of the row terms, a warp of its own: three copies a stage from one thread
-            //      (about 100 ns each, with the wait before them) set the pace of tiles of up to 128 tokens
+        };
+        auto load_x = [&](int s, const Cursor& c) {           // this CTA's half of the row terms
+            unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
+            const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
+            if (MERGED) {
+                tma_load_2d_pair(dst, &tmX, bar, c.kb * KB, rank * p.mpad + c.tok * nt);
+            } else {
+                const int r = c.tok * nt + rank * htok;
+                tma_load_2d_pair(dst, &tmX, bar, c.kb * KB, r);
+                tma_load_2d_pair(dst + xterm, &tmX, bar, c.kb * KB, p.mpad + r);
+            }
+        };
+        // The row terms come from a warp of their own where a K block is short: three copies a stage from one thread (about 100 ns each,
+        // with the wait before them) set the pace of tiles of up to 128 tokens.  Full tiles whose weights several token tiles share gain
+        // nothing, and under the power limit a second thread and a cache hint cost: prompts of the 7B shape at 513 / 700 / 768 tokens
+        // +0.8 / +0.9 / +0.9 %, one thread +0.65 / +0.4 / +0.4, and no hint level.
+        constexpr bool TWO = MERGED || PARTS;
+        if (warp == 0 && lane == 0) {
+            // ---- TMA producer of this CTA's weights, or of all it stages
+            const uint64_t once = policy_evict_first();
+            Cursor cw = first(), cx = cw;
+            const int pre = items < p.stages ? items : p.stages;
+#pragma unroll 1
+            for (int i = 0; i < pre; ++i) { load_w(i, cw, once); step(cw); }
+            if (!TWO) {
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll 1
+                for (int i = 0; i < pre; ++i) { load_x(i, cx); step(cx); }
+            }
+            int s = 0;
+            uint32_t ph = 0;
+#pragma unroll 1
+            for (int i = pre; i < items && !*abort_flag; ++i) {
+                if (!mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
+                load_w(s, cw, once);
+                step(cw);
+                if (!TWO) { load_x(s, cx); step(cx); }
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+            }
+        } else if (TWO && warp == 2 && lane == 0) {
+            // ---- TMA producer of its row terms
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            Cursor cur = first();
+            Cursor cx = first();
             int s = 0;
             uint32_t ph = 0;
 #pragma unroll 1
             for (int i = 0; i < items && !*abort_flag; ++i) {
                 if (i >= p.stages && !mbar_wait(&ctl->empty[s], ph)) { *abort_flag = 1; break; }
-                unsigned char* dst = ring + (size_t)s * stage_bytes + WB;
-                const uint32_t bar = map_to_cta(smem_u32(&ctl->full[s]), 0u);
-                if (MERGED) {
-                    tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, rank * p.mpad + cur.tok * nt);
-                } else {
-                    const int r = cur.tok * nt + rank * htok;
-                    tma_load_2d_pair(dst, &tmX, bar, cur.kb * KB, r);
-                    tma_load_2d_pair(dst + xterm, &tmX, bar, cur.kb * KB, p.mpad + r);
-                }
-                step(cur);
+                load_x(s, cx);
+                step(cx);
                 if (++s == p.stages) { s = 0; if (i >= p.stages) ph ^= 1u; }
             }
         } else if (warp == 1 && rank == 0 && lane == 0) {
